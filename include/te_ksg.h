@@ -340,6 +340,11 @@ te_status te_ctx_set_trace(te_ctx *ctx, te_trace_fn fn, void *user);
 
 /* ---- execution options (tuning and measurement; the paper has no counterpart) --
  *
+ * KSG estimates run on neighbour lists wherever a member's X values fit a
+ * CTA's shared memory (dx * points up to about 41,000).  The member-lane
+ * kernel serves the rest, and every estimate of a context in which one of its
+ * own options (tile, members per lane, persistent, order) is set.
+ *
  * te_ctx_set_option sets one option of a context for its later calls:
  *   TE_OPT_KSG_TILE              points per staged tile of the member-lane KSG
  *                                kernel: 64, 128 or 256; 0 (default) = the
@@ -377,17 +382,19 @@ typedef struct {
     uint64_t estimates;       /* CMI estimates (members) evaluated */
     uint64_t launches;        /* kernel launches issued (all kernels of the library) */
     uint64_t pair_evals;      /* member x point-pair distance evaluations the KSG kernel
-                                 executed (both passes; pairs of skipped chunks excluded) */
+                                 executed (both passes; pairs of skipped chunks, or beyond
+                                 the lists' prefixes, excluded) */
     double kernel_ms;         /* summed device time of the KSG kernels (CUDA events on the
                                  context's stream) */
-    uint64_t ksg_launches;    /* launches of the fused KSG kernel */
+    uint64_t ksg_launches;    /* launches of the KSG kernel (the list walk, or the member-lane kernel) */
     uint64_t h2d_bytes;       /* bytes copied host -> device by the library */
     uint64_t d2h_bytes;       /* bytes copied device -> host by the library */
     uint64_t pair_evals_bruteforce; /* member x ordered point pairs x 2 passes: the work of
                                        the unpruned all-pairs estimator */
     uint64_t ksg_ops;         /* algorithmic ops of the executed evaluations: 3 per kNN-pass
                                  pair (subtract, max, compare), 7 per count-pass pair
-                                 (subtract, 3 compares, 3 increments) */
+                                 (subtract, 3 compares, 3 increments); on neighbour lists 3
+                                 per pair (a count is a subtract, a compare, an increment) */
 } te_stats;
 
 te_status te_get_stats(const te_ctx *ctx, te_stats *out);

@@ -1,0 +1,1187 @@
+// Neighbour lists for the KSG estimator (sm_103a).
+//
+// The members of a group (candidates x surrogates) share Y, Z and the points
+// and differ in X only.  So for every query point the points near it in (Y, Z)
+// and in Z are found once per group and kept as two sorted lists; each
+// member then needs only a prefix of them:
+//   list A, ascending d_YZ: the joint distance is max(d_X, d_YZ) >= d_YZ, so
+//     a member's k nearest joint distances are known as soon as the next d_YZ
+//     is not below its k-th smallest so far; n_yz is a rank in this list;
+//   list B, ascending d_Z: n_z is a rank in it, n_xz a count over the prefix
+//     with d_Z < eps.
+// A list holds every valid point below its radius and no other, so a result
+// is exact whenever the member's k-th distance is at most the radius; the few
+// (member, point) pairs beyond it scan all points.  Masked points (the point
+// itself, the Theiler band) are in no list.
+//
+// Per member and point the estimate needs the points inside eps only: 9 for
+// the neighbours and 21 for n_z with eight Z variables at N = 10^4, 38 and 229
+// with two, 71 and 781 with one, against 900 to 10,000 visited by tiles that
+// are pruned for 64 members at once.  Measured on one GB300, tiled member-lane
+// kernel -> lists, whole calls: 89 candidates x 201 members, 8 Z variables,
+// N = 9995: 274 -> 24.1 ms; 45 x 201, 2 Z: 105 -> 41 ms; one call of 201, 1 Z:
+// 5.7 -> 2.5 ms; 9 x 201, Theiler window 12, N = 2994: 9.8 -> 1.5 ms.
+#include <cuda_runtime.h>
+#include <math_constants.h>
+#include <stdint.h>
+
+#include <algorithm>
+#include <cmath>
+
+#include "ksg_lists.h"
+
+namespace teksg {
+
+namespace {
+
+constexpr int kBins = 1024;          // counting-sort bins per list
+constexpr int kSample = 1024;        // points sampled for a list's radius
+constexpr int kBuildWarps = kListBuildThreads / 32;
+constexpr unsigned kFull = 0xffffffffu;
+
+struct Entry {   // 64 bits: unsigned order is (distance, point) order (distances are >= 0)
+    uint32_t j;
+    float d;
+};
+
+__device__ __forceinline__ uint64_t entry_key(Entry e)
+{
+    return ((uint64_t)__float_as_uint(e.d) << 32) | e.j;
+}
+
+template <typename F>
+__device__ __forceinline__ int last_at_or_below(int n, long long item, F first)
+{
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (first(mid) <= item) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+struct RowPtrs {
+    ListNear *near;
+    float *skip, *d_a, *d_b;
+    uint32_t *j_a, *j_b;
+};
+
+__device__ __forceinline__ RowPtrs row_ptrs(unsigned char *rows, int row, int cap_a, int cap_b)
+{
+    RowPtrs r;
+    unsigned char *p = rows + (size_t)row * list_row_bytes(cap_a, cap_b);
+    r.near = reinterpret_cast<ListNear *>(p);
+    r.skip = reinterpret_cast<float *>(p + sizeof(ListNear));
+    r.d_a = r.skip + kListSkip;
+    r.j_a = reinterpret_cast<uint32_t *>(r.d_a + cap_a);
+    r.d_b = reinterpret_cast<float *>(r.j_a + cap_a);
+    r.j_b = reinterpret_cast<uint32_t *>(r.d_b + cap_b);
+    return r;
+}
+
+// ---------------- list construction ----------------
+// d_Z and d_YZ of point j to Q query points (-inf over an empty Z).  qv holds
+// the query values dimension by dimension (Y first), so that a column's value
+// is loaded once for all queries.
+template <int Q>
+__device__ __forceinline__ void list_dist(const float *const *col, int dy, int dz, int j,
+                                          const float (*qv)[Q], float (&vz)[Q], float (&vyz)[Q])
+{
+#pragma unroll
+    for (int q = 0; q < Q; ++q) vz[q] = -CUDART_INF_F;
+#pragma unroll 2
+    for (int d = dy; d < dy + dz; ++d) {
+        const float v = __ldg(col[d] + j);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) vz[q] = fmaxf(vz[q], fabsf(__fsub_rn(qv[d][q], v)));
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) vyz[q] = vz[q];
+    for (int d = 0; d < dy; ++d) {
+        const float v = __ldg(col[d] + j);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) vyz[q] = fmaxf(vyz[q], fabsf(__fsub_rn(qv[d][q], v)));
+    }
+}
+
+// A team's barrier (team t: threads kTeam t .. of the CTA)
+constexpr int kTeam = 128;
+constexpr int kTeams = kListBuildThreads / kTeam;
+__device__ __forceinline__ void team_sync(int t)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(t + 1), "n"(kTeam) : "memory");
+}
+
+// One team sorts n entries (any order) ascending into its list of row R, pads
+// the list to a multiple of 32 and writes its near part (and B's skip row).
+// Counting sort into kBins equal parts of [0, top] (the bin is a
+// non-decreasing function of the distance), then every entry's rank inside
+// its bin by comparison.  bins: kBins ints, idx: n shorts.  Returns the
+// padded length.
+__device__ int team_list_sort(const Entry *ent, int n, float top, int *bins, uint16_t *idx,
+                              const RowPtrs &R, bool list_b, const int *__restrict__ rank, int team)
+{
+    const int tid = threadIdx.x % kTeam;
+    float *d = list_b ? R.d_b : R.d_a, *nd = list_b ? R.near->db : R.near->da;
+    uint32_t *j = list_b ? R.j_b : R.j_a, *no = list_b ? R.near->ob : R.near->oa;
+    const int n_near = list_b ? kNearB : kNearA;
+    const float scale = top > 0.f && top < 3e38f ? (float)kBins / top : 0.f;
+    auto bin_of = [&](float v) { return min((int)(v * scale), kBins - 1); };
+    for (int b = tid; b < kBins; b += kTeam) bins[b] = 0;
+    if (list_b) {
+        for (int b = tid; b < kListSkip; b += kTeam) R.skip[b] = CUDART_INF_F;
+        if (tid == 0) R.near->far = CUDART_INF_F;
+    }
+    for (int b = n + tid; b < n_near; b += kTeam) {
+        nd[b] = CUDART_INF_F;
+        no[b] = 0;
+    }
+    team_sync(team);
+    for (int e = tid; e < n; e += kTeam) atomicAdd(&bins[bin_of(ent[e].d)], 1);
+    team_sync(team);
+    if (tid < 32) {
+        int carry = 0;
+        for (int b0 = 0; b0 < kBins; b0 += 128) {   // exclusive scan in place, 4 bins per lane
+            int4 c = *reinterpret_cast<int4 *>(bins + b0 + 4 * tid);
+            const int t = c.x + c.y + c.z + c.w;
+            int s = t;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(kFull, s, o);
+                if (tid >= o) s += u;
+            }
+            const int before = carry + s - t;
+            *reinterpret_cast<int4 *>(bins + b0 + 4 * tid) =
+                make_int4(before, before + c.x, before + c.x + c.y, before + c.x + c.y + c.z);
+            carry += __shfl_sync(kFull, s, 31);
+        }
+    }
+    team_sync(team);
+    for (int e = tid; e < n; e += kTeam) idx[atomicAdd(&bins[bin_of(ent[e].d)], 1)] = (uint16_t)e;
+    team_sync(team);
+    // bins[b] is now the end of bin b, so bin b starts at bins[b - 1]
+    for (int p = tid; p < n; p += kTeam) {
+        const Entry me = ent[idx[p]];
+        const int b = bin_of(me.d);
+        const int lo = b ? bins[b - 1] : 0, hi = bins[b];
+        const uint64_t key = entry_key(me);
+        int r = lo;
+        for (int u = lo; u < hi; ++u) r += entry_key(ent[idx[u]]) < key ? 1 : 0;
+        const uint32_t place = 4u * (rank ? (uint32_t)__ldg(rank + me.j) : me.j);
+        d[r] = me.d;
+        j[r] = place;
+        if (r < n_near) {
+            nd[r] = me.d;
+            no[r] = place;
+        }
+        if (list_b) {
+            if ((r & 31) == 0) R.skip[r >> 5] = me.d;
+            if (r == kNearB) R.near->far = me.d;
+        }
+    }
+    const int padded = (n + 31) & ~31;
+    if (tid < padded - n) {
+        d[n + tid] = CUDART_INF_F;
+        j[n + tid] = 0;
+    }
+    team_sync(team);   // bins and idx are free again
+    return padded;
+}
+
+// One CTA builds the lists of Q consecutive query points.  The radius of a
+// list is chosen from a sample of the points so that about 0.7 of its capacity
+// is used; a list that overflows is collected again with a smaller radius.
+template <int Q>
+__global__ void __launch_bounds__(kListBuildThreads) list_build_kernel(const ListLaunch L,
+                                                                       int smem_a, int smem_b)
+{
+    extern __shared__ __align__(16) unsigned char lsm[];
+    // per team bins and the sort's index row; per query smem_a + smem_b
+    // entries (the sample before that)
+    const int per_q = smem_a + smem_b, idx_n = max(smem_a, smem_b);
+    int *bins = reinterpret_cast<int *>(lsm);
+    Entry *ent = reinterpret_cast<Entry *>(bins + kTeams * kBins);
+    uint16_t *idx = reinterpret_cast<uint16_t *>(ent + (size_t)Q * per_q);
+    __shared__ __align__(16) float qv[32][Q];
+    __shared__ const float *col[32];
+    __shared__ float s_r[Q][2];
+    __shared__ int s_cnt[Q][2];
+    __shared__ unsigned s_todo;
+
+    const long long item = blockIdx.x;
+    const ListSeg &S = L.segs[last_at_or_below(L.n_segs, item,
+                                               [&](int a) { return L.segs[a].build_item; })];
+    const ListGroup &G = L.groups[S.group];
+    const int N = G.N, w = G.theiler, dy = G.dy, dz = G.dz, dyz = dy + dz;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int r0 = (int)(item - S.build_item) * Q, nq = S.nq;   // first row of the segment
+    const int i0 = S.q0 + r0;
+    const int cap[2] = {G.cap_a, G.cap_b};
+    for (int e = tid; e < Q * dyz; e += kListBuildThreads) {
+        const int q = e / dyz, d = e - q * dyz;
+        const float *c = G.base + (d < dy ? L.cols[G.ycol + d] : L.cols[G.zcol + d - dy]);
+        qv[d][q] = c[i0 + min(q, nq - 1 - r0)];
+        if (q == 0) col[d] = c;
+    }
+    const int ns = min(N, kSample);
+    if (tid < 2 * Q) {
+        s_r[tid >> 1][tid & 1] = CUDART_INF_F;
+        s_cnt[tid >> 1][tid & 1] = 0;
+    }
+    __syncthreads();
+    auto masked = [&](int q, int j) { return abs(j - (i0 + q)) <= w; };
+    // per query [A sample | B sample], floats, in the entries' space
+    auto samp = [&](int q, int l) {
+        return reinterpret_cast<float *>(ent + (size_t)q * per_q) + l * kSample;
+    };
+    const bool sample[2] = {N > cap[0], cap[1] > 0 && N > cap[1]};
+    if (sample[0] || sample[1]) {
+        for (int s = tid; s < ns; s += kListBuildThreads) {
+            const int j = (int)((long long)s * N / ns);
+            float vz[Q], vyz[Q];
+            list_dist<Q>(col, dy, dz, j, qv, vz, vyz);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const bool m = masked(q, j);
+                samp(q, 0)[s] = m ? CUDART_INF_F : vyz[q];
+                samp(q, 1)[s] = m ? CUDART_INF_F : vz[q];
+            }
+        }
+        __syncthreads();
+        for (int t = warp; t < 2 * Q; t += kBuildWarps) {
+            const int q = t >> 1, l = t & 1;
+            if (!sample[l]) continue;
+            float v[kSample / 32];
+#pragma unroll
+            for (int a = 0; a < kSample / 32; ++a) {
+                const int s = a * 32 + lane;
+                v[a] = s < ns ? samp(q, l)[s] : CUDART_INF_F;
+            }
+            // largest radius (to 8 bits of mantissa) with at most `target`
+            // samples below it
+            const int target = (int)(0.7f * (float)cap[l] * (float)ns / (float)N);
+            unsigned lo = 0;
+            for (int bit = 30; bit >= 15; --bit) {
+                const unsigned c = lo | (1u << bit);
+                const float f = __uint_as_float(c);
+                int n = 0;
+#pragma unroll
+                for (int a = 0; a < kSample / 32; ++a) n += v[a] < f ? 1 : 0;
+                const int below = (int)__reduce_add_sync(kFull, n);
+                if (c <= 0x7f800000u && below <= target) lo = c;
+            }
+            if (lane == 0) s_r[q][l] = __uint_as_float(lo);
+        }
+        __syncthreads();
+    }
+    // B is needed up to A's radius only: a member beyond that scans all points
+    if (tid < Q) s_r[tid][1] = fminf(s_r[tid][1], s_r[tid][0]);
+    __syncthreads();
+    unsigned todo = 0;   // bit 2q + l: list still to be collected
+#pragma unroll
+    for (int b = 0; b < 2 * Q; ++b) todo |= (b & 1) && cap[1] == 0 ? 0u : 1u << b;
+    for (int sweep = 0; todo; ++sweep) {
+        float r[Q][2];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            // -inf: not collected in this sweep (d_Z itself is -inf over an empty Z)
+            r[q][0] = (todo >> (2 * q)) & 1u ? s_r[q][0] : -CUDART_INF_F;
+            r[q][1] = (todo >> (2 * q + 1)) & 1u ? s_r[q][1] : -CUDART_INF_F;
+        }
+        for (int j = tid; j < N; j += kListBuildThreads) {
+            float vz[Q], vyz[Q];
+            list_dist<Q>(col, dy, dz, j, qv, vz, vyz);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const bool ok = !masked(q, j);
+                if (ok && vyz[q] < r[q][0]) {
+                    const int at = atomicAdd(&s_cnt[q][0], 1);
+                    if (at < cap[0]) ent[(size_t)q * per_q + at] = Entry{(uint32_t)j, vyz[q]};
+                }
+                if (ok && vz[q] < r[q][1]) {
+                    const int at = atomicAdd(&s_cnt[q][1], 1);
+                    if (at < cap[1])
+                        ent[(size_t)q * per_q + smem_a + at] = Entry{(uint32_t)j, vz[q]};
+                }
+            }
+        }
+        if (tid == 0) s_todo = 0;
+        __syncthreads();
+        if (tid < 2 * Q && ((todo >> tid) & 1u)) {
+            const int q = tid >> 1, l = tid & 1;
+            if (s_cnt[q][l] > cap[l]) {
+                // too many: a smaller radius (the count goes with at most the
+                // dimension's power of it); an empty list in the end
+                const float f = 0.8f * (float)cap[l] / (float)s_cnt[q][l];
+                const float c = 1.f - (1.f - f) / (float)(l ? dz : dyz);
+                const float rn = s_r[q][l] * c;
+                s_r[q][l] = sweep < 8 && rn < s_r[q][l] ? rn : 0.f;
+                s_cnt[q][l] = 0;
+                atomicOr(&s_todo, 1u << tid);
+            }
+        }
+        __syncthreads();
+        todo = s_todo;
+        __syncthreads();
+    }
+    const int team = tid / kTeam;
+    for (int t = team; t < 2 * Q; t += kTeams) {
+        const int q = t >> 1, l = t & 1;
+        if (r0 + q >= nq || (l && cap[1] == 0)) continue;
+        const Entry *src = ent + (size_t)q * per_q + (l ? smem_a : 0);
+        const RowPtrs R = row_ptrs(S.rows, r0 + q, cap[0], cap[1]);
+        const int n = s_cnt[q][l];
+        float top = s_r[q][l];
+        if (!(top < 3e38f)) {   // no radius: the largest distance (each warp finds it)
+            float mx = 0.f;
+            for (int e = lane; e < n; e += 32) mx = fmaxf(mx, src[e].d);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
+            top = mx;
+        }
+        const int padded = team_list_sort(src, n, top, bins + team * kBins,
+                                          idx + (size_t)team * idx_n, R, l, G.rank, team);
+        if (tid % kTeam == 0) {
+            if (l) {
+                R.near->rb = s_r[q][1];
+                R.near->nb = (uint16_t)padded;
+            } else {
+                R.near->ra = s_r[q][0];
+                R.near->na = (uint16_t)padded;
+                R.near->place = 4u * (uint32_t)(G.rank ? __ldg(G.rank + i0 + q) : i0 + q);
+                if (cap[1] == 0) {
+                    R.near->rb = CUDART_INF_F;
+                    R.near->nb = 0;
+                    R.near->far = CUDART_INF_F;
+                }
+            }
+        }
+    }
+}
+
+// ---------------- sorted columns ----------------
+// A point's rank is the number of points before it in (value, index) order:
+// one CTA counts 64 points' against every point, staged in shared memory
+// (2^13 points sort in a few microseconds over all SMs; a sort by one CTA
+// takes a few hundred).
+__global__ void __launch_bounds__(256) rank_sort_kernel(const RankSortJob *jobs, int n_jobs)
+{
+    constexpr int T = 1024;
+    __shared__ __align__(16) float v[T];
+    __shared__ int s_rank[64];
+    const int item = blockIdx.x;
+    const RankSortJob J =
+        jobs[last_at_or_below(n_jobs, item, [&](int a) { return (long long)jobs[a].item; })];
+    const int p = (item - J.item) * 64 + (threadIdx.x & 63), part = threadIdx.x >> 6;
+    const float mine = p < J.N ? J.src[p] : 0.f;
+    if (threadIdx.x < 64) s_rank[threadIdx.x] = 0;
+    int r = 0;
+    for (int t0 = 0; t0 < J.N; t0 += T) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < T; e += 256)
+            v[e] = t0 + e < J.N ? J.src[t0 + e] : CUDART_INF_F;
+        __syncthreads();
+        const int a0 = part * (T / 4);
+#pragma unroll 4
+        for (int a = a0; a < a0 + T / 4; a += 4) {
+            const float4 x = *reinterpret_cast<const float4 *>(v + a);
+            const int j = t0 + a;
+            r += (x.x < mine || (x.x == mine && j < p)) ? 1 : 0;
+            r += (x.y < mine || (x.y == mine && j + 1 < p)) ? 1 : 0;
+            r += (x.z < mine || (x.z == mine && j + 2 < p)) ? 1 : 0;
+            r += (x.w < mine || (x.w == mine && j + 3 < p)) ? 1 : 0;
+        }
+    }
+    atomicAdd(&s_rank[threadIdx.x & 63], r);
+    __syncthreads();
+    if (threadIdx.x < 64 && p < J.N) {
+        const int k = s_rank[threadIdx.x];
+        if (J.sorted) J.sorted[k] = mine;
+        if (J.rank) J.rank[p] = k;
+    }
+}
+
+// ---------------- the walk ----------------
+// values of an ascending column within e > 0 of x, by exactly the pairwise
+// test (fl(col[u] - x) is non-decreasing in u, so they form one run)
+__device__ __forceinline__ int column_count(const float *__restrict__ col, int n, float x, float e)
+{
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__fsub_rn(__ldg(col + mid), x) >= e) hi = mid;
+        else lo = mid + 1;
+    }
+    const int a = lo;
+    lo = 0;
+    hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__fsub_rn(__ldg(col + mid), x) > -e) hi = mid;
+        else lo = mid + 1;
+    }
+    return a - lo;
+}
+
+// Ascending sort of the G lanes' values inside every group of G lanes.
+template <int G>
+__device__ __forceinline__ float group_sort(float v)
+{
+    const int u = threadIdx.x & (G - 1);
+#pragma unroll
+    for (int kk = 2; kk <= G; kk <<= 1)
+#pragma unroll
+        for (int jj = kk >> 1; jj > 0; jj >>= 1) {
+            const float o = __shfl_xor_sync(kFull, v, jj);
+            const bool low = ((u & jj) == 0) == ((u & kk) == 0 || kk == G);
+            v = low ? fminf(v, o) : fmaxf(v, o);
+        }
+    return v;
+}
+
+// The G smallest of buf (ascending over the group's lanes) and the lanes' new
+// values, ascending.
+template <int G>
+__device__ __forceinline__ float group_merge(float buf, float v)
+{
+    const int u = threadIdx.x & (G - 1);
+    v = group_sort<G>(v);
+    v = fminf(buf, __shfl_xor_sync(kFull, v, G - 1));   // lane u against the new lane G - 1 - u
+#pragma unroll
+    for (int jj = G >> 1; jj > 0; jj >>= 1) {
+        const float o = __shfl_xor_sync(kFull, v, jj);
+        v = (u & jj) == 0 ? fminf(v, o) : fmaxf(v, o);
+    }
+    return v;
+}
+
+// Per group of G lanes, the number of d[0, n) (ascending) below e: G-ary
+// search, the whole warp together.
+template <int G>
+__device__ __forceinline__ int group_rank(const float *__restrict__ d, int n, float e)
+{
+    const int lane = threadIdx.x & 31, u = lane & (G - 1), shift = lane & ~(G - 1);
+    const unsigned mask = G == 32 ? kFull : (1u << G) - 1u;
+    int lo = 0;
+    while (__any_sync(kFull, n > 0)) {
+        const int step = (n + G - 1) / G;
+        const int at = u * step;
+        const bool below = at < n && d[lo + at] < e;
+        const int c = __popc((__ballot_sync(kFull, below) >> shift) & mask);
+        const int end = lo + n;
+        if (c) lo += (c - 1) * step + 1;
+        n = c ? min(step - 1, end - lo) : 0;
+    }
+    return lo;
+}
+
+// One member at query point i over all points, by the whole CTA: its k-th
+// smallest joint distance and the three counts, added to the accumulators.
+// Blocks of 32 points go round the warps, four of a warp's in flight; every
+// warp keeps the smallest distances it meets, and the warps' k smallest are
+// merged through shared memory.  xm: the member's X values in shared memory,
+// dimension d of point j at d * xs + (j's place); col and q: the Y then Z columns and
+// the point's values in them; top: 32 * k floats, cnt: three ints.
+template <bool DX1>
+__device__ __noinline__ void scan_member(const ListLaunch &L, const ListGroup &G,
+                                         const float *const *col, const float *q, int i,
+                                         const float *xm, int xs, int out, float *top, int *cnt)
+{
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    const int N = G.N, dx = DX1 ? 1 : G.dx, dy = G.dy, dyz = G.dy + G.dz, k = G.k, w = G.theiler;
+    const int stride = 32 * n_warps;
+    const int pi = G.rank ? G.rank[i] : i;
+    auto dist = [&](int j0, float (&vx)[U], float (&vz)[U], float (&vyz)[U]) {
+        int j[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            j[u] = min(j0 + stride * u, N - 1);
+            vz[u] = -CUDART_INF_F;
+            const int pj = G.rank ? __ldg(G.rank + j[u]) : j[u];
+            vx[u] = fabsf(__fsub_rn(xm[pi], xm[pj]));
+            if (!DX1)
+                for (int d = 1; d < dx; ++d)
+                    vx[u] = fmaxf(vx[u], fabsf(__fsub_rn(xm[d * xs + pi], xm[d * xs + pj])));
+        }
+#pragma unroll 2
+        for (int d = dy; d < dyz; ++d) {
+            const float *c = col[d];
+            const float qd = q[d];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                vz[u] = fmaxf(vz[u], fabsf(__fsub_rn(qd, __ldg(c + j[u]))));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) vyz[u] = vz[u];
+        for (int d = 0; d < dy; ++d) {
+            const float *c = col[d];
+            const float qd = q[d];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                vyz[u] = fmaxf(vyz[u], fabsf(__fsub_rn(qd, __ldg(c + j[u]))));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)   // masked points: beyond every distance
+            if (j0 + stride * u >= N || abs(j[u] - i) <= w)
+                vx[u] = vz[u] = vyz[u] = CUDART_INF_F;
+    };
+    float buf = CUDART_INF_F, eps = CUDART_INF_F;
+    for (int j0 = 32 * warp + lane; j0 - lane < N; j0 += U * stride) {
+        float vx[U], vz[U], vyz[U];
+        dist(j0, vx, vz, vyz);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float D = fmaxf(vx[u], vyz[u]);
+            if (__any_sync(kFull, D < eps)) {
+                buf = group_merge<32>(buf, D);
+                eps = __shfl_sync(kFull, buf, k - 1);
+            }
+        }
+    }
+    if (lane < k) top[warp * k + lane] = buf;
+    if (threadIdx.x < 3) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    buf = CUDART_INF_F;
+    for (int a = 0; a < k; ++a)
+        buf = group_merge<32>(buf, lane < n_warps ? top[lane * k + a] : CUDART_INF_F);
+    eps = __shfl_sync(kFull, buf, k - 1);
+    int cxz = 0, cyz = 0, cz = 0;
+    for (int j0 = 32 * warp + lane; j0 - lane < N; j0 += U * stride) {
+        float vx[U], vz[U], vyz[U];
+        dist(j0, vx, vz, vyz);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            cz += vz[u] < eps ? 1 : 0;
+            cxz += fmaxf(vx[u], vz[u]) < eps ? 1 : 0;
+            cyz += vyz[u] < eps ? 1 : 0;
+        }
+    }
+    cz = (int)__reduce_add_sync(kFull, cz);
+    cxz = (int)__reduce_add_sync(kFull, cxz);
+    cyz = (int)__reduce_add_sync(kFull, cyz);
+    if (lane == 0) {
+        atomicAdd(&cnt[0], cz);
+        atomicAdd(&cnt[1], cxz);
+        atomicAdd(&cnt[2], cyz);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        // an empty Z: d_Z is below every eps for every point that is not masked
+        if (G.dz == 0) cnt[0] = N - (min(i + w, N - 1) - max(i - w, 0) + 1);
+        const long long t = L.q[cnt[0] + 1] - L.q[cnt[1] + 1] - L.q[cnt[2] + 1];
+        atomicAdd(&L.acc[2 * (size_t)out], (unsigned long long)t & 0xffffffffull);
+        atomicAdd(&L.acc[2 * (size_t)out + 1], (unsigned long long)(t >> 32));
+        if (L.dbg_eps && out == L.dbg_out) {
+            L.dbg_eps[i] = eps;
+            L.dbg_nz[i] = cnt[0];
+            L.dbg_nxz[i] = cnt[1];
+            L.dbg_nyz[i] = cnt[2];
+        }
+    }
+    __syncthreads();
+}
+
+// E consecutive entries of a list (E = 1, 2 or 4, aligned to E)
+template <int E>
+__device__ __forceinline__ void load_entries(const float *dp, const uint32_t *op, float (&d)[E],
+                                             uint32_t (&o)[E])
+{
+    if constexpr (E == 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(dp);
+        const uint4 w = *reinterpret_cast<const uint4 *>(op);
+        d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+        o[0] = w.x; o[1] = w.y; o[2] = w.z; o[3] = w.w;
+    } else if constexpr (E == 2) {
+        const float2 v = *reinterpret_cast<const float2 *>(dp);
+        const uint2 w = *reinterpret_cast<const uint2 *>(op);
+        d[0] = v.x; d[1] = v.y;
+        o[0] = w.x; o[1] = w.y;
+    } else {
+        d[0] = *dp;
+        o[0] = *op;
+    }
+}
+
+// The 4 smallest of two ascending lists of 4, ascending, into b.
+__device__ __forceinline__ void cmpx(float &a, float &b)
+{
+    const float lo = fminf(a, b);
+    b = fmaxf(a, b);
+    a = lo;
+}
+__device__ __forceinline__ void merge4(float (&b)[4], const float (&o)[4])
+{
+#pragma unroll
+    for (int a = 0; a < 4; ++a) b[a] = fminf(b[a], o[3 - a]);   // bitonic
+    cmpx(b[0], b[2]);
+    cmpx(b[1], b[3]);
+    cmpx(b[0], b[1]);
+    cmpx(b[2], b[3]);
+}
+
+// A member's k smallest joint distances so far.  K4 (k = 4): all four in
+// every lane of the member's group; otherwise the a-th in the group's lane a.
+template <int G, bool K4>
+struct Nearest {
+    float b[K4 ? 4 : 1];
+    float thr;   // the k-th
+    __device__ __forceinline__ Nearest()
+    {
+        thr = CUDART_INF_F;
+#pragma unroll
+        for (float &v : b) v = CUDART_INF_F;
+    }
+    // the lanes' E = 32 / G new distances each
+    __device__ __forceinline__ void add(const float (&D)[32 / G], int k)
+    {
+        constexpr int E = 32 / G;
+        if constexpr (K4) {
+            // sorted in the lane, then pairwise over the group's lanes
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = e < E ? D[e < E ? e : 0] : CUDART_INF_F;
+            if constexpr (E == 4) {
+                cmpx(v[0], v[1]);
+                cmpx(v[2], v[3]);
+                cmpx(v[0], v[2]);
+                cmpx(v[1], v[3]);
+                cmpx(v[1], v[2]);
+            } else if constexpr (E == 2) {
+                cmpx(v[0], v[1]);
+            }
+#pragma unroll
+            for (int o = 1; o < G; o <<= 1) {
+                float t[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) t[e] = __shfl_xor_sync(kFull, v[e], o);
+                merge4(v, t);
+            }
+            merge4(b, v);
+            thr = b[3];
+        } else {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (__any_sync(kFull, D[e] < thr)) {
+                    b[0] = group_merge<G>(b[0], D[e]);
+                    thr = __shfl_sync(kFull, b[0], k - 1, G);
+                }
+        }
+    }
+};
+
+// One CTA: 32 / G members of one group, their X values in shared memory, x a
+// range of query points.  A warp takes a query point at a time, G lanes per
+// member and 32 list entries per member at a time, all members at once; only
+// a long prefix of B (n_xz) goes over the whole warp, 128 entries at a time
+// for every member that reaches them.  A point's near lists are copied one
+// point ahead, and the digamma values that end its work are added one point
+// later: a warp's time is a chain of memory and shuffle latencies more than of
+// issue slots.
+template <int G, bool DX1, bool K4>
+__global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListLaunch L)
+{
+    constexpr int MW = 32 / G;
+    constexpr int E = 32 / G;       // entries per lane of a 32-entry step
+    // [2][warps] ListNear, [MW][dx][xs_dim] X, dz == 1: every 16th sorted Z
+    extern __shared__ __align__(16) unsigned char wsm[];
+    __shared__ const float *s_col[32];
+    __shared__ float s_q[32];                     // a point's Y and Z values
+    __shared__ int s_cnt[3];
+    // pairs beyond the lists' radii: bit (point of the CTA) * MW + member
+    __shared__ uint32_t s_slow[kListWalkSmem / 4 / 32 + 1];
+    const long long item = blockIdx.x;
+    const ListSeg &S = L.segs[last_at_or_below(L.n_segs, item,
+                                               [&](int a) { return L.segs[a].walk_item; })];
+    const ListGroup &Gr = L.groups[S.group];
+    const int N = Gr.N, dx = DX1 ? 1 : Gr.dx, w = Gr.theiler, k = K4 ? 4 : Gr.k, dz = Gr.dz;
+    const int dyz = Gr.dy + dz;
+    const long long local = item - S.walk_item;
+    const int mb = (int)(local / S.n_splits), split = (int)(local % S.n_splits);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    const int u = lane & (G - 1), g = lane / G;
+    const int cap_a = Gr.cap_a, cap_b = Gr.cap_b;
+    const int nm = min(MW, Gr.n_members - mb * MW);
+    const int xd = (N + 3) & ~3, xn = dx * xd;   // X values of a dimension, of a member
+    ListNear *near_buf = reinterpret_cast<ListNear *>(wsm) + 2 * warp;
+    float *xs = reinterpret_cast<float *>(reinterpret_cast<ListNear *>(wsm) + 2 * n_warps);
+    float *zc = xs + MW * xn;
+    const int nc = (N + 15) / 16;
+
+    for (int m = 0; m < MW; ++m) {
+        // past the last member: the last one again, its results dropped
+        const MemberDesc md = L.members[Gr.member_begin + mb * MW + min(m, nm - 1)];
+        for (int d = 0; d < dx; ++d) {
+            const float *src = Gr.base + L.cols[md.xcol + d];
+            float *dst = xs + m * xn + d * xd;
+#pragma unroll 4
+            for (int j = threadIdx.x; j < N; j += blockDim.x)
+                dst[dz == 1 ? __ldg(Gr.rank + j) : j] =
+                    __ldg(src + (md.perm ? __ldg(md.perm + j) : j));
+        }
+    }
+    if (dz == 1)
+        for (int c = threadIdx.x; c < nc; c += blockDim.x) zc[c] = Gr.zs[16 * c];
+    if (threadIdx.x < dyz)
+        s_col[threadIdx.x] = Gr.base + (threadIdx.x < Gr.dy
+                                            ? L.cols[Gr.ycol + threadIdx.x]
+                                            : L.cols[Gr.zcol + threadIdx.x - Gr.dy]);
+    const int q_first = split * S.per_cta, q_last = min(S.nq, q_first + S.per_cta);
+    for (int a = threadIdx.x; a <= (q_last - q_first) * MW / 32; a += blockDim.x) s_slow[a] = 0;
+    const char *xm = reinterpret_cast<const char *>(xs + g * xn);
+    // A member's sum of digamma values: its group's lanes 0, 1, 2 sum those of
+    // n_z, -n_xz and -n_yz (the low 32 bits and the rest apart, as the
+    // accumulators keep them: a long run would not fit in one int64).
+    unsigned long long sum_lo = 0;
+    long long sum_hi = 0, q_last_term = 0;
+    unsigned evals = 0;   // member-pairs evaluated by the warp
+    __syncthreads();
+
+    // d_X between the query point and the point at byte offset o, for the X
+    // values at x (xi: the query point's first one, oi: its byte offset)
+    auto dist_x = [&](const char *x, float xi, uint32_t oi, uint32_t o) {
+        float v = fabsf(__fsub_rn(xi, *reinterpret_cast<const float *>(x + o)));
+        if (!DX1)
+            for (int d = 1; d < dx; ++d) {
+                const char *r = x + 4 * d * xd;
+                v = fmaxf(v, fabsf(__fsub_rn(*reinterpret_cast<const float *>(r + oi),
+                                             *reinterpret_cast<const float *>(r + o))));
+            }
+        return v;
+    };
+    auto group_sum = [&](int v) {
+#pragma unroll
+        for (int o = G >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+        return v;
+    };
+    unsigned char *const rows = S.rows;
+    const int q0 = S.q0;
+    // copy a row's near part into buffer `half` (past the end: the last row again)
+    auto fetch = [&](int r, int half) {
+        const RowPtrs R = row_ptrs(rows, min(r, q_last - 1), cap_a, cap_b);
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(near_buf + half);
+        for (int e = 16 * lane; e < (int)sizeof(ListNear); e += 512)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + e),
+                         "l"(reinterpret_cast<const char *>(R.near) + e)
+                         : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto add_term = [&]() {
+        sum_lo += (unsigned long long)q_last_term & 0xffffffffull;
+        sum_hi += q_last_term >> 32;
+    };
+    int half = 0;
+    fetch(q_first + warp, 0);
+    for (int row = q_first + warp; row < q_last; row += n_warps, half ^= 1) {
+        const int i = q0 + row;
+        const RowPtrs R = row_ptrs(rows, row, cap_a, cap_b);
+        __syncwarp();   // the other half's readers are done
+        fetch(row + n_warps, half ^ 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const ListNear &h = near_buf[half];
+        const int na = h.na, nb = h.nb;
+        const uint32_t oi = h.place;
+        const float xi = *reinterpret_cast<const float *>(xm + oi);
+
+        // ---- k nearest joint distances over list A ----
+        Nearest<G, K4> near;
+        int c = 0, p = 0;
+        float da[E];   // the first 32 entries' d_YZ
+        {
+            uint32_t o[E];
+            float D[E];
+            load_entries<E>(h.da + E * u, h.oa + E * u, da, o);
+#pragma unroll
+            for (int e = 0; e < E; ++e) D[e] = fmaxf(dist_x(xm, xi, oi, o[e]), da[e]);
+            near.add(D, k);
+            evals += 32 * E;
+        }
+        for (p = 32; p < na; p += 32) {
+            float d[E], D[E], dmin = CUDART_INF_F;
+            uint32_t o[E];
+            load_entries<E>(R.d_a + p + E * u, R.j_a + p + E * u, d, o);
+            if (!__any_sync(kFull, d[0] < near.thr)) break;
+            evals += 32 * E;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                D[e] = fmaxf(dist_x(xm, xi, oi, o[e]), d[e]);
+                dmin = fminf(dmin, D[e]);
+            }
+            if (__any_sync(kFull, dmin < near.thr)) near.add(D, k);
+        }
+
+        // ---- n_yz: a rank in A ----
+        const float eps = near.thr;
+        const bool slow = eps > h.ra || (dz > 1 && eps > h.rb);
+        const float ec = slow ? -1.f : eps;   // below every distance for members that scan
+#pragma unroll
+        for (int e = 0; e < E; ++e) c += da[e] < ec ? 1 : 0;
+        int nyz = group_sum(c);
+        if (p > 32 && na > 32) nyz += group_rank<G>(R.d_a + 32, min(p, na) - 32, ec);
+
+        // ---- n_z and n_xz ----
+        int nz = 0, nxz = 0;
+        if (dz > 1 && !__any_sync(kFull, ec > h.far)) {
+            // every prefix of B ends within kNearB entries: counted by the groups
+            int cz = 0, cx = 0;
+            for (int b = 0; b < min(nb, kNearB); b += 32) {
+                float d[E];
+                uint32_t o[E];
+                load_entries<E>(h.db + b + E * u, h.ob + b + E * u, d, o);
+                if (!__any_sync(kFull, d[0] < ec)) break;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    cz += d[e] < ec ? 1 : 0;
+                    cx += fmaxf(dist_x(xm, xi, oi, o[e]), d[e]) < ec ? 1 : 0;
+                }
+                evals += 32 * E;
+            }
+            nz = group_sum(cz);
+            nxz = group_sum(cx);
+        } else if (dz > 1) {
+            // n_z: the last skip distance below eps, then the 32 entries from it
+            const float4 sk = *reinterpret_cast<const float4 *>(R.skip + 4 * lane);
+            float e[MW], xq[MW];
+            int n[MW], cm[MW], nmax = 0;
+#pragma unroll
+            for (int m = 0; m < MW; ++m) {
+                e[m] = __shfl_sync(kFull, ec, m * G);
+                xq[m] = __shfl_sync(kFull, xi, m * G);
+                cm[m] = 0;
+                n[m] = (int)__reduce_add_sync(
+                    kFull, (sk.x < e[m] ? 1 : 0) + (sk.y < e[m] ? 1 : 0) +
+                               (sk.z < e[m] ? 1 : 0) + (sk.w < e[m] ? 1 : 0));
+                if (g == m) nz = n[m];
+            }
+            const int from = 32 * max(nz - 1, 0);
+            {
+                float d[E];
+                uint32_t o[E];
+                load_entries<E>(R.d_b + from + E * u, R.j_b + from + E * u, d, o);
+                c = 0;
+#pragma unroll
+                for (int a = 0; a < E; ++a) c += d[a] < ec ? 1 : 0;
+            }
+            nz = from + group_sum(c);
+#pragma unroll
+            for (int m = 0; m < MW; ++m) {
+                n[m] = __shfl_sync(kFull, nz, m * G);
+                nmax = max(nmax, n[m]);
+                evals += n[m];
+            }
+            for (int b = 0; b < nmax; b += 128) {
+                const int at = b + 4 * lane;
+                const uint4 o = *reinterpret_cast<const uint4 *>(R.j_b + min(at, nb - 4));
+#pragma unroll
+                for (int m = 0; m < MW; ++m) {
+                    if (b >= n[m]) continue;
+                    const char *x = reinterpret_cast<const char *>(xs + m * xn);
+                    const float d0 = dist_x(x, xq[m], oi, o.x), d1 = dist_x(x, xq[m], oi, o.y);
+                    const float d2 = dist_x(x, xq[m], oi, o.z), d3 = dist_x(x, xq[m], oi, o.w);
+                    if (b + 128 <= n[m]) {
+                        cm[m] += (d0 < e[m] ? 1 : 0) + (d1 < e[m] ? 1 : 0) +
+                                 (d2 < e[m] ? 1 : 0) + (d3 < e[m] ? 1 : 0);
+                    } else {
+                        cm[m] += (at < n[m] && d0 < e[m] ? 1 : 0) +
+                                 (at + 1 < n[m] && d1 < e[m] ? 1 : 0) +
+                                 (at + 2 < n[m] && d2 < e[m] ? 1 : 0) +
+                                 (at + 3 < n[m] && d3 < e[m] ? 1 : 0);
+                    }
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < MW; ++m) {
+                const int t = (int)__reduce_add_sync(kFull, cm[m]);
+                if (g == m) nxz = t;
+            }
+        } else if (dz == 1) {
+            // The points with d_Z < eps are consecutive places lo .. hi - 1: rounding
+            // is monotone, so fl(z_i - z) >= eps holds for the first lo sorted z and
+            // fl(z - z_i) < eps for the first hi.  Even lanes find lo, odd lanes hi,
+            // over every 16th z in shared memory; then 16 z each by the group.
+            const float zi = __ldg(s_col[Gr.dy] + i);
+            int lo = 0, hi = 0;
+            {
+                const bool up = u & 1;
+                int a = 0, b = nc;   // entries for which the test holds: a prefix
+                while (__any_sync(kFull, a < b)) {
+                    const int mid = min((a + b) >> 1, nc - 1);
+                    const float z = zc[mid];
+                    const bool in = up ? __fsub_rn(z, zi) < ec : __fsub_rn(zi, z) >= ec;
+                    if (a < b) {
+                        if (in) a = mid + 1;
+                        else b = mid;
+                    }
+                }
+                const int cl = __shfl_sync(kFull, a, 0, G), ch = __shfl_sync(kFull, a, 1, G);
+                const int bl = 16 * max(cl - 1, 0), bh = 16 * max(ch - 1, 0);
+                int fl = 0, fh = 0;
+                for (int t = u; t < 16; t += G) {
+                    if (bl + t < N) fl += __fsub_rn(zi, __ldg(Gr.zs + bl + t)) >= ec ? 1 : 0;
+                    if (bh + t < N) fh += __fsub_rn(__ldg(Gr.zs + bh + t), zi) < ec ? 1 : 0;
+                }
+                lo = bl + group_sum(fl);
+                hi = bh + group_sum(fh);
+                if (!(ec > 0.f)) hi = lo;   // no point is nearer than 0
+            }
+            nz = hi - lo;
+#pragma unroll
+            for (int m = 0; m < MW; ++m) {
+                const int l = __shfl_sync(kFull, lo, m * G), n = __shfl_sync(kFull, nz, m * G);
+                const float e = __shfl_sync(kFull, ec, m * G);
+                const float xq = __shfl_sync(kFull, xi, m * G);
+                const char *x = reinterpret_cast<const char *>(xs + m * xn);
+                int cm = 0;
+                for (int b = l & ~3; b < l + n; b += 128) {
+                    const int at = min(b + 4 * lane, xd - 4);
+                    float v[4];
+                    if constexpr (DX1) {
+                        const float4 t = *reinterpret_cast<const float4 *>(x + 4 * at);
+                        v[0] = fabsf(__fsub_rn(xq, t.x));
+                        v[1] = fabsf(__fsub_rn(xq, t.y));
+                        v[2] = fabsf(__fsub_rn(xq, t.z));
+                        v[3] = fabsf(__fsub_rn(xq, t.w));
+                    } else {
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) v[a] = dist_x(x, xq, oi, 4u * (at + a));
+                    }
+                    if (b >= l && b + 128 <= l + n) {
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) cm += v[a] < e ? 1 : 0;
+                    } else {
+                        const unsigned f = b + 4 * lane - l;
+#pragma unroll
+                        for (int a = 0; a < 4; ++a)
+                            cm += f + a < (unsigned)n && v[a] < e ? 1 : 0;
+                    }
+                }
+                cm = (int)__reduce_add_sync(kFull, cm);
+                evals += n;
+                if (g == m) nxz = cm;
+            }
+            // less the point itself and its Theiler band
+            if (w == 0) {
+                if (ec > 0.f) {
+                    --nz;
+                    --nxz;
+                }
+            } else {
+                const int first = max(i - w, 0), last = min(i + w, N - 1);
+                int cz = 0, cx = 0;
+                for (int j = first + u; j <= last; j += G) {
+                    const float d = fabsf(__fsub_rn(zi, __ldg(s_col[Gr.dy] + j)));
+                    const float v = dist_x(xm, xi, oi, 4u * (uint32_t)__ldg(Gr.rank + j));
+                    cz += d < ec ? 1 : 0;
+                    cx += fmaxf(d, v) < ec ? 1 : 0;
+                }
+                nz -= group_sum(cz);
+                nxz -= group_sum(cx);
+            }
+        } else {
+            const int first = max(i - w, 0), last = min(i + w, N - 1);
+            nz = N - (last - first + 1);
+            const float *xsorted = L.members[Gr.member_begin + mb * MW + min(g, nm - 1)].xsorted;
+            c = 0;
+            if (DX1 && xsorted) {   // less the point itself and its band
+                for (int j = first + u; j <= last; j += G)
+                    c -= dist_x(xm, xi, oi, 4u * j) < ec ? 1 : 0;
+                if (u == 0 && ec > 0.f) c += column_count(xsorted, N, xi, ec);
+            } else {
+                for (int j = u; j < N; j += G)
+                    if (j < first || j > last) c += dist_x(xm, xi, oi, 4u * j) < ec ? 1 : 0;
+            }
+            nxz = group_sum(c);
+        }
+        if (slow) {
+            if (u == 0 && g < nm) {
+                const int bit = (row - q_first) * MW + g;
+                atomicOr(&s_slow[bit >> 5], 1u << (bit & 31));
+            }
+            nz = nxz = nyz = -1;   // the digamma table's first value, 0
+        }
+        add_term();
+        q_last_term = L.q[(u == 0 ? nz : u == 1 ? nxz : nyz) + 1];
+        if (u > 0) q_last_term = -q_last_term;
+        if (L.dbg_eps && u == 0 && g < nm && !slow &&
+            L.members[Gr.member_begin + mb * MW + g].out == L.dbg_out) {
+            L.dbg_eps[i] = eps;
+            L.dbg_nxz[i] = nxz;
+            L.dbg_nyz[i] = nyz;
+            L.dbg_nz[i] = nz;
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    add_term();
+    if (u < 3 && g < nm) {
+        const int out = L.members[Gr.member_begin + mb * MW + g].out;
+        atomicAdd(&L.acc[2 * (size_t)out], sum_lo);
+        atomicAdd(&L.acc[2 * (size_t)out + 1], (unsigned long long)sum_hi);
+    }
+    if (L.work && lane == 0) {
+        atomicAdd(&L.work[0], (unsigned long long)evals);
+        atomicAdd(&L.work[1], 3ull * evals);
+    }
+    // ---- pairs beyond the lists' radii: over all points, by the whole CTA ----
+    __syncthreads();
+    const int n_words = (q_last - q_first) * MW / 32 + 1;
+    for (int w0 = 0; w0 < n_words; w0 += 32) {   // the same in every warp
+        const uint32_t mine = w0 + lane < n_words ? s_slow[w0 + lane] : 0;
+        unsigned words = __ballot_sync(kFull, mine != 0);
+        while (words) {
+            const int src = __ffs(words) - 1;
+            words &= words - 1;
+            uint32_t bits = __shfl_sync(kFull, mine, src);
+            while (bits) {
+                const int b = 32 * (w0 + src) + __ffs(bits) - 1;
+                bits &= bits - 1;
+                const int i = q0 + q_first + b / MW, m = b % MW;
+                if (threadIdx.x < dyz) s_q[threadIdx.x] = __ldg(s_col[threadIdx.x] + i);
+                __syncthreads();
+                scan_member<DX1>(L, Gr, s_col, s_q, i, xs + m * xn, xd,
+                                 L.members[Gr.member_begin + mb * MW + m].out,
+                                 reinterpret_cast<float *>(wsm), s_cnt);
+            }
+        }
+    }
+}
+
+}  // namespace
+
+void list_caps(int N, int k, int dx, int dy, int dz, size_t members, int *cap_a, int *cap_b)
+{
+    // Expected counts when the joint space has m independent dimensions: a
+    // per-dimension slab of probability (k / N)^(1/m) holds the neighbours.
+    // The margins cover the members whose X value lies in a sparse region;
+    // the lists are built once per group, so many members pay for longer ones.
+    const double m = dx + dy + dz;
+    const double slab = std::pow((double)k / (double)N, 1.0 / m);
+    const double nyz = N * std::pow(slab, (double)(dy + dz));
+    const double nz = N * std::pow(slab, (double)dz);
+    const double more = members >= 1000 ? 2.0 : 1.0;
+    auto cap = [&](double c, int hi) {
+        const int all = (N + 31) & ~31;
+        const int v = ((int)std::min(c, 1e6) + 31) & ~31;
+        return std::min(all, std::max(128, std::min(v, hi)));
+    };
+    *cap_a = cap(more * (m >= 8 ? 16.0 : 28.0) * nyz, kListCapA);
+    *cap_b = dz > 1 ? cap(more * 14.0 * nz, kListCapB) : 0;
+}
+
+int list_width(int N, int dx, int dz, int k, size_t members)
+{
+    // as many members per CTA as shared memory holds; 32 / width lanes serve
+    // a member and must hold its k neighbours
+    int w = 4;
+    while (w > 1 && (list_walk_x_bytes(N, dx, dz, w) > kListWalkSmem || 32 / w < k ||
+                     (size_t)w / 2 >= members))
+        w /= 2;
+    return w;
+}
+
+bool list_fits(int N, int dx, int dz) { return list_walk_x_bytes(N, dx, dz, 1) <= kListWalkSmem; }
+
+static size_t list_build_smem(int cap_a, int cap_b, int queries)
+{
+    // a query's space also holds its sample: kSample distances of either kind
+    const int a = std::max(cap_a, kSample - cap_b), b = cap_b;
+    return (size_t)queries * (a + b) * sizeof(Entry) +
+           (size_t)kTeams * (kBins * 4 + 2 * (size_t)std::max(a, b));
+}
+
+int list_build_queries(int cap_a, int cap_b)
+{
+    for (int q = 8; q > 2; q >>= 1)
+        if (list_build_smem(cap_a, cap_b, q) <= 110 * 1024) return q;
+    return 2;
+}
+
+constexpr int kWalkSmemMax =
+    (int)(kListWalkSmem + 2 * (kListWalkThreads / 32) * sizeof(ListNear));
+
+template <int G>
+static const void *walk_kernel_g(bool dx1, bool k4)
+{
+    if (dx1)
+        return k4 ? reinterpret_cast<const void *>(&list_walk_kernel<G, true, true>)
+                  : reinterpret_cast<const void *>(&list_walk_kernel<G, true, false>);
+    return k4 ? reinterpret_cast<const void *>(&list_walk_kernel<G, false, true>)
+              : reinterpret_cast<const void *>(&list_walk_kernel<G, false, false>);
+}
+
+static const void *walk_kernel(int width, bool dx1, bool k4)
+{
+    switch (width) {
+    case 1: return walk_kernel_g<32>(dx1, k4);
+    case 2: return walk_kernel_g<16>(dx1, k4);
+    case 4: return walk_kernel_g<8>(dx1, k4);
+    default: return nullptr;
+    }
+}
+
+cudaError_t list_prepare_attributes()
+{
+    const struct {
+        const void *f;
+        int bytes;
+    } fs[] = {{reinterpret_cast<const void *>(&list_build_kernel<2>), 220 * 1024},
+              {reinterpret_cast<const void *>(&list_build_kernel<4>), 220 * 1024},
+              {reinterpret_cast<const void *>(&list_build_kernel<8>), 220 * 1024},
+              {walk_kernel(1, true, true), kWalkSmemMax},
+              {walk_kernel(2, true, true), kWalkSmemMax},
+              {walk_kernel(4, true, true), kWalkSmemMax},
+              {walk_kernel(1, false, true), kWalkSmemMax},
+              {walk_kernel(2, false, true), kWalkSmemMax},
+              {walk_kernel(4, false, true), kWalkSmemMax},
+              {walk_kernel(1, true, false), kWalkSmemMax},
+              {walk_kernel(2, true, false), kWalkSmemMax},
+              {walk_kernel(4, true, false), kWalkSmemMax},
+              {walk_kernel(1, false, false), kWalkSmemMax},
+              {walk_kernel(2, false, false), kWalkSmemMax},
+              {walk_kernel(4, false, false), kWalkSmemMax}};
+    for (const auto &f : fs) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(f.f, cudaFuncAttributeMaxDynamicSharedMemorySize, f.bytes);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_list_build(const ListLaunch &L, long long n_items, int queries, int cap_a,
+                              int cap_b, cudaStream_t st)
+{
+    if (n_items <= 0) return cudaSuccess;
+    const size_t smem = list_build_smem(cap_a, cap_b, queries);
+    if (n_items > 0x7fffffffLL || smem > 220 * 1024) return cudaErrorInvalidValue;
+    const int a = std::max(cap_a, kSample - cap_b), b = cap_b;
+    const unsigned grid = (unsigned)n_items;
+    if (queries == 8) list_build_kernel<8><<<grid, kListBuildThreads, smem, st>>>(L, a, b);
+    else if (queries == 4) list_build_kernel<4><<<grid, kListBuildThreads, smem, st>>>(L, a, b);
+    else if (queries == 2) list_build_kernel<2><<<grid, kListBuildThreads, smem, st>>>(L, a, b);
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_list_walk(const ListLaunch &L, long long n_items, int width, bool dx1, bool k4,
+                             size_t smem, cudaStream_t st)
+{
+    if (n_items <= 0) return cudaSuccess;
+    const void *f = walk_kernel(width, dx1, k4);
+    if (!f || n_items > 0x7fffffffLL || smem > kListWalkSmem) return cudaErrorInvalidValue;
+    // one CTA per SM where its X values fill the shared memory, else two
+    const int threads = smem > kListHalfSmem ? kListWalkThreads : kListWalkThreads / 2;
+    smem += 2 * (size_t)(threads / 32) * sizeof(ListNear);
+    ListLaunch arg = L;
+    void *args[] = {&arg};
+    return cudaLaunchKernel(f, dim3((unsigned)n_items), dim3(threads), args, smem, st);
+}
+
+cudaError_t launch_rank_sort(const RankSortJob *jobs, int n_jobs, int n_items, cudaStream_t st)
+{
+    if (n_items <= 0) return cudaSuccess;
+    rank_sort_kernel<<<n_items, 256, 0, st>>>(jobs, n_jobs);
+    return cudaGetLastError();
+}
+
+}  // namespace teksg

@@ -1,0 +1,118 @@
+// Neighbour-list form of the KSG estimator: interface between the host plans
+// (te_lists.cu, te_static.cu) and the kernels (ksg_lists.cu).
+#pragma once
+
+#include "ksg_internal.h"
+
+namespace teksg {
+
+// Lists of one query point, one row of memory (list_row_bytes):
+//   ListNear | B skip | A distances | A points | B distances | B points
+// A holds exactly the valid points with d_YZ < ra, ascending by d_YZ, B those
+// with d_Z < rb, ascending by d_Z; distances are float, points byte offsets
+// into a row of X values (as the walk's shared-memory loads take them).  Both are padded to a
+// multiple of 32 entries with (+inf, 0).  skip[b] is B's distance 32 b, +inf
+// past its end.  ListNear repeats the beginning of both (+inf past their
+// ends): what most points need, in one piece that the walk copies ahead.
+//
+// Point j's place in a row of X values is j, and for one Z variable its rank
+// in the Z column: the points with d_Z < eps are then consecutive, and the
+// group has no list B.
+constexpr int kNearA = 32, kNearB = 64;
+struct __align__(16) ListNear {
+    float ra, rb;
+    uint16_t na, nb;   // entries, padding included
+    float far;         // B's distance kNearB (+inf past its end)
+    uint32_t place;    // byte offset of the query point itself
+    uint32_t pad[3];
+    float da[kNearA];
+    uint32_t oa[kNearA];
+    float db[kNearB];
+    uint32_t ob[kNearB];
+};
+static_assert(sizeof(ListNear) % 16 == 0, "copied in 16-byte pieces");
+constexpr int kListCapA = 2048, kListCapB = 4096;   // largest lists
+constexpr int kListSkip = kListCapB / 32;
+constexpr size_t kListWalkSmem = 164 * 1024;   // X values of a walking CTA
+constexpr size_t kListHalfSmem = 72 * 1024;    // of each of two CTAs on an SM
+
+__host__ __device__ inline size_t list_row_bytes(int cap_a, int cap_b)
+{
+    return sizeof(ListNear) + 4 * kListSkip + 8 * (size_t)(cap_a + cap_b);
+}
+
+// A group of members (as GroupDesc) on the list path; member block b holds
+// members b * width .. of the group.
+struct ListGroup {
+    const float *base;
+    int N, k, theiler;
+    int dy, dz, dx;
+    int ycol, zcol;          // first index into cols[] of the Y / Z column offsets
+    int member_begin, n_members, n_mblocks;
+    int cap_a, cap_b;        // list capacities, multiples of 32; cap_b = 0 when dz < 2
+    const float *zs;         // dz == 1: the Z column ascending, every point's rank in it
+    const int *rank;
+};
+
+// Query points q0 .. q0 + nq - 1 of one group, whose lists are in the pool at
+// once (a launch works through the points in such segments).
+struct ListSeg {
+    int group, q0, nq;
+    int per_cta;             // query points per walking CTA
+    int n_splits;            // walking CTAs per member block
+    long long build_item, walk_item;   // first CTA in the build / walk launch
+    unsigned char *rows;     // nq rows
+};
+
+struct ListLaunch {
+    const ListGroup *groups;
+    const ListSeg *segs;
+    int n_segs;
+    const MemberDesc *members;
+    const int *cols;
+    const int64_t *q;
+    unsigned long long *acc;
+    float *dbg_eps;
+    int *dbg_nxz, *dbg_nyz, *dbg_nz;
+    int dbg_out;
+    unsigned long long *work;   // as KsgLaunch::work [0], [1]; nullptr: not counted
+};
+
+constexpr int kListBuildThreads = 512;
+constexpr int kListWalkThreads = 1024;   // of all walking CTAs on an SM
+
+// capacities of the two lists for a group
+void list_caps(int N, int k, int dx, int dy, int dz, size_t members, int *cap_a, int *cap_b);
+// shared memory of a walking CTA: X values of width members, and for one Z
+// variable every 16th sorted Z value
+inline size_t list_walk_x_bytes(int N, int dx, int dz, int width)
+{
+    return (size_t)width * dx * (((size_t)N + 3) & ~(size_t)3) * 4 +
+           (dz == 1 ? ((size_t)(N + 15) / 16 * 4 + 15 & ~(size_t)15) : 0);
+}
+// whether a group can take the list path, and the members per walking CTA
+bool list_fits(int N, int dx, int dz);
+int list_width(int N, int dx, int dz, int k, size_t members);
+// queries per CTA of the build kernel
+int list_build_queries(int cap_a, int cap_b);
+
+// Ascending copies of columns (sorted) and the points' ranks in them (rank;
+// either may be nullptr), equal values in the order of their points.
+struct RankSortJob {
+    const float *src;
+    float *sorted;
+    int *rank;
+    int N;
+    int item;   // first CTA of the job: rank_sort_items(N) each
+};
+inline int rank_sort_items(int N) { return (N + 63) / 64; }
+cudaError_t launch_rank_sort(const RankSortJob *jobs, int n_jobs, int n_items, cudaStream_t st);
+
+cudaError_t list_prepare_attributes();
+cudaError_t launch_list_build(const ListLaunch &L, long long n_items, int queries, int cap_a,
+                              int cap_b, cudaStream_t st);
+// smem: the largest list_walk_x_bytes of the launch's groups; width members per CTA
+cudaError_t launch_list_walk(const ListLaunch &L, long long n_items, int width, bool dx1, bool k4,
+                             size_t smem, cudaStream_t st);
+
+}  // namespace teksg

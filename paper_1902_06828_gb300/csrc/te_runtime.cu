@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "te_runtime.h"
+#include "ksg_lists.h"
 #include "ksg_tune_table.h"
 
 using namespace teksg;
@@ -301,6 +302,31 @@ te_status finish_groups(te_ctx *ctx)
     return TE_OK;
 }
 
+te_status submit_work(te_ctx *ctx, const std::function<te_status()> &work)
+{
+    if (!ctx->opt_graph) return work();
+    CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal),
+       "cudaStreamBeginCapture");
+    const te_status ws = work();
+    cudaGraph_t g = nullptr;
+    const cudaError_t ce = cudaStreamEndCapture(ctx->stream, &g);
+    if (ws) {
+        if (g) cudaGraphDestroy(g);
+        return ws;
+    }
+    CK(ce, "cudaStreamEndCapture");
+    cudaGraphExec_t ge = nullptr;
+    const cudaError_t ie = cudaGraphInstantiate(&ge, g, 0);
+    cudaGraphDestroy(g);
+    CK(ie, "cudaGraphInstantiate");
+    cudaError_t le = cudaEventRecord(ctx->ev_a, ctx->stream);
+    if (le == cudaSuccess) le = cudaGraphLaunch(ge, ctx->stream);
+    if (le == cudaSuccess) le = cudaEventRecord(ctx->ev_b, ctx->stream);
+    cudaGraphExecDestroy(ge);   // released once the launched graph completes
+    CK(le, "cudaGraphLaunch");
+    return TE_OK;
+}
+
 te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n_out, int dbg_out,
                         float *dbg_eps, int *dbg_nxz, int *dbg_nyz, int *dbg_nz)
 {
@@ -312,6 +338,14 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
     if ((st = ensure_dev(ctx, ctx->ws_acc, (size_t)std::max(n_out, 1) * 16))) return st;
     if ((st = ensure_dev(ctx, ctx->ws_keys, (size_t)std::max(n_out, 1) * 16))) return st;
     CK(cudaMemsetAsync(ctx->ws_acc.p, 0, (size_t)n_out * 16, ctx->stream), "cudaMemsetAsync");
+    // Neighbour lists wherever a member's X values fit a CTA's shared memory;
+    // an option of the member-lane kernel asks for that kernel.
+    bool lists = !ctx->opt_jt && !ctx->opt_ms && !ctx->opt_persistent && !ctx->opt_order;
+    for (const HostGroup &g : groups)
+        lists = lists && list_fits(g.data->T - g.max_lag, g.dx, (int)g.z.size());
+    if (lists)
+        return launch_groups_lists(ctx, groups, n_out, dbg_out, dbg_eps, dbg_nxz, dbg_nyz,
+                                   dbg_nz);
 
     std::map<ClassKey, std::vector<const HostGroup *>> classes;
     for (const HostGroup &g : groups) {
@@ -663,9 +697,6 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
         CK(ksg_prepare_attributes(), "cudaFuncSetAttribute");
         ctx->prepared = 1;
     }
-    // The batch's device work.  With the graph option it is captured on the
-    // stream into a CUDA graph, instantiated and launched as one graph (the
-    // timing events then bracket the graph launch).
     const bool graph = ctx->opt_graph != 0;
     auto device_work = [&]() -> te_status {
         if (!ojobs.empty()) {
@@ -732,29 +763,7 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
         ctx->stats.launches++;
         return TE_OK;
     };
-    if (!graph) {
-        if ((st = device_work())) return st;
-    } else {
-        CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal),
-           "cudaStreamBeginCapture");
-        const te_status ws = device_work();
-        cudaGraph_t g = nullptr;
-        const cudaError_t ce = cudaStreamEndCapture(ctx->stream, &g);
-        if (ws) {
-            if (g) cudaGraphDestroy(g);
-            return ws;
-        }
-        CK(ce, "cudaStreamEndCapture");
-        cudaGraphExec_t ge = nullptr;
-        const cudaError_t ie = cudaGraphInstantiate(&ge, g, 0);
-        cudaGraphDestroy(g);
-        CK(ie, "cudaGraphInstantiate");
-        cudaError_t le = cudaEventRecord(ctx->ev_a, ctx->stream);
-        if (le == cudaSuccess) le = cudaGraphLaunch(ge, ctx->stream);
-        if (le == cudaSuccess) le = cudaEventRecord(ctx->ev_b, ctx->stream);
-        cudaGraphExecDestroy(ge);   // released once the launched graph completes
-        CK(le, "cudaGraphLaunch");
-    }
+    if ((st = submit_work(ctx, device_work))) return st;
     ctx->pend_timed = 1;
     ctx->pend_pair_evals = pair_evals;
     ctx->pend_members = members_total;
@@ -852,7 +861,8 @@ void te_ctx_destroy(te_ctx *ctx)
     DevBuf *bufs[] = {&ctx->ws_groups, &ctx->ws_members, &ctx->ws_cols,  &ctx->ws_acc,
                       &ctx->ws_keys,   &ctx->ws_perm,    &ctx->ws_stat,  &ctx->ws_dbg,
                       &ctx->ws_order,  &ctx->ws_ojobs,  &ctx->ws_cperm, &ctx->ws_gauss,
-                      &ctx->ws_vsort,  &ctx->ws_xval,   &ctx->ws_gtile};
+                      &ctx->ws_vsort,  &ctx->ws_xval,   &ctx->ws_gtile,
+                      &ctx->ws_lists};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);
     if (ctx->q_dev) cudaFree(ctx->q_dev);

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -67,6 +68,7 @@ struct te_ctx {
     teksg::DevBuf ws_groups, ws_members, ws_cols, ws_acc, ws_keys, ws_perm, ws_stat, ws_dbg;
     teksg::DevBuf ws_order, ws_ojobs, ws_cperm, ws_gauss, ws_vsort;
     teksg::DevBuf ws_xval;   // X-value rows of the TMA-staged lane kernel
+    teksg::DevBuf ws_lists;  // neighbour lists of the points in work
     teksg::DevBuf ws_gtile;  // cmi_gauss: the contraction's prepared B tiles and centred X
     // pinned host staging
     void *pin = nullptr;
@@ -85,7 +87,7 @@ struct te_ctx {
     // first use) and the events that fork to it and join back
     cudaStream_t aux_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    int prepared = 0;
+    int prepared = 0, prepared_lists = 0;
     te_trace_fn trace_fn = nullptr;   // te_ctx_set_trace
     void *trace_user = nullptr;
     // te_ctx_set_option: forced member-lane tile / members per lane (0 = the
@@ -141,6 +143,14 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
                         int dbg_out = -1, float *dbg_eps = nullptr, int *dbg_nxz = nullptr,
                         int *dbg_nyz = nullptr, int *dbg_nz = nullptr);
 te_status finish_groups(te_ctx *ctx);
+// launch_groups by neighbour lists (te_lists.cu), after the accumulators are set
+te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups, int n_out,
+                              int dbg_out, float *dbg_eps, int *dbg_nxz, int *dbg_nyz,
+                              int *dbg_nz);
+// Queue a batch's device work on ctx->stream: directly, or with the graph
+// option captured on the stream, instantiated and launched as one graph (the
+// timing events then bracket the graph launch).
+te_status submit_work(te_ctx *ctx, const std::function<te_status()> &work);
 
 double key_to_cmi(const te_ctx *ctx, int64_t hi, uint64_t lo, int k, int N);
 

@@ -1,0 +1,109 @@
+"""The neighbour-list kernels (the default) against the member-lane kernel,
+which a forced tile length selects: the keys are exact integers, so they are
+equal, at the sizes where the lists can go wrong: fewer points than a step of
+32 entries, one to five members (a CTA holds four, two or one), every count
+of Z variables that has its own form (none, one, several), k beyond the lanes
+of a member's group, several X variables, Theiler bands, tied distances (lists
+that stay empty) and the largest point counts of every CTA width.  The
+unpermuted estimates also equal the oracle's at the small sizes."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import paper_1902_06828_gb300 as te
+    ctx = te.Context(0)
+    yield te, ctx
+    ctx.close()
+
+
+def _both(te, ctx, jobs):
+    ctx.set_option("ksg_tile", 0)
+    _, got = te.cmi_ksg_batch(ctx, jobs, return_keys=True)
+    try:
+        ctx.set_option("ksg_tile", 256)
+        _, ref = te.cmi_ksg_batch(ctx, jobs, return_keys=True)
+    finally:
+        ctx.set_option("ksg_tile", 0)
+    return got, ref
+
+
+Z = [(0, 1), (4, 2), (0, 2), (7, 1), (1, 4), (5, 3), (8, 2), (9, 1), (6, 2)]
+
+
+@pytest.mark.parametrize("T,dz,dx,S,k,w", [
+    (13, 2, 1, 0, 4, 0), (13, 0, 1, 3, 1, 1), (40, 1, 1, 4, 4, 0), (41, 3, 1, 2, 4, 3),
+    (69, 0, 2, 1, 4, 0), (69, 2, 3, 4, 4, 2), (300, 1, 1, 5, 8, 0), (300, 1, 2, 3, 4, 5),
+    (301, 2, 1, 6, 9, 0), (301, 0, 1, 6, 16, 4), (700, 9, 1, 3, 4, 0), (700, 1, 1, 7, 16, 7),
+    (1203, 2, 1, 70, 4, 0), (1203, 1, 1, 66, 4, 11), (1203, 0, 1, 65, 4, 0),
+    (1203, 5, 4, 9, 3, 0)])
+def test_lists_equal_the_member_lane_kernel_and_the_oracle(env, T, dz, dx, S, k, w):
+    from oracle import ksg as oksg
+    te, ctx = env
+    s = np.asarray(synth.workload_var10(T=T, seed=T + dz)["series"], dtype=np.float32)
+    data = te.te_data_create(ctx, s)
+    z = Z[:dz]
+    xs = [[(2, 1 + a) for a in range(dx)], [(3, 1 + a) for a in range(dx)]]
+    jobs = [te.Job(data, x, [(0, 0)], z, k=k, theiler=w, max_lag=5, n_surr=S, seed=4,
+                   stream_tag=9) for x in xs]
+    got, ref = _both(te, ctx, jobs)
+    assert got == ref
+    for x, keys in zip(xs, got):
+        assert keys[0] == oksg.cmi_ksg(s, x, [(0, 0)], z, k=k, theiler=w, max_lag=5)["key"]
+    data.close()
+
+
+@pytest.mark.parametrize("dz", [0, 1, 2])
+@pytest.mark.parametrize("levels", [2, 7, 40])
+def test_tied_distances(env, dz, levels):
+    """Few distinct values: most distances are equal, radii end at ties, lists
+    hold nothing or stop short, and pairs scan all points."""
+    from oracle import ksg as oksg
+    te, ctx = env
+    rng = np.random.default_rng(levels + dz)
+    s = rng.integers(0, levels, size=(10, 2600)).astype(np.float32)
+    data = te.te_data_create(ctx, s)
+    jobs = [te.Job(data, [(2, 1)], [(0, 0)], Z[:dz], k=4, max_lag=5, n_surr=5, seed=1)]
+    got, _ = _both(te, ctx, jobs) if dz else (te.cmi_ksg_batch(ctx, jobs, return_keys=True)[1], 0)
+    perms = np.stack([oksg.permutation(1, 0, 0, 0, a, 2595) for a in range(1, 6)])
+    ok, _, _ = oksg.cmi_ksg_batch(s, [[(2, 1)]] * 6, [(0, 0)], Z[:dz], perms=perms,
+                                  perm_idx=[-1] + list(range(5)), k=4, max_lag=5)
+    assert got[0] == ok
+    data.close()
+
+
+@pytest.mark.parametrize("N", [10496, 10497, 20992, 20993, 41984, 41985])
+def test_largest_point_counts_of_every_width(env, N):
+    """The last N at which a CTA holds four, two and one members' X values, and
+    the first beyond (past the last, the member-lane kernel is the default)."""
+    te, ctx = env
+    rng = np.random.default_rng(N)
+    s = rng.normal(size=(3, N + 1)).astype(np.float32)
+    s[1, 1:] += 0.5 * s[0, :-1]
+    data = te.te_data_create(ctx, s)
+    for z in ([(1, 1), (2, 1)], [(1, 1)]):
+        jobs = [te.Job(data, [(0, 1)], [(1, 0)], z, k=4, max_lag=1, n_surr=4, seed=2)]
+        got, ref = _both(te, ctx, jobs)
+        assert got == ref
+    data.close()
+
+
+def test_columns_of_different_point_sets_in_one_batch(env):
+    """Jobs whose maximum lags differ read the same memory as columns of
+    different lengths; each sorts its own."""
+    from oracle import ksg as oksg
+    te, ctx = env
+    s = np.asarray(synth.workload_var10(T=400, seed=8)["series"], dtype=np.float32)
+    data = te.te_data_create(ctx, s)
+    jobs = [te.Job(data, [(2, ml)], [(0, 0)], z, k=4, max_lag=ml, n_surr=3, seed=2)
+            for ml in (2, 5) for z in ([], [(0, ml)])]
+    _, got = te.cmi_ksg_batch(ctx, jobs, return_keys=True)
+    for j, keys in zip(jobs, got):
+        o = oksg.cmi_ksg(s, j.x, j.y, j.z, k=4, max_lag=j.max_lag)
+        assert keys[0] == o["key"], (j.max_lag, j.z)
+    data.close()
