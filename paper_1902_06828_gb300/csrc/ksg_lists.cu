@@ -63,7 +63,7 @@ __device__ __forceinline__ int last_at_or_below(int n, long long item, F first)
 
 struct RowPtrs {
     ListNear *near;
-    float *skip, *d_a, *d_b;
+    float *skip_a, *skip_b, *d_a, *d_b;
     uint32_t *j_a, *j_b;
 };
 
@@ -72,8 +72,9 @@ __device__ __forceinline__ RowPtrs row_ptrs(unsigned char *rows, int row, int ca
     RowPtrs r;
     unsigned char *p = rows + (size_t)row * list_row_bytes(cap_a, cap_b);
     r.near = reinterpret_cast<ListNear *>(p);
-    r.skip = reinterpret_cast<float *>(p + sizeof(ListNear));
-    r.d_a = r.skip + kListSkip;
+    r.skip_a = reinterpret_cast<float *>(p + sizeof(ListNear));
+    r.skip_b = r.skip_a + kSkipA;
+    r.d_a = r.skip_b + kSkipB;
     r.j_a = reinterpret_cast<uint32_t *>(r.d_a + cap_a);
     r.d_b = reinterpret_cast<float *>(r.j_a + cap_a);
     r.j_b = reinterpret_cast<uint32_t *>(r.d_b + cap_b);
@@ -114,7 +115,7 @@ __device__ __forceinline__ void team_sync(int t)
 }
 
 // One team sorts n entries (any order) ascending into its list of row R, pads
-// the list to a multiple of 32 and writes its near part (and B's skip row).
+// the list to a multiple of 32 and writes its near part and skip row.
 // Counting sort into kBins equal parts of [0, top] (the bin is a
 // non-decreasing function of the distance), then every entry's rank inside
 // its bin by comparison.  bins: kBins ints, idx: n shorts.  Returns the
@@ -125,14 +126,14 @@ __device__ int team_list_sort(const Entry *ent, int n, float top, int *bins, uin
     const int tid = threadIdx.x % kTeam;
     float *d = list_b ? R.d_b : R.d_a, *nd = list_b ? R.near->db : R.near->da;
     uint32_t *j = list_b ? R.j_b : R.j_a, *no = list_b ? R.near->ob : R.near->oa;
-    const int n_near = list_b ? kNearB : kNearA;
+    float *skip = list_b ? R.skip_b : R.skip_a;
+    const int n_near = list_b ? kNearB : kNearA, n_skip = list_b ? kSkipB : kSkipA;
     const float scale = top > 0.f && top < 3e38f ? (float)kBins / top : 0.f;
     auto bin_of = [&](float v) { return min((int)(v * scale), kBins - 1); };
     for (int b = tid; b < kBins; b += kTeam) bins[b] = 0;
-    if (list_b) {
-        for (int b = tid; b < kListSkip; b += kTeam) R.skip[b] = CUDART_INF_F;
-        if (tid == 0) R.near->far = CUDART_INF_F;
-    }
+    for (int b = tid; b < n_skip; b += kTeam) skip[b] = CUDART_INF_F;
+    float *far = list_b ? &R.near->far_b : &R.near->far_a;
+    if (tid == 0) *far = CUDART_INF_F;
     for (int b = n + tid; b < n_near; b += kTeam) {
         nd[b] = CUDART_INF_F;
         no[b] = 0;
@@ -175,10 +176,8 @@ __device__ int team_list_sort(const Entry *ent, int n, float top, int *bins, uin
             nd[r] = me.d;
             no[r] = place;
         }
-        if (list_b) {
-            if ((r & 31) == 0) R.skip[r >> 5] = me.d;
-            if (r == kNearB) R.near->far = me.d;
-        }
+        if ((r & 31) == 0) skip[r >> 5] = me.d;
+        if (r == n_near) *far = me.d;
     }
     const int padded = (n + 31) & ~31;
     if (tid < padded - n) {
@@ -353,7 +352,7 @@ __global__ void __launch_bounds__(kListBuildThreads) list_build_kernel(const Lis
                 if (cap[1] == 0) {
                     R.near->rb = CUDART_INF_F;
                     R.near->nb = 0;
-                    R.near->far = CUDART_INF_F;
+                    R.near->far_b = CUDART_INF_F;
                 }
             }
         }
@@ -403,27 +402,6 @@ __global__ void __launch_bounds__(256) rank_sort_kernel(const RankSortJob *jobs,
 }
 
 // ---------------- the walk ----------------
-// values of an ascending column within e > 0 of x, by exactly the pairwise
-// test (fl(col[u] - x) is non-decreasing in u, so they form one run)
-__device__ __forceinline__ int column_count(const float *__restrict__ col, int n, float x, float e)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__fsub_rn(__ldg(col + mid), x) >= e) hi = mid;
-        else lo = mid + 1;
-    }
-    const int a = lo;
-    lo = 0;
-    hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__fsub_rn(__ldg(col + mid), x) > -e) hi = mid;
-        else lo = mid + 1;
-    }
-    return a - lo;
-}
-
 // Ascending sort of the G lanes' values inside every group of G lanes.
 template <int G>
 __device__ __forceinline__ float group_sort(float v)
@@ -476,21 +454,59 @@ __device__ __forceinline__ int group_rank(const float *__restrict__ d, int n, fl
     return lo;
 }
 
+// The places of an ascending column's values within e of v: rounding is
+// monotone, so fl(v - z) >= e holds for its first lo values and fl(z - v) < e
+// for its first hi, and the values within are lo .. hi - 1 (none for e <= 0).
+// Even lanes of a group find lo, odd lanes hi, over every 16th value (coarse,
+// nc of them, in shared memory); then the group reads 16 values for each.
+template <int G>
+__device__ __forceinline__ void group_window(const float *__restrict__ z, int n,
+                                             const float *coarse, int nc, float v, float e, int &lo,
+                                             int &hi)
+{
+    const int u = threadIdx.x & (G - 1);
+    const bool up = u & 1;
+    int a = 0, b = nc;   // entries for which the test holds: a prefix
+    while (__any_sync(kFull, a < b)) {
+        const int mid = min((a + b) >> 1, nc - 1);
+        const float x = coarse[mid];
+        const bool in = up ? __fsub_rn(x, v) < e : __fsub_rn(v, x) >= e;
+        if (a < b) {
+            if (in) a = mid + 1;
+            else b = mid;
+        }
+    }
+    const int cl = __shfl_sync(kFull, a, 0, G), ch = __shfl_sync(kFull, a, 1, G);
+    const int bl = 16 * max(cl - 1, 0), bh = 16 * max(ch - 1, 0);
+    int fl = 0, fh = 0;
+#pragma unroll
+    for (int t = u; t < 16; t += G) {
+        if (bl + t < n) fl += __fsub_rn(v, __ldg(z + bl + t)) >= e ? 1 : 0;
+        if (bh + t < n) fh += __fsub_rn(__ldg(z + bh + t), v) < e ? 1 : 0;
+    }
+    int s = fl | (fh << 16);   // both below 17
+#pragma unroll
+    for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    lo = bl + (s & 0xffff);
+    hi = bh + (s >> 16);
+    if (!(e > 0.f)) hi = lo;
+}
+
 // One member at query point i over all points, by the whole CTA: its k-th
 // smallest joint distance and the three counts, added to the accumulators.
 // Blocks of 32 points go round the warps, four of a warp's in flight; every
 // warp keeps the smallest distances it meets, and the warps' k smallest are
 // merged through shared memory.  xm: the member's X values in shared memory,
-// dimension d of point j at d * xs + (j's place); col and q: the Y then Z columns and
+// dimension d of point j at sp * (j's place) + d * sd; col and q: the Y then Z columns and
 // the point's values in them; top: 32 * k floats, cnt: three ints.
-template <bool DX1>
 __device__ __noinline__ void scan_member(const ListLaunch &L, const ListGroup &G,
                                          const float *const *col, const float *q, int i,
-                                         const float *xm, int xs, int out, float *top, int *cnt)
+                                         const float *xm, int sp, int sd, int out, float *top,
+                                         int *cnt)
 {
     constexpr int U = 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    const int N = G.N, dx = DX1 ? 1 : G.dx, dy = G.dy, dyz = G.dy + G.dz, k = G.k, w = G.theiler;
+    const int N = G.N, dx = G.dx, dy = G.dy, dyz = G.dy + G.dz, k = G.k, w = G.theiler;
     const int stride = 32 * n_warps;
     const int pi = G.rank ? G.rank[i] : i;
     auto dist = [&](int j0, float (&vx)[U], float (&vz)[U], float (&vyz)[U]) {
@@ -500,10 +516,10 @@ __device__ __noinline__ void scan_member(const ListLaunch &L, const ListGroup &G
             j[u] = min(j0 + stride * u, N - 1);
             vz[u] = -CUDART_INF_F;
             const int pj = G.rank ? __ldg(G.rank + j[u]) : j[u];
-            vx[u] = fabsf(__fsub_rn(xm[pi], xm[pj]));
-            if (!DX1)
-                for (int d = 1; d < dx; ++d)
-                    vx[u] = fmaxf(vx[u], fabsf(__fsub_rn(xm[d * xs + pi], xm[d * xs + pj])));
+            vx[u] = fabsf(__fsub_rn(xm[sp * pi], xm[sp * pj]));
+            for (int d = 1; d < dx; ++d)
+                vx[u] = fmaxf(vx[u],
+                              fabsf(__fsub_rn(xm[sp * pi + d * sd], xm[sp * pj + d * sd])));
         }
 #pragma unroll 2
         for (int d = dy; d < dyz; ++d) {
@@ -581,6 +597,21 @@ __device__ __noinline__ void scan_member(const ListLaunch &L, const ListGroup &G
         }
     }
     __syncthreads();
+}
+
+// E consecutive distances (E = 1, 2 or 4, aligned to E)
+template <int E>
+__device__ __forceinline__ void load_vec(const float *dp, float (&d)[E])
+{
+    if constexpr (E == 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(dp);
+        d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+    } else if constexpr (E == 2) {
+        const float2 v = *reinterpret_cast<const float2 *>(dp);
+        d[0] = v.x; d[1] = v.y;
+    } else {
+        d[0] = *dp;
+    }
 }
 
 // E consecutive entries of a list (E = 1, 2 or 4, aligned to E)
@@ -671,66 +702,85 @@ struct Nearest {
     }
 };
 
-// One CTA: 32 / G members of one group, their X values in shared memory, x a
-// range of query points.  A warp takes a query point at a time, G lanes per
-// member and 32 list entries per member at a time, all members at once; only
-// a long prefix of B (n_xz) goes over the whole warp, 128 entries at a time
-// for every member that reaches them.  A point's near lists are copied one
-// point ahead, and the digamma values that end its work are added one point
-// later: a warp's time is a chain of memory and shuffle latencies more than of
-// issue slots.
-template <int G, bool DX1, bool K4>
-__global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListLaunch L)
+// One CTA: `width` members of one group, their X values in shared memory, x a
+// range of query points.  A warp serves NG = 32 / G (point, member) pairs at a
+// time, G lanes each and 32 list entries at a time: `width` members at
+// NG / width points.  Only a long prefix (n_xz) goes over the whole warp, 128
+// entries at a time.  With NG members (NEAR) the warp's one point has its
+// near lists copied a point ahead; the digamma values that end a pair's work
+// are added a point later: a warp's time is a chain of memory and shuffle
+// latencies more than of issue slots.
+// DXP: X variables as stored, dimensions of a point together: 1, 2 or 4 (three
+// or four variables), so that a point's values are one load; 0: any number, a
+// row per dimension.
+template <int G, bool NEAR, int DXP, bool K4>
+__global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListLaunch L,
+                                                                     const int width)
 {
-    constexpr int MW = 32 / G;
+    constexpr int NG = 32 / G;
     constexpr int E = 32 / G;       // entries per lane of a 32-entry step
-    // [2][warps] ListNear, [MW][dx][xs_dim] X, dz == 1: every 16th sorted Z
+    constexpr int XR = DXP > 0 ? DXP : 1;
+    // NEAR: [2][warps] ListNear; X of every member; coarse sorted columns
     extern __shared__ __align__(16) unsigned char wsm[];
     __shared__ const float *s_col[32];
     __shared__ float s_q[32];                     // a point's Y and Z values
+    __shared__ float s_top[32 * 16];
     __shared__ int s_cnt[3];
-    // pairs beyond the lists' radii: bit (point of the CTA) * MW + member
+    // pairs beyond the lists' radii: bit (point of the CTA) * width + member
     __shared__ uint32_t s_slow[kListWalkSmem / 4 / 32 + 1];
     const long long item = blockIdx.x;
     const ListSeg &S = L.segs[last_at_or_below(L.n_segs, item,
                                                [&](int a) { return L.segs[a].walk_item; })];
     const ListGroup &Gr = L.groups[S.group];
-    const int N = Gr.N, dx = DX1 ? 1 : Gr.dx, w = Gr.theiler, k = K4 ? 4 : Gr.k, dz = Gr.dz;
+    const int N = Gr.N, dx = DXP == 1 ? 1 : Gr.dx, w = Gr.theiler, k = K4 ? 4 : Gr.k, dz = Gr.dz;
     const int dyz = Gr.dy + dz;
     const long long local = item - S.walk_item;
     const int mb = (int)(local / S.n_splits), split = (int)(local % S.n_splits);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const int u = lane & (G - 1), g = lane / G;
+    const int gm = NEAR ? g : g & (width - 1);         // the group's member and
+    const int qw = NEAR ? 1 : NG / width;              // point, of qw at a time
     const int cap_a = Gr.cap_a, cap_b = Gr.cap_b;
-    const int nm = min(MW, Gr.n_members - mb * MW);
-    const int xd = (N + 3) & ~3, xn = dx * xd;   // X values of a dimension, of a member
+    const int nm = min(width, Gr.n_members - mb * width);
+    const int xd = (N + 3) & ~3;
+    const int xn = (DXP > 0 ? DXP : dx) * xd;          // X values of a member
+    const int sp = XR, sd = DXP > 0 ? 1 : xd;          // strides of a point, of a dimension
     ListNear *near_buf = reinterpret_cast<ListNear *>(wsm) + 2 * warp;
-    float *xs = reinterpret_cast<float *>(reinterpret_cast<ListNear *>(wsm) + 2 * n_warps);
-    float *zc = xs + MW * xn;
+    float *xs = reinterpret_cast<float *>(reinterpret_cast<ListNear *>(wsm) +
+                                          (NEAR ? 2 * n_warps : 0));
+    float *coarse = xs + width * xn;
     const int nc = (N + 15) / 16;
+    const bool xsorted = DXP == 1 && dz == 0;
 
-    for (int m = 0; m < MW; ++m) {
+    for (int m = 0; m < width; ++m) {
         // past the last member: the last one again, its results dropped
-        const MemberDesc md = L.members[Gr.member_begin + mb * MW + min(m, nm - 1)];
+        const MemberDesc md = L.members[Gr.member_begin + mb * width + min(m, nm - 1)];
         for (int d = 0; d < dx; ++d) {
             const float *src = Gr.base + L.cols[md.xcol + d];
-            float *dst = xs + m * xn + d * xd;
+            float *dst = xs + m * xn + d * sd;
 #pragma unroll 4
             for (int j = threadIdx.x; j < N; j += blockDim.x)
-                dst[dz == 1 ? __ldg(Gr.rank + j) : j] =
+                dst[sp * (dz == 1 ? __ldg(Gr.rank + j) : j)] =
                     __ldg(src + (md.perm ? __ldg(md.perm + j) : j));
         }
+        if (DXP > 2 && dx < DXP)   // the unused dimensions add nothing to a maximum
+            for (int j = threadIdx.x; j < N; j += blockDim.x)
+                for (int d = dx; d < DXP; ++d) xs[m * xn + DXP * j + d] = 0.f;
+        if (xsorted)
+            for (int c = threadIdx.x; c < nc; c += blockDim.x)
+                coarse[m * nc + c] = __ldg(md.xsorted + 16 * c);
     }
     if (dz == 1)
-        for (int c = threadIdx.x; c < nc; c += blockDim.x) zc[c] = Gr.zs[16 * c];
+        for (int c = threadIdx.x; c < nc; c += blockDim.x) coarse[c] = __ldg(Gr.zs + 16 * c);
     if (threadIdx.x < dyz)
         s_col[threadIdx.x] = Gr.base + (threadIdx.x < Gr.dy
                                             ? L.cols[Gr.ycol + threadIdx.x]
                                             : L.cols[Gr.zcol + threadIdx.x - Gr.dy]);
     const int q_first = split * S.per_cta, q_last = min(S.nq, q_first + S.per_cta);
-    for (int a = threadIdx.x; a <= (q_last - q_first) * MW / 32; a += blockDim.x) s_slow[a] = 0;
-    const char *xm = reinterpret_cast<const char *>(xs + g * xn);
-    // A member's sum of digamma values: its group's lanes 0, 1, 2 sum those of
+    const int n_words = (q_last - q_first) * width / 32 + 1;
+    for (int a = threadIdx.x; a < n_words; a += blockDim.x) s_slow[a] = 0;
+    const char *xm = reinterpret_cast<const char *>(xs + gm * xn);
+    // A pair's sum of digamma values: its group's lanes 0, 1, 2 sum those of
     // n_z, -n_xz and -n_yz (the low 32 bits and the rest apart, as the
     // accumulators keep them: a long run would not fit in one int64).
     unsigned long long sum_lo = 0;
@@ -738,11 +788,26 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
     unsigned evals = 0;   // member-pairs evaluated by the warp
     __syncthreads();
 
-    // d_X between the query point and the point at byte offset o, for the X
-    // values at x (xi: the query point's first one, oi: its byte offset)
-    auto dist_x = [&](const char *x, float xi, uint32_t oi, uint32_t o) {
-        float v = fabsf(__fsub_rn(xi, *reinterpret_cast<const float *>(x + o)));
-        if (!DX1)
+    // the X values at byte offset o of the row x
+    auto load_x = [&](const char *x, uint32_t o, float (&v)[XR]) {
+        if constexpr (DXP == 4) {
+            const float4 t = *reinterpret_cast<const float4 *>(x + 4 * o);
+            v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+        } else if constexpr (DXP == 2) {
+            const float2 t = *reinterpret_cast<const float2 *>(x + 2 * o);
+            v[0] = t.x; v[1] = t.y;
+        } else {
+            v[0] = *reinterpret_cast<const float *>(x + o);
+        }
+    };
+    // d_X between the query point (values xi, byte offset oi) and the point at o
+    auto dist_x = [&](const char *x, const float (&xi)[XR], uint32_t oi, uint32_t o) {
+        float t[XR];
+        load_x(x, o, t);
+        float v = fabsf(__fsub_rn(xi[0], t[0]));
+#pragma unroll
+        for (int d = 1; d < XR; ++d) v = fmaxf(v, fabsf(__fsub_rn(xi[d], t[d])));
+        if (DXP == 0)
             for (int d = 1; d < dx; ++d) {
                 const char *r = x + 4 * d * xd;
                 v = fmaxf(v, fabsf(__fsub_rn(*reinterpret_cast<const float *>(r + oi),
@@ -772,25 +837,34 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
         sum_hi += q_last_term >> 32;
     };
     int half = 0;
-    fetch(q_first + warp, 0);
-    for (int row = q_first + warp; row < q_last; row += n_warps, half ^= 1) {
+    if (NEAR) fetch(q_first + warp, 0);
+    for (int first_row = q_first + warp * qw; first_row < q_last;
+         first_row += n_warps * qw, half ^= 1) {
+        // a group past the last point repeats it, its result dropped
+        const int row_g = NEAR ? first_row : first_row + g / width;
+        const int row = NEAR ? first_row : min(row_g, q_last - 1);
+        const bool live = gm < nm && row_g < q_last;
         const int i = q0 + row;
         const RowPtrs R = row_ptrs(rows, row, cap_a, cap_b);
-        __syncwarp();   // the other half's readers are done
-        fetch(row + n_warps, half ^ 1);
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncwarp();
-        const ListNear &h = near_buf[half];
+        if (NEAR) {
+            __syncwarp();   // the other half's readers are done
+            fetch(first_row + n_warps, half ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
+        }
+        const ListNear &h = NEAR ? near_buf[half] : *R.near;
         const int na = h.na, nb = h.nb;
         const uint32_t oi = h.place;
-        const float xi = *reinterpret_cast<const float *>(xm + oi);
+        float xi[XR];
+        load_x(xm, oi, xi);
 
         // ---- k nearest joint distances over list A ----
         Nearest<G, K4> near;
-        int c = 0, p = 0;
+        int c = 0, p = 32;
         float da[E];   // the first 32 entries' d_YZ
+        float d[E];
+        uint32_t o[E];
         {
-            uint32_t o[E];
             float D[E];
             load_entries<E>(h.da + E * u, h.oa + E * u, da, o);
 #pragma unroll
@@ -798,37 +872,80 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
             near.add(D, k);
             evals += 32 * E;
         }
-        for (p = 32; p < na; p += 32) {
-            float d[E], D[E], dmin = CUDART_INF_F;
-            uint32_t o[E];
-            load_entries<E>(R.d_a + p + E * u, R.j_a + p + E * u, d, o);
-            if (!__any_sync(kFull, d[0] < near.thr)) break;
-            evals += 32 * E;
+        if (__any_sync(kFull, h.far_a < near.thr))
+            for (; NEAR ? p < na : __any_sync(kFull, p < na); p += 32) {
+                float D[E], dmin = CUDART_INF_F;
+                if (NEAR || p < na) {
+                    load_entries<E>(R.d_a + p + E * u, R.j_a + p + E * u, d, o);
+                } else {
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                D[e] = fmaxf(dist_x(xm, xi, oi, o[e]), d[e]);
-                dmin = fminf(dmin, D[e]);
+                    for (int e = 0; e < E; ++e) {
+                        d[e] = CUDART_INF_F;
+                        o[e] = 0;
+                    }
+                }
+                if (!__any_sync(kFull, d[0] < near.thr)) break;
+                evals += 32 * E;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    D[e] = fmaxf(dist_x(xm, xi, oi, o[e]), d[e]);
+                    dmin = fminf(dmin, D[e]);
+                }
+                if (__any_sync(kFull, dmin < near.thr)) near.add(D, k);
             }
-            if (__any_sync(kFull, dmin < near.thr)) near.add(D, k);
-        }
 
         // ---- n_yz: a rank in A ----
         const float eps = near.thr;
         const bool slow = eps > h.ra || (dz > 1 && eps > h.rb);
-        const float ec = slow ? -1.f : eps;   // below every distance for members that scan
+        const float ec = slow ? -1.f : eps;   // below every distance for pairs that scan
+        int nz = 0, nyz = 0, nxz = 0;
+        int n[NG];
+        int from = 0;   // n_z: the entries before the 32 that hold its end
+        const bool far = dz > 1 && __any_sync(kFull, ec > h.far_b);
+        if constexpr (NEAR) {
+            // the last skip distance below eps, then the 32 entries from it
+            int fa = 0;
+            const bool far_a = p > 32;
+            float2 ska = make_float2(CUDART_INF_F, CUDART_INF_F);
+            float4 skb = make_float4(CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, CUDART_INF_F);
+            if (far_a) ska = *reinterpret_cast<const float2 *>(R.skip_a + 2 * lane);
+            if (far) skb = *reinterpret_cast<const float4 *>(R.skip_b + 4 * lane);
 #pragma unroll
-        for (int e = 0; e < E; ++e) c += da[e] < ec ? 1 : 0;
-        int nyz = group_sum(c);
-        if (p > 32 && na > 32) nyz += group_rank<G>(R.d_a + 32, min(p, na) - 32, ec);
+            for (int m = 0; m < NG; ++m) {
+                const float e = __shfl_sync(kFull, ec, m * G);
+                if (far_a) {
+                    const int t = __popc(__ballot_sync(kFull, ska.x < e)) +
+                                  __popc(__ballot_sync(kFull, ska.y < e));
+                    if (g == m) fa = 32 * max(t - 1, 0);
+                }
+                if (far) {
+                    const int t = (int)__reduce_add_sync(
+                        kFull, (skb.x < e ? 1 : 0) + (skb.y < e ? 1 : 0) + (skb.z < e ? 1 : 0) +
+                                   (skb.w < e ? 1 : 0));
+                    if (g == m) from = 32 * max(t - 1, 0);
+                }
+            }
+            if (far_a) load_vec<E>(R.d_a + fa + E * u, da);
+            if (far) load_vec<E>(R.d_b + from + E * u, d);
+#pragma unroll
+            for (int e = 0; e < E; ++e) nyz += da[e] < ec ? 1 : 0;
+            nyz = fa + group_sum(nyz);
+        } else {
+#pragma unroll
+            for (int e = 0; e < E; ++e) nyz += da[e] < ec ? 1 : 0;
+            nyz = group_sum(nyz);
+            if (p > 32) nyz += group_rank<G>(R.d_a + 32, max(min(p, na) - 32, 0), ec);
+            if (far) {
+                from = 32 * max(group_rank<G>(R.skip_b, kSkipB, ec) - 1, 0);
+                load_vec<E>(R.d_b + from + E * u, d);
+            }
+        }
 
         // ---- n_z and n_xz ----
-        int nz = 0, nxz = 0;
-        if (dz > 1 && !__any_sync(kFull, ec > h.far)) {
+        if (dz > 1 && !far) {
             // every prefix of B ends within kNearB entries: counted by the groups
             int cz = 0, cx = 0;
-            for (int b = 0; b < min(nb, kNearB); b += 32) {
-                float d[E];
-                uint32_t o[E];
+            for (int b = 0; b < kNearB; b += 32) {
                 load_entries<E>(h.db + b + E * u, h.ob + b + E * u, d, o);
                 if (!__any_sync(kFull, d[0] < ec)) break;
 #pragma unroll
@@ -841,111 +958,113 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
             nz = group_sum(cz);
             nxz = group_sum(cx);
         } else if (dz > 1) {
-            // n_z: the last skip distance below eps, then the 32 entries from it
-            const float4 sk = *reinterpret_cast<const float4 *>(R.skip + 4 * lane);
-            float e[MW], xq[MW];
-            int n[MW], cm[MW], nmax = 0;
+            uint4 o_next = make_uint4(0, 0, 0, 0);
+            if (NEAR && DXP == 1)
+                o_next = *reinterpret_cast<const uint4 *>(R.j_b + min(4 * lane, nb - 4));
 #pragma unroll
-            for (int m = 0; m < MW; ++m) {
-                e[m] = __shfl_sync(kFull, ec, m * G);
-                xq[m] = __shfl_sync(kFull, xi, m * G);
-                cm[m] = 0;
-                n[m] = (int)__reduce_add_sync(
-                    kFull, (sk.x < e[m] ? 1 : 0) + (sk.y < e[m] ? 1 : 0) +
-                               (sk.z < e[m] ? 1 : 0) + (sk.w < e[m] ? 1 : 0));
-                if (g == m) nz = n[m];
-            }
-            const int from = 32 * max(nz - 1, 0);
-            {
-                float d[E];
-                uint32_t o[E];
-                load_entries<E>(R.d_b + from + E * u, R.j_b + from + E * u, d, o);
-                c = 0;
+            for (int e = 0; e < E; ++e) c += d[e] < ec ? 1 : 0;
+            c = group_sum(c);
+            nz = nb ? from + c : 0;
+            int nmax = 0;
 #pragma unroll
-                for (int a = 0; a < E; ++a) c += d[a] < ec ? 1 : 0;
-            }
-            nz = from + group_sum(c);
-#pragma unroll
-            for (int m = 0; m < MW; ++m) {
+            for (int m = 0; m < NG; ++m) {
                 n[m] = __shfl_sync(kFull, nz, m * G);
                 nmax = max(nmax, n[m]);
                 evals += n[m];
             }
-            for (int b = 0; b < nmax; b += 128) {
-                const int at = b + 4 * lane;
-                const uint4 o = *reinterpret_cast<const uint4 *>(R.j_b + min(at, nb - 4));
+            if constexpr (NEAR && DXP == 1) {   // one list: its entries are read once
+                float e[NG], xq[NG][1];
+                int cm[NG];
 #pragma unroll
-                for (int m = 0; m < MW; ++m) {
-                    if (b >= n[m]) continue;
-                    const char *x = reinterpret_cast<const char *>(xs + m * xn);
-                    const float d0 = dist_x(x, xq[m], oi, o.x), d1 = dist_x(x, xq[m], oi, o.y);
-                    const float d2 = dist_x(x, xq[m], oi, o.z), d3 = dist_x(x, xq[m], oi, o.w);
-                    if (b + 128 <= n[m]) {
-                        cm[m] += (d0 < e[m] ? 1 : 0) + (d1 < e[m] ? 1 : 0) +
-                                 (d2 < e[m] ? 1 : 0) + (d3 < e[m] ? 1 : 0);
-                    } else {
-                        cm[m] += (at < n[m] && d0 < e[m] ? 1 : 0) +
-                                 (at + 1 < n[m] && d1 < e[m] ? 1 : 0) +
-                                 (at + 2 < n[m] && d2 < e[m] ? 1 : 0) +
-                                 (at + 3 < n[m] && d3 < e[m] ? 1 : 0);
+                for (int m = 0; m < NG; ++m) {
+                    e[m] = __shfl_sync(kFull, ec, m * G);
+                    xq[m][0] = __shfl_sync(kFull, xi[0], m * G);
+                    cm[m] = 0;
+                }
+                for (int b = 0; b < nmax; b += 128) {
+                    const int at = b + 4 * lane;
+                    const uint4 o = o_next;
+                    if (b + 128 < nmax)
+                        o_next = *reinterpret_cast<const uint4 *>(R.j_b + min(at + 128, nb - 4));
+#pragma unroll
+                    for (int m = 0; m < NG; ++m) {
+                        if (b >= n[m]) continue;
+                        const char *x = reinterpret_cast<const char *>(xs + m * xn);
+                        const float d0 = dist_x(x, xq[m], oi, o.x), d1 = dist_x(x, xq[m], oi, o.y);
+                        const float d2 = dist_x(x, xq[m], oi, o.z), d3 = dist_x(x, xq[m], oi, o.w);
+                        if (b + 128 <= n[m]) {
+                            cm[m] += (d0 < e[m] ? 1 : 0) + (d1 < e[m] ? 1 : 0) +
+                                     (d2 < e[m] ? 1 : 0) + (d3 < e[m] ? 1 : 0);
+                        } else {
+                            cm[m] += (at < n[m] && d0 < e[m] ? 1 : 0) +
+                                     (at + 1 < n[m] && d1 < e[m] ? 1 : 0) +
+                                     (at + 2 < n[m] && d2 < e[m] ? 1 : 0) +
+                                     (at + 3 < n[m] && d3 < e[m] ? 1 : 0);
+                        }
                     }
                 }
-            }
 #pragma unroll
-            for (int m = 0; m < MW; ++m) {
-                const int t = (int)__reduce_add_sync(kFull, cm[m]);
-                if (g == m) nxz = t;
+                for (int m = 0; m < NG; ++m) {
+                    const int t = (int)__reduce_add_sync(kFull, cm[m]);
+                    if (g == m) nxz = t;
+                }
+            } else {
+#pragma unroll 1
+                for (int m = 0; m < NG; ++m) {
+                    const int nn = __shfl_sync(kFull, nz, m * G);
+                    if (nn == 0) continue;
+                    const float e = __shfl_sync(kFull, ec, m * G);
+                    const uint32_t oq = __shfl_sync(kFull, oi, m * G);
+                    float xq[XR];
+#pragma unroll
+                    for (int d = 0; d < XR; ++d) xq[d] = __shfl_sync(kFull, xi[d], m * G);
+                    const uint32_t *list =
+                        row_ptrs(rows, __shfl_sync(kFull, row, m * G), cap_a, cap_b).j_b;
+                    const char *x = reinterpret_cast<const char *>(
+                        xs + (NEAR ? m : m & (width - 1)) * xn);
+                    int cm = 0;
+                    for (int b = 0; b < nn; b += 128) {
+                        const int at = b + 4 * lane;
+                        if (at >= nn) continue;
+                        const uint4 o = *reinterpret_cast<const uint4 *>(list + at);
+                        cm += dist_x(x, xq, oq, o.x) < e ? 1 : 0;
+                        cm += at + 1 < nn && dist_x(x, xq, oq, o.y) < e ? 1 : 0;
+                        cm += at + 2 < nn && dist_x(x, xq, oq, o.z) < e ? 1 : 0;
+                        cm += at + 3 < nn && dist_x(x, xq, oq, o.w) < e ? 1 : 0;
+                    }
+                    cm = (int)__reduce_add_sync(kFull, cm);
+                    if (g == m) nxz = cm;
+                }
             }
         } else if (dz == 1) {
-            // The points with d_Z < eps are consecutive places lo .. hi - 1: rounding
-            // is monotone, so fl(z_i - z) >= eps holds for the first lo sorted z and
-            // fl(z - z_i) < eps for the first hi.  Even lanes find lo, odd lanes hi,
-            // over every 16th z in shared memory; then 16 z each by the group.
+            // the points with d_Z < eps are consecutive places
             const float zi = __ldg(s_col[Gr.dy] + i);
-            int lo = 0, hi = 0;
-            {
-                const bool up = u & 1;
-                int a = 0, b = nc;   // entries for which the test holds: a prefix
-                while (__any_sync(kFull, a < b)) {
-                    const int mid = min((a + b) >> 1, nc - 1);
-                    const float z = zc[mid];
-                    const bool in = up ? __fsub_rn(z, zi) < ec : __fsub_rn(zi, z) >= ec;
-                    if (a < b) {
-                        if (in) a = mid + 1;
-                        else b = mid;
-                    }
-                }
-                const int cl = __shfl_sync(kFull, a, 0, G), ch = __shfl_sync(kFull, a, 1, G);
-                const int bl = 16 * max(cl - 1, 0), bh = 16 * max(ch - 1, 0);
-                int fl = 0, fh = 0;
-                for (int t = u; t < 16; t += G) {
-                    if (bl + t < N) fl += __fsub_rn(zi, __ldg(Gr.zs + bl + t)) >= ec ? 1 : 0;
-                    if (bh + t < N) fh += __fsub_rn(__ldg(Gr.zs + bh + t), zi) < ec ? 1 : 0;
-                }
-                lo = bl + group_sum(fl);
-                hi = bh + group_sum(fh);
-                if (!(ec > 0.f)) hi = lo;   // no point is nearer than 0
-            }
+            int lo, hi;
+            group_window<G>(Gr.zs, N, coarse, nc, zi, ec, lo, hi);
             nz = hi - lo;
 #pragma unroll
-            for (int m = 0; m < MW; ++m) {
+            for (int m = 0; m < NG; ++m) {
                 const int l = __shfl_sync(kFull, lo, m * G), n = __shfl_sync(kFull, nz, m * G);
                 const float e = __shfl_sync(kFull, ec, m * G);
-                const float xq = __shfl_sync(kFull, xi, m * G);
-                const char *x = reinterpret_cast<const char *>(xs + m * xn);
+                const uint32_t oq = __shfl_sync(kFull, oi, m * G);
+                float xq[XR];
+#pragma unroll
+                for (int d = 0; d < XR; ++d) xq[d] = __shfl_sync(kFull, xi[d], m * G);
+                const char *x = reinterpret_cast<const char *>(
+                    xs + (NEAR ? m : m & (width - 1)) * xn);
                 int cm = 0;
                 for (int b = l & ~3; b < l + n; b += 128) {
                     const int at = min(b + 4 * lane, xd - 4);
                     float v[4];
-                    if constexpr (DX1) {
+                    if constexpr (DXP == 1) {
                         const float4 t = *reinterpret_cast<const float4 *>(x + 4 * at);
-                        v[0] = fabsf(__fsub_rn(xq, t.x));
-                        v[1] = fabsf(__fsub_rn(xq, t.y));
-                        v[2] = fabsf(__fsub_rn(xq, t.z));
-                        v[3] = fabsf(__fsub_rn(xq, t.w));
+                        v[0] = fabsf(__fsub_rn(xq[0], t.x));
+                        v[1] = fabsf(__fsub_rn(xq[0], t.y));
+                        v[2] = fabsf(__fsub_rn(xq[0], t.z));
+                        v[3] = fabsf(__fsub_rn(xq[0], t.w));
                     } else {
 #pragma unroll
-                        for (int a = 0; a < 4; ++a) v[a] = dist_x(x, xq, oi, 4u * (at + a));
+                        for (int a = 0; a < 4; ++a) v[a] = dist_x(x, xq, oq, 4u * (at + a));
                     }
                     if (b >= l && b + 128 <= l + n) {
 #pragma unroll
@@ -976,46 +1095,55 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
                     cz += d < ec ? 1 : 0;
                     cx += fmaxf(d, v) < ec ? 1 : 0;
                 }
+                __syncwarp();
                 nz -= group_sum(cz);
                 nxz -= group_sum(cx);
             }
         } else {
             const int first = max(i - w, 0), last = min(i + w, N - 1);
             nz = N - (last - first + 1);
-            const float *xsorted = L.members[Gr.member_begin + mb * MW + min(g, nm - 1)].xsorted;
-            c = 0;
-            if (DX1 && xsorted) {   // less the point itself and its band
+            if (xsorted) {
+                // the member's X values are its column's, in another order: a
+                // window of the sorted column, less the point itself and its band
+                int lo, hi;
+                group_window<G>(
+                    L.members[Gr.member_begin + mb * width + min(gm, nm - 1)].xsorted, N,
+                    coarse + gm * nc, nc, xi[0], ec, lo, hi);
+                c = 0;
                 for (int j = first + u; j <= last; j += G)
-                    c -= dist_x(xm, xi, oi, 4u * j) < ec ? 1 : 0;
-                if (u == 0 && ec > 0.f) c += column_count(xsorted, N, xi, ec);
+                    c += dist_x(xm, xi, oi, 4u * j) < ec ? 1 : 0;
+                __syncwarp();
+                nxz = hi - lo - group_sum(c);
             } else {
+                c = 0;
                 for (int j = u; j < N; j += G)
                     if (j < first || j > last) c += dist_x(xm, xi, oi, 4u * j) < ec ? 1 : 0;
+                __syncwarp();
+                nxz = group_sum(c);
             }
-            nxz = group_sum(c);
         }
         if (slow) {
-            if (u == 0 && g < nm) {
-                const int bit = (row - q_first) * MW + g;
+            if (u == 0 && live) {
+                const int bit = (row - q_first) * width + gm;
                 atomicOr(&s_slow[bit >> 5], 1u << (bit & 31));
             }
-            nz = nxz = nyz = -1;   // the digamma table's first value, 0
         }
+        if (slow || !live) nz = nxz = nyz = -1;   // the digamma table's first value, 0
         add_term();
         q_last_term = L.q[(u == 0 ? nz : u == 1 ? nxz : nyz) + 1];
         if (u > 0) q_last_term = -q_last_term;
-        if (L.dbg_eps && u == 0 && g < nm && !slow &&
-            L.members[Gr.member_begin + mb * MW + g].out == L.dbg_out) {
+        if (L.dbg_eps && u == 0 && live && !slow &&
+            L.members[Gr.member_begin + mb * width + gm].out == L.dbg_out) {
             L.dbg_eps[i] = eps;
             L.dbg_nxz[i] = nxz;
             L.dbg_nyz[i] = nyz;
             L.dbg_nz[i] = nz;
         }
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (NEAR) asm volatile("cp.async.wait_group 0;" ::: "memory");
     add_term();
-    if (u < 3 && g < nm) {
-        const int out = L.members[Gr.member_begin + mb * MW + g].out;
+    if (u < 3 && gm < nm) {
+        const int out = L.members[Gr.member_begin + mb * width + gm].out;
         atomicAdd(&L.acc[2 * (size_t)out], sum_lo);
         atomicAdd(&L.acc[2 * (size_t)out + 1], (unsigned long long)sum_hi);
     }
@@ -1025,7 +1153,6 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
     }
     // ---- pairs beyond the lists' radii: over all points, by the whole CTA ----
     __syncthreads();
-    const int n_words = (q_last - q_first) * MW / 32 + 1;
     for (int w0 = 0; w0 < n_words; w0 += 32) {   // the same in every warp
         const uint32_t mine = w0 + lane < n_words ? s_slow[w0 + lane] : 0;
         unsigned words = __ballot_sync(kFull, mine != 0);
@@ -1036,12 +1163,11 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
             while (bits) {
                 const int b = 32 * (w0 + src) + __ffs(bits) - 1;
                 bits &= bits - 1;
-                const int i = q0 + q_first + b / MW, m = b % MW;
+                const int i = q0 + q_first + b / width, m = b % width;
                 if (threadIdx.x < dyz) s_q[threadIdx.x] = __ldg(s_col[threadIdx.x] + i);
                 __syncthreads();
-                scan_member<DX1>(L, Gr, s_col, s_q, i, xs + m * xn, xd,
-                                 L.members[Gr.member_begin + mb * MW + m].out,
-                                 reinterpret_cast<float *>(wsm), s_cnt);
+                scan_member(L, Gr, s_col, s_q, i, xs + m * xn, sp, sd,
+                            L.members[Gr.member_begin + mb * width + m].out, s_top, s_cnt);
             }
         }
     }
@@ -1069,18 +1195,50 @@ void list_caps(int N, int k, int dx, int dy, int dz, size_t members, int *cap_a,
     *cap_b = dz > 1 ? cap(more * 14.0 * nz, kListCapB) : 0;
 }
 
-int list_width(int N, int dx, int dz, int k, size_t members)
+// X variables as stored for the walk (ListWalk's DXP): the dimensions of a
+// point together where that fits, a row per dimension (0) otherwise
+static int list_dxp(int N, int dx, int k)
 {
-    // as many members per CTA as shared memory holds; 32 / width lanes serve
-    // a member and must hold its k neighbours
-    int w = 4;
-    while (w > 1 && (list_walk_x_bytes(N, dx, dz, w) > kListWalkSmem || 32 / w < k ||
-                     (size_t)w / 2 >= members))
-        w /= 2;
-    return w;
+    if (dx == 1) return 1;
+    const int p = dx == 2 ? 2 : 4;
+    return k == 4 && dx <= 4 && (size_t)p * (((size_t)N + 3) & ~(size_t)3) * 4 <= kListWalkSmem ? p
+                                                                                               : 0;
 }
 
-bool list_fits(int N, int dx, int dz) { return list_walk_x_bytes(N, dx, dz, 1) <= kListWalkSmem; }
+size_t list_walk_x_bytes(int N, int dx, int dz, int k, int width)
+{
+    const int dxp = list_dxp(N, dx, k);
+    const size_t coarse = (((size_t)N + 15) / 16 * 4 + 15) & ~(size_t)15;
+    return (size_t)width * (dxp ? dxp : dx) * (((size_t)N + 3) & ~(size_t)3) * 4 +
+           (dz == 1 ? coarse : dz == 0 && dx == 1 ? width * coarse : 0);
+}
+
+ListShape list_shape(int N, int dx, int dz, int k, size_t members)
+{
+    // G lanes serve a pair and must hold its k neighbours; as many of a
+    // warp's pairs as shared memory allows are members of one point
+    ListShape s;
+    s.dxp = list_dxp(N, dx, k);
+    s.k4 = k == 4;
+    s.lanes = k <= 8 ? 8 : 16;
+    s.width = 32 / s.lanes;
+    // one member: a warp per point (fewer than 2^17 pairs leave warps idle, and
+    // a point's chain of steps is shorter over 32 lanes)
+    if (members == 1 && N <= 131072) {
+        s.lanes = 32;
+        s.width = 1;
+        return s;
+    }
+    while (s.width > 1 && (list_walk_x_bytes(N, dx, dz, k, s.width) > kListWalkSmem ||
+                           (size_t)s.width / 2 >= members))
+        s.width /= 2;
+    return s;
+}
+
+bool list_fits(int N, int dx, int dz, int k)
+{
+    return list_walk_x_bytes(N, dx, dz, k, 1) <= kListWalkSmem;
+}
 
 static size_t list_build_smem(int cap_a, int cap_b, int queries)
 {
@@ -1100,51 +1258,52 @@ int list_build_queries(int cap_a, int cap_b)
 constexpr int kWalkSmemMax =
     (int)(kListWalkSmem + 2 * (kListWalkThreads / 32) * sizeof(ListNear));
 
-template <int G>
-static const void *walk_kernel_g(bool dx1, bool k4)
+template <int G, bool NEAR>
+static const void *walk_kernel_g(const ListShape &s)
 {
-    if (dx1)
-        return k4 ? reinterpret_cast<const void *>(&list_walk_kernel<G, true, true>)
-                  : reinterpret_cast<const void *>(&list_walk_kernel<G, true, false>);
-    return k4 ? reinterpret_cast<const void *>(&list_walk_kernel<G, false, true>)
-              : reinterpret_cast<const void *>(&list_walk_kernel<G, false, false>);
+    if (s.k4) {
+        if constexpr (G != 16) {
+            switch (s.dxp) {
+            case 1: return reinterpret_cast<const void *>(&list_walk_kernel<G, NEAR, 1, true>);
+            case 2: return reinterpret_cast<const void *>(&list_walk_kernel<G, NEAR, 2, true>);
+            case 4: return reinterpret_cast<const void *>(&list_walk_kernel<G, NEAR, 4, true>);
+            default: return reinterpret_cast<const void *>(&list_walk_kernel<G, NEAR, 0, true>);
+            }
+        }
+        return nullptr;
+    }
+    if (s.dxp == 1) return reinterpret_cast<const void *>(&list_walk_kernel<G, NEAR, 1, false>);
+    return reinterpret_cast<const void *>(&list_walk_kernel<G, NEAR, 0, false>);
 }
 
-static const void *walk_kernel(int width, bool dx1, bool k4)
+static const void *walk_kernel(const ListShape &s)
 {
-    switch (width) {
-    case 1: return walk_kernel_g<32>(dx1, k4);
-    case 2: return walk_kernel_g<16>(dx1, k4);
-    case 4: return walk_kernel_g<8>(dx1, k4);
-    default: return nullptr;
-    }
+    if (s.lanes == 32) return walk_kernel_g<32, true>(s);
+    if (s.lanes == 8) return s.width == 4 ? walk_kernel_g<8, true>(s) : walk_kernel_g<8, false>(s);
+    return s.width == 2 ? walk_kernel_g<16, true>(s) : walk_kernel_g<16, false>(s);
 }
 
 cudaError_t list_prepare_attributes()
 {
-    const struct {
-        const void *f;
-        int bytes;
-    } fs[] = {{reinterpret_cast<const void *>(&list_build_kernel<2>), 220 * 1024},
-              {reinterpret_cast<const void *>(&list_build_kernel<4>), 220 * 1024},
-              {reinterpret_cast<const void *>(&list_build_kernel<8>), 220 * 1024},
-              {walk_kernel(1, true, true), kWalkSmemMax},
-              {walk_kernel(2, true, true), kWalkSmemMax},
-              {walk_kernel(4, true, true), kWalkSmemMax},
-              {walk_kernel(1, false, true), kWalkSmemMax},
-              {walk_kernel(2, false, true), kWalkSmemMax},
-              {walk_kernel(4, false, true), kWalkSmemMax},
-              {walk_kernel(1, true, false), kWalkSmemMax},
-              {walk_kernel(2, true, false), kWalkSmemMax},
-              {walk_kernel(4, true, false), kWalkSmemMax},
-              {walk_kernel(1, false, false), kWalkSmemMax},
-              {walk_kernel(2, false, false), kWalkSmemMax},
-              {walk_kernel(4, false, false), kWalkSmemMax}};
-    for (const auto &f : fs) {
+    const void *build[] = {reinterpret_cast<const void *>(&list_build_kernel<2>),
+                           reinterpret_cast<const void *>(&list_build_kernel<4>),
+                           reinterpret_cast<const void *>(&list_build_kernel<8>)};
+    for (const void *f : build) {
         const cudaError_t e =
-            cudaFuncSetAttribute(f.f, cudaFuncAttributeMaxDynamicSharedMemorySize, f.bytes);
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         if (e != cudaSuccess) return e;
     }
+    for (int lanes = 8; lanes <= 32; lanes *= 2)
+        for (int width = 32 / lanes; width >= 1; width /= 2)
+            for (int dxp : {1, 2, 4, 0})
+                for (int k4 = 0; k4 < 2; ++k4) {
+                    const void *f = walk_kernel(ListShape{lanes, width, dxp, k4 != 0});
+                    if (!f) continue;
+                    const cudaError_t e = cudaFuncSetAttribute(
+                        f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                        (int)(kListWalkSmem + 2 * (kListWalkThreads / 32) * sizeof(ListNear)));
+                    if (e != cudaSuccess) return e;
+                }
     return cudaSuccess;
 }
 
@@ -1163,17 +1322,18 @@ cudaError_t launch_list_build(const ListLaunch &L, long long n_items, int querie
     return cudaGetLastError();
 }
 
-cudaError_t launch_list_walk(const ListLaunch &L, long long n_items, int width, bool dx1, bool k4,
+cudaError_t launch_list_walk(const ListLaunch &L, long long n_items, const ListShape &s,
                              size_t smem, cudaStream_t st)
 {
     if (n_items <= 0) return cudaSuccess;
-    const void *f = walk_kernel(width, dx1, k4);
+    const void *f = walk_kernel(s);
     if (!f || n_items > 0x7fffffffLL || smem > kListWalkSmem) return cudaErrorInvalidValue;
     // one CTA per SM where its X values fill the shared memory, else two
     const int threads = smem > kListHalfSmem ? kListWalkThreads : kListWalkThreads / 2;
-    smem += 2 * (size_t)(threads / 32) * sizeof(ListNear);
+    if (s.width == 32 / s.lanes) smem += 2 * (size_t)(threads / 32) * sizeof(ListNear);
     ListLaunch arg = L;
-    void *args[] = {&arg};
+    int width = s.width;
+    void *args[] = {&arg, &width};
     return cudaLaunchKernel(f, dim3((unsigned)n_items), dim3(threads), args, smem, st);
 }
 

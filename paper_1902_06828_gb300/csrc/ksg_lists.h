@@ -2,17 +2,19 @@
 // (te_lists.cu, te_static.cu) and the kernels (ksg_lists.cu).
 #pragma once
 
+#include <tuple>
+
 #include "ksg_internal.h"
 
 namespace teksg {
 
 // Lists of one query point, one row of memory (list_row_bytes):
-//   ListNear | B skip | A distances | A points | B distances | B points
+//   ListNear | A skip | B skip | A distances | A points | B distances | B points
 // A holds exactly the valid points with d_YZ < ra, ascending by d_YZ, B those
 // with d_Z < rb, ascending by d_Z; distances are float, points byte offsets
 // into a row of X values (as the walk's shared-memory loads take them).  Both are padded to a
-// multiple of 32 entries with (+inf, 0).  skip[b] is B's distance 32 b, +inf
-// past its end.  ListNear repeats the beginning of both (+inf past their
+// multiple of 32 entries with (+inf, 0).  skip[b] is a list's distance 32 b,
+// +inf past its end.  ListNear repeats the beginning of both (+inf past their
 // ends): what most points need, in one piece that the walk copies ahead.
 //
 // Point j's place in a row of X values is j, and for one Z variable its rank
@@ -22,9 +24,9 @@ constexpr int kNearA = 32, kNearB = 64;
 struct __align__(16) ListNear {
     float ra, rb;
     uint16_t na, nb;   // entries, padding included
-    float far;         // B's distance kNearB (+inf past its end)
-    uint32_t place;    // byte offset of the query point itself
-    uint32_t pad[3];
+    float far_a, far_b;   // A's distance kNearA, B's distance kNearB (+inf past their ends)
+    uint32_t place;       // byte offset of the query point itself
+    uint32_t pad[2];
     float da[kNearA];
     uint32_t oa[kNearA];
     float db[kNearB];
@@ -32,13 +34,13 @@ struct __align__(16) ListNear {
 };
 static_assert(sizeof(ListNear) % 16 == 0, "copied in 16-byte pieces");
 constexpr int kListCapA = 2048, kListCapB = 4096;   // largest lists
-constexpr int kListSkip = kListCapB / 32;
+constexpr int kSkipA = kListCapA / 32, kSkipB = kListCapB / 32;
 constexpr size_t kListWalkSmem = 164 * 1024;   // X values of a walking CTA
 constexpr size_t kListHalfSmem = 72 * 1024;    // of each of two CTAs on an SM
 
 __host__ __device__ inline size_t list_row_bytes(int cap_a, int cap_b)
 {
-    return sizeof(ListNear) + 4 * kListSkip + 8 * (size_t)(cap_a + cap_b);
+    return sizeof(ListNear) + 4 * (kSkipA + kSkipB) + 8 * (size_t)(cap_a + cap_b);
 }
 
 // A group of members (as GroupDesc) on the list path; member block b holds
@@ -83,16 +85,23 @@ constexpr int kListWalkThreads = 1024;   // of all walking CTAs on an SM
 
 // capacities of the two lists for a group
 void list_caps(int N, int k, int dx, int dy, int dz, size_t members, int *cap_a, int *cap_b);
-// shared memory of a walking CTA: X values of width members, and for one Z
-// variable every 16th sorted Z value
-inline size_t list_walk_x_bytes(int N, int dx, int dz, int width)
-{
-    return (size_t)width * dx * (((size_t)N + 3) & ~(size_t)3) * 4 +
-           (dz == 1 ? ((size_t)(N + 15) / 16 * 4 + 15 & ~(size_t)15) : 0);
-}
-// whether a group can take the list path, and the members per walking CTA
-bool list_fits(int N, int dx, int dz);
-int list_width(int N, int dx, int dz, int k, size_t members);
+// Walk variant of a group: lanes per (point, member) pair, members per CTA, X
+// storage (1, 2, 4: a point's dimensions together; 0: a row per dimension),
+// k = 4.
+struct ListShape {
+    int lanes, width, dxp;
+    bool k4;
+    bool operator<(const ListShape &o) const
+    {
+        return std::tie(lanes, width, dxp, k4) < std::tie(o.lanes, o.width, o.dxp, o.k4);
+    }
+};
+ListShape list_shape(int N, int dx, int dz, int k, size_t members);
+// shared memory of a walking CTA: X values of width members, and every 16th
+// value of the sorted columns that the group's counts search
+size_t list_walk_x_bytes(int N, int dx, int dz, int k, int width);
+// whether a group can take the list path
+bool list_fits(int N, int dx, int dz, int k);
 // queries per CTA of the build kernel
 int list_build_queries(int cap_a, int cap_b);
 
@@ -111,8 +120,8 @@ cudaError_t launch_rank_sort(const RankSortJob *jobs, int n_jobs, int n_items, c
 cudaError_t list_prepare_attributes();
 cudaError_t launch_list_build(const ListLaunch &L, long long n_items, int queries, int cap_a,
                               int cap_b, cudaStream_t st);
-// smem: the largest list_walk_x_bytes of the launch's groups; width members per CTA
-cudaError_t launch_list_walk(const ListLaunch &L, long long n_items, int width, bool dx1, bool k4,
+// smem: the largest list_walk_x_bytes of the launch's groups, all of shape s
+cudaError_t launch_list_walk(const ListLaunch &L, long long n_items, const ListShape &s,
                              size_t smem, cudaStream_t st);
 
 }  // namespace teksg

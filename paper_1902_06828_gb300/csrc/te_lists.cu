@@ -23,10 +23,10 @@ constexpr size_t kListPoolBytes = (size_t)256 << 20;
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// Groups of one walk variant (one or several X variables, members per CTA).
+// Groups of one walk variant.
 struct ClassPlan {
-    int first_group = 0, width = 1;
-    bool dx1 = true, k4 = true;
+    int first_group = 0;
+    ListShape shape{};
     size_t smem = 0;
 };
 
@@ -47,14 +47,12 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device),
        "cudaDeviceGetAttribute");
-    // (one X variable, k == 4, members per CTA)
-    std::map<std::tuple<bool, bool, int>, std::vector<const HostGroup *>> classes;
+    std::map<ListShape, std::vector<const HostGroup *>> classes;
     for (const HostGroup &g : groups)
-        if (!g.members.empty()) {
-            const int width = list_width(g.data->T - g.max_lag, g.dx, (int)g.z.size(), g.k,
-                                         g.members.size());
-            classes[{g.dx == 1, g.k == 4, width}].push_back(&g);
-        }
+        if (!g.members.empty())
+            classes[list_shape(g.data->T - g.max_lag, g.dx, (int)g.z.size(), g.k,
+                               g.members.size())]
+                .push_back(&g);
 
     std::vector<ListGroup> lg;
     std::vector<MemberDesc> mdesc;
@@ -75,10 +73,11 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
     for (auto &kv : classes) {
         ClassPlan cp;
         cp.first_group = (int)lg.size();
-        std::tie(cp.dx1, cp.k4, cp.width) = kv.first;
+        cp.shape = kv.first;
         for (const HostGroup *g : kv.second)
             cp.smem = std::max(cp.smem, list_walk_x_bytes(g->data->T - g->max_lag, g->dx,
-                                                          (int)g->z.size(), cp.width));
+                                                          (int)g->z.size(), g->k,
+                                                          cp.shape.width));
         Chunk ch;
         size_t used = 0;
         auto close_chunk = [&]() {
@@ -153,7 +152,7 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
             const bool xsorted = g.z.empty() && g.dx == 1;
             G.member_begin = (int)mdesc.size();
             G.n_members = (int)g.members.size();
-            G.n_mblocks = (G.n_members + cp.width - 1) / cp.width;
+            G.n_mblocks = (G.n_members + cp.shape.width - 1) / cp.shape.width;
             for (const HostMember &hm : g.members) {
                 if (xsorted)
                     msorted.emplace_back(mdesc.size(), sorted_job(off(g.xvars[hm.xcol_first])));
@@ -274,8 +273,7 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
             L.n_segs = ch.n_segs;
             CK(launch_list_build(L, ch.build_items, ch.queries, ch.cap_a, ch.cap_b, ctx->stream),
                "list build launch");
-            CK(launch_list_walk(L, ch.walk_items, cp.width, cp.dx1, cp.k4, cp.smem,
-                                ctx->stream),
+            CK(launch_list_walk(L, ch.walk_items, cp.shape, cp.smem, ctx->stream),
                "list walk launch");
             ctx->stats.launches += 2;
             ctx->stats.ksg_launches++;

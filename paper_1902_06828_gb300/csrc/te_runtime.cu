@@ -342,7 +342,7 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
     // an option of the member-lane kernel asks for that kernel.
     bool lists = !ctx->opt_jt && !ctx->opt_ms && !ctx->opt_persistent && !ctx->opt_order;
     for (const HostGroup &g : groups)
-        lists = lists && list_fits(g.data->T - g.max_lag, g.dx, (int)g.z.size());
+        lists = lists && list_fits(g.data->T - g.max_lag, g.dx, (int)g.z.size(), g.k);
     if (lists)
         return launch_groups_lists(ctx, groups, n_out, dbg_out, dbg_eps, dbg_nxz, dbg_nyz,
                                    dbg_nz);
