@@ -1443,7 +1443,7 @@ __device__ __forceinline__ int fy_draw(uint64_t st, int n, int i)
 }
 
 // The same shuffle for n <= 65535 with the permutation as 16-bit values in
-// shared memory (2 bytes per point), the result widened into out.  Warp 0
+// shared memory (2 bytes per point).  Warp 0
 // walks the steps i = n-1 down to 1 in windows of 32, lane l holding step
 // hi - l and its draw j.  Each round applies at once the longest leading run
 // of steps whose swaps touch pairwise distinct positions: a step with j != i
@@ -1453,7 +1453,7 @@ __device__ __forceinline__ int fy_draw(uint64_t st, int n, int i)
 // window's draws come from this window's (shifted) and from draws computed
 // one window ahead.  No draw is stored, so a CTA needs only the permutation
 // and one warp.  Called by the whole CTA.
-__device__ void fy_shuffle16(uint16_t *p, int n, uint64_t st, int32_t *out)
+__device__ void fy_shuffle16(uint16_t *p, int n, uint64_t st)
 {
     for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = (uint16_t)i;
     __syncthreads();
@@ -1500,70 +1500,100 @@ __device__ void fy_shuffle16(uint16_t *p, int n, uint64_t st, int32_t *out)
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = (int32_t)p[i];
 }
 
-// One round of fy_shuffle16's warp walk for a permutation p (state: the top
-// step hi and this lane's draw jc).  Called by the whole warp while hi >= 1.
-__device__ __forceinline__ void fy16_round(uint16_t *p, int n, uint64_t st, int &hi, int &jc)
+// The shuffle for n <= kFyLinkMaxN without its serial chain.  Step i swaps
+// positions i and j_i and leaves position i final, so p[i] is what position
+// j_i holds at that time: what the last earlier step s > i with the same draw
+// moved there, i.e. what position s held before its own step, or j_i itself if
+// there is none.  Position s held, by the same argument, what the position
+// first(s) held, first(x) = the smallest step above x that drew x, and so on
+// until a position that no earlier step drew.  So with the steps grouped by
+// their draw (linked lists built by atomic exchanges, one step per position
+// on average) and the chains of first links shortened by pointer jumping (they
+// are about ln(n / x) long), every p[i] is found by itself.  The result equals the
+// sequential loop for any draws.
+// The swapping walk is a chain of 380 dependent rounds of one warp at n = 10^4;
+// here a CTA's threads work side by side, bound by issue (78%) and
+// shared-memory wavefronts (60%) once the chip is full.  Walk -> links, one
+// launch on one GB300: n = 10^4, 200 permutations 138 -> 34 us, 1000 141 -> 104,
+// 4000 451 -> 380; n = 3000, 1000 56 -> 36; n = 1000, 200 29 -> 15.
+// smem: fy_link_bytes(n) bytes; the permutation is left in the returned array.
+constexpr int kFyLinkMaxN = 20480;
+__host__ __device__ inline size_t fy_link_bytes(int n) { return 10 * (((size_t)n + 7) & ~(size_t)7); }
+// about ten points a thread: with 10 bytes a point, the CTAs that fit an SM's
+// shared memory then fill its threads
+inline int fy_link_threads(int n)
 {
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const unsigned lower = (1u << lane) - 1u;
-    const int i = hi - lane;
-    const bool valid = i >= 1;
-    const int j = valid ? jc : -1 - lane;   // invalid lanes: distinct dummies
-    const int is = hi - 32 - lane;
-    const int js = is >= 1 ? fy_draw(st, n, is) : 0;
-    int lim = !valid ? 0 : (j == i ? 32 : hi - j);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(full, lim, o);
-        if (lane >= o) lim = min(lim, t);
-    }
-    const unsigned same = __match_any_sync(full, j);
-    const unsigned run = __ballot_sync(full, valid && lane < lim && (same & lower) == 0);
-    const int k = run == full ? 32 : __ffs(~run) - 1;   // >= 1: step hi always applies
-    const bool act = lane < k && j != i;
-    uint16_t a = 0, b = 0;
-    if (act) {
-        a = p[i];
-        b = p[j];
-    }
-    __syncwarp();
-    if (act) {
-        p[i] = b;
-        p[j] = a;
-    }
-    __syncwarp();
-    const int from_cur = __shfl_down_sync(full, j, k & 31);
-    const int from_ahead = __shfl_sync(full, js, (lane + k - 32) & 31);
-    jc = lane < 32 - k ? from_cur : from_ahead;
-    hi -= k;
+    int t = 128;
+    while (t < 1024 && 10 * t < n) t *= 2;
+    return t;
 }
 
-// The same permutations as fisher_yates_kernel (16-bit mode), written as
-// 16-bit rows of `pitch` entries (a multiple of 8, zeros past n): one warp per
-// permutation, the rounds of fy_shuffle16.  (Two walks interleaved in one warp
-// were measured 1.5x slower: the rounds' warp collectives and __syncwarp keep
-// the two chains from overlapping, and half as many warps remain.)
+__device__ const uint16_t *fy_links(unsigned char *smem, int n, uint64_t st)
+{
+    const int m = (n + 7) & ~7;
+    uint32_t *head = reinterpret_cast<uint32_t *>(smem);        // last step with this draw, 0 none
+    uint16_t *next = reinterpret_cast<uint16_t *>(head + m);    // next step of the list
+    uint16_t *first = next + m;                                 // first(x), 0 none
+    uint16_t *p = first + m;
+    for (int x = threadIdx.x; x < n; x += blockDim.x) head[x] = 0;
+    __syncthreads();
+    for (int i = 1 + threadIdx.x; i < n; i += blockDim.x) {
+        const int j = fy_draw(st, n, i);
+        p[i] = (uint16_t)j;   // kept here until p[i] is known
+        next[i] = (uint16_t)atomicExch(&head[j], (uint32_t)i);
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < n; x += blockDim.x) {
+        int f = 0;
+        for (int i = (int)head[x]; i; i = next[i])
+            if (i > x && (f == 0 || i < f)) f = i;
+        first[x] = (uint16_t)f;
+    }
+    // first[x] -> the end of x's chain, by pointer jumping (any value read on the
+    // way is a step further up the same chain, so the order does not matter)
+    for (bool on = true; __syncthreads_or(on);) {
+        on = false;
+        for (int x = threadIdx.x; x < n; x += blockDim.x) {
+            const int f = first[x], g = f ? first[f] : 0;
+            if (g) {
+                first[x] = (uint16_t)g;
+                on = true;
+            }
+        }
+    }
+    auto held = [&](int s) { return first[s] ? first[s] : s; };
+    for (int i = 1 + threadIdx.x; i < n; i += blockDim.x) {
+        const int j = p[i];
+        int s = 0;   // the last earlier step with this draw
+        for (int t = (int)head[j]; t; t = next[t])
+            if (t > i && (s == 0 || t < s)) s = t;
+        p[i] = (uint16_t)(s ? held(s) : j);
+    }
+    if (threadIdx.x == 0) p[0] = (uint16_t)held(0);
+    __syncthreads();
+    return p;
+}
+
+// The same permutations as fisher_yates_kernel, written as 16-bit rows of
+// `pitch` entries (a multiple of 8, zeros past n).
 __global__ void fisher_yates16_kernel(uint16_t *out, int pitch, int n, uint64_t seed,
                                       uint64_t target, uint64_t stage, uint64_t iter,
                                       uint64_t s_first)
 {
-    extern __shared__ int32_t sperm16[];
-    uint16_t *p = reinterpret_cast<uint16_t *>(sperm16);
+    extern __shared__ __align__(16) unsigned char fsm[];
     uint64_t h = sm64_once(seed ^ target);
     h = sm64_once(h ^ stage);
     h = sm64_once(h ^ iter);
     const uint64_t st = sm64_once(h ^ (s_first + blockIdx.x));
-    for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = (uint16_t)i;
-    __syncwarp();
-    const int lane = threadIdx.x & 31;
-    int hi = n - 1;
-    int jc = (hi - lane >= 1) ? fy_draw(st, n, hi - lane) : 0;
-    while (hi >= 1) fy16_round(p, n, st, hi, jc);
-    __syncwarp();
+    const uint16_t *p;
+    if (n <= kFyLinkMaxN) {
+        p = fy_links(fsm, n, st);
+    } else {
+        fy_shuffle16(reinterpret_cast<uint16_t *>(fsm), n, st);
+        p = reinterpret_cast<const uint16_t *>(fsm);
+    }
     uint16_t *o = out + (long long)blockIdx.x * pitch;
     for (int i = 8 * threadIdx.x; i < pitch; i += 8 * blockDim.x) {
         uint16_t v[8];
@@ -1580,8 +1610,8 @@ __global__ void fisher_yates16_kernel(uint16_t *out, int pitch, int n, uint64_t 
 
 // in_smem: bit 0 = the permutation is built in shared memory, bit 1 = the
 // draws are computed in parallel into shared memory after it, 4 = the
-// permutation as 16-bit values with the draws computed by the swapping warp
-// (n <= 65535)
+// permutation as 16-bit values (n <= 65535): by links, or beyond kFyLinkMaxN
+// with the draws computed by the swapping warp
 __global__ void fisher_yates_kernel(int32_t *out, long long stride, int n, uint64_t seed,
                                     uint64_t target, uint64_t stage, uint64_t iter,
                                     uint64_t s_first, int in_smem)
@@ -1592,8 +1622,12 @@ __global__ void fisher_yates_kernel(int32_t *out, long long stride, int n, uint6
         uint64_t h = sm64_once(seed ^ target);
         h = sm64_once(h ^ stage);
         h = sm64_once(h ^ iter);
-        uint16_t *p16 = reinterpret_cast<uint16_t *>(sperm);
-        fy_shuffle16(p16, n, sm64_once(h ^ s), out + (long long)blockIdx.x * stride);
+        const uint64_t st = sm64_once(h ^ s);
+        int32_t *dst = out + (long long)blockIdx.x * stride;
+        const uint16_t *p16 = reinterpret_cast<const uint16_t *>(sperm);
+        if (n <= kFyLinkMaxN) p16 = fy_links(reinterpret_cast<unsigned char *>(sperm), n, st);
+        else fy_shuffle16(reinterpret_cast<uint16_t *>(sperm), n, st);
+        for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = (int32_t)p16[i];
         return;
     }
     int32_t *p = (in_smem & 1) ? sperm : out + (long long)blockIdx.x * stride;
@@ -1946,7 +1980,8 @@ __global__ void compose_kernel(const ComposeJob *jobs)
 
 // Many permutation requests in one launch: CTA g is permutation g of the
 // concatenated request list (binary search over the requests' first index).
-__global__ void fisher_yates_multi_kernel(const PermJob *jobs, int n_jobs, int smem_n, int jb_ok)
+__global__ void fisher_yates_multi_kernel(const PermJob *jobs, int n_jobs, int smem_n, int jb_ok,
+                                          int links)
 {
     extern __shared__ int32_t sperm[];
     const long long g = blockIdx.x;
@@ -1964,9 +1999,16 @@ __global__ void fisher_yates_multi_kernel(const PermJob *jobs, int n_jobs, int s
     uint64_t h0 = sm64_once(J.seed ^ J.target);
     h0 = sm64_once(h0 ^ J.stage);
     h0 = sm64_once(h0 ^ J.iter);
+    if (n <= kFyLinkMaxN && links) {
+        const uint16_t *p16 = fy_links(reinterpret_cast<unsigned char *>(sperm), n,
+                                       sm64_once(h0 ^ (J.s_first + (uint64_t)r)));
+        for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = (int32_t)p16[i];
+        return;
+    }
     if (in_smem && n <= 65535) {
         uint16_t *p16 = reinterpret_cast<uint16_t *>(sperm);
-        fy_shuffle16(p16, n, sm64_once(h0 ^ (J.s_first + (uint64_t)r)), dst);
+        fy_shuffle16(p16, n, sm64_once(h0 ^ (J.s_first + (uint64_t)r)));
+        for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = (int32_t)p16[i];
         return;
     }
     int32_t *p = in_smem ? sperm : dst;
@@ -2277,8 +2319,8 @@ cudaError_t launch_perms(int32_t *out, long long stride, int n, uint64_t seed, u
     int threads = 256;
     if (n <= 65535) {
         mode = 4;
-        bytes = (size_t)n * 2;   // the permutation alone, one warp per CTA
-        threads = 32;
+        bytes = n <= kFyLinkMaxN ? fy_link_bytes(n) : (size_t)n * 2;   // else the permutation
+        threads = n <= kFyLinkMaxN ? fy_link_threads(n) : 32;          // alone, one warp
     } else if (2 * smem <= 200 * 1024) {
         mode = 3;
         bytes = 2 * smem;
@@ -2306,8 +2348,10 @@ cudaError_t launch_perms16(uint16_t *out, int pitch, int n, uint64_t seed, uint6
                            200 * 1024, attr_done);
         if (e != cudaSuccess) return e;
     }
-    fisher_yates16_kernel<<<n_perm, 32, (size_t)n * 2, st>>>(out, pitch, n, seed, target, stage,
-                                                            iter, s_first);
+    const bool links = n <= kFyLinkMaxN;
+    fisher_yates16_kernel<<<n_perm, links ? fy_link_threads(n) : 32,
+                            links ? fy_link_bytes(n) : (size_t)n * 2, st>>>(
+        out, pitch, n, seed, target, stage, iter, s_first);
     return cudaGetLastError();
 }
 
@@ -2315,7 +2359,8 @@ cudaError_t launch_perms16(uint16_t *out, int pitch, int n, uint64_t seed, uint6
 // One CTA per surrogate s = s_first + blockIdx.x, state keyed as in
 // fisher_yates_kernel.  mode 0: Fisher-Yates of the R trials, point r*n + t
 // reads sigma[r]*n + t; mode 1: one Fisher-Yates shuffle per trial, trial 0
-// first, all from one continuing generator (R = 1 gives the flat permutation).
+// first, all from one continuing generator (R = 1 gives the flat permutation):
+// by links (in_smem 2) where a trial fits, else one thread's loop.
 __global__ void fisher_yates_trials_kernel(int32_t *out, int R, int n, uint64_t seed,
                                            uint64_t target, uint64_t stage, uint64_t iter,
                                            uint64_t s_first, int mode, int in_smem)
@@ -2344,6 +2389,17 @@ __global__ void fisher_yates_trials_kernel(int32_t *out, int R, int n, uint64_t 
         for (long long p = threadIdx.x; p < total; p += blockDim.x) {
             const int r = (int)(p / n), t = (int)(p - (long long)r * n);
             dst[p] = sigma[r] * n + t;
+        }
+        return;
+    }
+    if (in_smem == 2) {   // trial r's draws continue the generator after r (n - 1) outputs
+        for (int r = 0; r < R; ++r) {
+            const uint16_t *p16 =
+                fy_links(reinterpret_cast<unsigned char *>(sbuf), n,
+                         st + (uint64_t)r * (uint64_t)(n - 1) * 0x9E3779B97F4A7C15ull);
+            for (int i = threadIdx.x; i < n; i += blockDim.x)
+                dst[(long long)r * n + i] = r * n + (int32_t)p16[i];
+            __syncthreads();
         }
         return;
     }
@@ -2387,8 +2443,8 @@ cudaError_t launch_perms_trials(int32_t *out, int R, int n, uint64_t seed, uint6
         smem = (size_t)R * sizeof(int32_t);
         if (smem > 200 * 1024) return cudaErrorInvalidValue;
     } else {
-        in_smem = whole <= 200 * 1024;
-        smem = in_smem ? whole : 0;
+        in_smem = n <= kFyLinkMaxN ? 2 : whole <= 200 * 1024;
+        smem = in_smem == 2 ? fy_link_bytes(n) : in_smem ? whole : 0;
     }
     fisher_yates_trials_kernel<<<n_perm, 256, smem, st>>>(out, R, n, seed, target, stage, iter,
                                                           s_first, mode, in_smem);
@@ -2407,10 +2463,15 @@ cudaError_t launch_perms_multi(const PermJob *jobs, int n_jobs, long long total,
                            200 * 1024, attr_done);
         if (e != cudaSuccess) return e;
     }
+    if (max_n <= kFyLinkMaxN) {
+        fisher_yates_multi_kernel<<<(unsigned)total, fy_link_threads(max_n), fy_link_bytes(max_n),
+                                    st>>>(jobs, n_jobs, max_n, 0, 1);
+        return cudaGetLastError();
+    }
     if (max_n <= 65535) {
         // every job shuffles in 16 bits (2 bytes per point), one warp per CTA
         fisher_yates_multi_kernel<<<(unsigned)total, 32, (size_t)max_n * 2, st>>>(jobs, n_jobs,
-                                                                                 max_n, 0);
+                                                                                 max_n, 0, 0);
         return cudaGetLastError();
     }
     const int smem_n = max_n * 4 <= 200 * 1024 ? max_n : 0;
@@ -2418,7 +2479,7 @@ cudaError_t launch_perms_multi(const PermJob *jobs, int n_jobs, long long total,
     // fits; jobs of at most 65535 points still shuffle in 16 bits
     const int jb_ok = smem_n > 0 && (size_t)max_n * 8 <= 200 * 1024;
     fisher_yates_multi_kernel<<<(unsigned)total, 256, (size_t)smem_n * (jb_ok ? 8 : 4), st>>>(
-        jobs, n_jobs, smem_n, jb_ok);
+        jobs, n_jobs, smem_n, jb_ok, 0);
     return cudaGetLastError();
 }
 
