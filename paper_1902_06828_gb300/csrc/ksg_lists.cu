@@ -1255,9 +1255,6 @@ int list_build_queries(int cap_a, int cap_b)
     return 2;
 }
 
-constexpr int kWalkSmemMax =
-    (int)(kListWalkSmem + 2 * (kListWalkThreads / 32) * sizeof(ListNear));
-
 template <int G, bool NEAR>
 static const void *walk_kernel_g(const ListShape &s)
 {

@@ -1077,10 +1077,9 @@ te_status cmi_ksg_batch(te_ctx *ctx, const te_cmi_job *jobs, int32_t n_jobs, dou
     if (n_jobs < 0 || (n_jobs > 0 && (!jobs || !out)))
         return fail(ctx, TE_EINVAL, "jobs or out is NULL");
     if (n_jobs == 0) return TE_OK;
-    size_t perm_elems = 0;
     int n_out = 0;
-    std::vector<int> job_out(n_jobs), job_N(n_jobs);
-    std::vector<size_t> job_perm(n_jobs);
+    std::vector<int> job_out(n_jobs), job_N(n_jobs), job_set(n_jobs);
+    PermSets sets;
     for (int j = 0; j < n_jobs; ++j) {
         const te_cmi_job &J = jobs[j];
         if ((st = validate_estimate(ctx, J.data, J.x, J.dx, J.y, J.dy, J.z, J.dz, J.params.k,
@@ -1091,48 +1090,26 @@ te_status cmi_ksg_batch(te_ctx *ctx, const te_cmi_job *jobs, int32_t n_jobs, dou
         job_N[j] = J.data->T - J.params.max_lag;
         job_out[j] = n_out;
         n_out += 1 + J.params.n_surr;
-        job_perm[j] = perm_elems;
-        perm_elems += (size_t)J.params.n_surr * job_N[j];
+        job_set[j] = sets.add(J.params.seed, J.params.stream_tag, job_N[j], J.params.n_surr);
     }
     CK(cudaSetDevice(ctx->device), "cudaSetDevice");
-    if ((st = ensure_dev(ctx, ctx->ws_perm, std::max<size_t>(perm_elems, 1) * 4))) return st;
-    int32_t *perm = (int32_t *)ctx->ws_perm.p;
+    if ((st = ensure_dev(ctx, ctx->ws_perm, std::max<size_t>(sets.elems(), 1) * 4))) return st;
+    sets.place((int32_t *)ctx->ws_perm.p);
     // jobs with the same data, point set, k, window, Y and Z share a group
     std::map<std::vector<long long>, int> gid;
     std::vector<HostGroup> groups;
-    // every job's surrogate permutations in one launch
-    std::vector<PermJob> pj;
-    long long perm_total = 0;
-    int max_n = 0;
-    for (int j = 0; j < n_jobs; ++j) {
-        const int S = jobs[j].params.n_surr;
-        if (S <= 0) continue;
-        PermJob q{};
-        q.out = perm + job_perm[j];
-        q.n = job_N[j];
-        q.n_perm = S;
-        q.s_first = 1;
-        q.seed = jobs[j].params.seed;
-        q.target = jobs[j].params.stream_tag;
-        q.stage = 0;
-        q.iter = 0;
-        q.perm_begin = perm_total;
-        perm_total += S;
-        max_n = std::max(max_n, job_N[j]);
-        pj.push_back(q);
-    }
-    if (!pj.empty()) {
-        const size_t bytes = pj.size() * sizeof(PermJob);
+    if (!sets.jobs().empty()) {   // every set's permutations in one launch
+        const size_t bytes = sets.jobs().size() * sizeof(PermJob);
         if ((st = ensure_dev(ctx, ctx->ws_stat, bytes + 16))) return st;
-        CK(copy_h2d(ctx, ctx->ws_stat.p, pj.data(), bytes), "cudaMemcpyAsync");
-        CK(launch_perms_multi((const PermJob *)ctx->ws_stat.p, (int)pj.size(), perm_total, max_n,
-                              ctx->stream),
+        CK(copy_h2d(ctx, ctx->ws_stat.p, sets.jobs().data(), bytes), "cudaMemcpyAsync");
+        CK(launch_perms_multi((const PermJob *)ctx->ws_stat.p, (int)sets.jobs().size(),
+                              sets.total(), sets.max_n(), ctx->stream),
            "permutation launch");
         ctx->stats.launches++;
     }
     for (int j = 0; j < n_jobs; ++j) {
         const te_cmi_job &J = jobs[j];
-        const int N = job_N[j], S = J.params.n_surr;
+        const int S = J.params.n_surr;
         std::vector<long long> key{(long long)(uintptr_t)J.data, J.params.max_lag, J.params.k,
                                    J.params.theiler, J.dx, J.dy, J.dz};
         for (int d = 0; d < J.dy; ++d) key.push_back(((long long)J.y[d].proc << 32) | J.y[d].lag);
@@ -1159,9 +1136,7 @@ te_status cmi_ksg_batch(te_ctx *ctx, const te_cmi_job *jobs, int32_t n_jobs, dou
         const int xfirst = (int)hg.xvars.size();
         hg.xvars.insert(hg.xvars.end(), J.x, J.x + J.dx);
         for (int s = 0; s <= S; ++s)
-            hg.members.push_back(HostMember{
-                xfirst, s == 0 ? nullptr : perm + job_perm[j] + (size_t)(s - 1) * N,
-                job_out[j] + s});
+            hg.members.push_back(HostMember{xfirst, sets.perm(job_set[j], s), job_out[j] + s});
     }
     if ((st = run_groups(ctx, groups, n_out))) return st;
     std::vector<int64_t> keys((size_t)2 * n_out);

@@ -5,8 +5,10 @@
 #include <stdint.h>
 
 #include <functional>
+#include <map>
 #include <mutex>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "te_ksg.h"
@@ -34,6 +36,59 @@ struct HostGroup {
     int dx = 1;
     std::vector<te_var> xvars;     // dx variables per member, member-major
     std::vector<HostMember> members;
+};
+
+// The surrogate permutations of a batch: surrogate s of a job depends on the
+// job's seed, stream tag and point count only, so jobs that agree in these (the
+// candidates of one test) share one set, drawn once with as many permutations
+// as the largest of them needs.
+class PermSets {
+public:
+    int add(uint64_t seed, uint64_t tag, int N, int S)   // -> set index
+    {
+        auto ins = index_.emplace(std::make_tuple(seed, tag, N), (int)sets_.size());
+        if (ins.second) {
+            PermJob q{};
+            q.n = N;
+            q.s_first = 1;
+            q.seed = seed;
+            q.target = tag;
+            sets_.push_back(q);
+        }
+        PermJob &q = sets_[ins.first->second];
+        q.n_perm = q.n_perm > S ? q.n_perm : S;
+        return ins.first->second;
+    }
+    size_t elems() const   // ints that all sets take
+    {
+        size_t n = 0;
+        for (const PermJob &q : sets_) n += (size_t)q.n_perm * q.n;
+        return n;
+    }
+    void place(int32_t *base)   // sets the output addresses; then jobs() can be launched
+    {
+        for (PermJob &q : sets_) {
+            q.out = base;
+            base += (size_t)q.n_perm * q.n;
+            q.perm_begin = total_;
+            total_ += q.n_perm;
+            max_n_ = max_n_ > q.n ? max_n_ : q.n;
+            if (q.n_perm) jobs_.push_back(q);
+        }
+    }
+    const int32_t *perm(int set, int s) const   // surrogate s (1 ..); nullptr for the original
+    {
+        return s == 0 ? nullptr : sets_[set].out + (size_t)(s - 1) * sets_[set].n;
+    }
+    const std::vector<PermJob> &jobs() const { return jobs_; }
+    long long total() const { return total_; }
+    int max_n() const { return max_n_; }
+
+private:
+    std::map<std::tuple<uint64_t, uint64_t, int>, int> index_;
+    std::vector<PermJob> sets_, jobs_;
+    long long total_ = 0;
+    int max_n_ = 0;
 };
 
 struct te_status_error {

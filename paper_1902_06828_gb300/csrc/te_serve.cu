@@ -94,48 +94,28 @@ te_status launch_batch(Slot &sl)
 {
     te_ctx *ctx = sl.ctx;
     te_status st;
-    size_t perm_elems = 0;
     int n_out = 0;
     sl.out0.resize(sl.jobs.size());
-    std::vector<size_t> perm_at(sl.jobs.size());
-    int max_n = 0;
+    std::vector<int> set(sl.jobs.size());
+    PermSets sets;
     for (size_t a = 0; a < sl.jobs.size(); ++a) {
         ServeJob *j = sl.jobs[a];
         sl.out0[a] = n_out;
         n_out += j->S + 1;
-        perm_at[a] = perm_elems;
-        perm_elems += (size_t)j->S * j->N;
-        max_n = std::max(max_n, j->N);
+        set[a] = sets.add(j->p.seed, j->p.stream_tag, j->N, j->S);
     }
     sl.n_out = n_out;
-    if ((st = ensure_dev(ctx, ctx->ws_perm, std::max<size_t>(perm_elems, 1) * 4))) return st;
-    int32_t *perm = (int32_t *)ctx->ws_perm.p;
-    std::vector<PermJob> pj;
-    long long total = 0;
-    for (size_t a = 0; a < sl.jobs.size(); ++a) {
-        ServeJob *j = sl.jobs[a];
-        if (j->S == 0) continue;
-        PermJob q;
-        q.out = perm + perm_at[a];
-        q.n = j->N;
-        q.n_perm = j->S;
-        q.s_first = 1;
-        q.seed = j->p.seed;
-        q.target = j->p.stream_tag;
-        q.stage = 0;
-        q.iter = 0;
-        q.perm_begin = total;
-        total += j->S;
-        pj.push_back(q);
-    }
-    if (!pj.empty()) {
-        const size_t bytes = pj.size() * sizeof(PermJob);
+    if ((st = ensure_dev(ctx, ctx->ws_perm, std::max<size_t>(sets.elems(), 1) * 4))) return st;
+    sets.place((int32_t *)ctx->ws_perm.p);
+    if (!sets.jobs().empty()) {
+        const size_t bytes = sets.jobs().size() * sizeof(PermJob);
         if ((st = ensure_dev(ctx, ctx->ws_stat, bytes + 16))) return st;
-        // pageable source: the copy has left pj when the call returns
-        CK(cudaMemcpyAsync(ctx->ws_stat.p, pj.data(), bytes, cudaMemcpyHostToDevice, ctx->stream),
+        // pageable source: the copy has left the vector when the call returns
+        CK(cudaMemcpyAsync(ctx->ws_stat.p, sets.jobs().data(), bytes, cudaMemcpyHostToDevice,
+                           ctx->stream),
            "cudaMemcpyAsync");
-        CK(launch_perms_multi((const PermJob *)ctx->ws_stat.p, (int)pj.size(), total, max_n,
-                              ctx->stream),
+        CK(launch_perms_multi((const PermJob *)ctx->ws_stat.p, (int)sets.jobs().size(),
+                              sets.total(), sets.max_n(), ctx->stream),
            "permutation launch");
         ctx->stats.launches++;
     }
@@ -170,9 +150,7 @@ te_status launch_batch(Slot &sl)
         const int xfirst = (int)hg.xvars.size();
         hg.xvars.insert(hg.xvars.end(), j->x.begin(), j->x.end());
         for (int s = 0; s <= j->S; ++s)
-            hg.members.push_back(HostMember{
-                xfirst, s == 0 ? nullptr : perm + perm_at[a] + (size_t)(s - 1) * j->N,
-                sl.out0[a] + s});
+            hg.members.push_back(HostMember{xfirst, sets.perm(set[a], s), sl.out0[a] + s});
     }
     if ((st = launch_groups(ctx, groups, n_out))) return st;
     if ((size_t)n_out * 16 > sl.keys_cap) {

@@ -107,3 +107,42 @@ def test_columns_of_different_point_sets_in_one_batch(env):
         o = oksg.cmi_ksg(s, j.x, j.y, j.z, k=4, max_lag=j.max_lag)
         assert keys[0] == o["key"], (j.max_lag, j.z)
     data.close()
+
+
+@pytest.mark.parametrize("N", [6, 33, 511, 513, 2048, 2049, 4099])
+def test_permutations_at_every_launch_shape(env, N):
+    """Surrogate keys equal the oracle's, whose permutations come from the
+    sequential shuffle, at point counts on both sides of every thread count of
+    the parallel one; two jobs of different length share their permutations."""
+    from oracle import ksg as oksg
+    te, ctx = env
+    rng = np.random.default_rng(N)
+    s = rng.normal(size=(3, N)).astype(np.float32)
+    data = te.te_data_create(ctx, s)
+    jobs = [te.Job(data, [(p, 0)], [(1, 0)], [], k=2, max_lag=0, n_surr=S, seed=5, stream_tag=6)
+            for p, S in ((0, 2), (2, 5))]
+    _, got = te.cmi_ksg_batch(ctx, jobs, return_keys=True)
+    perms = np.stack([oksg.permutation(5, 6, 0, 0, a, N) for a in range(1, 6)])
+    for j, keys in zip(jobs, got):
+        ok, _, _ = oksg.cmi_ksg_batch(s, [j.x] * (j.n_surr + 1), j.y, [], perms=perms,
+                                      perm_idx=[-1] + list(range(j.n_surr)), k=2, max_lag=0)
+        assert keys == ok
+    data.close()
+
+
+@pytest.mark.parametrize("N", [20480, 20481])
+def test_permutations_past_the_parallel_shuffle(env, N):
+    """The largest N of the parallel shuffle and the first past it: a
+    surrogate's X values, read back through the Gaussian estimate, give the
+    estimate of the permuted column."""
+    from oracle import ksg as oksg
+    te, ctx = env
+    rng = np.random.default_rng(N)
+    s = rng.normal(size=(2, N)).astype(np.float32)
+    data = te.te_data_create(ctx, s)
+    got, _ = te.cmi_gauss(ctx, data, [(0, 0)], [(1, 0)], max_lag=0, n_surr=3, seed=8, stream_tag=1)
+    for a in range(1, 4):
+        x = s[0].astype(np.float64)[oksg.permutation(8, 1, 0, 0, a, N)]
+        r = np.corrcoef(x, s[1].astype(np.float64))[0, 1]
+        assert abs(got[a] - -0.5 * np.log1p(-r * r)) < 1e-7
+    data.close()
