@@ -477,7 +477,9 @@ te_status te_serve_get_stats(te_ctx *ctx, te_serve_stats *out);
  *   4 (dx + dy + dz)     column offsets
  *   16 (S + 1), twice    key accumulators and keys
  * with N = T - max_lag and S = n_surr <= TE_STATIC_MAX_SURR; it returns
- * TE_EINVAL when the sum exceeds TE_STATIC_SCRATCH_BYTES.
+ * TE_EINVAL when the sum exceeds TE_STATIC_SCRATCH_BYTES.  What the scratch has
+ * left beyond the sum holds neighbour lists, as many points' at a time as fit;
+ * where that is less than a 64th of the points, the call runs without lists.
  *
  * series_dev: device float32 [n_proc][T] on the current device, owned by the
  * caller; TE_EINVAL if it is not device memory of the current device.  x, y, z, params: as cmi_ksg.  cuda_stream: a cudaStream_t of the

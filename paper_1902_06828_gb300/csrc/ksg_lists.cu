@@ -1240,6 +1240,24 @@ bool list_fits(int N, int dx, int dz, int k)
     return list_walk_x_bytes(N, dx, dz, k, 1) <= kListWalkSmem;
 }
 
+int list_splits(long long blocks, int max_nq, size_t smem, int sms)
+{
+    // CTAs that fill whole waves; a CTA first loads its members' X values,
+    // which costs about 1/32 of a walk over all points
+    const long long resident = (long long)sms * (smem > kListHalfSmem ? 1 : 2);
+    int splits = 1;
+    double best = 1e300;
+    for (int t = 1; t <= std::min(512, (max_nq + 15) / 16); ++t) {
+        const double waves = (double)((blocks * t + resident - 1) / resident);
+        const double cost = waves * (1.0 / t + 1.0 / 32.0);
+        if (cost < 0.98 * best) {
+            best = cost;
+            splits = t;
+        }
+    }
+    return splits;
+}
+
 static size_t list_build_smem(int cap_a, int cap_b, int queries)
 {
     // a query's space also holds its sample: kSample distances of either kind

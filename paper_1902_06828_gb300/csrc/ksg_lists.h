@@ -102,6 +102,9 @@ ListShape list_shape(int N, int dx, int dz, int k, size_t members);
 size_t list_walk_x_bytes(int N, int dx, int dz, int k, int width);
 // whether a group can take the list path
 bool list_fits(int N, int dx, int dz, int k);
+// Parts into which the walk splits the points of a launch, given its member
+// blocks, the most points of a segment, its CTAs' X bytes and the SM count
+int list_splits(long long blocks, int max_nq, size_t smem, int sms);
 // queries per CTA of the build kernel
 int list_build_queries(int cap_a, int cap_b);
 

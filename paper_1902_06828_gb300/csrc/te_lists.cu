@@ -82,28 +82,13 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
         size_t used = 0;
         auto close_chunk = [&]() {
             ch.queries = list_build_queries(ch.cap_a, ch.cap_b);
-            // Split the points so that the CTAs fill whole waves; a CTA
-            // first loads its members' X values, which costs about 1/32 of a
-            // walk over all points.
-            const long long resident =
-                (long long)sms *
-                (cp.smem > kListHalfSmem ? 1 : 2);
             long long blocks = 0;
             int max_nq = 1;
             for (int s = ch.first_seg; s < ch.first_seg + ch.n_segs; ++s) {
                 blocks += lg[cp.first_group + segs[s].group].n_mblocks;
                 max_nq = std::max(max_nq, segs[s].nq);
             }
-            int splits = 1;
-            double best = 1e300;
-            for (int t = 1; t <= std::min(512, (max_nq + 15) / 16); ++t) {
-                const double waves = (double)((blocks * t + resident - 1) / resident);
-                const double cost = waves * (1.0 / t + 1.0 / 32.0);
-                if (cost < 0.98 * best) {
-                    best = cost;
-                    splits = t;
-                }
-            }
+            const int splits = list_splits(blocks, max_nq, cp.smem, sms);
             for (int s = ch.first_seg; s < ch.first_seg + ch.n_segs; ++s) {
                 segs[s].build_item = ch.build_items;
                 ch.build_items += (segs[s].nq + ch.queries - 1) / ch.queries;

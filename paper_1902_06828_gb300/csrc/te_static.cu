@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "ksg_lists.h"
 #include "te_runtime.h"
 
 using namespace teksg;
@@ -51,6 +52,14 @@ int64_t g_q_host[kStaticMaxN + 2];
 int g_q_host_n = -1;
 unsigned char g_desc_host[sizeof(GroupDesc) + (kStaticMaxSurr + 1) * sizeof(MemberDesc) +
                           4 * TE_MAX_DIMS + 64];
+constexpr int kStaticMaxSegs = 64;   // pieces of the points whose lists are in the scratch at once
+struct StaticListTables {
+    ListGroup group;
+    RankSortJob sort;
+    ListSeg segs[kStaticMaxSegs];
+};
+StaticListTables g_tables_host;
+int g_sms[kStaticMaxDevices];
 int64_t g_keys_host[2 * (kStaticMaxSurr + 1)];
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -63,7 +72,9 @@ te_status setup_device(int dev)
     if (g_ready[dev]) return TE_OK;
     void *p = nullptr;
     if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return TE_ECUDA;
-    if (ksg_prepare_attributes() != cudaSuccess) return TE_ECUDA;
+    if (ksg_prepare_attributes() != cudaSuccess || list_prepare_attributes() != cudaSuccess ||
+        cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return TE_ECUDA;
     g_scratch_addr[dev] = p;
     g_ready[dev] = true;
     return TE_OK;
@@ -140,24 +151,45 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
     if (launch_perms(perms, N, N, p->seed, p->stream_tag, 0, 0, 1, S, stream) != cudaSuccess)
         return TE_ECUDA;
 
+    // Neighbour lists (as the context path) where the scratch beyond the seven
+    // parts holds the lists of at least a 64th of the points (the tables and
+    // sorted columns lie before them); else the member-lane kernel, which
+    // needs no more.  A call of 201 members at T = 1000: 426 us with the
+    // member-lane kernel, 213 with lists.
+    const ListShape shape = list_shape(N, dx, dz, p->k, (size_t)S + 1);
+    ListGroup lg{};
+    list_caps(N, p->k, dx, dy, dz, (size_t)S + 1, &lg.cap_a, &lg.cap_b);
+    const bool sorted_column = dz == 1 || (dz == 0 && dx == 1);
+    const size_t np = ((size_t)N + 3) & ~(size_t)3;
+    const size_t tab_off = total;
+    const size_t sort_off = align256(tab_off + sizeof(StaticListTables));
+    const size_t row_off = align256(sort_off + (sorted_column ? np * 8 : 0));
+    const size_t row = list_row_bytes(lg.cap_a, lg.cap_b);
+    const size_t room = row_off < kStaticScratchBytes ? (kStaticScratchBytes - row_off) / row : 0;
+    const int seg_rows = (int)std::min<size_t>((size_t)N, room);
+    const bool lists = list_fits(N, dx, dz, p->k) && seg_rows > 0 &&
+                       (N + seg_rows - 1) / seg_rows <= kStaticMaxSegs;
+
     // one group in time order, members = identity + S surrogates
     const bool dx1 = dx == 1;
     KsgVariant v = dx1 ? KsgVariant{32, p->k == 4 ? 4 : 0, kLaneThreads}
                        : KsgVariant{2, p->k == 4 ? 4 : 0, 128};
     const int qsz = dx1 ? kLaneQueries : 128;
-    int jt;
-    size_t smem;
-    if (dx1) {
+    int jt = 0;
+    size_t smem = 0;
+    if (lists) {
+        // no tile
+    } else if (dx1) {
         jt = 256;
         if (N < jt) jt = std::max(64, (N + 63) & ~63);
         smem = ksg_lane_smem_bytes(dy + dz, jt);
     } else {
         const int rows_t = dy + dz + v.m * dx, rows_q = rows_t;
-        long long room = 40 * 1024 - 4LL * rows_q * 128 - 64 - 8 * 8 * 128;
-        jt = (int)std::min<long long>((room / (4LL * rows_t + 8)) & ~7LL, 2048);
+        long long room_t = 40 * 1024 - 4LL * rows_q * 128 - 64 - 8 * 8 * 128;
+        jt = (int)std::min<long long>((room_t / (4LL * rows_t + 8)) & ~7LL, 2048);
         if (jt < 64) {
-            room = 190 * 1024 - 4LL * rows_q * 128 - 64 - 8 * 8 * 128;
-            jt = (int)std::min<long long>((room / (4LL * rows_t + 8)) & ~7LL, 2048);
+            room_t = 190 * 1024 - 4LL * rows_q * 128 - 64 - 8 * 8 * 128;
+            jt = (int)std::min<long long>((room_t / (4LL * rows_t + 8)) & ~7LL, 2048);
         }
         if (jt < 8) return TE_EINVAL;
         jt = std::min(jt, (N + 7) & ~7);
@@ -185,34 +217,93 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
         hm[s].perm = s == 0 ? nullptr : perms + (size_t)(s - 1) * N;
         hm[s].xcol = 0;
         hm[s].out = s;
-        hm[s].xsorted = nullptr;
+        hm[s].xsorted = lists && dz == 0 && dx == 1 ? (const float *)(sc + sort_off) : nullptr;
     }
     int *hc = (int *)(hm + S + 1);
     int c = 0;
     for (int d = 0; d < dx; ++d) hc[c++] = x[d].proc * T + p->max_lag - x[d].lag;
     for (int d = 0; d < dy; ++d) hc[c++] = y[d].proc * T + p->max_lag - y[d].lag;
     for (int d = 0; d < dz; ++d) hc[c++] = z[d].proc * T + p->max_lag - z[d].lag;
-    if (cudaMemcpyAsync(sc + grp_off, h, sizeof(GroupDesc), cudaMemcpyHostToDevice, stream) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(sc + mem_off, hm, (size_t)(S + 1) * sizeof(MemberDesc),
+    if (cudaMemcpyAsync(sc + mem_off, hm, (size_t)(S + 1) * sizeof(MemberDesc),
                         cudaMemcpyHostToDevice, stream) != cudaSuccess ||
         cudaMemcpyAsync(sc + col_off, hc, (size_t)c * 4, cudaMemcpyHostToDevice, stream) !=
             cudaSuccess ||
         cudaMemsetAsync(acc, 0, (size_t)(S + 1) * 16, stream) != cudaSuccess)
         return TE_ECUDA;
 
-    KsgLaunch L{};
-    L.groups = (const GroupDesc *)(sc + grp_off);
-    L.n_groups = 1;
-    L.members = (const MemberDesc *)(sc + mem_off);
-    L.cols = (const int *)(sc + col_off);
-    L.q = q;
-    L.acc = acc;
-    L.dbg_out = -1;
-    L.jt = jt;
-    L.work = nullptr;
-    const long long items = (long long)gd.n_qtiles * gd.n_mblocks;
-    if (launch_ksg(L, v, items, dx1, smem, stream) != cudaSuccess) return TE_ECUDA;
+    if (lists) {
+        StaticListTables &t = g_tables_host;
+        lg.base = series_dev;
+        lg.N = N;
+        lg.k = p->k;
+        lg.theiler = p->theiler;
+        lg.dy = dy;
+        lg.dz = dz;
+        lg.dx = dx;
+        lg.ycol = dx;
+        lg.zcol = dx + dy;
+        lg.n_members = S + 1;
+        lg.n_mblocks = (S + shape.width) / shape.width;
+        t.sort = RankSortJob{series_dev + hc[dz ? dx + dy : 0], (float *)(sc + sort_off),
+                             (int *)((float *)(sc + sort_off) + np), N, 0};
+        if (dz == 1) {
+            lg.zs = t.sort.sorted;
+            lg.rank = t.sort.rank;
+        }
+        t.group = lg;
+        const size_t xbytes = list_walk_x_bytes(N, dx, dz, p->k, shape.width);
+        int n_segs = 0;
+        for (int q0 = 0; q0 < N; q0 += seg_rows) {
+            ListSeg &g = t.segs[n_segs++];
+            g = ListSeg{};
+            g.q0 = q0;
+            g.nq = std::min(seg_rows, N - q0);
+            const int splits = list_splits(lg.n_mblocks, g.nq, xbytes, g_sms[dev]);
+            g.per_cta = (g.nq + splits - 1) / splits;
+            g.n_splits = (g.nq + g.per_cta - 1) / g.per_cta;
+            g.rows = sc + row_off;
+        }
+        if (cudaMemcpyAsync(sc + tab_off, &t, sizeof t, cudaMemcpyHostToDevice, stream) !=
+            cudaSuccess)
+            return TE_ECUDA;
+        const StaticListTables *dt = (const StaticListTables *)(sc + tab_off);
+        if (sorted_column &&
+            launch_rank_sort(&dt->sort, 1, rank_sort_items(N), stream) != cudaSuccess)
+            return TE_ECUDA;
+        const int queries = list_build_queries(lg.cap_a, lg.cap_b);
+        for (int a = 0; a < n_segs; ++a) {
+            ListLaunch L{};
+            L.groups = &dt->group;
+            L.segs = dt->segs + a;
+            L.n_segs = 1;
+            L.members = (const MemberDesc *)(sc + mem_off);
+            L.cols = (const int *)(sc + col_off);
+            L.q = q;
+            L.acc = acc;
+            L.dbg_out = -1;
+            if (launch_list_build(L, (t.segs[a].nq + queries - 1) / queries, queries, lg.cap_a,
+                                  lg.cap_b, stream) != cudaSuccess ||
+                launch_list_walk(L, (long long)t.segs[a].n_splits * lg.n_mblocks, shape, xbytes,
+                                 stream) != cudaSuccess)
+                return TE_ECUDA;
+        }
+    } else {
+        if (cudaMemcpyAsync(sc + grp_off, h, sizeof(GroupDesc), cudaMemcpyHostToDevice, stream) !=
+            cudaSuccess)
+            return TE_ECUDA;
+        KsgLaunch L{};
+        L.groups = (const GroupDesc *)(sc + grp_off);
+        L.n_groups = 1;
+        L.members = (const MemberDesc *)(sc + mem_off);
+        L.cols = (const int *)(sc + col_off);
+        L.q = q;
+        L.acc = acc;
+        L.dbg_out = -1;
+        L.jt = jt;
+        L.work = nullptr;
+        const long long items = (long long)gd.n_qtiles * gd.n_mblocks;
+        if (launch_ksg(L, v, items, dx1, smem, stream) != cudaSuccess) return TE_ECUDA;
+    }
     if (launch_finalize(acc, keys, S + 1, stream) != cudaSuccess) return TE_ECUDA;
 
     int64_t *kh = g_keys_host;

@@ -146,3 +146,23 @@ def test_permutations_past_the_parallel_shuffle(env, N):
         r = np.corrcoef(x, s[1].astype(np.float64))[0, 1]
         assert abs(got[a] - -0.5 * np.log1p(-r * r)) < 1e-7
     data.close()
+
+
+@pytest.mark.parametrize("T,dz,dx,S,k", [(300, 2, 1, 6, 4), (300, 0, 1, 3, 4), (300, 1, 2, 3, 5),
+                                         (6000, 2, 1, 300, 4), (6000, 1, 1, 300, 4),
+                                         (9000, 2, 1, 900, 4)])
+def test_static_entry_point_in_pieces(env, T, dz, dx, S, k):
+    """The allocation-free call keeps the lists of as many points as its scratch
+    has left: all of them, a few pieces, or (last) too few, where the
+    member-lane kernel serves the call."""
+    torch = pytest.importorskip("torch")
+    te, ctx = env
+    s = np.asarray(synth.workload_var10(T=T, seed=3)["series"], dtype=np.float32)
+    data = te.te_data_create(ctx, s)
+    dev = torch.from_numpy(s).cuda()
+    kw = dict(k=k, max_lag=5, n_surr=S, seed=7, stream_tag=2, return_keys=True)
+    x = [(2, 1 + a) for a in range(dx)]
+    _, ref = te.cmi_ksg(ctx, data, x, [(0, 0)], Z[:dz], **kw)
+    _, got = te.cmi_ksg_static(dev, x, [(0, 0)], Z[:dz], **kw)
+    assert got == ref
+    data.close()
