@@ -20,6 +20,10 @@ struct GaussArgs {
     // of 8), or nullptr: read by the tensor-core contraction when set
     const uint16_t *perms16;
     int perm_pitch;
+    // batched contraction: the permutations turned, entry s of point t (0: the
+    // point itself) at perm_t[t * perm_t_pitch + s], or nullptr
+    const uint16_t *perm_t;
+    int perm_t_pitch;
     int w0;                 // tensor-core contraction: first W column of this pass (32 per pass)
     // tensor-core contraction inputs prepared once per call: W's B tiles
     // (split TF32, core-matrix layout, 8 KB per 32-point chunk and pass) and
@@ -28,8 +32,10 @@ struct GaussArgs {
     float *btile;
     float *xcen;
     int xcen_pitch;
-    double *mean;           // [d]
-    double *cov;            // [d][d] sample covariance, ddof = 1
+    double *mean;           // [d] (X only where own_w = 0)
+    const double *meanw;    // [dw] means of the W columns: mean + dx, or another estimate's
+    double *cov;            // [d][d] sample covariance, ddof = 1 (its X-W blocks are not formed:
+                            // cross holds them, for every surrogate)
     double *LW, *LZ;        // [dw][dw] lower Cholesky factors of S_WW and S_ZZ
     double *norms;          // ||L_W^-1||_F^2, ||L_Z^-1||_F^2
     double *scratch;        // [kGaussMaxDims]
@@ -73,6 +79,17 @@ __host__ __device__ inline double gauss_f64_gamma(int N)
 // 3 * 2^-48 per product and at most 128^2 * 2^-48 per window of kGaussFFWindow
 // 32-point chunks (2^-34 covers both), then the FP64 sums
 constexpr int kGaussFFMaxW = 16;
+// points whose centred X column (8 bytes each) fits a CTA's shared memory; such
+// estimates with dw <= kGaussFFMaxW and perm_t set gather there
+constexpr int kGaussFFColMax = 26000;
+// perm_t of one set: S permutations of N <= 65535 points as 32-bit rows
+struct PermTurnJob {
+    const int32_t *src;
+    uint16_t *dst;
+    int S, N, pitch;
+};
+cudaError_t gauss_launch_turn(const PermTurnJob *jobs_dev, const PermTurnJob *jobs_host, int n,
+                              cudaStream_t st);
 constexpr int kGaussFFWindow = 4;
 __host__ __device__ inline double gauss_batch_gamma(int N, int dw)
 {

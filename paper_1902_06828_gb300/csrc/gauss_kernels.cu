@@ -40,6 +40,7 @@ __device__ __forceinline__ double block_sum(double v, double *red)
 __device__ __forceinline__ void gauss_mean_body(const GaussArgs &A, int d)
 {
     __shared__ double red[32];
+    if (!A.own_w && d >= A.dx) return;   // meanw is another estimate's
     const float *col = A.base + A.cols[d];
     double s = 0.0;
     for (int t = threadIdx.x; t < A.N; t += blockDim.x) s += (double)col[t];
@@ -56,11 +57,13 @@ __device__ __forceinline__ void gauss_cov_body(const GaussArgs &A, int p)
         p -= A.d - i;
         ++i;
     }
-    if (!A.own_w && i >= A.dx) return;   // a W-W entry: taken from covw
     const int j = i + p;
+    if (!A.own_w && i >= A.dx) return;   // a W-W entry: taken from covw
+    if (i < A.dx && j >= A.dx) return;   // an X-W entry: in cross
     const float *ci = A.base + A.cols[i];
     const float *cj = A.base + A.cols[j];
-    const double mi = A.mean[i], mj = A.mean[j];
+    const double mi = i < A.dx ? A.mean[i] : A.meanw[i - A.dx];
+    const double mj = j < A.dx ? A.mean[j] : A.meanw[j - A.dx];
     double s = 0.0;
     for (int t = threadIdx.x; t < A.N; t += blockDim.x)
         s += ((double)ci[t] - mi) * ((double)cj[t] - mj);
@@ -406,7 +409,7 @@ __global__ void gauss_tc_prep_w(GaussArgs A, int nchunks)
         const int t = c * kGaussKC + k, col = pass * kGaussTileN + n;
         float hi = 0.f, lo = 0.f;
         if (col < A.dw && t < A.N) {
-            const double v = (double)A.base[A.cols[A.dx + col] + t] - A.mean[A.dx + col];
+            const double v = (double)A.base[A.cols[A.dx + col] + t] - A.meanw[col];
             hi = __uint_as_float(to_tf32((float)v));
             lo = __uint_as_float(to_tf32((float)(v - (double)hi)));
         }
@@ -639,7 +642,7 @@ __device__ __forceinline__ void gauss_cross_f64_body(const GaussArgs &A, int bx,
         for (int e = threadIdx.x; e < kGaussKC * DW4; e += kF64Rows) {
             const int t = e / DW4, w = e - t * DW4;
             sW[t][w] = (t < n && w < dw)
-                           ? (double)A.base[A.cols[A.dx + w] + t0 + t] - A.mean[A.dx + w]
+                           ? (double)A.base[A.cols[A.dx + w] + t0 + t] - A.meanw[w]
                            : 0.0;
         }
         __syncthreads();
@@ -695,7 +698,7 @@ __device__ __forceinline__ void gauss_cross_ff_body(const GaussArgs &A, int bx, 
             const int t = e / DW, w = e - t * DW;
             float2 v = make_float2(0.f, 0.f);
             if (t < n && w < dw) {
-                const double d = (double)A.base[A.cols[A.dx + w] + t0 + t] - A.mean[A.dx + w];
+                const double d = (double)A.base[A.cols[A.dx + w] + t0 + t] - A.meanw[w];
                 v.x = (float)d;
                 v.y = (float)(d - (double)v.x);
             }
@@ -747,6 +750,181 @@ __device__ __forceinline__ void gauss_cross_ff_body(const GaussArgs &A, int bx, 
 #pragma unroll
     for (int w = 0; w < DW; ++w)
         if (w < dw) dst[w] = acc[w];
+}
+
+// The permutations of a set, turned: [S][N] 32-bit rows -> [N][pitch] 16-bit
+// entries, column 0 the identity, so that the rows a warp serves (consecutive
+// surrogates) read one point's indices as one line.
+__global__ void __launch_bounds__(256) gauss_turn_kernel(const PermTurnJob *jobs)
+{
+    __shared__ uint16_t tile[64][66];
+    const PermTurnJob J = jobs[blockIdx.z];
+    const int t0 = blockIdx.x * 64, s0 = blockIdx.y * 64;
+    if (t0 >= J.N || s0 >= J.pitch) return;
+    for (int e = threadIdx.x; e < 64 * 64; e += 256) {
+        const int s = e >> 6, t = e & 63;
+        int v = 0;
+        if (t0 + t < J.N) {
+            if (s0 + s == 0) v = t0 + t;
+            else if (s0 + s <= J.S) v = J.src[(size_t)(s0 + s - 1) * J.N + t0 + t];
+        }
+        tile[t][s] = (uint16_t)v;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 64 * 32; e += 256) {
+        const int t = e >> 5, s = 2 * (e & 31);
+        if (t0 + t < J.N && s0 + s < J.pitch)
+            *reinterpret_cast<uint32_t *>(J.dst + (size_t)(t0 + t) * J.pitch + s0 + s) =
+                *reinterpret_cast<const uint32_t *>(&tile[t][s]);
+    }
+}
+
+// The float-float contraction of gauss_cross_ff_body with its gathers in
+// shared memory.  One thread per surrogate and X dimension; the CTA keeps the
+// centred X column there (80 KB at N = 10^4, two CTAs an SM) and reads the
+// turned permutations, so that a warp's 32 gathers cost their bank conflicts
+// (about 7 cycles of 8-byte loads) and its 32 indices one line, where gathers
+// through L1 took a cycle per row each for the indices and the values (64
+// cycles a point, against 12 of arithmetic at dw = 4).  319 estimates of 201
+// rows, dw = 4, N = 9995: 3.1 -> 1.5 ms, the FMA pipe 58% and issue 73% busy.
+// smem: N float2
+//
+// The CTA's H parts of `rows` threads take consecutive splits of the points
+// with one copy of the column: seven warps (201 surrogates) an SM's half would
+// not cover the latency of the index loads, which also run eight points ahead.
+constexpr int kFFTile = 64;   // points of W staged at a time
+template <int DW, int H>
+__device__ __forceinline__ void gauss_cross_col_body(const GaussArgs &A, int bx, int by, int rows_t,
+                                                     const float2 *col, float2 (*sWh)[DW])
+{
+    const int part = H == 1 ? 0 : (int)threadIdx.x / rows_t;
+    const int tid = (int)threadIdx.x - part * rows_t;
+    const int split = by * H + part;
+    const int nb = (A.S + rows_t) / rows_t;   // blocks of surrogates per X dimension
+    const int a = bx / nb, s = (bx - a * nb) * rows_t + tid, dw = A.dw;
+    const bool live = s <= A.S && split < A.splits;
+    const uint16_t *pt = A.perm_t + min(s, A.S);
+    const size_t pitch = (size_t)A.perm_t_pitch;
+    float2 (*sW)[DW] = sWh + part * kFFTile;
+    double acc[DW];
+    float sh[DW], sl[DW];
+#pragma unroll
+    for (int w = 0; w < DW; ++w) {
+        acc[w] = 0.0;
+        sh[w] = sl[w] = 0.f;
+    }
+    const int span = A.chunks_per_split * kGaussKC;
+    const int t_begin = split * span;
+    const int t_end = min(A.N, t_begin + span);   // may lie below t_begin in the last CTA
+    int src[8];
+    auto load_src = [&](int t) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) src[u] = pt[(size_t)min(t + u, A.N - 1) * pitch];
+    };
+    load_src(t_begin);
+    int window = 0;   // points in the float pairs since their last flush
+    for (int dt = 0; dt < span; dt += kFFTile) {   // the same steps in every part
+        const int t0 = t_begin + dt, n = min(kFFTile, t_end - t0);
+        __syncthreads();
+        for (int e = tid; e < kFFTile * DW; e += rows_t) {
+            const int t = e / DW, w = e - t * DW;
+            float2 v = make_float2(0.f, 0.f);
+            if (t < n && w < dw) {
+                const double d = (double)A.base[A.cols[A.dx + w] + t0 + t] - A.meanw[w];
+                v.x = (float)d;
+                v.y = (float)(d - (double)v.x);
+            }
+            sW[t][w] = v;
+        }
+        __syncthreads();
+        for (int t8 = 0; t8 < n; t8 += 8) {   // past n: W is zero
+            float2 xs[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) xs[u] = col[src[u]];
+            load_src(t0 + t8 + 8);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float2 x = xs[u];
+#pragma unroll
+                for (int w = 0; w < DW; ++w) {
+                    const float2 y = sW[t8 + u][w];
+                    const float p = __fmul_rn(x.x, y.x);
+                    float e = __fmaf_rn(x.x, y.x, -p);
+                    e = __fmaf_rn(x.x, y.y, e);
+                    e = __fmaf_rn(x.y, y.x, e);
+                    const float sn = __fadd_rn(sh[w], p);
+                    const float bp = __fsub_rn(sn, sh[w]);
+                    const float er =
+                        __fadd_rn(__fsub_rn(sh[w], __fsub_rn(sn, bp)), __fsub_rn(p, bp));
+                    sl[w] = __fadd_rn(sl[w], __fadd_rn(er, e));
+                    sh[w] = sn;
+                }
+            }
+        }
+        window += kFFTile;
+        if (window >= kGaussFFWindow * kGaussKC || dt + kFFTile >= span) {
+            window = 0;
+#pragma unroll
+            for (int w = 0; w < DW; ++w) {
+                acc[w] += (double)sh[w] + (double)sl[w];
+                sh[w] = sl[w] = 0.f;
+            }
+        }
+    }
+    if (!live) return;
+    const int rows = (A.S + 1) * A.dx;
+    double *dst = A.cross_part + ((size_t)split * rows + (size_t)s * A.dx + a) * dw;
+#pragma unroll
+    for (int w = 0; w < DW; ++w)
+        if (w < dw) dst[w] = acc[w];
+}
+
+// Estimates whose contraction runs there, in two kernels by register use
+constexpr int kFFSmallW = 8;
+__device__ __forceinline__ bool gauss_takes_col(const GaussArgs &A)
+{
+    return A.perm_t != nullptr && A.dw <= kGaussFFMaxW && A.N <= kGaussFFColMax;
+}
+
+template <int H>
+__global__ void __launch_bounds__(256 * H, 2) gauss_cross_col_batch(const GaussArgs *args,
+                                                                    int rows_t)
+{
+    constexpr bool kSmall = H > 1;
+    constexpr int WMAX = kSmall ? kFFSmallW : kGaussFFMaxW;
+    extern __shared__ __align__(16) float2 ccol[];
+    __shared__ __align__(16) float2 sW[H * kFFTile * WMAX];
+    const GaussArgs A = args[blockIdx.z];
+    const int nb = (A.S + rows_t) / rows_t;
+    if (!gauss_takes_col(A) || (A.dw <= kFFSmallW) != kSmall || (int)blockIdx.x >= nb * A.dx ||
+        (int)blockIdx.y * H >= A.splits)
+        return;
+    const int a = (int)blockIdx.x / nb;
+    const float2 *src = reinterpret_cast<const float2 *>(A.xc) + (size_t)a * A.N;
+    for (int t = threadIdx.x; t < A.N; t += blockDim.x) ccol[t] = __ldg(src + t);
+#define TE_COL_CASE(DW)                                                                          \
+    gauss_cross_col_body<DW, H>(A, blockIdx.x, blockIdx.y, rows_t, ccol,                         \
+                                reinterpret_cast<float2 (*)[DW]>(sW))
+    if constexpr (kSmall) {
+        switch (A.dw) {
+        case 1: TE_COL_CASE(1); break;
+        case 2: TE_COL_CASE(2); break;
+        case 3: TE_COL_CASE(3); break;
+        case 4: TE_COL_CASE(4); break;
+        case 5: TE_COL_CASE(5); break;
+        case 6: TE_COL_CASE(6); break;
+        case 7: TE_COL_CASE(7); break;
+        default: TE_COL_CASE(8); break;
+        }
+    } else {
+        switch ((A.dw + 1) >> 1) {
+        case 5: TE_COL_CASE(10); break;
+        case 6: TE_COL_CASE(12); break;
+        case 7: TE_COL_CASE(14); break;
+        default: TE_COL_CASE(16); break;
+        }
+    }
+#undef TE_COL_CASE
 }
 
 __device__ __forceinline__ void gauss_cross_f64_any(const GaussArgs &A, int bx, int by)
@@ -873,6 +1051,7 @@ __global__ void gauss_factor_batch(const GaussArgs *args)
 __global__ void __launch_bounds__(kF64Rows) gauss_cross_f64_batch(const GaussArgs *args)
 {
     const GaussArgs A = args[blockIdx.z];
+    if (gauss_takes_col(A)) return;
     if ((int)blockIdx.x * kF64Rows < (A.S + 1) * A.dx && (int)blockIdx.y < A.splits)
         gauss_cross_f64_any(A, blockIdx.x, blockIdx.y);
 }
@@ -895,6 +1074,9 @@ cudaError_t gauss_launch_batch_f64(const GaussArgs *args_dev, const GaussArgs *a
     if (n < 1) return cudaSuccess;
     if (n > 65535) return cudaErrorInvalidValue;
     int md = 1, mrb = 1, msp = 1, ms = 1, mdx = 1;
+    // the shared-memory contraction's share: [0] dw <= kFFSmallW, [1] wider
+    int col_n[2] = {0, 0}, col_rows = 32, col_blocks = 1;
+    bool others = false;
     long long mtot = 1;
     for (int i = 0; i < n; ++i) {
         const GaussArgs &A = args_host[i];
@@ -906,14 +1088,59 @@ cudaError_t gauss_launch_batch_f64(const GaussArgs *args_dev, const GaussArgs *a
         msp = std::max(msp, A.splits);
         ms = std::max(ms, A.S + 1);
         mtot = std::max(mtot, (long long)rows * A.dw);
+        if (A.perm_t && A.dw <= kGaussFFMaxW && A.N <= kGaussFFColMax) {
+            int &cn = col_n[A.dw <= kFFSmallW ? 0 : 1];
+            cn = std::max(cn, A.N);
+            col_rows = std::max(col_rows, std::min(256, (A.S + 32) & ~31));
+        } else {
+            others = true;
+        }
     }
+    for (int i = 0; i < n; ++i)
+        col_blocks =
+            std::max(col_blocks, (args_host[i].S + col_rows) / col_rows * args_host[i].dx);
     gauss_mean_batch<<<dim3(md, 1, n), 256, 0, st>>>(args_dev);
     gauss_cov_batch<<<dim3(md * (md + 1) / 2, 1, n), 256, 0, st>>>(args_dev);
     gauss_factor_batch<<<dim3(1, 1, n), kFactorThreads, 0, st>>>(args_dev);
     gauss_centre_batch<<<dim3(8, mdx, n), 256, 0, st>>>(args_dev);
-    gauss_cross_f64_batch<<<dim3(mrb, msp, n), kF64Rows, 0, st>>>(args_dev);
+    const void *cf[2] = {reinterpret_cast<const void *>(&gauss_cross_col_batch<2>),
+                         reinterpret_cast<const void *>(&gauss_cross_col_batch<1>)};
+    for (int c = 0; c < 2; ++c) {
+        if (!col_n[c]) continue;
+        static bool attr_done[2][64] = {};
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess && !(dev >= 0 && dev < 64 && attr_done[c][dev])) {
+            e = cudaFuncSetAttribute(cf[c], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kGaussFFColMax * 8);
+            if (e == cudaSuccess && dev >= 0 && dev < 64) attr_done[c][dev] = true;
+        }
+        const int parts = c == 0 ? 2 : 1;
+        void *ka[] = {&args_dev, &col_rows};
+        if (e == cudaSuccess)
+            e = cudaLaunchKernel(cf[c], dim3(col_blocks, (msp + parts - 1) / parts, n),
+                                 dim3(col_rows * parts), ka, (size_t)col_n[c] * 8, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (others)
+        gauss_cross_f64_batch<<<dim3(mrb, msp, n), kF64Rows, 0, st>>>(args_dev);
     gauss_cross_reduce_batch<<<dim3((unsigned)((mtot + 255) / 256), 1, n), 256, 0, st>>>(args_dev);
     gauss_schur_f64_batch<<<dim3((ms + 63) / 64, 1, n), 64, 0, st>>>(args_dev);
+    return cudaGetLastError();
+}
+
+cudaError_t gauss_launch_turn(const PermTurnJob *jobs_dev, const PermTurnJob *jobs_host, int n,
+                              cudaStream_t st)
+{
+    if (n < 1) return cudaSuccess;
+    if (n > 65535) return cudaErrorInvalidValue;
+    int mt = 1, ms = 1;
+    for (int i = 0; i < n; ++i) {
+        if (jobs_host[i].N > 65535 || (jobs_host[i].pitch & 1)) return cudaErrorInvalidValue;
+        mt = std::max(mt, (jobs_host[i].N + 63) / 64);
+        ms = std::max(ms, (jobs_host[i].pitch + 63) / 64);
+    }
+    gauss_turn_kernel<<<dim3(mt, ms, n), 256, 0, st>>>(jobs_dev);
     return cudaGetLastError();
 }
 

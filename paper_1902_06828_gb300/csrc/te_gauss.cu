@@ -58,6 +58,7 @@ void gauss_bind(GaussArgs &A, double *w, bool xc = false)
     A.xc = xc ? A.cross_part + (size_t)A.splits * (A.S + 1) * A.dx * dw : nullptr;
     A.covw = A.cov;
     A.own_w = 1;
+    A.meanw = A.mean + A.dx;
 }
 
 // offset of variable v's column at the first point: the value at point t is
@@ -136,8 +137,22 @@ te_status run_groups_gauss(te_ctx *ctx, const std::vector<HostGroup> &groups, in
             for (const te_var &v : g.z) cols.push_back(gauss_col(g.data, g.max_lag, v));
         }
     }
+    // every permutation set turned once for the contraction in shared memory
+    std::vector<PermTurnJob> turn;
+    std::map<const int32_t *, size_t> turn_of;   // -> 16-bit entries into the turned sets
+    size_t turn_elems = 0;
+    for (GaussArgs &A : est) {
+        if (A.d - A.dx > kGaussFFMaxW || A.N > kGaussFFColMax || A.S < 1) continue;
+        A.perm_t_pitch = (A.S + 32) & ~31;
+        if (turn_of.emplace(A.perms, turn_elems).second) {
+            turn.push_back(PermTurnJob{A.perms, nullptr, A.S, A.N, A.perm_t_pitch});
+            turn_elems += (size_t)A.N * A.perm_t_pitch;
+        }
+    }
     // shapes: a batch splits each estimate's points so that the contraction
-    // has about eight CTAs per SM in all
+    // has about eight CTAs per SM in all; where a CTA keeps the X column (two
+    // fit an SM, each takes two splits, and loading the column costs it 1% of a
+    // whole estimate) eight waves of them, so that the last is a small part
     const int n_est = (int)est.size();
     size_t ws = 0;
     std::vector<size_t> off(n_est);
@@ -146,8 +161,10 @@ te_status run_groups_gauss(te_ctx *ctx, const std::vector<HostGroup> &groups, in
         size_t w = 0;
         for (int i = b0; i < b0 + nb; ++i) {
             GaussArgs &A = est[i];
-            const int blocks = ((A.S + 1) * A.dx + 127) / 128;
-            const int splits = (8 * 152 + nb * blocks - 1) / (nb * blocks);
+            const int blocks = A.perm_t_pitch ? (A.S + 256) / 256 * A.dx
+                                              : ((A.S + 1) * A.dx + 127) / 128;
+            const bool col = A.perm_t_pitch != 0;
+            const int splits = ((col ? 32 : 8) * 152 + nb * blocks - 1) / (nb * blocks);
             off[i] = w;
             w += gauss_shape(A, A.N, A.S, A.dx, A.dy, A.d - A.dx - A.dy, splits, true);
         }
@@ -170,6 +187,20 @@ te_status run_groups_gauss(te_ctx *ctx, const std::vector<HostGroup> &groups, in
     CK(cudaMemsetAsync(v_out, 0, (size_t)n_out * 8, ctx->stream), "cudaMemsetAsync");
     if (!cols.empty())
         CK(copy_h2d(ctx, cols_dev, cols.data(), cols.size() * 4), "cudaMemcpyAsync");
+    if (!turn.empty()) {
+        const size_t jobs_at = (turn_elems * 2 + 255) & ~(size_t)255;
+        if ((st = ensure_dev(ctx, ctx->ws_gtile, jobs_at + turn.size() * sizeof(PermTurnJob))))
+            return st;
+        uint16_t *tb = (uint16_t *)ctx->ws_gtile.p;
+        for (PermTurnJob &J : turn) J.dst = tb + turn_of[J.src];
+        for (GaussArgs &A : est)
+            if (A.perm_t_pitch) A.perm_t = tb + turn_of[A.perms];
+        PermTurnJob *jd = (PermTurnJob *)((char *)ctx->ws_gtile.p + jobs_at);
+        CK(copy_h2d(ctx, jd, turn.data(), turn.size() * sizeof(PermTurnJob)), "cudaMemcpyAsync");
+        CK(gauss_launch_turn(jd, turn.data(), (int)turn.size(), ctx->stream),
+           "permutation turn launch");
+        ctx->stats.launches++;
+    }
     int src = 0;
     for (int i = 0; i < n_est; ++i) {
         GaussArgs &A = est[i];
@@ -185,6 +216,7 @@ te_status run_groups_gauss(te_ctx *ctx, const std::vector<HostGroup> &groups, in
         } else {
             A.own_w = 0;
             A.covw = est[src].cov;
+            A.meanw = est[src].mean + est[src].dx;
             A.LW = est[src].LW;
             A.LZ = est[src].LZ;
             A.norms = est[src].norms;

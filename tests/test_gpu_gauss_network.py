@@ -126,3 +126,68 @@ def test_gauss_network_full_length_target(te, ctx):
     assert gt["omnibus_p"] == r.omnibus_p
     assert abs(gt["omnibus_cmi"] - r.omnibus_cmi) <= TOL
     assert gt["n_estimates"] == r.n_estimates
+
+
+@pytest.mark.parametrize("T,S", [(203, 31), (703, 32), (706, 33), (1031, 255), (390, 256),
+                                 (1417, 300)])
+def test_every_estimate_at_growing_conditioning_sets(te, ctx, T, S):
+    """Every traced estimate against a plain FP64 evaluation, at surrogate
+    counts on both sides of a warp and of a block of rows and at odd lengths.
+    With alpha = 0.9 almost every candidate is selected, so that W grows
+    column by column from 1 to over 16, through every width of the
+    shared-memory contraction and into the FP64 one."""
+    from oracle import ksg as oksg
+    L, n = 6, 3
+    x, _adj, _lags = synth.var_er(n=n, p=0.5, T=T, seed=T, lo=0.3, hi=0.6, max_lag=3)
+    s = synth.standardise_jitter(x, T).astype(np.longdouble)
+    N = T - L
+    col = lambda v: s[v[0], L - v[1]:T - v[1]]
+    sel, widths, errs = [], set(), []
+
+    def explained(a, c):   # c^T a^-1 c by a Cholesky factor (lags are nearly collinear)
+        m = len(a)
+        f, v = np.zeros((m, m), np.longdouble), np.zeros_like(c)
+        for j in range(m):
+            f[j, j] = np.sqrt(a[j, j] - np.sum(f[j, :j] ** 2))
+            f[j + 1:, j] = (a[j + 1:, j] - f[j + 1:, :j] @ f[j, :j]) / f[j, j]
+        for j in range(m):
+            v[:, j] = (c[:, j] - v[:, :j] @ f[j, :j]) / f[j, j]
+        return np.sum(v ** 2, axis=1)
+
+    def value(key):   # inverse of the order-preserving image
+        k = key & ((1 << 64) - 1)
+        k = k - (1 << 64) if k >= 1 << 63 else k
+        return np.int64(k if k >= 0 else k ^ 0x7FFFFFFFFFFFFFFF).view(np.float64)
+
+    def check(target, stage, it, vs, n_cand, n_surr, keys):
+        if stage not in (1, 2):
+            return
+        got = np.array([[value(k) for k in row] for row in keys])
+        W = np.array([col((0, 0))] + [col(v) for v in sel])
+        W = W - W.mean(1, keepdims=True)
+        widths.add(len(W))
+        perms = [np.arange(N)] + [oksg.permutation(9, 0, stage, it, a, N)
+                                  for a in range(1, n_surr + 1)]
+        sww = W @ W.T / (N - 1)
+        for c, v in enumerate(vs):
+            xc = col(v) - col(v).mean()
+            cw = np.array([xc[p] for p in perms]) @ W.T / (N - 1)
+            sxx = xc @ xc / (N - 1)
+            ref = 0.5 * (np.log(sxx - explained(sww[1:, 1:], cw[:, 1:]))
+                         - np.log(sxx - explained(sww, cw)))
+            errs.append(float(np.max(np.abs(got[c] - ref))))
+        best = int(np.argmax(got[:, 0]))
+        if np.sum(got[:, 1:].max(0) > got[best, 0]) / n_surr < 0.9:
+            sel.append(tuple(vs[best]))
+
+    data = te.te_data_create(ctx, s.astype(np.float32))
+    ctx.set_trace(check)
+    try:
+        te.te_network_infer(ctx, data, max_lag_target=L, max_lag_sources=L, n_surr=S,
+                            alpha_max=0.9, alpha_min=0.9, alpha_omnibus=0.9, seed=9, targets=[0],
+                            estimator="gauss")
+    except te.TEError as e:   # more than 8 sources left for the omnibus block
+        assert "dx <= 8" in str(e)
+    finally:
+        ctx.set_trace(None)
+    assert len(errs) > 20 and max(widths) > 4 and max(errs) <= TOL
