@@ -32,6 +32,11 @@ struct GaussArgs {
     float *btile;
     float *xcen;
     int xcen_pitch;
+    // cmi_gauss's statistics: all columns centred in FP64, cen[c * xcen_pitch + t],
+    // zero past N; partial sums of the columns and of the products of column
+    // pairs over kGaussParts ranges of the points; inverse factors [dw][dw] (lower)
+    // and {||L_W^-1||_F^2, ||L_Z^-1||_F^2, tr S_WW, tr S_ZZ, tr S_XX}
+    double *cen, *sum_part, *cov_part, *inv_w, *inv_z, *traces;
     double *mean;           // [d] (X only where own_w = 0)
     const double *meanw;    // [dw] means of the W columns: mean + dx, or another estimate's
     double *cov;            // [d][d] sample covariance, ddof = 1 (its X-W blocks are not formed:
@@ -61,10 +66,15 @@ struct GaussArgs {
 int gauss_cross_splits(int rows, int N);
 // splits of the tensor-core contraction: one FP32 accumulation group each
 int gauss_tc_splits(int N);
-// bytes of the tensor-core contraction's prepared inputs (btile, xcen)
+// bytes of the tensor-core contraction's prepared inputs and the statistics
+// (btile .. traces), and their pointers in a buffer at base
+constexpr int kGaussParts = 8;
 size_t gauss_tc_workspace(int N, int dx, int dw);
+void gauss_tc_bind(GaussArgs &A, void *base);
 
-cudaError_t gauss_launch_stats(const GaussArgs &A, cudaStream_t st);
+// column sums and the contraction's inputs, then covariances and factors
+cudaError_t gauss_launch_prepare(const GaussArgs &A, cudaStream_t st);
+cudaError_t gauss_launch_factor(const GaussArgs &A, cudaStream_t st);
 cudaError_t gauss_launch_cross_tc(const GaussArgs &A, cudaStream_t st);
 double gauss_tc_gamma();   // relative error factor of the tensor-core contraction
 // relative error factor of the FP64 contraction: a sum of N FP64 products

@@ -397,37 +397,211 @@ __device__ __forceinline__ uint32_t cm_offset(int row, int k)
 
 constexpr int kGaussColMax = 16384;   // X column points kept in shared memory
 
-// W's B tiles: tile (pass p, chunk c) at btile + (p * nchunks + c) * 2048
-// floats, hi then lo, each in the core-matrix layout of 32 columns x 32 points
-__global__ void gauss_tc_prep_w(GaussArgs A, int nchunks)
+// ---- the statistics of one call (gauss_launch_prepare, gauss_launch_factor) ----
+// GB300's FP64 pipe takes two lanes a clock and SM, so the sums are spread
+// over the chip (kGaussParts ranges of the points each, added in order) and a
+// term costs one FP64 operation: columns are centred once.  N = 9995: sums 24 ->
+// 9 us, covariances of 39 columns 109 -> 21 us (one CTA for each before).
+
+// partial sum of column c over range `part`: grid (d, kGaussParts)
+__global__ void __launch_bounds__(128) gauss_sum_kernel(GaussArgs A)
 {
+    __shared__ double red[32];
+    const int c = blockIdx.x, part = blockIdx.y;
+    const int t0 = (int)((long long)A.N * part / kGaussParts);
+    const int t1 = (int)((long long)A.N * (part + 1) / kGaussParts);
+    const float *col = A.base + A.cols[c];
+    double s = 0.0;
+    for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) s += (double)col[t];
+    s = block_sum(s, red);
+    if (threadIdx.x == 0) A.sum_part[c * kGaussParts + part] = s;
+}
+
+// Chunk blockIdx.x of 32 points: for pass blockIdx.y < passes, W's B tile
+// (tile (pass, chunk) at btile + (pass * nchunks + chunk) * 2048 floats, hi
+// then lo, each in the core-matrix layout of 32 columns x 32 points) and W's
+// centred columns; for blockIdx.y == passes the X columns, centred in FP64
+// and rounded once to FP32 for the gathers.
+__global__ void __launch_bounds__(256) gauss_prep_kernel(GaussArgs A, int nchunks, int passes)
+{
+    __shared__ double s_mean[kGaussTileN];
     const int c = blockIdx.x, pass = blockIdx.y;
+    const bool is_x = pass == passes;
+    const int col0 = is_x ? 0 : A.dx + pass * kGaussTileN;
+    const int n_cols = is_x ? A.dx : min(kGaussTileN, A.dw - pass * kGaussTileN);
+    if (threadIdx.x < n_cols) {
+        double s = 0.0;
+        for (int p = 0; p < kGaussParts; ++p)
+            s += A.sum_part[(col0 + threadIdx.x) * kGaussParts + p];
+        s_mean[threadIdx.x] = s / (double)A.N;
+    }
+    __syncthreads();
     float *hb = A.btile + ((size_t)pass * nchunks + c) * 2048;
     float *lb = hb + 1024;
     for (int e = threadIdx.x; e < kGaussTileN * kGaussKC; e += blockDim.x) {
         const int n = e / kGaussKC, k = e % kGaussKC;
-        const int t = c * kGaussKC + k, col = pass * kGaussTileN + n;
-        float hi = 0.f, lo = 0.f;
-        if (col < A.dw && t < A.N) {
-            const double v = (double)A.base[A.cols[A.dx + col] + t] - A.meanw[col];
-            hi = __uint_as_float(to_tf32((float)v));
-            lo = __uint_as_float(to_tf32((float)(v - (double)hi)));
+        const int t = c * kGaussKC + k;
+        double v = 0.0;
+        if (n < n_cols && t < A.N) v = (double)A.base[A.cols[col0 + n] + t] - s_mean[n];
+        if (n < n_cols) A.cen[(size_t)(col0 + n) * A.xcen_pitch + t] = v;
+        if (is_x) {
+            if (n < n_cols) A.xcen[(size_t)n * A.xcen_pitch + t] = (float)v;
+        } else {
+            const float hi = __uint_as_float(to_tf32((float)v));
+            const uint32_t off = cm_offset(n, k) / 4;
+            hb[off] = hi;
+            lb[off] = __uint_as_float(to_tf32((float)(v - (double)hi)));
         }
-        const uint32_t off = cm_offset(n, k) / 4;
-        hb[off] = hi;
-        lb[off] = lo;
     }
 }
 
-// X centred in FP64, rounded once to FP32: xcen[i * xcen_pitch + t]
-__global__ void gauss_tc_prep_x(GaussArgs A)
+// Products of the centred columns summed over range blockIdx.y for a tile of
+// 4 x 4 column pairs (W-W tiles first, then X-X; X-W pairs are cross's): 16
+// FP64 FMAs for 8 loads a point and thread, then a sum in thread order.
+__device__ __forceinline__ void gauss_tile_pair(int t, int &i, int &j)
 {
-    const int i = blockIdx.y;
-    const float *col = A.base + A.cols[i];
-    const double m = A.mean[i];
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < A.xcen_pitch;
-         t += gridDim.x * blockDim.x)
-        A.xcen[(size_t)i * A.xcen_pitch + t] = t < A.N ? (float)((double)col[t] - m) : 0.f;
+    j = 0;
+    while (t > j) {
+        t -= j + 1;
+        ++j;
+    }
+    i = t;
+}
+__global__ void __launch_bounds__(128) gauss_cov_tiles_kernel(GaussArgs A)
+{
+    __shared__ double s_sum[16][129];
+    const int tw = (A.dw + 3) / 4, nw = tw * (tw + 1) / 2;
+    int ti, tj;
+    const bool is_x = (int)blockIdx.x >= nw;
+    gauss_tile_pair(is_x ? (int)blockIdx.x - nw : (int)blockIdx.x, ti, tj);
+    const int c0 = is_x ? 0 : A.dx, n = is_x ? A.dx : A.dw;
+    const int part = blockIdx.y, tid = threadIdx.x;
+    const int t0 = (int)((long long)A.N * part / kGaussParts);
+    const int t1 = (int)((long long)A.N * (part + 1) / kGaussParts);
+    const double *pa[4], *pb[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {   // past the last column: the last again, not stored
+        pa[a] = A.cen + (size_t)(c0 + min(4 * ti + a, n - 1)) * A.xcen_pitch;
+        pb[a] = A.cen + (size_t)(c0 + min(4 * tj + a, n - 1)) * A.xcen_pitch;
+    }
+    double acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
+    for (int t = t0 + tid; t < t1; t += 128) {
+        double va[4], vb[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            va[a] = __ldg(pa[a] + t);
+            vb[a] = __ldg(pb[a] + t);
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) acc[a][b] = fma(va[a], vb[b], acc[a][b]);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) s_sum[4 * a + b][tid] = acc[a][b];
+    __syncthreads();
+    const int v = tid >> 3, l = tid & 7;
+    double s = 0.0;
+    for (int e = 0; e < 16; ++e) s += s_sum[v][16 * l + e];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const int i = 4 * ti + (v >> 2), j = 4 * tj + (v & 3);
+    if (l == 0 && i < n && j < n && i <= j)
+        A.cov_part[((size_t)part * A.d + c0 + i) * A.d + c0 + j] = s;
+}
+
+// Covariances from their parts, and the inverse of the Cholesky factor of S_WW
+// (block 0) and S_ZZ (block 1; Z is the trailing block of W), as the unit
+// lower inverse of an L D L^T factorisation scaled by D^-1/2 at the end.
+// Right-looking, the inverse's rows updated beside the trailing block, sixteen
+// lanes a row: each of the n steps is a chain of one division and one update
+// (an FP64 operation's latency is some 60 clocks), where a warp's row-oriented
+// factorisation and a thread's column solve were chains of ~800 (39 columns:
+// 190 -> 75 us; 5 columns: 13 -> 11).
+constexpr int kFactorLanes = 16;
+__global__ void __launch_bounds__(kFactorLanes * 40) gauss_factor_inv_kernel(GaussArgs A)
+{
+    __shared__ double sA[kFacW * kFacW], sX[kFacW * kFacW];
+    __shared__ double s_f[kFacW], s_red[kFactorLanes * 40 / 32];
+    static_assert(kFacW <= 40, "a row per sixteen threads");
+    const int tid = threadIdx.x, d = A.d, dx = A.dx;
+    const int off = blockIdx.x == 0 ? 0 : A.dy, n = A.dw - off;
+    auto cov = [&](int i, int j) {   // i <= j
+        double v[kGaussParts], s = 0.0;
+#pragma unroll
+        for (int p = 0; p < kGaussParts; ++p)
+            v[p] = __ldg(A.cov_part + ((size_t)p * d + i) * d + j);
+#pragma unroll
+        for (int p = 0; p < kGaussParts; ++p) s += v[p];
+        return s / (double)(A.N - 1);
+    };
+    const int i = tid / kFactorLanes, l = tid % kFactorLanes;   // this thread's row and lane
+    if (i < n)
+        for (int c = l; c <= i; c += kFactorLanes) {
+            const double v = cov(dx + off + c, dx + off + i);
+            sA[i * n + c] = v;
+            sX[i * n + c] = i == c ? 1.0 : 0.0;
+            if (blockIdx.x == 0)
+                A.cov[(dx + i) * d + dx + c] = A.cov[(dx + c) * d + dx + i] = v;
+        }
+    if (blockIdx.x == 0)
+        for (int e = tid; e < dx * dx; e += blockDim.x) {
+            const int r = e / dx, c = e - r * dx;
+            if (c <= r) A.cov[r * d + c] = A.cov[c * d + r] = cov(c, r);
+        }
+    __syncthreads();
+    if (tid < 32) {   // trace of the W (or Z) block
+        double s = 0.0;
+        for (int r = tid; r < n; r += 32) s += sA[r * n + r];
+        s = warp_sum_d(s);
+        if (tid == 0) A.traces[2 + blockIdx.x] = s;
+    } else if (tid == 32 && blockIdx.x == 0) {   // and of X's
+        double s = 0.0;
+        for (int a = 0; a < dx; ++a) s += cov(a, a);
+        A.traces[4] = s;
+    }
+    for (int j = 0; j < n; ++j) {
+        __syncthreads();
+        const double pivot = sA[j * n + j];
+        if (!(pivot > 0.0)) {   // the same value for every thread
+            if (tid == 0) A.status[0] = 1;
+            return;
+        }
+        if (tid > j && tid < n) s_f[tid] = sA[tid * n + j] / pivot;
+        __syncthreads();
+        if (i > j && i < n) {
+            const double f = s_f[i];
+            for (int c = l; c <= i; c += kFactorLanes) {
+                if (c <= j) sX[i * n + c] -= f * sX[j * n + c];
+                else sA[i * n + c] -= f * sA[c * n + j];
+            }
+        }
+    }
+    __syncthreads();
+    if (tid < n) s_f[tid] = sqrt(sA[tid * n + tid]);
+    __syncthreads();
+    double *inv = blockIdx.x == 0 ? A.inv_w : A.inv_z;
+    double s = 0.0;
+    for (int e = tid; e < n * n; e += blockDim.x) {
+        const int r = e / n, c = e - r * n;
+        const double v = c <= r ? sX[e] / s_f[r] : 0.0;
+        inv[e] = v;
+        s += v * v;
+    }
+    s = warp_sum_d(s);
+    if ((tid & 31) == 0) s_red[tid >> 5] = s;
+    __syncthreads();
+    if (tid == 0) {
+        double t = 0.0;
+        for (int w = 0; w < kFactorLanes * 40 / 32; ++w) t += s_red[w];
+        A.traces[blockIdx.x] = t;
+    }
 }
 
 // 256 threads: thread (half h = tid / 128, row r = tid % 128) stages points
@@ -602,7 +776,15 @@ __device__ __forceinline__ void gauss_cross_reduce_body(const GaussArgs &A, long
     const long long total = (long long)(A.S + 1) * A.dx * A.dw;
     if (e >= total) return;
     double s = 0.0;
-    for (int p = 0; p < A.splits; ++p) s += A.cross_part[(size_t)p * total + e];
+    int p = 0;
+    for (; p + 16 <= A.splits; p += 16) {   // the loads of 16 splits together, added in order
+        double v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = __ldg(A.cross_part + (size_t)(p + u) * total + e);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) s += v[u];
+    }
+    for (; p < A.splits; ++p) s += A.cross_part[(size_t)p * total + e];
     A.cross[e] = s * (1.0 / (double)(A.N - 1));
 }
 
@@ -975,33 +1157,98 @@ __global__ void gauss_keys_kernel(const double *v, int n, long long *keys, int *
     keys[2 * (size_t)i + 1] = k;
 }
 
-__global__ void gauss_mean_kernel(GaussArgs A) { gauss_mean_body(A, blockIdx.x); }
-__global__ void gauss_cov_kernel(GaussArgs A) { gauss_cov_body(A, blockIdx.x); }
-__global__ void gauss_factor_kernel(GaussArgs A) { gauss_factor_body(A); }
-// Single-call Schur step: the two halves of a surrogate run on a pair of
-// adjacent threads (the chains are independent and GB300's FP64 pipe is
-// narrow, so more threads in flight hide more of their latency), with both
-// factors read from shared memory; same arithmetic as gauss_schur_body.
-constexpr int kSchurThreads = 64;
+// Single-call Schur step.  V = L^-1 C_V by the inverse factor, eight lanes
+// per surrogate and block (Z, W) taking every eighth row, so that no lane waits
+// on another's rows; S_XX - V^T V, its log-determinant and the bound are then
+// done for all of the CTA's surrogates by one warp (FP64 instructions cost 16
+// clocks a warp however many lanes take part).  1001 rows of 39 columns: 123 ->
+// 19 us, of 5 columns: 15 -> 8 (a thread per row and block, solving by rows).  DX: X dimensions, 1 or up to 8.
+constexpr int kSchurS = 8;        // surrogates per CTA
+constexpr int kSchurThreads = kSchurS * 16;
+template <int DX>
 __global__ void __launch_bounds__(kSchurThreads) gauss_schur_kernel(GaussArgs A, double gamma)
 {
-    __shared__ double sL[2][kFacW * kFacW];
-    const int dw = A.dw, dz = dw - A.dy;
-    for (int e = threadIdx.x; e < dw * dw; e += blockDim.x) {
-        sL[0][e] = (e / dw < dz && e % dw < dz) ? A.LZ[e] : 0.0;
-        sL[1][e] = A.LW[e];
+    constexpr int NP = DX * (DX + 1) / 2;
+    __shared__ double s_inv[2][kFacW * kFacW];
+    __shared__ double s_c[kSchurS][DX * (kGaussMaxDims - DX)];
+    __shared__ double s_dot[kSchurS * 2][NP];
+    const int tid = threadIdx.x, dx = DX == 1 ? 1 : A.dx, dw = A.dw, dy = A.dy, dz = dw - dy;
+    const int d = A.d, s0 = blockIdx.x * kSchurS;
+    for (int e = tid; e < dw * dw; e += kSchurThreads) s_inv[1][e] = A.inv_w[e];
+    for (int e = tid; e < dz * dz; e += kSchurThreads) s_inv[0][e] = A.inv_z[e];
+    const int per = dx * dw;
+    for (int e = tid; e < kSchurS * per; e += kSchurThreads) {
+        const int s = e / per;
+        s_c[s][e - s * per] = s0 + s <= A.S ? A.cross[(size_t)(s0 + s) * per + e - s * per] : 0.0;
     }
     __syncthreads();
-    const int s = blockIdx.x * (kSchurThreads / 2) + (int)(threadIdx.x >> 1);
-    const int which = threadIdx.x & 1;
+    const int s = tid >> 4, which = (tid >> 3) & 1, l = tid & 7;
+    const int n = which == 0 ? dz : dw, off = which == 0 ? dy : 0;
+    double dot[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) dot[p] = 0.0;
+    for (int r = l; r < n; r += 8) {
+        double v[DX];
+#pragma unroll
+        for (int a = 0; a < DX; ++a) {
+            v[a] = 0.0;
+            if (a < dx) {
+                double t0 = 0.0, t1 = 0.0;
+                int k = 0;
+                for (; k + 1 <= r; k += 2) {
+                    t0 = fma(s_inv[which][r * n + k], s_c[s][a * dw + off + k], t0);
+                    t1 = fma(s_inv[which][r * n + k + 1], s_c[s][a * dw + off + k + 1], t1);
+                }
+                if (k <= r) t0 = fma(s_inv[which][r * n + k], s_c[s][a * dw + off + k], t0);
+                v[a] = t0 + t1;
+            }
+        }
+#pragma unroll
+        for (int a = 0, p = 0; a < DX; ++a)
+#pragma unroll
+            for (int b = 0; b <= a; ++b, ++p) dot[p] = fma(v[a], v[b], dot[p]);
+    }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) dot[p] += __shfl_xor_sync(0xffffffffu, dot[p], o);
+        if (l == 0) s_dot[2 * s + which][p] = dot[p];
+    }
+    __syncthreads();
+    if (tid >= 32) return;
+    // lane 2 s + which
     double ld = 0.0, bound = 0.0;
-    if (s <= A.S) gauss_schur_half(A, gamma, s, which, sL[which], ld, bound);
+    const int sl = tid >> 1, w = tid & 1;
+    if (tid < 2 * kSchurS) {
+        double Sm[DX * DX], tmp[DX], vnorm2 = 0.0;
+#pragma unroll
+        for (int a = 0, p = 0; a < DX; ++a)
+#pragma unroll
+            for (int b = 0; b <= a; ++b, ++p)
+                if (a < dx) {
+                    const double t = s_dot[tid][p];
+                    if (a == b) vnorm2 += t;
+                    Sm[a * dx + b] = Sm[b * dx + a] = A.cov[a * d + b] - t;
+                }
+        if (!chol(Sm, dx, dx)) {
+            ld = CUDART_NAN;
+            bound = CUDART_INF;
+        } else {
+            for (int a = 0; a < dx; ++a) ld += 2.0 * log(Sm[a * dx + a]);
+            // d ln|Sm| <= ||Sm^-1||_F ||dSm||_F,  ||dSm||_F <= 2 ||dC||_F ||L^-1||_F ||V||_F
+            const double sinv = sqrt(inv_frob2(Sm, dx, dx, tmp));
+            const double linv = (w == 0 ? dz : dw) > 0 ? sqrt(A.traces[1 - w]) : 0.0;
+            const double svv = (w == 0 ? dz : dw) > 0 ? A.traces[3 - w] : 0.0;
+            const double dcnorm2 = gamma * gamma * A.traces[4] * svv;
+            bound = sinv * 2.0 * sqrt(dcnorm2) * linv * sqrt(vnorm2);
+        }
+    }
     const double ld_o = __shfl_xor_sync(0xffffffffu, ld, 1);
     const double bound_o = __shfl_xor_sync(0xffffffffu, bound, 1);
-    if (s <= A.S && which == 0) {
-        A.out[s] = 0.5 * (ld - ld_o);
+    if (tid < 2 * kSchurS && w == 0 && s0 + sl <= A.S) {
+        A.out[s0 + sl] = 0.5 * (ld - ld_o);
         // factor 2 for second-order terms
-        A.err[s] = 2.0 * 0.5 * (bound + bound_o);
+        A.err[s0 + sl] = 2.0 * 0.5 * (bound + bound_o);
     }
 }
 __global__ void gauss_cross_reduce_kernel(GaussArgs A)
@@ -1166,24 +1413,66 @@ int gauss_cross_splits(int rows, int N)
     return splits < 1 ? 1 : (splits > groups ? groups : splits);
 }
 
-cudaError_t gauss_launch_stats(const GaussArgs &A, cudaStream_t st)
-{
-    gauss_mean_kernel<<<A.d, 256, 0, st>>>(A);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    gauss_cov_kernel<<<A.d * (A.d + 1) / 2, 256, 0, st>>>(A);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    gauss_factor_kernel<<<1, kFactorThreads, 0, st>>>(A);
-    return cudaGetLastError();
-}
+static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-size_t gauss_tc_workspace(int N, int dx, int dw)
+// byte offsets of the parts of the buffer (btile first), and their end
+struct GaussTcLayout {
+    size_t xcen, cen, sum_part, cov_part, inv_w, inv_z, traces, end;
+};
+static GaussTcLayout gauss_tc_layout(int N, int dx, int dw)
 {
     const size_t nchunks = (size_t)(N + kGaussKC - 1) / kGaussKC;
     const size_t passes = (size_t)(dw + kGaussTileN - 1) / kGaussTileN;
-    const size_t pitch = ((size_t)N + 31) & ~(size_t)31;
-    return passes * nchunks * 2048 * 4 + (size_t)dx * pitch * 4;
+    const size_t pitch = ((size_t)N + 31) & ~(size_t)31, d = (size_t)(dx + dw);
+    GaussTcLayout o;
+    o.xcen = align256(passes * nchunks * 2048 * 4);
+    o.cen = align256(o.xcen + (size_t)dx * pitch * 4);
+    o.sum_part = align256(o.cen + d * pitch * 8);
+    o.cov_part = align256(o.sum_part + d * kGaussParts * 8);
+    o.inv_w = align256(o.cov_part + (size_t)kGaussParts * d * d * 8);
+    o.inv_z = align256(o.inv_w + (size_t)dw * dw * 8);
+    o.traces = align256(o.inv_z + (size_t)dw * dw * 8);
+    o.end = align256(o.traces + 8 * 8);
+    return o;
+}
+
+size_t gauss_tc_workspace(int N, int dx, int dw) { return gauss_tc_layout(N, dx, dw).end; }
+
+void gauss_tc_bind(GaussArgs &A, void *base)
+{
+    const GaussTcLayout o = gauss_tc_layout(A.N, A.dx, A.dw);
+    char *b = (char *)base;
+    A.btile = (float *)b;
+    A.xcen = (float *)(b + o.xcen);
+    A.xcen_pitch = (A.N + 31) & ~31;
+    A.cen = (double *)(b + o.cen);
+    A.sum_part = (double *)(b + o.sum_part);
+    A.cov_part = (double *)(b + o.cov_part);
+    A.inv_w = (double *)(b + o.inv_w);
+    A.inv_z = (double *)(b + o.inv_z);
+    A.traces = (double *)(b + o.traces);
+}
+
+cudaError_t gauss_launch_prepare(const GaussArgs &A, cudaStream_t st)
+{
+    gauss_sum_kernel<<<dim3(A.d, kGaussParts), 128, 0, st>>>(A);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const int nchunks = (A.N + kGaussKC - 1) / kGaussKC;
+    const int passes = (A.dw + kGaussTileN - 1) / kGaussTileN;
+    gauss_prep_kernel<<<dim3(nchunks, passes + 1), 256, 0, st>>>(A, nchunks, passes);
+    return cudaGetLastError();
+}
+
+cudaError_t gauss_launch_factor(const GaussArgs &A, cudaStream_t st)
+{
+    const int tw = (A.dw + 3) / 4, tx = (A.dx + 3) / 4;
+    gauss_cov_tiles_kernel<<<dim3(tw * (tw + 1) / 2 + tx * (tx + 1) / 2, kGaussParts), 128, 0,
+                             st>>>(A);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    gauss_factor_inv_kernel<<<2, kFactorLanes * 40, 0, st>>>(A);
+    return cudaGetLastError();
 }
 
 int gauss_tc_splits(int N)
@@ -1203,12 +1492,7 @@ cudaError_t gauss_launch_cross_tc(const GaussArgs &A, cudaStream_t st)
     if (A.perms16 && (A.perm_pitch < A.N || (A.perm_pitch & 7) ||
                       (reinterpret_cast<uintptr_t>(A.perms16) & 15)))
         return cudaErrorInvalidValue;
-    const int passes = (A.dw + kGaussTileN - 1) / kGaussTileN;
-    gauss_tc_prep_w<<<dim3(nchunks, passes), 256, 0, st>>>(A, nchunks);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    gauss_tc_prep_x<<<dim3((A.xcen_pitch + 255) / 256, A.dx), 256, 0, st>>>(A);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    cudaError_t e;
     const bool colsmem = A.dx == 1 && A.xcen_pitch <= kGaussColMax;
     const size_t smem = 1024 + (size_t)4 * (2 * kGaussTileM * kGaussKC + kGaussGroup * 2048 +
                                             (colsmem ? A.xcen_pitch : 0));
@@ -1234,7 +1518,7 @@ cudaError_t gauss_launch_cross_tc(const GaussArgs &A, cudaStream_t st)
         if (e != cudaSuccess) return e;
     }
     const long long total = (long long)rows * A.dw;
-    gauss_cross_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(A);
+    gauss_cross_reduce_kernel<<<(unsigned)((total + 63) / 64), 64, 0, st>>>(A);
     return cudaGetLastError();
 }
 
@@ -1250,8 +1534,9 @@ double gauss_tc_gamma()
 
 cudaError_t gauss_launch_schur(const GaussArgs &A, double gamma, cudaStream_t st)
 {
-    gauss_schur_kernel<<<(A.S + 1 + kSchurThreads / 2 - 1) / (kSchurThreads / 2), kSchurThreads, 0, st>>>(
-        A, gamma);
+    const int grid = (A.S + kSchurS) / kSchurS;
+    if (A.dx == 1) gauss_schur_kernel<1><<<grid, kSchurThreads, 0, st>>>(A, gamma);
+    else gauss_schur_kernel<kGaussMaxX><<<grid, kSchurThreads, 0, st>>>(A, gamma);
     return cudaGetLastError();
 }
 

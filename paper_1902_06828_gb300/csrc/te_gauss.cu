@@ -282,13 +282,7 @@ extern "C" te_status cmi_gauss(te_ctx *ctx, const te_data *data, const te_var *x
         A.perms16 = p16 ? (const uint16_t *)ctx->ws_perm.p : nullptr;
         A.perm_pitch = p16 ? pitch16 : 0;
         if ((st = ensure_dev(ctx, ctx->ws_gtile, gauss_tc_workspace(N, dx, dy + dz)))) return st;
-        {
-            const size_t nchunks = (size_t)(N + 31) / 32;
-            const size_t passes = (size_t)(dy + dz + 31) / 32;
-            A.btile = (float *)ctx->ws_gtile.p;
-            A.xcen = A.btile + passes * nchunks * 2048;
-            A.xcen_pitch = (N + 31) & ~31;
-        }
+        gauss_tc_bind(A, ctx->ws_gtile.p);
         A.out = w + ws;
         A.err = A.out + (S + 1);
         int *ip = (int *)(w + nd);
@@ -303,12 +297,15 @@ extern "C" te_status cmi_gauss(te_ctx *ctx, const te_data *data, const te_var *x
         CK(cudaMemsetAsync(A.status, 0, 2 * sizeof(int), ctx->stream), "cudaMemsetAsync");
         // the statistics (means, covariance, FP64 factors) do not depend on
         // the permutations: they run on the auxiliary stream while the
-        // permutations are drawn, and the contraction waits for both
+        // permutations are drawn; the contraction waits for the permutations
+        // and its inputs, the Schur step for the factors
         if ((st = ensure_aux(ctx))) return st;
         CK(cudaEventRecord(ctx->ev_fork, ctx->stream), "cudaEventRecord");
         CK(cudaStreamWaitEvent(ctx->aux_stream, ctx->ev_fork, 0), "cudaStreamWaitEvent");
-        CK(gauss_launch_stats(A, ctx->aux_stream), "Gaussian statistics launch");
+        CK(gauss_launch_prepare(A, ctx->aux_stream), "Gaussian preparation launch");
         CK(cudaEventRecord(ctx->ev_join, ctx->aux_stream), "cudaEventRecord");
+        CK(gauss_launch_factor(A, ctx->aux_stream), "Gaussian statistics launch");
+        CK(cudaEventRecord(ctx->ev_join2, ctx->aux_stream), "cudaEventRecord");
         if (p16)
             CK(launch_perms16((uint16_t *)ctx->ws_perm.p, pitch16, N, p->seed, p->stream_tag, 0,
                               0, 1, S, ctx->stream),
@@ -319,20 +316,23 @@ extern "C" te_status cmi_gauss(te_ctx *ctx, const te_data *data, const te_var *x
                "permutation launch");
         CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0), "cudaStreamWaitEvent");
         CK(gauss_launch_cross_tc(A, ctx->stream), "tensor-core cross-covariance launch");
+        CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_join2, 0), "cudaStreamWaitEvent");
         const double gamma = gauss_tc_gamma();
         CK(gauss_launch_schur(A, gamma, ctx->stream), "Schur launch");
         ctx->stats.launches += 7;
-        std::vector<double> res(2 * (size_t)(S + 1));
-        int status[2] = {0, 0};
-        CK(copy_d2h(ctx, res.data(), A.out, res.size() * 8), "cudaMemcpyAsync");
-        CK(copy_d2h(ctx, status, A.status, 8), "cudaMemcpyAsync");
+        // estimates, bounds and the status words behind them in one copy
+        const size_t res_bytes = 2 * (size_t)(S + 1) * 8;
+        if ((st = ensure_pin(ctx, res_bytes + 8))) return st;
+        CK(copy_d2h(ctx, ctx->pin, A.out, res_bytes + 8), "cudaMemcpyAsync");
         CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+        const double *res = (const double *)ctx->pin;
+        const int *status = (const int *)((const char *)ctx->pin + res_bytes);
         if (status[1])
             return fail(ctx, TE_ETIMEOUT, "tensor-core contraction did not complete in time");
         if (status[0])
             return fail(ctx, TE_EINVAL, "covariance of the conditioning variables is singular");
-        std::memcpy(out_cmi, res.data(), (size_t)(S + 1) * 8);
-        if (out_err_bound) std::memcpy(out_err_bound, res.data() + S + 1, (size_t)(S + 1) * 8);
+        std::memcpy(out_cmi, res, (size_t)(S + 1) * 8);
+        if (out_err_bound) std::memcpy(out_err_bound, res + S + 1, (size_t)(S + 1) * 8);
         return TE_OK;
     } catch (...) {
         return fail(ctx, TE_EINTERNAL, "unexpected C++ exception");

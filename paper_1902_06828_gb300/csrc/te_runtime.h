@@ -141,7 +141,7 @@ struct te_ctx {
     // second stream for work that overlaps the context's stream (created on
     // first use) and the events that fork to it and join back
     cudaStream_t aux_stream = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
     int prepared = 0, prepared_lists = 0;
     te_trace_fn trace_fn = nullptr;   // te_ctx_set_trace
     void *trace_user = nullptr;
