@@ -166,3 +166,24 @@ def test_static_entry_point_in_pieces(env, T, dz, dx, S, k):
     _, got = te.cmi_ksg_static(dev, x, [(0, 0)], Z[:dz], **kw)
     assert got == ref
     data.close()
+
+
+@pytest.mark.parametrize("T,dz,dx,k,w,S,levels", [
+    (38, 2, 1, 4, 0, 2, 0), (505, 0, 1, 4, 3, 9, 0), (505, 1, 1, 12, 0, 9, 0),
+    (1500, 2, 1, 4, 0, 33, 0), (1500, 3, 2, 4, 5, 9, 0), (1500, 1, 4, 16, 0, 9, 0),
+    (2600, 2, 1, 4, 0, 400, 7), (2600, 1, 1, 4, 0, 400, 300)])
+def test_pairs_beyond_the_radii(env, T, dz, dx, k, w, S, levels):
+    """Heavy tails (and, with levels, ties) put many pairs beyond their lists'
+    radii: fewer than a batch of the scan and more, more than a CTA can put
+    aside, and with more distances up to the bound than a pair can keep."""
+    te, ctx = env
+    rng = np.random.default_rng(T + dz)
+    s = rng.standard_cauchy(size=(10, T)).astype(np.float32)
+    if levels:
+        s = np.clip(np.round(s * levels / 20), -levels, levels).astype(np.float32)
+    data = te.te_data_create(ctx, s)
+    jobs = [te.Job(data, [(2, 1 + a) for a in range(dx)], [(0, 0)], Z[:dz], k=k, theiler=w,
+                   max_lag=5, n_surr=S, seed=3)]
+    got, ref = _both(te, ctx, jobs)
+    assert got == ref
+    data.close()
