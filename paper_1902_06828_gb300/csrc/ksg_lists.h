@@ -84,7 +84,7 @@ constexpr int kListBuildThreads = 512;
 constexpr int kListWalkThreads = 1024;   // of all walking CTAs on an SM
 
 // capacities of the two lists for a group
-void list_caps(int N, int k, int dx, int dy, int dz, size_t members, int *cap_a, int *cap_b);
+void list_caps(int N, int k, int dx, int dy, int dz, int *cap_a, int *cap_b);
 // Walk variant of a group: lanes per (point, member) pair, members per CTA, X
 // storage (1, 2, 4: a point's dimensions together; 0: a row per dimension),
 // k = 4.

@@ -143,7 +143,7 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
                     msorted.emplace_back(mdesc.size(), sorted_job(off(g.xvars[hm.xcol_first])));
                 mdesc.push_back(MemberDesc{hm.perm, xbase + hm.xcol_first, hm.out, nullptr});
             }
-            list_caps(N, g.k, g.dx, G.dy, G.dz, g.members.size(), &G.cap_a, &G.cap_b);
+            list_caps(N, g.k, g.dx, G.dy, G.dz, &G.cap_a, &G.cap_b);
             lg.push_back(G);
             const size_t row = list_row_bytes(G.cap_a, G.cap_b);
             for (int q0 = 0; q0 < N;) {

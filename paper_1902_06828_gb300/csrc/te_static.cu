@@ -158,7 +158,7 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
     // member-lane kernel, 213 with lists.
     const ListShape shape = list_shape(N, dx, dz, p->k, (size_t)S + 1);
     ListGroup lg{};
-    list_caps(N, p->k, dx, dy, dz, (size_t)S + 1, &lg.cap_a, &lg.cap_b);
+    list_caps(N, p->k, dx, dy, dz, &lg.cap_a, &lg.cap_b);
     const bool sorted_column = dz == 1 || (dz == 0 && dx == 1);
     const size_t np = ((size_t)N + 3) & ~(size_t)3;
     const size_t tab_off = total;
