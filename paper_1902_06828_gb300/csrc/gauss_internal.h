@@ -24,7 +24,6 @@ struct GaussArgs {
     // point itself) at perm_t[t * perm_t_pitch + s], or nullptr
     const uint16_t *perm_t;
     int perm_t_pitch;
-    int w0;                 // tensor-core contraction: first W column of this pass (32 per pass)
     // tensor-core contraction inputs prepared once per call: W's B tiles
     // (split TF32, core-matrix layout, 8 KB per 32-point chunk and pass) and
     // the centred X columns in FP32, xcen[i * xcen_pitch + t] (pitch a
@@ -58,14 +57,16 @@ struct GaussArgs {
     // the contraction is split along the points: split p sums chunks
     // [p * chunks_per_split, ...) into cross_part[p][S + 1][dx][dw]
     int splits, chunks_per_split;
+    int group;              // chunks per FP32 accumulation group of the tensor-core contraction
     double *cross_part;
 };
 // splits of the points for (S + 1) * dx rows of N points in the batched
 // FP64 / float-float contraction (every split keeps at least one accumulation
 // group)
 int gauss_cross_splits(int rows, int N);
-// splits of the tensor-core contraction: one FP32 accumulation group each
-int gauss_tc_splits(int N);
+// chunks of 32 points per split of the tensor-core contraction (two CTAs an SM)
+// and per FP32 accumulation group
+int gauss_tc_split_chunks(int N, int rows, int sms, int *group);
 // bytes of the tensor-core contraction's prepared inputs and the statistics
 // (btile .. traces), and their pointers in a buffer at base
 constexpr int kGaussParts = 8;

@@ -308,15 +308,15 @@ __device__ __forceinline__ void gauss_schur_body(const GaussArgs &A, double gamm
 // tcgen05.mma.kind::tf32 per K step, FP32 accumulation in tensor memory.
 //
 // What does not depend on the surrogate is prepared once per call
-// (gauss_tc_prep_*): W centred in FP64 and split, already laid out as the
-// MMA's B tiles (one 8 KB hi + lo tile per 32-point chunk and 32-column pass),
+// (gauss_prep_kernel): W centred in FP64 and split, already laid out as the
+// MMA's B tiles (one 8 KB hi + lo tile per 32-point chunk and 32 columns),
 // and X centred in FP64 and rounded to FP32 (one rounding of 2^-24).  A CTA
-// owns 128 rows and one FP32 accumulation group of at most kGaussGroup chunks:
-// it copies its B tiles with cp.async.bulk, keeps the X column in shared memory
-// (one X dimension and N <= kGaussColMax) or reads it through L1, gathers each
-// chunk's A operand through the 16-bit permutation rows (loaded one chunk
-// ahead), lets one thread issue the MMAs, and at the end reads the accumulator
-// once (tcgen05.ld) into its FP64 partial-sum row.  Operands use the canonical
+// owns 128 rows and a range of chunks: it copies B tiles with cp.async.bulk two
+// chunks ahead, keeps the X column in shared memory (one X dimension and
+// N <= kGaussColMax) or reads it through L1, gathers a chunk's A operand
+// through the 16-bit permutation rows (both a chunk ahead), lets one thread
+// issue the MMAs, and after every kGaussGroup chunks reads the FP32 accumulators
+// (tcgen05.ld) and adds them to FP64 sums.  Operands use the canonical
 // K-major layout without swizzle: 8-row x 16-byte core matrices, K-adjacent
 // core matrices 128 bytes apart (leading byte offset), 8-row groups 1024 bytes
 // apart (stride byte offset).
@@ -605,17 +605,25 @@ __global__ void __launch_bounds__(kFactorLanes * 40) gauss_factor_inv_kernel(Gau
 }
 
 // 256 threads: thread (half h = tid / 128, row r = tid % 128) stages points
-// 16 h .. 16 h + 15 of every chunk of row r
-template <bool COLSMEM>
+// 16 h .. 16 h + 15 of every chunk of row r.  A CTA works through
+// chunks_per_split chunks (the grid is one wave of two CTAs an SM, so that the
+// X column and the launch's other fixed work are paid once per ten chunks): the
+// accumulators start anew every A.group chunks and are added to FP64 sums
+// in registers.  TILES: 32-column tiles of W, all from the one staged A tile.
+// Bound by a chunk's chain of gathers, operand stores, MMAs and waits (3.3 us
+// with at most two CTAs an SM).  N = 9995, 1001 rows: 5 columns 39.5 us, 39
+// columns 66; with a CTA per group of four chunks, a pass per 32 columns,
+// per-entry bounds and operand stores of four bytes in four-way conflict: 45, 99.
+template <bool COLSMEM, int TILES, bool P16>
 __global__ void __launch_bounds__(256, 2) gauss_cross_tc_kernel(GaussArgs A, int nchunks)
 {
     extern __shared__ unsigned char gsm_raw[];
     unsigned char *gsm = gsm_raw + ((1024u - (smem_u32(gsm_raw) & 1023u)) & 1023u);
     float *sA_hi = reinterpret_cast<float *>(gsm);
     float *sA_lo = sA_hi + kGaussTileM * kGaussKC;
-    float *sB = sA_lo + kGaussTileM * kGaussKC;          // [kGaussGroup][2][1024]
-    float *scol = sB + kGaussGroup * 2048;               // [xcen_pitch] with COLSMEM
-    __shared__ __align__(8) unsigned long long s_mbar_b, s_mbar_m;
+    float *sB = sA_lo + kGaussTileM * kGaussKC;          // [2][TILES][2][1024]
+    float *scol = sB + 2 * TILES * 2048;                 // [xcen_pitch] with COLSMEM
+    __shared__ __align__(8) unsigned long long s_mbar_b[2], s_mbar_m;
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
 
@@ -627,42 +635,48 @@ __global__ void __launch_bounds__(256, 2) gauss_cross_tc_kernel(GaussArgs A, int
     const bool mvalid = m < rows;
     const int ms = mvalid ? m / A.dx : 0, mi = mvalid ? m % A.dx : 0;
     const uint16_t *perm16 =
-        (mvalid && ms > 0 && A.perms16) ? A.perms16 + (size_t)(ms - 1) * A.perm_pitch : nullptr;
-    const int32_t *perm32 =
-        (mvalid && ms > 0 && !A.perms16) ? A.perms + (size_t)(ms - 1) * A.N : nullptr;
+        P16 && ms > 0 ? A.perms16 + (size_t)(ms - 1) * A.perm_pitch : nullptr;
+    const int32_t *perm32 = !P16 && ms > 0 ? A.perms + (size_t)(ms - 1) * A.N : nullptr;
     const float *xg = A.xcen + (size_t)mi * A.xcen_pitch;
-    const int w0 = A.w0, pass = w0 / kGaussTileN;
     const int ch0 = split * A.chunks_per_split;
-    const int nch = min(nchunks, ch0 + A.chunks_per_split) - ch0;   // 1 .. kGaussGroup
-    const uint32_t mbar_b = smem_u32(&s_mbar_b), mbar_m = smem_u32(&s_mbar_m);
+    const int nch = min(nchunks, ch0 + A.chunks_per_split) - ch0;   // at least 1
+    const uint32_t mbar_m = smem_u32(&s_mbar_m);
+    const uint32_t mbar_b[2] = {smem_u32(&s_mbar_b[0]), smem_u32(&s_mbar_b[1])};
 
+    // W's B tiles of the CTA's chunk c, into slot c & 1: one bulk copy of 8 KB a tile
+    auto load_b = [&](int c) {
+        const uint32_t bar = mbar_b[c & 1];
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                     "r"((uint32_t)(TILES * 8192))
+                     : "memory");
+        for (int t = 0; t < TILES; ++t) {
+            const float *src = A.btile + ((size_t)t * nchunks + ch0 + c) * 2048;
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], "
+                "8192, [%2];" ::"r"(smem_u32(sB + ((c & 1) * TILES + t) * 2048)),
+                "l"(reinterpret_cast<uint64_t>(src)), "r"(bar)
+                : "memory");
+        }
+    };
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&s_tmem)),
-                     "r"((uint32_t)kGaussTileN));
+                     "r"((uint32_t)(TILES * kGaussTileN)));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
         s_fail = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar_b));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar_b[0]));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar_b[1]));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar_m));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        // this group's B tiles: one bulk copy of 8 KB per chunk
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar_b),
-                     "r"((uint32_t)(nch * 8192))
-                     : "memory");
-        for (int c = 0; c < nch; ++c) {
-            const float *src = A.btile + ((size_t)pass * nchunks + ch0 + c) * 2048;
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], "
-                "8192, [%2];" ::"r"(smem_u32(sB + c * 2048)),
-                "l"(reinterpret_cast<uint64_t>(src)), "r"(mbar_b)
-                : "memory");
-        }
+        load_b(0);
+        if (nch > 1) load_b(1);
     }
     if (COLSMEM) {   // the (single) X column, centred, into shared memory
         const float4 *src = reinterpret_cast<const float4 *>(A.xcen);
         float4 *dst = reinterpret_cast<float4 *>(scol);
+#pragma unroll 4
         for (int e = tid; e < A.xcen_pitch / 4; e += 256) dst[e] = __ldg(src + e);
     }
     __syncthreads();
@@ -673,101 +687,150 @@ __global__ void __launch_bounds__(256, 2) gauss_cross_tc_kernel(GaussArgs A, int
                            ((uint32_t)(kGaussTileM >> 4) << 24);
     const uint32_t aHi = smem_u32(sA_hi), aLo = smem_u32(sA_lo);
 
-    // permutation entries of this thread's half chunk: 16 indices (-1 past N)
-    uint4 pv[2];
+    // Permutation entries of this thread's half chunk, two a word.  Past N any
+    // index of the column will do (W's tile is zero there), and a row past the
+    // last repeats row 0.
+    uint32_t pv[8] = {};
     auto load_perm = [&](int ch) {
         const int k0 = ch * kGaussKC + 16 * half;
-        if (perm16) {
-            const uint4 *q = reinterpret_cast<const uint4 *>(perm16 + k0);
-            pv[0] = __ldg(q);
-            pv[1] = __ldg(q + 1);
+        if (!P16) return;
+        if (perm16) {   // a row has perm_pitch entries, a multiple of 8, zeros past N
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+                if (k0 + 8 * a < A.perm_pitch) {
+                    const uint4 q = __ldg(reinterpret_cast<const uint4 *>(perm16 + k0) + a);
+                    pv[4 * a] = q.x;
+                    pv[4 * a + 1] = q.y;
+                    pv[4 * a + 2] = q.z;
+                    pv[4 * a + 3] = q.w;
+                }
+        } else {
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                const uint32_t t = min(k0 + 2 * a, A.N - 1), t1 = min(k0 + 2 * a + 1, A.N - 1);
+                pv[a] = t | t1 << 16;
+            }
         }
     };
-    auto index_of = [&](int ch, int k) {   // k: 0 .. 15 within the half
-        const int t = ch * kGaussKC + 16 * half + k;
-        if (!mvalid || t >= A.N) return -1;
-        if (perm16) {
-            const uint32_t wv = (&pv[k >> 3].x)[(k >> 1) & 3];
-            return (int)((wv >> (16 * (k & 1))) & 0xFFFFu);
+    float xv[16];
+    auto gather = [&](int ch) {   // this thread's half of its row's chunk
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            int idx;
+            if (P16) {
+                idx = (int)(k & 1 ? pv[k >> 1] >> 16 : pv[k >> 1] & 0xffffu);
+            } else {
+                const int t = min(ch * kGaussKC + 16 * half + k, A.N - 1);
+                idx = perm32 ? __ldg(perm32 + t) : t;
+            }
+            xv[k] = COLSMEM ? scol[idx] : __ldg(xg + idx);
         }
-        return perm32 ? perm32[t] : t;
     };
+    double sum[TILES][16];
+#pragma unroll
+    for (int t = 0; t < TILES; ++t)
+#pragma unroll
+        for (int n = 0; n < 16; ++n) sum[t][n] = 0.0;
     load_perm(ch0);
-    // the B tiles have landed, or the copy timed out: decided by the whole CTA
-    bool failed = __syncthreads_or(!mbar_wait(mbar_b, 0)) != 0;
-    uint32_t phase = 0;
-    for (int c = 0; c < nch && !failed; ++c) {
-        const int ch = ch0 + c;
-        // stage A: this thread's half of its row's chunk, all gathers before any use
-        {
-            unsigned char *hb = reinterpret_cast<unsigned char *>(sA_hi);
-            unsigned char *lb = reinterpret_cast<unsigned char *>(sA_lo);
-            float xv[16];
+    gather(ch0);
+    if (nch > 1) load_perm(ch0 + 1);
+    bool failed = false;
+    int c = 0;
+    for (; c < nch && !failed; ++c) {
+        // stage A, a core matrix row (four values) a store
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const int idx = index_of(ch, k);
-                xv[k] = idx < 0 ? 0.f : (COLSMEM ? scol[idx] : __ldg(xg + idx));
-            }
+        for (int k = 0; k < 16; k += 4) {
+            float hi[4], lo[4];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const float hi = __uint_as_float(to_tf32(xv[k]));
-                const float lo = __uint_as_float(to_tf32(__fsub_rn(xv[k], hi)));
-                const uint32_t off = cm_offset(r, 16 * half + k);
-                *reinterpret_cast<float *>(hb + off) = hi;
-                *reinterpret_cast<float *>(lb + off) = lo;
+            for (int q = 0; q < 4; ++q) {
+                hi[q] = __uint_as_float(to_tf32(xv[k + q]));
+                lo[q] = __uint_as_float(to_tf32(__fsub_rn(xv[k + q], hi[q])));
             }
+            const uint32_t off = cm_offset(r, 16 * half + k);
+            *reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(sA_hi) + off) =
+                make_float4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(sA_lo) + off) =
+                make_float4(lo[0], lo[1], lo[2], lo[3]);
         }
-        if (c + 1 < nch) load_perm(ch + 1);   // in flight while the MMAs run
         // generic-proxy smem writes -> visible to the tensor core (async proxy)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t bHi = smem_u32(sB + c * 2048), bLo = bHi + 4096;
+            // without its B tiles the chunk's commit stays out and every wait below ends
+            if (!mbar_wait(mbar_b[c & 1], (uint32_t)(c >> 1) & 1u)) {
+                atomicExch(&s_fail, 1);
+            } else {
 #pragma unroll
-            for (int q = 0; q < kGaussKC / 8; ++q) {   // K = 8 TF32 per MMA
-                const uint32_t ko = q * 256;            // two core matrices along K
-                const uint64_t dAh = smem_desc(aHi + ko, 128, 1024);
-                const uint64_t dAl = smem_desc(aLo + ko, 128, 1024);
-                const uint64_t dBh = smem_desc(bHi + ko, 128, 1024);
-                const uint64_t dBl = smem_desc(bLo + ko, 128, 1024);
-                mma_tf32(tmem, dAh, dBh, idesc, (c == 0 && q == 0) ? 0u : 1u);
-                mma_tf32(tmem, dAh, dBl, idesc, 1u);
-                mma_tf32(tmem, dAl, dBh, idesc, 1u);
+                for (int t = 0; t < TILES; ++t) {
+                    const uint32_t bHi = smem_u32(sB + ((c & 1) * TILES + t) * 2048);
+                    const uint32_t bLo = bHi + 4096, acc = tmem + (uint32_t)(t * kGaussTileN);
+#pragma unroll
+                    for (int q = 0; q < kGaussKC / 8; ++q) {   // K = 8 TF32 per MMA
+                        const uint32_t ko = q * 256;            // two core matrices along K
+                        const uint64_t dAh = smem_desc(aHi + ko, 128, 1024);
+                        const uint64_t dAl = smem_desc(aLo + ko, 128, 1024);
+                        const uint64_t dBh = smem_desc(bHi + ko, 128, 1024);
+                        const uint64_t dBl = smem_desc(bLo + ko, 128, 1024);
+                        mma_tf32(acc, dAh, dBh, idesc,
+                                 (c % A.group == 0 && q == 0) ? 0u : 1u);
+                        mma_tf32(acc, dAh, dBl, idesc, 1u);
+                        mma_tf32(acc, dAl, dBh, idesc, 1u);
+                    }
+                }
+                asm volatile(
+                    "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                    ::"r"(mbar_m)
+                    : "memory");
             }
-            asm volatile(
-                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                    mbar_m)
-                : "memory");
         }
-        // every thread waits: the MMAs have read the A tile before it is
-        // restaged (and, after the last chunk, written the accumulator)
-        if (!mbar_wait(mbar_m, phase)) atomicExch(&s_fail, 1);
-        phase ^= 1u;
+        if (c + 1 < nch) {   // the next chunk's values while the MMAs run
+            gather(ch0 + c + 1);
+            if (c + 2 < nch) load_perm(ch0 + c + 2);
+        }
+        // every thread waits: the MMAs have read the A and B tiles before they
+        // are written again, and have written the accumulators
+        if (!mbar_wait(mbar_m, (uint32_t)c & 1u)) atomicExch(&s_fail, 1);
         __syncthreads();
-        if (s_fail) {
-            mbar_wait(mbar_m, phase ^ 1u);   // a second bounded wait before TMEM is freed
-            failed = true;
+        failed = s_fail != 0;
+        if (failed) break;
+        if (tid == 0 && c + 2 < nch) load_b(c + 2);
+        if ((c + 1) % A.group == 0 || c + 1 == nch) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+            for (int t = 0; t < TILES; ++t) {
+                // warps w and w + 4 share TMEM lanes 32 (w % 4) ..; each reads 16 columns
+                float v[16];
+                tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) +
+                              (uint32_t)(t * kGaussTileN) + 16u * half,
+                          v);
+#pragma unroll
+                for (int n = 0; n < 16; ++n) sum[t][n] += (double)v[n];
+            }
         }
     }
-    if (failed && tid == 0) atomicExch(A.status + 1, 1);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!failed) {
-        // warps w and w + 4 share TMEM lanes 32 (w % 4) ..; each reads 16 columns
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + 16u * half, v);
-        if (mvalid) {
-            double *part = A.cross_part + ((size_t)split * rows + m) * A.dw + w0 + 16 * half;
+    if (failed) {
+        // bounded waits for the copies and the MMAs in flight before anything is freed
+        if (tid == 0) {
+            atomicExch(A.status + 1, 1);
+            mbar_wait(mbar_b[c & 1], (uint32_t)(c >> 1) & 1u);
+            if (c + 1 < nch) mbar_wait(mbar_b[(c + 1) & 1], (uint32_t)((c + 1) >> 1) & 1u);
+        }
+        mbar_wait(mbar_m, (uint32_t)c & 1u);
+    } else if (mvalid) {
+        double *part = A.cross_part + ((size_t)split * rows + m) * A.dw + 16 * half;
+#pragma unroll
+        for (int t = 0; t < TILES; ++t)
 #pragma unroll
             for (int n = 0; n < 16; ++n)
-                if (w0 + 16 * half + n < A.dw) part[n] = (double)v[n];
-        }
+                if (t * kGaussTileN + 16 * half + n < A.dw) part[t * kGaussTileN + n] = sum[t][n];
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"((uint32_t)kGaussTileN));
+                     "r"((uint32_t)(TILES * kGaussTileN)));
 }
 
 // cross = (sum of the splits' partial sums, in split order) / (N - 1)
@@ -1475,48 +1538,59 @@ cudaError_t gauss_launch_factor(const GaussArgs &A, cudaStream_t st)
     return cudaGetLastError();
 }
 
-int gauss_tc_splits(int N)
+int gauss_tc_split_chunks(int N, int rows, int sms, int *group)
 {
     const int nchunks = (N + kGaussKC - 1) / kGaussKC;
-    return (nchunks + kGaussGroup - 1) / kGaussGroup;
+    const int groups = (nchunks + kGaussGroup - 1) / kGaussGroup;
+    *group = (nchunks + groups - 1) / groups;
+    // whole accumulation groups, so that no sum depends on the split
+    const int tiles = (rows + kGaussTileM - 1) / kGaussTileM;
+    const int ctas = std::max(1, 2 * sms / tiles);
+    return *group * ((groups + ctas - 1) / ctas);
+}
+
+template <bool COLSMEM, int TILES, bool P16>
+static cudaError_t gauss_cross_tc(const GaussArgs &A, int rows, int nchunks, cudaStream_t st)
+{
+    const size_t smem = 1024 + (size_t)4 * (2 * kGaussTileM * kGaussKC + 2 * TILES * 2048 +
+                                            (COLSMEM ? A.xcen_pitch : 0));
+    const auto f = &gauss_cross_tc_kernel<COLSMEM, TILES, P16>;
+    static bool attr_done[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64 && !attr_done[dev]) {
+        if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      200 * 1024)) != cudaSuccess)
+            return e;
+        attr_done[dev] = true;
+    }
+    f<<<dim3((rows + kGaussTileM - 1) / kGaussTileM, A.splits), 256, smem, st>>>(A, nchunks);
+    return cudaGetLastError();
 }
 
 cudaError_t gauss_launch_cross_tc(const GaussArgs &A, cudaStream_t st)
 {
     const int rows = (A.S + 1) * A.dx;
     const int nchunks = (A.N + kGaussKC - 1) / kGaussKC;
-    if (A.splits < 1 || A.splits > 65535 || A.chunks_per_split > kGaussGroup || !A.btile ||
-        !A.xcen || (A.xcen_pitch & 31) || A.xcen_pitch < A.N ||
+    if (A.splits < 1 || A.splits > 65535 || A.group < 1 || A.group > kGaussGroup ||
+        A.chunks_per_split < 1 || A.chunks_per_split % A.group ||
+        (long long)(A.splits - 1) * A.chunks_per_split >= nchunks || A.dw > 2 * kGaussTileN ||
+        !A.btile || !A.xcen || (A.xcen_pitch & 31) || A.xcen_pitch < A.N ||
         (reinterpret_cast<uintptr_t>(A.btile) & 15) || (reinterpret_cast<uintptr_t>(A.xcen) & 15))
         return cudaErrorInvalidValue;
     if (A.perms16 && (A.perm_pitch < A.N || (A.perm_pitch & 7) ||
                       (reinterpret_cast<uintptr_t>(A.perms16) & 15)))
         return cudaErrorInvalidValue;
-    cudaError_t e;
-    const bool colsmem = A.dx == 1 && A.xcen_pitch <= kGaussColMax;
-    const size_t smem = 1024 + (size_t)4 * (2 * kGaussTileM * kGaussKC + kGaussGroup * 2048 +
-                                            (colsmem ? A.xcen_pitch : 0));
-    const void *f = colsmem ? reinterpret_cast<const void *>(&gauss_cross_tc_kernel<true>)
-                            : reinterpret_cast<const void *>(&gauss_cross_tc_kernel<false>);
-    static bool attr_done[64][2] = {};
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && !attr_done[dev][colsmem]) {
-        if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      200 * 1024)) != cudaSuccess)
-            return e;
-        attr_done[dev][colsmem] = true;
-    }
-    // W wider than one 32-column tile: one pass per 32 columns
-    for (int w0 = 0; w0 < A.dw; w0 += kGaussTileN) {
-        GaussArgs P = A;
-        P.w0 = w0;
-        int nc = nchunks;
-        void *args[] = {&P, &nc};
-        e = cudaLaunchKernel(f, dim3((rows + kGaussTileM - 1) / kGaussTileM, A.splits), dim3(256),
-                             args, smem, st);
-        if (e != cudaSuccess) return e;
-    }
+    const bool colsmem = A.dx == 1 && A.xcen_pitch <= kGaussColMax, wide = A.dw > kGaussTileN;
+    const cudaError_t e =
+        !A.perms16 ? (wide ? gauss_cross_tc<false, 2, false>(A, rows, nchunks, st)
+                           : gauss_cross_tc<false, 1, false>(A, rows, nchunks, st))
+        : colsmem  ? (wide ? gauss_cross_tc<true, 2, true>(A, rows, nchunks, st)
+                           : gauss_cross_tc<true, 1, true>(A, rows, nchunks, st))
+                   : (wide ? gauss_cross_tc<false, 2, true>(A, rows, nchunks, st)
+                           : gauss_cross_tc<false, 1, true>(A, rows, nchunks, st));
+    if (e != cudaSuccess) return e;
     const long long total = (long long)rows * A.dw;
     gauss_cross_reduce_kernel<<<(unsigned)((total + 63) / 64), 64, 0, st>>>(A);
     return cudaGetLastError();

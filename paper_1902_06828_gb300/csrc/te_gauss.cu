@@ -26,7 +26,7 @@ constexpr int kGaussBatch = 4096;   // estimates per batched launch (grid z)
 // sums, and with xc the centred X columns.  The estimates and error bounds
 // are bound elsewhere.
 size_t gauss_shape(GaussArgs &A, int N, int S, int dx, int dy, int dz, int splits,
-                   bool xc = false)
+                   bool xc = false, int split_chunks = 0)
 {
     A.N = N;
     A.S = S;
@@ -36,7 +36,7 @@ size_t gauss_shape(GaussArgs &A, int N, int S, int dx, int dy, int dz, int split
     A.d = dx + dy + dz;
     const int nchunks = (N + 31) / 32;
     splits = std::max(1, std::min(splits, nchunks));
-    A.chunks_per_split = (nchunks + splits - 1) / splits;
+    A.chunks_per_split = split_chunks ? split_chunks : (nchunks + splits - 1) / splits;
     A.splits = (nchunks + A.chunks_per_split - 1) / A.chunks_per_split;
     const size_t d = (size_t)A.d, dw = (size_t)A.dw;
     return d + d * d + 2 * dw * dw + 2 + kGaussMaxDims +
@@ -264,7 +264,9 @@ extern "C" te_status cmi_gauss(te_ctx *ctx, const te_data *data, const te_var *x
         CK(cudaSetDevice(ctx->device), "cudaSetDevice");
         // workspace: the estimate's doubles, its estimates and bounds, then ints
         GaussArgs A{};
-        const size_t ws = gauss_shape(A, N, S, dx, dy, dz, gauss_tc_splits(N));
+        const size_t ws =
+            gauss_shape(A, N, S, dx, dy, dz, 1, false,
+                        gauss_tc_split_chunks(N, (S + 1) * dx, 152, &A.group));
         const size_t nd = ws + 2 * (size_t)(S + 1);
         if ((st = ensure_dev(ctx, ctx->ws_gauss, nd * 8 + (size_t)(d + 8) * 4))) return st;
         // permutations as 16-bit rows (pitch a multiple of 8 entries) when the
