@@ -1478,28 +1478,46 @@ static const void *walk_kernel(const ListShape &s)
     return s.width == 2 ? walk_kernel_g<16, true>(s) : walk_kernel_g<16, false>(s);
 }
 
+static cudaError_t prepare_build(int queries)
+{
+    const void *f = queries == 2   ? reinterpret_cast<const void *>(&list_build_kernel<2>)
+                    : queries == 4 ? reinterpret_cast<const void *>(&list_build_kernel<4>)
+                                   : reinterpret_cast<const void *>(&list_build_kernel<8>);
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+}
+
+static cudaError_t prepare_walk(const ListShape &s)
+{
+    const void *f = walk_kernel(s);
+    if (!f) return cudaSuccess;   // no group has this shape
+    return cudaFuncSetAttribute(
+        f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)(kListWalkSmem + list_walk_head(true, kListWalkThreads / 32)));
+}
+
+cudaError_t list_prepare(const ListShape &s, int queries, uint64_t *done)
+{
+    const int near = s.width == 32 / s.lanes;
+    const int bit = ((s.lanes / 16 * 2 + near) * 5 + s.dxp) * 2 + (s.k4 ? 1 : 0);   // below 60
+    const int build = 60 + queries / 4;   // 2, 4 or 8
+    cudaError_t e = cudaSuccess;
+    if (!(*done >> build & 1)) e = prepare_build(queries);
+    if (e == cudaSuccess && !(*done >> bit & 1)) e = prepare_walk(s);
+    if (e == cudaSuccess) *done |= 1ull << build | 1ull << bit;
+    return e;
+}
+
 cudaError_t list_prepare_attributes()
 {
-    const void *build[] = {reinterpret_cast<const void *>(&list_build_kernel<2>),
-                           reinterpret_cast<const void *>(&list_build_kernel<4>),
-                           reinterpret_cast<const void *>(&list_build_kernel<8>)};
-    for (const void *f : build) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-        if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = cudaSuccess;
+    for (int queries = 2; queries <= 8 && e == cudaSuccess; queries *= 2)
+        e = prepare_build(queries);
     for (int lanes = 8; lanes <= 32; lanes *= 2)
         for (int width = 32 / lanes; width >= 1; width /= 2)
             for (int dxp : {1, 2, 4, 0})
-                for (int k4 = 0; k4 < 2; ++k4) {
-                    const void *f = walk_kernel(ListShape{lanes, width, dxp, k4 != 0});
-                    if (!f) continue;
-                    const cudaError_t e = cudaFuncSetAttribute(
-                        f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                        (int)(kListWalkSmem + list_walk_head(true, kListWalkThreads / 32)));
-                    if (e != cudaSuccess) return e;
-                }
-    return cudaSuccess;
+                for (int k4 = 0; k4 < 2 && e == cudaSuccess; ++k4)
+                    e = prepare_walk(ListShape{lanes, width, dxp, k4 != 0});
+    return e;
 }
 
 cudaError_t launch_list_build(const ListLaunch &L, long long n_items, int queries, int cap_a,

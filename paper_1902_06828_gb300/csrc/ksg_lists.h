@@ -120,7 +120,11 @@ struct RankSortJob {
 inline int rank_sort_items(int N) { return (N + 63) / 64; }
 cudaError_t launch_rank_sort(const RankSortJob *jobs, int n_jobs, int n_items, cudaStream_t st);
 
+// Kernel attributes before the first launch on a device: of every kernel, or
+// of those a chunk uses that are not marked in *done yet (loading all of them
+// takes longer than a small call).
 cudaError_t list_prepare_attributes();
+cudaError_t list_prepare(const ListShape &s, int queries, uint64_t *done);
 cudaError_t launch_list_build(const ListLaunch &L, long long n_items, int queries, int cap_a,
                               int cap_b, cudaStream_t st);
 // smem: the largest list_walk_x_bytes of the launch's groups, all of shape s

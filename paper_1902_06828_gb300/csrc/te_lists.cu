@@ -220,10 +220,9 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
         if (t.bytes) std::memcpy((char *)ctx->pin + t.at, t.src, t.bytes);
     CK(copy_h2d(ctx, ctx->ws_groups.p, ctx->pin, bytes), "cudaMemcpyAsync");
     char *dtab = (char *)ctx->ws_groups.p;
-    if (!ctx->prepared_lists) {
-        CK(list_prepare_attributes(), "cudaFuncSetAttribute");
-        ctx->prepared_lists = 1;
-    }
+    for (const Chunk &ch : chunks)
+        CK(list_prepare(plans[ch.cls].shape, ch.queries, &ctx->prepared_lists),
+           "cudaFuncSetAttribute");
 
     const bool graph = ctx->opt_graph != 0;
     auto device_work = [&]() -> te_status {

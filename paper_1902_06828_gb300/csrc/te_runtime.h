@@ -142,7 +142,8 @@ struct te_ctx {
     // first use) and the events that fork to it and join back
     cudaStream_t aux_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
-    int prepared = 0, prepared_lists = 0;
+    int prepared = 0;
+    uint64_t prepared_lists = 0;   // kernels, as list_prepare marks them
     te_trace_fn trace_fn = nullptr;   // te_ctx_set_trace
     void *trace_user = nullptr;
     // te_ctx_set_option: forced member-lane tile / members per lane (0 = the
