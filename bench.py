@@ -36,7 +36,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "KSG CMI estimates/s incl. surrogates at T=10000"
 UNIT = "estimates/s"
-TRAFFIC_PER_MEMBER_POINT = (146883584.0 + 4136448.0) / (9045 * 3995)
+TRAFFIC_PER_MEMBER_POINT = 3453012224.0 / (9045 * 9995)
 
 
 def _peaks():
@@ -652,12 +652,10 @@ def main():
     achieved = ops / (kernel_ms / 1e3) / 1e12 if kernel_ms > 0 else None
     sm_count = torch.cuda.get_device_properties(local).multi_processor_count
     peak = sm_count * 128 * sm_max * 1e6 / 1e12
-    # DRAM traffic of the KSG kernel per launch: the ncu capture of the same
-    # kernel (var10 at T = 4000, step-2 launch of target 0, 9045 members x 3995
-    # points) read 147.02 MB and wrote 4.22 MB, i.e. 4.19 bytes per
-    # member-point (each member's X row read once); scaled here by the
-    # member-points one launch processes.  Algorithmic bytes: 4 N per member
-    # (its X row) + 16 (key).
+    # DRAM traffic of the KSG kernels per launch pair (lists built, then walked):
+    # the ncu capture of the same kernels (profiles/list_walk_kernel_*) by
+    # member-point; scaled here by the member-points one launch processes.
+    # Algorithmic bytes: 4 N per member (its X values) + 16 (key).
     n_pts = args.T - 5
     mp_per_launch = (n_est / world) * n_pts / max(ksg_launches, 1)   # this rank's launches
     traffic = TRAFFIC_PER_MEMBER_POINT * mp_per_launch if ksg_launches else None
@@ -692,9 +690,9 @@ def main():
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s",
                      "frac": (achieved / peak) if achieved else None, "traffic": traffic,
                      "traffic_note": "dram read+write bytes per launch, scaled from the ncu "
-                                     "capture of this kernel at T=4000 by member-points",
+                                     "capture of these kernels at T=10000 by member-points",
                      "algorithmic_bytes_per_launch": alg_bytes,
-                     "kernel": "ksg_lane_kernel", "kernel_ms_per_launch":
+                     "kernel": "list_build_kernel + list_walk_kernel", "kernel_ms_per_launch":
                      kernel_ms / max(ksg_launches, 1), "launches": ksg_launches,
                      "peak_note": f"{sm_count} SMs x 128 FP32 lanes x {sm_max:.0f} MHz "
                                   "(derived; SM count read from the device)",
@@ -707,7 +705,8 @@ def main():
                                        "note": "te_alu_peak: each pass's counted instruction "
                                                "pattern from registers at full occupancy, this "
                                                "run; the mix weights them by this run's ops"},
-                     "work": "3 ops per executed kNN-pass member-pair, 7 per count-pass one",
+                     "work": "3 ops per list entry evaluated for a member (member-lane kernel: 3 per "
+                             "kNN-pass member-pair, 7 per count-pass one)",
                      "pair_evals_executed": pair_evals, "pair_evals_bruteforce": pair_evals_bf,
                      "pruned_fraction": (1.0 - pair_evals / pair_evals_bf) if pair_evals_bf
                      else None},

@@ -19,8 +19,8 @@
 // with two, 71 and 781 with one, against 900 to 10,000 visited by tiles that
 // are pruned for 64 members at once.  Measured on one GB300, tiled member-lane
 // kernel -> lists, whole calls: 89 candidates x 201 members, 8 Z variables,
-// N = 9995: 274 -> 24.1 ms; 45 x 201, 2 Z: 105 -> 41 ms; one call of 201, 1 Z:
-// 5.7 -> 2.5 ms; 9 x 201, Theiler window 12, N = 2994: 9.8 -> 1.5 ms.
+// N = 9995: 277 -> 22.9 ms; 45 x 201, 2 Z: 104 -> 35.9 ms; one call of 201, 1 Z:
+// 5.7 -> 2.1 ms; 9 x 201, Theiler window 12, N = 2994: 9.8 -> 1.5 ms.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 #include <stdint.h>
@@ -624,8 +624,8 @@ struct ScanScratch {
 // by one warp, then everything is counted.  The warps meet four times a batch
 // and take its pairs one after another without waiting for each other, where
 // scan_member meets four times a pair and sorts as it goes.  10^4 points and a
-// few pairs in a thousand: 90 candidates of 201 members 40.0 -> 36.0 ms, one
-// 2.43 -> 2.18, four X variables 8.5 -> 6.7.  A pair with more than kScanNear distances up to its bound
+// few pairs in a thousand: 45 candidates of 201 members 40.0 -> 36.0 ms, one
+// 2.43 -> 2.18, three X variables 8.5 -> 6.7.  A pair with more than kScanNear distances up to its bound
 // is set in `left`, for scan_member.  xs: X values, member m's at xs + m * sm.
 __device__ __noinline__ void scan_aside(const ListLaunch &L, const ListGroup &G,
                                         const float *const *col, const Aside *aside, int n,
@@ -869,8 +869,10 @@ struct Nearest {
 // NG / width points.  Only a long prefix (n_xz) goes over the whole warp, 128
 // entries at a time.  With NG members (NEAR) the warp's one point has its
 // near lists copied a point ahead; the digamma values that end a pair's work
-// are added a point later: a warp's time is a chain of memory and shuffle
-// latencies more than of issue slots.
+// are added a point later: in a small call a warp's time is a chain of memory
+// and shuffle latencies.  In a large one (45 x 201 members, N = 9995, 2 Z: 33.9
+// ms) the kernel issues in 75% of the slots, 344 warp instructions a pair, with the
+// shared-memory pipe busy 72%, 63% of its load wavefronts bank conflicts of gathers.
 // DXP: X variables as stored, dimensions of a point together: 1, 2 or 4 (three
 // or four variables), so that a point's values are one load; 0: any number, a
 // row per dimension.
@@ -1360,7 +1362,7 @@ void list_caps(int N, int k, int dx, int dy, int dz, int *cap_a, int *cap_b)
     // Expected counts when the joint space has m independent dimensions: a
     // per-dimension slab of probability (k / N)^(1/m) holds the neighbours.
     // The margins cover the members whose X value lies in a sparse region.
-    // Half of either, N = 10^4: one call of 201 members 2.15 -> 2.19 ms, 89
+    // Half of either, N = 10^4: one call of 201 members 2.15 -> 2.19 ms, 45
     // candidates 35.8 -> 44.9; more of either changes nothing.
     const double m = dx + dy + dz;
     const double slab = std::pow((double)k / (double)N, 1.0 / m);

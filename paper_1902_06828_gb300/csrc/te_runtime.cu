@@ -344,7 +344,9 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
     if ((st = ensure_dev(ctx, ctx->ws_keys, (size_t)std::max(n_out, 1) * 16))) return st;
     CK(cudaMemsetAsync(ctx->ws_acc.p, 0, (size_t)n_out * 16, ctx->stream), "cudaMemsetAsync");
     // Neighbour lists wherever a member's X values fit a CTA's shared memory;
-    // an option of the member-lane kernel asks for that kernel.
+    // an option of the member-lane kernel asks for that kernel.  Member-lane ->
+    // lists over the sizes: one estimate at T = 203 128 -> 79 us, 201 members at
+    // T = 1000 366 -> 190 us, at T = 10^4 5.7 -> 2.1 ms, 9045 members 104 -> 36 ms.
     bool lists = !ctx->opt_jt && !ctx->opt_ms && !ctx->opt_persistent && !ctx->opt_order;
     for (const HostGroup &g : groups)
         lists = lists && list_fits(g.data->T - g.max_lag, g.dx, (int)g.z.size(), g.k);

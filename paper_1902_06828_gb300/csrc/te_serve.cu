@@ -58,10 +58,12 @@ struct Slot {
     size_t fp = 0;
 };
 
-// device bytes of one job: permutations and their composed copies (8 S N),
-// the X-value rows of the TMA-staged kernel (4 (S + 1) N, rows padded to a
-// multiple of 8 points), the order and sorted Y/Z columns, the chunk boxes,
-// accumulators, keys and descriptors
+// device bytes of one job, as the member-lane path needs them: permutations
+// and their composed copies (8 S N), the X-value rows of the TMA-staged kernel
+// (4 (S + 1) N, rows padded to a multiple of 8 points), the order and sorted Y/Z
+// columns, the chunk boxes, accumulators, keys and descriptors.  The list path
+// keeps the permutations alone and, per batch in flight and whatever its
+// size, at most 256 MiB of lists.
 size_t footprint(int N, int S, int dyz)
 {
     const size_t pitch = (size_t)std::max(32, (N + 7) & ~7);
