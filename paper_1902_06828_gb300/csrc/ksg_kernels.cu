@@ -1197,19 +1197,21 @@ __device__ __forceinline__ void ksg_lane_item(const KsgLaunch &L, const CUtensor
     // Empty Z with one X and one Y variable and no Theiler window: n_z = N - 1
     // and n_xz, n_yz are 1-D range counts.  The member's X values over the
     // points are the column's values (a permutation only reorders them), so
-    // both counts come from sorted columns, minus the point itself (distance 0
-    // counts iff eps > 0).  Exactly the counts of the pairwise loop below.
+    // both counts come from sorted columns, minus the point itself.  Exactly the counts of the pairwise loop below.
     if (G.ysorted) {
 #pragma unroll
         for (int a = 0; a < LQ; ++a)
 #pragma unroll
             for (int q = 0; q < MS; ++q) {
                 const float e = eps[a][q];
-                const int self = e > 0.f ? 1 : 0;
                 cz[a][q] = (float)(N - 1);
-                cxz[a][q] = (float)(range_count(md[q].xsorted, N, xi[a][q], e) - self);
+                // no distance is below eps = 0, where the searches' ends would cross
+                cxz[a][q] =
+                    e > 0.f ? (float)(range_count(md[q].xsorted, N, xi[a][q], e) - 1) : 0.f;
                 cyz[a][q] =
-                    (float)(range_count(G.ysorted, N, s_q[(warp * LQ + a) * dyz], e) - self);
+                    e > 0.f
+                        ? (float)(range_count(G.ysorted, N, s_q[(warp * LQ + a) * dyz], e) - 1)
+                        : 0.f;
             }
     }
     for (int t = 0; t < (G.ysorted ? 0 : ntiles); ++t) {

@@ -187,3 +187,16 @@ def test_pairs_beyond_the_radii(env, T, dz, dx, k, w, S, levels):
     got, ref = _both(te, ctx, jobs)
     assert got == ref
     data.close()
+
+
+@pytest.mark.parametrize("levels", [2, 3])
+def test_member_lane_kernel_with_distances_of_zero(env, levels):
+    """Empty Z and k-th distances of 0: nothing is below them, in either kernel."""
+    te, ctx = env
+    rng = np.random.default_rng(levels)
+    s = rng.integers(0, levels, size=(3, 300)).astype(np.float32)
+    data = te.te_data_create(ctx, s)
+    jobs = [te.Job(data, [(2, 1)], [(0, 0)], [], k=4, max_lag=5, n_surr=5, seed=1)]
+    got, ref = _both(te, ctx, jobs)
+    assert got == ref
+    data.close()
