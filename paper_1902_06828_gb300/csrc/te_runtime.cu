@@ -429,25 +429,27 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
 
     // Sorted groups with an empty Z, one Y and one X variable and no Theiler
     // window count by 1-D range searches: sorted copies of their X columns and
-    // of the Y column (one per distinct column of a data set).
-    std::map<std::pair<const te_data *, int>, size_t> vsorted_of;
+    // of the Y column (one per distinct column and number of points of a data
+    // set: point sets of different maximum lags may begin at the same value).
+    using ColumnKey = std::tuple<const te_data *, int, int>;   // data, offset, points
+    std::map<ColumnKey, size_t> vsorted_of;
     size_t vs_elems = 0;
     auto col_off = [](const HostGroup *g, te_var v) {
         return v.proc * g->data->T + g->max_lag - v.lag;
     };
-    auto want_sorted = [&](const HostGroup *g, int off) {
-        auto key = std::make_pair(g->data, off);
-        if (!vsorted_of.count(key)) {
-            vsorted_of[key] = vs_elems;
+    auto column_key = [&](const HostGroup *g, te_var v) {
+        return ColumnKey(g->data, col_off(g, v), g->data->T - g->max_lag);
+    };
+    auto want_sorted = [&](const HostGroup *g, te_var v) {
+        if (vsorted_of.emplace(column_key(g, v), vs_elems).second)
             vs_elems += ((size_t)(g->data->T - g->max_lag) + 3) & ~(size_t)3;
-        }
     };
     std::vector<const HostGroup *> fast_groups;
     for (const HostGroup *g : to_order) {
         if (!g->z.empty() || g->y.size() != 1 || g->dx != 1 || g->theiler != 0) continue;
         fast_groups.push_back(g);
-        want_sorted(g, col_off(g, g->y[0]));
-        for (te_var v : g->xvars) want_sorted(g, col_off(g, v));
+        want_sorted(g, g->y[0]);
+        for (te_var v : g->xvars) want_sorted(g, v);
     }
     if (vs_elems) {
         if ((st = ensure_dev(ctx, ctx->ws_vsort, vs_elems * 4))) return st;
@@ -597,8 +599,7 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
                 if (grp_sorted && hm.perm) md.perm = cbase + (*mc)[i];
                 md.xsorted = nullptr;
                 if (grp_fast)
-                    md.xsorted = vbase + vsorted_of[std::make_pair(
-                                             g->data, col_off(g, g->xvars[hm.xcol_first]))];
+                    md.xsorted = vbase + vsorted_of[column_key(g, g->xvars[hm.xcol_first])];
                 md.xcol = xbase + hm.xcol_first;
                 md.out = hm.out;
                 mdesc.push_back(md);
@@ -612,7 +613,7 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
                 gd.tbox = (const float2 *)(obase + oit->second.tbox);
                 gd.n_tiles256 = oit->second.ntl;
                 if (fast_set.count(g))
-                    gd.ysorted = vbase + vsorted_of[std::make_pair(g->data, col_off(g, g->y[0]))];
+                    gd.ysorted = vbase + vsorted_of[column_key(g, g->y[0])];
             }
             gd.n_qtiles = (N + qsz - 1) / qsz;
             gd.n_mblocks = (gd.n_members + v.m - 1) / v.m;
@@ -665,12 +666,9 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
     std::vector<ValueSortJob> vjobs;
     for (auto &kv : vsorted_of) {
         ValueSortJob J;
-        J.src = kv.first.first->d_series + kv.first.second;
+        J.src = std::get<0>(kv.first)->d_series + std::get<1>(kv.first);
         J.dst = vbase + kv.second;
-        int n = 0;
-        for (const HostGroup *g : fast_groups)
-            if (g->data == kv.first.first) n = g->data->T - g->max_lag;
-        J.N = n;
+        J.N = std::get<2>(kv.first);
         vjobs.push_back(J);
     }
     const size_t gbytes = gdesc.size() * sizeof(GroupDesc);

@@ -128,3 +128,24 @@ def test_bad_options_rejected(env):
         ctx.set_option("graph", 2)
     with pytest.raises(ValueError):
         ctx.set_option("no_such_option", 1)
+
+
+def test_member_lane_columns_of_different_point_sets_in_one_batch(env):
+    """With a forced tile, jobs over an empty Z whose maximum lags differ read
+    the same memory as columns of different lengths: each sorts its own, the
+    longer one neither taken for the shorter nor written past its part."""
+    from oracle import ksg as oksg
+    te, ctx = env
+    s = synth.workload_var10(T=403, seed=8)["series"]
+    data = te.te_data_create(ctx, s)
+    jobs = [te.Job(data, [(2, ml)], [(0, ml)], [], k=4, max_lag=ml, n_surr=3, seed=2)
+            for ml in (7, 5, 1, 4)]
+    _reset(ctx)
+    try:
+        ctx.set_option("ksg_tile", 64)
+        _, got = te.cmi_ksg_batch(ctx, jobs, return_keys=True)
+    finally:
+        _reset(ctx)
+    for j, keys in zip(jobs, got):
+        assert keys[0] == oksg.cmi_ksg(s, j.x, j.y, [], k=4, max_lag=j.max_lag)["key"]
+    data.close()
