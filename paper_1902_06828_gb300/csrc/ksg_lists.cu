@@ -82,15 +82,16 @@ __device__ __forceinline__ RowPtrs row_ptrs(unsigned char *rows, int row, int ca
 }
 
 // ---------------- list construction ----------------
-// d_Z and d_YZ of point j to Q query points (-inf over an empty Z).  qv holds
-// the query values dimension by dimension (Y first), so that a column's value
-// is loaded once for all queries.
+// d_Z and d_YZ of point j to Q query points (0 over an empty Z, whose list is
+// not built).  qv holds the query values dimension by dimension (Y first), so
+// that a column's value is loaded once for all queries.  The maximum starts at
+// 0, so that no difference of non-finite values leaves a distance below it.
 template <int Q>
 __device__ __forceinline__ void list_dist(const float *const *col, int dy, int dz, int j,
                                           const float (*qv)[Q], float (&vz)[Q], float (&vyz)[Q])
 {
 #pragma unroll
-    for (int q = 0; q < Q; ++q) vz[q] = -CUDART_INF_F;
+    for (int q = 0; q < Q; ++q) vz[q] = 0.f;
 #pragma unroll 2
     for (int d = dy; d < dy + dz; ++d) {
         const float v = __ldg(col[d] + j);
@@ -220,7 +221,9 @@ __global__ void __launch_bounds__(kListBuildThreads) list_build_kernel(const Lis
     for (int e = tid; e < Q * dyz; e += kListBuildThreads) {
         const int q = e / dyz, d = e - q * dyz;
         const float *c = G.base + (d < dy ? L.cols[G.ycol + d] : L.cols[G.zcol + d - dy]);
-        qv[d][q] = c[i0 + min(q, nq - 1 - r0)];
+        const float v = c[i0 + min(q, nq - 1 - r0)];
+        qv[d][q] = v;
+        if (L.nonfinite && !(fabsf(v) < CUDART_INF_F)) *L.nonfinite = 1;
         if (q == 0) col[d] = c;
     }
     const int ns = min(N, kSample);
@@ -284,7 +287,7 @@ __global__ void __launch_bounds__(kListBuildThreads) list_build_kernel(const Lis
         float r[Q][2];
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
-            // -inf: not collected in this sweep (d_Z itself is -inf over an empty Z)
+            // -inf: not collected in this sweep
             r[q][0] = (todo >> (2 * q)) & 1u ? s_r[q][0] : -CUDART_INF_F;
             r[q][1] = (todo >> (2 * q + 1)) & 1u ? s_r[q][1] : -CUDART_INF_F;
         }
@@ -489,7 +492,7 @@ __device__ __forceinline__ void group_window(const float *__restrict__ z, int n,
     for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
     lo = bl + (s & 0xffff);
     hi = bh + (s >> 16);
-    if (!(e > 0.f)) hi = lo;
+    if (!(e > 0.f) || hi < lo) hi = lo;   // hi < lo: values out of order (not finite)
 }
 
 // One member at query point i over all points, by the whole CTA: its k-th
@@ -935,6 +938,9 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
             for (int j = threadIdx.x; j < N; j += blockDim.x)
                 dst[sp * (dz == 1 ? __ldg(Gr.rank + j) : j)] =
                     __ldg(src + (md.perm ? __ldg(md.perm + j) : j));
+            if (L.nonfinite && !md.perm)   // a permutation has the original's values
+                for (int j = threadIdx.x; j < N; j += blockDim.x)
+                    if (!(fabsf(__ldg(src + j)) < CUDART_INF_F)) *L.nonfinite = 1;
         }
         if (DXP > 2 && dx < DXP)   // the unused dimensions add nothing to a maximum
             for (int j = threadIdx.x; j < N; j += blockDim.x)
@@ -1308,7 +1314,8 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
         }
         if (slow || !live) nz = nxz = nyz = -1;   // the digamma table's first value, 0
         add_term();
-        q_last_term = L.q[(u == 0 ? nz : u == 1 ? nxz : nyz) + 1];
+        // (a band can hold more than the window of values that are not finite)
+        q_last_term = L.q[max(u == 0 ? nz : u == 1 ? nxz : nyz, -1) + 1];
         if (u > 0) q_last_term = -q_last_term;
         if (L.dbg_eps && u == 0 && live && !slow &&
             L.members[Gr.member_begin + mb * width + gm].out == L.dbg_out) {

@@ -78,6 +78,7 @@ struct ListLaunch {
     int *dbg_nxz, *dbg_nyz, *dbg_nz;
     int dbg_out;
     unsigned long long *work;   // as KsgLaunch::work [0], [1]; nullptr: not counted
+    unsigned *nonfinite;        // set if a value is not finite; nullptr: checked by the caller
 };
 
 constexpr int kListBuildThreads = 512;

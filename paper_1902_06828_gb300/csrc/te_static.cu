@@ -54,13 +54,15 @@ unsigned char g_desc_host[sizeof(GroupDesc) + (kStaticMaxSurr + 1) * sizeof(Memb
                           4 * TE_MAX_DIMS + 64];
 constexpr int kStaticMaxSegs = 64;   // pieces of the points whose lists are in the scratch at once
 struct StaticListTables {
+    unsigned nonfinite, pad[3];   // set by the kernels, read back with the keys before it
     ListGroup group;
     RankSortJob sort;
     ListSeg segs[kStaticMaxSegs];
 };
 StaticListTables g_tables_host;
 int g_sms[kStaticMaxDevices];
-int64_t g_keys_host[2 * (kStaticMaxSurr + 1)];
+// the keys, the padding behind them and the list tables' first words
+alignas(16) unsigned char g_keys_host[16 * (kStaticMaxSurr + 1) + 256 + 16];
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 static_assert(sizeof(GroupDesc) <= 256, "the documented scratch size counts 256 bytes for it");
@@ -233,6 +235,7 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
 
     if (lists) {
         StaticListTables &t = g_tables_host;
+        t.nonfinite = 0;
         lg.base = series_dev;
         lg.N = N;
         lg.k = p->k;
@@ -281,6 +284,7 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
             L.q = q;
             L.acc = acc;
             L.dbg_out = -1;
+            L.nonfinite = (unsigned *)(sc + tab_off);
             if (launch_list_build(L, (t.segs[a].nq + queries - 1) / queries, queries, lg.cap_a,
                                   lg.cap_b, stream) != cudaSuccess ||
                 launch_list_walk(L, (long long)t.segs[a].n_splits * lg.n_mblocks, shape, xbytes,
@@ -306,11 +310,16 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
     }
     if (launch_finalize(acc, keys, S + 1, stream) != cudaSuccess) return TE_ECUDA;
 
-    int64_t *kh = g_keys_host;
-    if (cudaMemcpyAsync(kh, keys, (size_t)(S + 1) * 16, cudaMemcpyDeviceToHost, stream) !=
-            cudaSuccess ||
+    // with lists the flag lies at most 256 bytes behind the keys: one copy
+    const size_t flag_at = tab_off - key_off;
+    if (cudaMemcpyAsync(g_keys_host, keys, lists ? flag_at + 16 : (size_t)(S + 1) * 16,
+                        cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
         cudaStreamSynchronize(stream) != cudaSuccess)
         return TE_ECUDA;
+    unsigned nonfinite = 0;
+    if (lists) std::memcpy(&nonfinite, g_keys_host + flag_at, sizeof nonfinite);
+    if (nonfinite) return TE_EINVAL;
+    const int64_t *kh = (const int64_t *)g_keys_host;
     if (out_key) std::memcpy(out_key, kh, (size_t)(S + 1) * 16);
     const double psi_k = std::ldexp((double)g_q_host[p->k], -52);
     const double dN = 4503599627370496.0 * (double)N;

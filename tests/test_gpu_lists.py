@@ -200,3 +200,26 @@ def test_member_lane_kernel_with_distances_of_zero(env, levels):
     got, ref = _both(te, ctx, jobs)
     assert got == ref
     data.close()
+
+
+@pytest.mark.parametrize("dz,w", [(0, 0), (0, 3), (1, 0), (1, 3), (2, 0)])
+def test_static_entry_point_refuses_values_that_are_not_finite(env, dz, w):
+    """The allocation-free call gets a device pointer that no host check has
+    read: single and whole-column values that are not finite, in X, Y and Z,
+    are refused, and the next call is as good as one before."""
+    torch = pytest.importorskip("torch")
+    te, ctx = env
+    T = 3300
+    s = np.asarray(synth.workload_var10(T=T, seed=5)["series"], dtype=np.float32)
+    dev = torch.from_numpy(s).cuda()
+    kw = dict(k=4, theiler=w, max_lag=5, n_surr=3, seed=7, return_keys=True)
+    call = lambda d: te.cmi_ksg_static(d, [(2, 1)], [(0, 0)], Z[:dz], **kw)
+    ref = call(dev)[1]
+    for proc in [2, 0] + ([4] if dz > 1 else []):
+        for value in (np.nan, np.inf, -np.inf):
+            for where in (slice(1700, 1701), slice(0, T)):
+                bad = s.copy()
+                bad[proc, where] = value
+                with pytest.raises(te.TEError, match="TE_EINVAL"):
+                    call(torch.from_numpy(bad).cuda())
+    assert call(dev)[1] == ref
