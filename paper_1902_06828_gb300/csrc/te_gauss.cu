@@ -18,6 +18,7 @@ using namespace teksg;
 namespace {
 
 constexpr int kGaussBatch = 4096;   // estimates per batched launch (grid z)
+constexpr size_t kGaussTurn = (size_t)1 << 29;   // 16-bit entries of a batch's turned permutations
 
 // Shape of one estimate (N points, S surrogates, X / Y / Z dimensions, the
 // points split `splits` ways for the contraction) and the number of doubles
@@ -137,38 +138,47 @@ te_status run_groups_gauss(te_ctx *ctx, const std::vector<HostGroup> &groups, in
             for (const te_var &v : g.z) cols.push_back(gauss_col(g.data, g.max_lag, v));
         }
     }
-    // every permutation set turned once for the contraction in shared memory
-    std::vector<PermTurnJob> turn;
-    std::map<const int32_t *, size_t> turn_of;   // -> 16-bit entries into the turned sets
-    size_t turn_elems = 0;
-    for (GaussArgs &A : est) {
-        if (A.d - A.dx > kGaussFFMaxW || A.N > kGaussFFColMax || A.S < 1) continue;
-        A.perm_t_pitch = (A.S + 32) & ~31;
-        if (turn_of.emplace(A.perms, turn_elems).second) {
-            turn.push_back(PermTurnJob{A.perms, nullptr, A.S, A.N, A.perm_t_pitch});
-            turn_elems += (size_t)A.N * A.perm_t_pitch;
-        }
-    }
     // shapes: a batch splits each estimate's points so that the contraction
     // has about eight CTAs per SM in all; where a CTA keeps the X column (two
     // fit an SM, each takes two splits, and loading the column costs it 1% of a
     // whole estimate) eight waves of them, so that the last is a small part
+    // The contraction in shared memory reads its permutations turned: a batch
+    // turns the sets of its own estimates and ends where they pass kGaussTurn
+    // (independent surrogates make a set per candidate: 201 x 10^4 points take 4.5 MB).
     const int n_est = (int)est.size();
-    size_t ws = 0;
+    struct Batch {
+        int begin, n;
+        std::vector<PermTurnJob> turn;
+        std::map<const int32_t *, size_t> turn_of;   // -> entries into the turned sets
+    };
+    std::vector<Batch> batches;
+    size_t ws = 0, turn_elems = 0;   // of the largest batch
     std::vector<size_t> off(n_est);
-    for (int b0 = 0; b0 < n_est; b0 += kGaussBatch) {
-        const int nb = std::min(kGaussBatch, n_est - b0);
-        size_t w = 0;
-        for (int i = b0; i < b0 + nb; ++i) {
+    for (int b0 = 0; b0 < n_est;) {
+        Batch b{b0, 0, {}, {}};
+        size_t w = 0, elems = 0;
+        for (; b0 + b.n < n_est && b.n < kGaussBatch && elems < kGaussTurn; ++b.n) {
+            GaussArgs &A = est[b0 + b.n];
+            if (A.d - A.dx > kGaussFFMaxW || A.N > kGaussFFColMax || A.S < 1) continue;
+            A.perm_t_pitch = (A.S + 32) & ~31;
+            if (b.turn_of.emplace(A.perms, elems).second) {
+                b.turn.push_back(PermTurnJob{A.perms, nullptr, A.S, A.N, A.perm_t_pitch});
+                elems += (size_t)A.N * A.perm_t_pitch;
+            }
+        }
+        for (int i = b0; i < b0 + b.n; ++i) {
             GaussArgs &A = est[i];
             const int blocks = A.perm_t_pitch ? (A.S + 256) / 256 * A.dx
                                               : ((A.S + 1) * A.dx + 127) / 128;
             const bool col = A.perm_t_pitch != 0;
-            const int splits = ((col ? 32 : 8) * 152 + nb * blocks - 1) / (nb * blocks);
+            const int splits = ((col ? 32 : 8) * 152 + b.n * blocks - 1) / (b.n * blocks);
             off[i] = w;
             w += gauss_shape(A, A.N, A.S, A.dx, A.dy, A.d - A.dx - A.dy, splits, true);
         }
         ws = std::max(ws, w);
+        turn_elems = std::max(turn_elems, elems);
+        b0 += b.n;
+        batches.push_back(std::move(b));
     }
     // doubles: batch workspace, then estimates and bounds of all slots;
     // then the batch's argument blocks; ints: status flags, the columns
@@ -187,48 +197,48 @@ te_status run_groups_gauss(te_ctx *ctx, const std::vector<HostGroup> &groups, in
     CK(cudaMemsetAsync(v_out, 0, (size_t)n_out * 8, ctx->stream), "cudaMemsetAsync");
     if (!cols.empty())
         CK(copy_h2d(ctx, cols_dev, cols.data(), cols.size() * 4), "cudaMemcpyAsync");
-    if (!turn.empty()) {
-        const size_t jobs_at = (turn_elems * 2 + 255) & ~(size_t)255;
-        if ((st = ensure_dev(ctx, ctx->ws_gtile, jobs_at + turn.size() * sizeof(PermTurnJob))))
-            return st;
-        uint16_t *tb = (uint16_t *)ctx->ws_gtile.p;
-        for (PermTurnJob &J : turn) J.dst = tb + turn_of[J.src];
-        for (GaussArgs &A : est)
-            if (A.perm_t_pitch) A.perm_t = tb + turn_of[A.perms];
-        PermTurnJob *jd = (PermTurnJob *)((char *)ctx->ws_gtile.p + jobs_at);
-        CK(copy_h2d(ctx, jd, turn.data(), turn.size() * sizeof(PermTurnJob)), "cudaMemcpyAsync");
-        CK(gauss_launch_turn(jd, turn.data(), (int)turn.size(), ctx->stream),
-           "permutation turn launch");
-        ctx->stats.launches++;
-    }
-    int src = 0;
-    for (int i = 0; i < n_est; ++i) {
-        GaussArgs &A = est[i];
-        gauss_bind(A, w + off[i], true);
-        A.cols = cols_dev + col0[i];
-        A.status = status;
-        A.out = v_out + slot0[i];
-        A.err = v_err + slot0[i];
-        // the group's first estimate in each batch forms the W-W covariance and
-        // the factors; the group's later ones in the batch use them
-        if (i % kGaussBatch == 0 || gid[i] != gid[i - 1]) {
-            src = i;
-        } else {
-            A.own_w = 0;
-            A.covw = est[src].cov;
-            A.meanw = est[src].mean + est[src].dx;
-            A.LW = est[src].LW;
-            A.LZ = est[src].LZ;
-            A.norms = est[src].norms;
+    const size_t turn_at = (turn_elems * 2 + 255) & ~(size_t)255;   // the batch's turn jobs
+    if (turn_elems &&
+        (st = ensure_dev(ctx, ctx->ws_gtile, turn_at + kGaussBatch * sizeof(PermTurnJob))))
+        return st;
+    uint16_t *tb = (uint16_t *)ctx->ws_gtile.p;
+    for (Batch &b : batches) {
+        int src = b.begin;
+        for (int i = b.begin; i < b.begin + b.n; ++i) {
+            GaussArgs &A = est[i];
+            if (A.perm_t_pitch) A.perm_t = tb + b.turn_of[A.perms];
+            gauss_bind(A, w + off[i], true);
+            A.cols = cols_dev + col0[i];
+            A.status = status;
+            A.out = v_out + slot0[i];
+            A.err = v_err + slot0[i];
+            // the group's first estimate in each batch forms the W-W covariance
+            // and the factors; the group's later ones in the batch use them
+            if (i == b.begin || gid[i] != gid[i - 1]) {
+                src = i;
+            } else {
+                A.own_w = 0;
+                A.covw = est[src].cov;
+                A.meanw = est[src].mean + est[src].dx;
+                A.LW = est[src].LW;
+                A.LZ = est[src].LZ;
+                A.norms = est[src].norms;
+            }
+            ctx->stats.estimates += (uint64_t)A.S + 1;
         }
-        ctx->stats.estimates += (uint64_t)A.S + 1;
-    }
-    for (int b0 = 0; b0 < n_est; b0 += kGaussBatch) {
-        const int nb = std::min(kGaussBatch, n_est - b0);
-        // the previous batch's kernels precede this copy on the stream
-        CK(copy_h2d(ctx, args_dev, est.data() + b0, (size_t)nb * sizeof(GaussArgs)),
+        // the previous batch's kernels precede these copies on the stream
+        if (!b.turn.empty()) {
+            for (PermTurnJob &J : b.turn) J.dst = tb + b.turn_of[J.src];
+            PermTurnJob *jd = (PermTurnJob *)((char *)tb + turn_at);
+            CK(copy_h2d(ctx, jd, b.turn.data(), b.turn.size() * sizeof(PermTurnJob)),
+               "cudaMemcpyAsync");
+            CK(gauss_launch_turn(jd, b.turn.data(), (int)b.turn.size(), ctx->stream),
+               "permutation turn launch");
+            ctx->stats.launches++;
+        }
+        CK(copy_h2d(ctx, args_dev, est.data() + b.begin, (size_t)b.n * sizeof(GaussArgs)),
            "cudaMemcpyAsync");
-        CK(gauss_launch_batch_f64(args_dev, est.data() + b0, nb, ctx->stream),
+        CK(gauss_launch_batch_f64(args_dev, est.data() + b.begin, b.n, ctx->stream),
            "Gaussian batch launch");
         ctx->stats.launches += 7;
     }
