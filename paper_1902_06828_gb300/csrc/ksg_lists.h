@@ -101,6 +101,13 @@ ListShape list_shape(int N, int dx, int dz, int k, size_t members);
 // shared memory of a walking CTA: X values of width members, and every 16th
 // value of the sorted columns that the group's counts search
 size_t list_walk_x_bytes(int N, int dx, int dz, int k, int width);
+// whether neighbour lists are the faster path for a group of a batch of
+// n_groups with `rows` points and `pairs` (member, point) pairs in all
+struct ListCall {
+    int N, k, theiler, dx, dy, dz;
+    size_t members;
+};
+bool list_serves(const ListCall &c, int n_groups, long long rows, long long pairs);
 // whether a group can take the list path
 bool list_fits(int N, int dx, int dz, int k);
 // Parts into which the walk splits the points of a launch, given its member

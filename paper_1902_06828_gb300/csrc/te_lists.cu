@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <tuple>
@@ -39,20 +40,82 @@ struct Chunk {
 
 }  // namespace
 
-te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups, int n_out,
-                              int dbg_out, float *dbg_eps, int *dbg_nxz, int *dbg_nyz,
-                              int *dbg_nz)
+// Measured line between the two paths (whole calls on one GB300, member-lane
+// or fused kernel / lists, microseconds).  Lists pay for themselves by a row
+// per point that all members of the group walk; the member-lane kernel shares
+// its tiles among 32 members (64 from 64 on) and wins
+// - over an empty Z, where n_z needs no list and n_xz is a range count for
+//   either, once the chip is full: 2000 members at N = 10^4 13,700 / 15,800, 9045
+//   57,900 / 66,700, 401 2940 / 2120; 12 groups of 64 at N = 2000 719 / 1572;
+// - where few members share a row and there are many groups: 64 groups of 21,
+//   N = 4000: one Z 8005 / 12,670, two 8323 / 21,559 (their lists are the longest),
+//   three 9317 / 13,002, five 12,134 / 9605; one group of 21 933 / 401, 64 of 201
+//   at N = 1000 and two Z 7095 / 4901.
+// Several X variables: a member's neighbours lie the deeper in list A the fewer
+// Y and Z variables there are, and pairs beyond its capacity scan all points.
+// The line is at the expected depth: 201 members at N = 9000, k = 4, empty Z, two X
+// variables (depth 686) 17,220 / 18,689, four (1922) 28,342 / 147,900; one Z and four
+// (686) equal; two Z 3.3 to 7 times in the lists' favour.  With k other than 4
+// a point's dimensions lie apart (list_shape) and the line is nearer: k = 6,
+// one Z, four X variables, N = 4000 9981 / 12,455.
+bool list_serves(const ListCall &c, int n_groups, long long rows, long long pairs)
+{
+    const int N = c.N, dz = c.dz;
+    const long long m = (long long)c.members;
+    if (!list_fits(N, c.dx, dz, c.k)) return false;
+    if (c.dx > 1) {
+        if (dz > 1 || m < 8) return true;
+        const double d = c.dx + c.dy + dz;
+        const double depth = N * std::pow((double)c.k / N, (c.dy + dz) / d);   // mean n_yz
+        const bool packed = list_shape(N, c.dx, dz, c.k, c.members).dxp > 0;
+        double most;
+        if (dz == 0)
+            most = m >= 64 ? (packed ? 650 : std::min(290.0, 0.42 * N))
+                           : packed ? 1150 : m >= 24 ? 430 : 700;
+        else if (packed)
+            most = 680;
+        else
+            most = m >= 64 && (c.dx > 2 || (m >= 100 && N < 5000)) ? 0 : 500;
+        return depth <= most;
+    }
+    if (c.theiler > 0 || N > kMaxOrderN) return true;   // the member lanes cannot prune then
+    const bool full = rows >= 24000;   // points of all groups: several waves of CTAs
+    const bool block = m <= 32 || (m >= 48 && m <= 64);   // one well-filled block of members
+    if (n_groups >= 200 && m <= 8 && N <= 700 && dz > 0) return false;
+    if (N < 250) return true;
+    switch (dz) {
+    case 0:
+        return !((pairs >= 1600LL * N && N >= 700) ||
+                 (n_groups >= 4 && rows >= 8000 && m >= 16 && (N >= 350 || m <= 64)) ||
+                 (full && (m >= 4 || N <= 3000) && (N >= 350 || m <= 64)));
+    case 1:
+        return !(full && block && n_groups >= (m >= 16 ? 10 : 32) && (m >= 4 || N <= 3000));
+    case 2:
+        return !(full && (block || (m < 64 && N >= 3500)) &&
+                 n_groups >= (m >= 16 ? (N >= 3500 ? 5 : 10)
+                                      : N >= 3500 ? 8 : N >= 1500 ? 16 : 32));
+    case 3:
+        return !(full && block && n_groups >= (m >= 16 && N >= 3500 ? 12 : 32));
+    case 4:
+    case 5:
+        return !(full && m <= 32 && n_groups >= 64 && N <= (dz == 4 ? 1500 : 700));
+    default:
+        return !(full && m <= 32 && n_groups >= 200 && N <= 700);
+    }
+}
+
+te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &groups,
+                        const KsgDebug &dbg, KsgPart &part)
 {
     te_status st;
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device),
        "cudaDeviceGetAttribute");
     std::map<ListShape, std::vector<const HostGroup *>> classes;
-    for (const HostGroup &g : groups)
-        if (!g.members.empty())
-            classes[list_shape(g.data->T - g.max_lag, g.dx, (int)g.z.size(), g.k,
-                               g.members.size())]
-                .push_back(&g);
+    for (const HostGroup *g : groups)
+        classes[list_shape(g->data->T - g->max_lag, g->dx, (int)g->z.size(), g->k,
+                           g->members.size())]
+            .push_back(g);
 
     std::vector<ListGroup> lg;
     std::vector<MemberDesc> mdesc;
@@ -176,20 +239,13 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
         close_chunk();
         plans.push_back(cp);
     }
-    if (plans.empty()) {
-        CK(launch_finalize((const unsigned long long *)ctx->ws_acc.p, (long long *)ctx->ws_keys.p,
-                           n_out, ctx->stream),
-           "finalize launch");
-        return TE_OK;
-    }
-
     // workspaces, then the pointers into them, then one upload of all tables
     if ((st = ensure_dev(ctx, ctx->ws_lists, pool))) return st;
-    if (vs_words && (st = ensure_dev(ctx, ctx->ws_vsort, vs_words * 4))) return st;
+    if (vs_words && (st = ensure_dev(ctx, ctx->ws_lsort, vs_words * 4))) return st;
     int vitems = 0;
     for (size_t a = 0; a < vjobs.size(); ++a) {
         RankSortJob &J = vjobs[a];
-        J.sorted = (float *)ctx->ws_vsort.p + vjob_off[a];
+        J.sorted = (float *)ctx->ws_lsort.p + vjob_off[a];
         J.rank = (int *)(J.sorted + (((size_t)J.N + 3) & ~(size_t)3));
         J.item = vitems;
         vitems += rank_sort_items(J.N);
@@ -214,46 +270,44 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
         t.at = bytes;
         bytes += (t.bytes + 15) & ~(size_t)15;
     }
-    if ((st = ensure_pin(ctx, bytes))) return st;
-    if ((st = ensure_dev(ctx, ctx->ws_groups, bytes))) return st;
+    if ((st = ensure_pin_lists(ctx, bytes))) return st;
+    if ((st = ensure_dev(ctx, ctx->ws_ltables, bytes))) return st;
     for (const Table &t : tab)
-        if (t.bytes) std::memcpy((char *)ctx->pin + t.at, t.src, t.bytes);
-    CK(copy_h2d(ctx, ctx->ws_groups.p, ctx->pin, bytes), "cudaMemcpyAsync");
-    char *dtab = (char *)ctx->ws_groups.p;
+        if (t.bytes) std::memcpy((char *)ctx->pin_lists + t.at, t.src, t.bytes);
+    CK(copy_h2d(ctx, ctx->ws_ltables.p, ctx->pin_lists, bytes), "cudaMemcpyAsync");
+    char *dtab = (char *)ctx->ws_ltables.p;
     for (const Chunk &ch : chunks)
         CK(list_prepare(plans[ch.cls].shape, ch.queries, &ctx->prepared_lists),
            "cudaFuncSetAttribute");
 
-    const bool graph = ctx->opt_graph != 0;
-    auto device_work = [&]() -> te_status {
-        if (!vjobs.empty()) {
-            CK(launch_rank_sort((const RankSortJob *)(dtab + tab[3].at), (int)vjobs.size(), vitems,
-                                ctx->stream),
-               "column sort launch");
+    part.pair_evals = pair_evals;
+    part.members = members_total;
+    if (!vjobs.empty())
+        part.before = [ctx, jobs = (const RankSortJob *)(dtab + tab[3].at),
+                       n = (int)vjobs.size(), vitems]() -> te_status {
+            CK(launch_rank_sort(jobs, n, vitems, ctx->stream), "column sort launch");
             ctx->stats.launches++;
-        }
-        CK(cudaMemsetAsync(ctx->work_dev, 0, 3 * sizeof(unsigned long long), ctx->stream),
-           "cudaMemsetAsync");
-        if (!graph) CK(cudaEventRecord(ctx->ev_a, ctx->stream), "cudaEventRecord");
-        auto launch_args = [&](const ClassPlan &cp) {
-            ListLaunch L{};
-            L.groups = (const ListGroup *)(dtab + tab[0].at) + cp.first_group;
-            L.members = (const MemberDesc *)(dtab + tab[2].at);
-            L.cols = (const int *)(dtab + tab[4].at);
-            L.q = ctx->q_dev;
-            L.acc = (unsigned long long *)ctx->ws_acc.p;
-            L.dbg_eps = dbg_eps;
-            L.dbg_nxz = dbg_nxz;
-            L.dbg_nyz = dbg_nyz;
-            L.dbg_nz = dbg_nz;
-            L.dbg_out = dbg_out;
-            L.work = ctx->work_dev;
-            return L;
+            return TE_OK;
         };
+    ListLaunch base{};
+    base.groups = (const ListGroup *)(dtab + tab[0].at);
+    base.segs = (const ListSeg *)(dtab + tab[1].at);
+    base.members = (const MemberDesc *)(dtab + tab[2].at);
+    base.cols = (const int *)(dtab + tab[4].at);
+    base.q = ctx->q_dev;
+    base.acc = (unsigned long long *)ctx->ws_acc.p;
+    base.dbg_eps = dbg.eps;
+    base.dbg_nxz = dbg.nxz;
+    base.dbg_nyz = dbg.nyz;
+    base.dbg_nz = dbg.nz;
+    base.dbg_out = dbg.out;
+    base.work = ctx->work_dev;
+    part.kernels = [ctx, plans, chunks, base]() -> te_status {
         for (const Chunk &ch : chunks) {
             const ClassPlan &cp = plans[ch.cls];
-            ListLaunch L = launch_args(cp);
-            L.segs = (const ListSeg *)(dtab + tab[1].at) + ch.first_seg;
+            ListLaunch L = base;
+            L.groups += cp.first_group;
+            L.segs += ch.first_seg;
             L.n_segs = ch.n_segs;
             CK(launch_list_build(L, ch.build_items, ch.queries, ch.cap_a, ch.cap_b, ctx->stream),
                "list build launch");
@@ -262,19 +316,8 @@ te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups,
             ctx->stats.launches += 2;
             ctx->stats.ksg_launches++;
         }
-        if (!graph) CK(cudaEventRecord(ctx->ev_b, ctx->stream), "cudaEventRecord");
-        CK(copy_d2h(ctx, ctx->work_host, ctx->work_dev, 3 * sizeof(unsigned long long)),
-           "cudaMemcpyAsync");
-        CK(launch_finalize((const unsigned long long *)ctx->ws_acc.p,
-                           (long long *)ctx->ws_keys.p, n_out, ctx->stream),
-           "finalize launch");
-        ctx->stats.launches++;
         return TE_OK;
     };
-    if ((st = submit_work(ctx, device_work))) return st;
-    ctx->pend_timed = 1;
-    ctx->pend_pair_evals = pair_evals;
-    ctx->pend_members = members_total;
     return TE_OK;
 }
 

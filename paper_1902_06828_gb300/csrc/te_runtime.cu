@@ -63,19 +63,29 @@ te_status ensure_dev(te_ctx *ctx, DevBuf &b, size_t bytes)
     return TE_OK;
 }
 
+static te_status grow_pinned(te_ctx *ctx, void *&p, size_t &cap, size_t bytes)
+{
+    if (bytes <= cap) return TE_OK;
+    const size_t want = std::max(bytes, cap + cap / 2);
+    if (p) {
+        CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+        CK(cudaFreeHost(p), "cudaFreeHost");
+        p = nullptr;
+        cap = 0;
+    }
+    CK(cudaMallocHost(&p, want), "cudaMallocHost");
+    cap = want;
+    return TE_OK;
+}
+
 te_status ensure_pin(te_ctx *ctx, size_t bytes)
 {
-    if (bytes <= ctx->pin_cap) return TE_OK;
-    size_t want = std::max(bytes, ctx->pin_cap + ctx->pin_cap / 2);
-    if (ctx->pin) {
-        CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
-        CK(cudaFreeHost(ctx->pin), "cudaFreeHost");
-        ctx->pin = nullptr;
-        ctx->pin_cap = 0;
-    }
-    CK(cudaMallocHost(&ctx->pin, want), "cudaMallocHost");
-    ctx->pin_cap = want;
-    return TE_OK;
+    return grow_pinned(ctx, ctx->pin, ctx->pin_cap, bytes);
+}
+
+te_status ensure_pin_lists(te_ctx *ctx, size_t bytes)
+{
+    return grow_pinned(ctx, ctx->pin_lists, ctx->pin_lists_cap, bytes);
 }
 
 te_status ensure_aux(te_ctx *ctx)
@@ -343,22 +353,62 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
     if ((st = ensure_dev(ctx, ctx->ws_acc, (size_t)std::max(n_out, 1) * 16))) return st;
     if ((st = ensure_dev(ctx, ctx->ws_keys, (size_t)std::max(n_out, 1) * 16))) return st;
     CK(cudaMemsetAsync(ctx->ws_acc.p, 0, (size_t)n_out * 16, ctx->stream), "cudaMemsetAsync");
-    // Neighbour lists wherever a member's X values fit a CTA's shared memory;
-    // an option of the member-lane kernel asks for that kernel.  Member-lane ->
-    // lists over the sizes: one estimate at T = 203 128 -> 79 us, 201 members at
-    // T = 1000 366 -> 190 us, at T = 10^4 5.7 -> 2.1 ms, 9045 members 104 -> 36 ms.
-    bool lists = !ctx->opt_jt && !ctx->opt_ms && !ctx->opt_persistent && !ctx->opt_order;
-    for (const HostGroup &g : groups)
-        lists = lists && list_fits(g.data->T - g.max_lag, g.dx, (int)g.z.size(), g.k);
-    if (lists)
-        return launch_groups_lists(ctx, groups, n_out, dbg_out, dbg_eps, dbg_nxz, dbg_nyz,
-                                   dbg_nz);
-
-    std::map<ClassKey, std::vector<const HostGroup *>> classes;
+    const KsgDebug dbg{dbg_out, dbg_eps, dbg_nxz, dbg_nyz, dbg_nz};
+    // each group by neighbour lists or by the member-lane kernel; an option of
+    // the latter asks for it
+    const bool lane_only = ctx->opt_jt || ctx->opt_ms || ctx->opt_persistent || ctx->opt_order;
+    int n_groups = 0;
+    long long rows = 0, pairs = 0;
+    for (const HostGroup &g : groups) {
+        const long long N = g.data->T - g.max_lag;
+        if (g.members.empty()) continue;
+        n_groups++;
+        rows += N;
+        pairs += N * (long long)g.members.size();
+    }
+    std::vector<const HostGroup *> by_lists, by_lanes;
     for (const HostGroup &g : groups) {
         if (g.members.empty()) continue;
-        classes[ClassKey{g.dx == 1, g.k == 4}].push_back(&g);
+        const ListCall c{g.data->T - g.max_lag, g.k, g.theiler, g.dx, (int)g.y.size(),
+                         (int)g.z.size(), g.members.size()};
+        (!lane_only && list_serves(c, n_groups, rows, pairs) ? by_lists : by_lanes).push_back(&g);
     }
+    KsgPart lanes, lists;
+    if (!by_lanes.empty() && (st = prepare_lanes(ctx, by_lanes, dbg, lanes))) return st;
+    if (!by_lists.empty() && (st = prepare_lists(ctx, by_lists, dbg, lists))) return st;
+    const bool graph = ctx->opt_graph != 0;
+    auto device_work = [&]() -> te_status {
+        te_status st;
+        CK(cudaMemsetAsync(ctx->work_dev, 0, 3 * sizeof(unsigned long long), ctx->stream),
+           "cudaMemsetAsync");
+        for (const KsgPart *p : {&lanes, &lists})
+            if (p->before && (st = p->before())) return st;
+        if (!graph) CK(cudaEventRecord(ctx->ev_a, ctx->stream), "cudaEventRecord");
+        for (const KsgPart *p : {&lanes, &lists})
+            if (p->kernels && (st = p->kernels())) return st;
+        if (!graph) CK(cudaEventRecord(ctx->ev_b, ctx->stream), "cudaEventRecord");
+        CK(copy_d2h(ctx, ctx->work_host, ctx->work_dev, 3 * sizeof(unsigned long long)),
+           "cudaMemcpyAsync");
+        CK(launch_finalize((const unsigned long long *)ctx->ws_acc.p, (long long *)ctx->ws_keys.p,
+                           n_out, ctx->stream),
+           "finalize launch");
+        ctx->stats.launches++;
+        return TE_OK;
+    };
+    if ((st = submit_work(ctx, device_work))) return st;
+    if (!lanes.members && !lists.members) return TE_OK;
+    ctx->pend_timed = 1;
+    ctx->pend_pair_evals = lanes.pair_evals + lists.pair_evals;
+    ctx->pend_members = lanes.members + lists.members;
+    return TE_OK;
+}
+
+te_status prepare_lanes(te_ctx *ctx, const std::vector<const HostGroup *> &groups,
+                        const KsgDebug &dbg, KsgPart &part)
+{
+    te_status st;
+    std::map<ClassKey, std::vector<const HostGroup *>> classes;
+    for (const HostGroup *g : groups) classes[ClassKey{g->dx == 1, g->k == 4}].push_back(g);
 
     // Spatial order for every group without a Theiler window that fits one
     // sorting CTA: sigma [N], sorted coordinates [dyz][N], chunk boxes.
@@ -370,11 +420,10 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
     std::vector<const HostGroup *> to_order;
     size_t order_bytes = 0;
     auto align16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
-    for (const HostGroup &g : groups) {
-        const int N = g.data->T - g.max_lag;
-        const int dyz = (int)(g.y.size() + g.z.size());
-        if (g.members.empty() || g.theiler != 0 || N > kMaxOrderN || N < 16 || dyz > 32)
-            continue;
+    for (const HostGroup *g : groups) {
+        const int N = g->data->T - g->max_lag;
+        const int dyz = (int)(g->y.size() + g->z.size());
+        if (g->theiler != 0 || N > kMaxOrderN || N < 16 || dyz > 32) continue;
         OrderOut o;
         o.nch = (N + 7) / 8;
         o.sigma = order_bytes;
@@ -386,8 +435,8 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
         o.ntl = (N + 255) / 256;
         o.tbox = order_bytes;
         order_bytes += align16((size_t)dyz * o.ntl * 8);
-        order_of[&g] = o;
-        to_order.push_back(&g);
+        order_of[g] = o;
+        to_order.push_back(g);
     }
     if (!to_order.empty()) {
         if ((st = ensure_dev(ctx, ctx->ws_order, order_bytes))) return st;
@@ -626,12 +675,6 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
         p.items = item;
         plans.push_back(p);
     }
-    if (plans.empty()) {
-        CK(launch_finalize((const unsigned long long *)ctx->ws_acc.p, (long long *)ctx->ws_keys.p,
-                           n_out, ctx->stream),
-           "finalize launch");
-        return TE_OK;
-    }
 
     std::vector<OrderJob> ojobs;
     for (const HostGroup *g : to_order) {
@@ -702,28 +745,29 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
         CK(ksg_prepare_attributes(), "cudaFuncSetAttribute");
         ctx->prepared = 1;
     }
-    const bool graph = ctx->opt_graph != 0;
-    auto device_work = [&]() -> te_status {
-        if (!ojobs.empty()) {
-            CK(launch_order((const OrderJob *)ctx->ws_ojobs.p, (int)ojobs.size(), ctx->stream),
-               "order launch");
+    part.pair_evals = pair_evals;
+    part.members = members_total;
+    part.before = [ctx, n_order = (int)ojobs.size(), n_compose = (int)cjobs.size(),
+                   n_sort = (int)vjobs.size(), obytes, jbytes, max_cn]() -> te_status {
+        const char *jobs = (const char *)ctx->ws_ojobs.p;
+        if (n_order) {
+            CK(launch_order((const OrderJob *)jobs, n_order, ctx->stream), "order launch");
             ctx->stats.launches++;
         }
-        if (!cjobs.empty()) {
-            CK(launch_compose((const ComposeJob *)((char *)ctx->ws_ojobs.p + obytes),
-                              (int)cjobs.size(), max_cn, ctx->stream),
+        if (n_compose) {
+            CK(launch_compose((const ComposeJob *)(jobs + obytes), n_compose, max_cn, ctx->stream),
                "compose launch");
             ctx->stats.launches++;
         }
-        if (!vjobs.empty()) {
-            CK(launch_value_sort((const ValueSortJob *)((char *)ctx->ws_ojobs.p + obytes + jbytes),
-                                 (int)vjobs.size(), ctx->stream),
+        if (n_sort) {
+            CK(launch_value_sort((const ValueSortJob *)(jobs + obytes + jbytes), n_sort,
+                                 ctx->stream),
                "value sort launch");
             ctx->stats.launches++;
         }
-        CK(cudaMemsetAsync(ctx->work_dev, 0, 3 * sizeof(unsigned long long), ctx->stream),
-           "cudaMemsetAsync");
-        if (!graph) CK(cudaEventRecord(ctx->ev_a, ctx->stream), "cudaEventRecord");
+        return TE_OK;
+    };
+    part.kernels = [ctx, plans, dbg]() -> te_status {
         for (const Plan &p : plans) {
             KsgLaunch L{};
             L.groups = (const GroupDesc *)ctx->ws_groups.p + p.g_off;
@@ -732,11 +776,11 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
             L.cols = (const int *)ctx->ws_cols.p + p.c_off;
             L.q = ctx->q_dev;
             L.acc = (unsigned long long *)ctx->ws_acc.p;
-            L.dbg_eps = dbg_eps;
-            L.dbg_nxz = dbg_nxz;
-            L.dbg_nyz = dbg_nyz;
-            L.dbg_nz = dbg_nz;
-            L.dbg_out = dbg_out;
+            L.dbg_eps = dbg.eps;
+            L.dbg_nxz = dbg.nxz;
+            L.dbg_nyz = dbg.nyz;
+            L.dbg_nz = dbg.nz;
+            L.dbg_out = dbg.out;
             L.jt = p.jt;
             L.work = ctx->work_dev;
             if (p.v.persist) {
@@ -759,19 +803,8 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
             ctx->stats.launches++;
             ctx->stats.ksg_launches++;
         }
-        if (!graph) CK(cudaEventRecord(ctx->ev_b, ctx->stream), "cudaEventRecord");
-        CK(copy_d2h(ctx, ctx->work_host, ctx->work_dev, 3 * sizeof(unsigned long long)),
-           "cudaMemcpyAsync");
-        CK(launch_finalize((const unsigned long long *)ctx->ws_acc.p,
-                           (long long *)ctx->ws_keys.p, n_out, ctx->stream),
-           "finalize launch");
-        ctx->stats.launches++;
         return TE_OK;
     };
-    if ((st = submit_work(ctx, device_work))) return st;
-    ctx->pend_timed = 1;
-    ctx->pend_pair_evals = pair_evals;
-    ctx->pend_members = members_total;
     return TE_OK;
 }
 
@@ -867,11 +900,12 @@ void te_ctx_destroy(te_ctx *ctx)
                       &ctx->ws_keys,   &ctx->ws_perm,    &ctx->ws_stat,  &ctx->ws_dbg,
                       &ctx->ws_order,  &ctx->ws_ojobs,  &ctx->ws_cperm, &ctx->ws_gauss,
                       &ctx->ws_vsort,  &ctx->ws_xval,   &ctx->ws_gtile,
-                      &ctx->ws_lists};
+                      &ctx->ws_lists,  &ctx->ws_ltables, &ctx->ws_lsort};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);
     if (ctx->q_dev) cudaFree(ctx->q_dev);
     if (ctx->pin) cudaFreeHost(ctx->pin);
+    if (ctx->pin_lists) cudaFreeHost(ctx->pin_lists);
     if (ctx->work_dev) cudaFree(ctx->work_dev);
     if (ctx->work_host) cudaFreeHost(ctx->work_host);
     if (ctx->ev_a) cudaEventDestroy(ctx->ev_a);

@@ -123,11 +123,15 @@ struct te_ctx {
     teksg::DevBuf ws_groups, ws_members, ws_cols, ws_acc, ws_keys, ws_perm, ws_stat, ws_dbg;
     teksg::DevBuf ws_order, ws_ojobs, ws_cperm, ws_gauss, ws_vsort;
     teksg::DevBuf ws_xval;   // X-value rows of the TMA-staged lane kernel
-    teksg::DevBuf ws_lists;  // neighbour lists of the points in work
+    // neighbour lists of the points in work, the list launches' tables and
+    // sorted columns (a batch may need the member-lane kernel's beside them)
+    teksg::DevBuf ws_lists, ws_ltables, ws_lsort;
     teksg::DevBuf ws_gtile;  // cmi_gauss: the contraction's prepared B tiles and centred X
     // pinned host staging
     void *pin = nullptr;
     size_t pin_cap = 0;
+    void *pin_lists = nullptr;   // the list launches' tables
+    size_t pin_lists_cap = 0;
     te_stats stats{};
     // counters of the launch in flight, added to stats by finish_groups
     int pend_timed = 0;
@@ -167,6 +171,7 @@ te_status cuda_fail(te_ctx *ctx, cudaError_t e, const char *what);
 
 te_status ensure_dev(te_ctx *ctx, DevBuf &b, size_t bytes);
 te_status ensure_pin(te_ctx *ctx, size_t bytes);
+te_status ensure_pin_lists(te_ctx *ctx, size_t bytes);
 te_status ensure_aux(te_ctx *ctx);   // ctx->aux_stream, ev_fork, ev_join
 te_status ensure_q(te_ctx *ctx, int n_needed);   // Q[0..n_needed] on the device
 // Q[0..n_max] into a caller buffer (host), same arithmetic as ensure_q
@@ -199,10 +204,22 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
                         int dbg_out = -1, float *dbg_eps = nullptr, int *dbg_nxz = nullptr,
                         int *dbg_nyz = nullptr, int *dbg_nz = nullptr);
 te_status finish_groups(te_ctx *ctx);
-// launch_groups by neighbour lists (te_lists.cu), after the accumulators are set
-te_status launch_groups_lists(te_ctx *ctx, const std::vector<HostGroup> &groups, int n_out,
-                              int dbg_out, float *dbg_eps, int *dbg_nxz, int *dbg_nyz,
-                              int *dbg_nz);
+// A launch's groups on one path: what precedes the timed kernels (orders,
+// sorted columns) and the kernels themselves, to be called on ctx->stream (or
+// under capture) once the tables are uploaded, which prepare_* has done.
+struct KsgDebug {
+    int out;
+    float *eps;
+    int *nxz, *nyz, *nz;
+};
+struct KsgPart {
+    std::function<te_status()> before, kernels;
+    uint64_t pair_evals = 0, members = 0;   // of the unpruned estimator; estimates
+};
+te_status prepare_lanes(te_ctx *ctx, const std::vector<const HostGroup *> &groups,
+                        const KsgDebug &dbg, KsgPart &part);   // member-lane / fused kernel
+te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &groups,
+                        const KsgDebug &dbg, KsgPart &part);   // te_lists.cu
 // Queue a batch's device work on ctx->stream: directly, or with the graph
 // option captured on the stream, instantiated and launched as one graph (the
 // timing events then bracket the graph launch).

@@ -169,8 +169,11 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
     const size_t row = list_row_bytes(lg.cap_a, lg.cap_b);
     const size_t room = row_off < kStaticScratchBytes ? (kStaticScratchBytes - row_off) / row : 0;
     const int seg_rows = (int)std::min<size_t>((size_t)N, room);
-    const bool lists = list_fits(N, dx, dz, p->k) && seg_rows > 0 &&
-                       (N + seg_rows - 1) / seg_rows <= kStaticMaxSegs;
+    // (its member-lane kernel has no spatial order to prune by, so one X variable
+    // takes the lists at any number of pairs)
+    const bool lists =
+        seg_rows > 0 && (N + seg_rows - 1) / seg_rows <= kStaticMaxSegs &&
+        list_serves(ListCall{N, p->k, p->theiler, dx, dy, dz, (size_t)S + 1}, 1, N, 0);
 
     // one group in time order, members = identity + S surrogates
     const bool dx1 = dx == 1;

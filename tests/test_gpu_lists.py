@@ -223,3 +223,27 @@ def test_static_entry_point_refuses_values_that_are_not_finite(env, dz, w):
                 with pytest.raises(te.TEError, match="TE_EINVAL"):
                     call(torch.from_numpy(bad).cuda())
     assert call(dev)[1] == ref
+
+
+@pytest.mark.parametrize("T,n_groups,S", [(360, 70, 3), (1005, 30, 20), (3005, 12, 20)])
+def test_batches_whose_groups_take_both_paths(env, T, n_groups, S):
+    """One batch of many groups: of few members over zero to five Z variables,
+    of 201 members, of several X variables with and without Z, and (at the
+    longest) of an X block past a CTA's shared memory.  Some take lists, some
+    the member-lane or the fused kernel; the keys are those of the latter."""
+    te, ctx = env
+    s = np.asarray(synth.workload_var10(T=T, seed=T)["series"], dtype=np.float32)
+    data = te.te_data_create(ctx, s)
+    jobs = []
+    for g in range(n_groups):
+        y = [(g % 10, g // 10 % 5)] + ([((g + 1) % 10, 5)] if g >= 50 else [])
+        z = [((g + 1 + d) % 10, 1 + d) for d in range(g % 6 if g % 6 < 5 else 0)]
+        jobs.append(te.Job(data, [((g + 7) % 10, 1 + g % 4)], y, z, k=4, max_lag=5, n_surr=S,
+                           seed=3, stream_tag=g % 3))
+    for a, (dx, dz, surr) in enumerate([(1, 2, 200), (1, 0, 200), (3, 0, 70), (4, 2, 12),
+                                        (16, 1, 9)]):
+        jobs.append(te.Job(data, [(a, 1 + d % 5) if d < 5 else (a + 1 + d % 4, 5) for d in range(dx)],
+                           [(a, 0)], Z[:dz], k=4, max_lag=5, n_surr=surr, seed=3))
+    got, ref = _both(te, ctx, jobs)
+    assert got == ref
+    data.close()
