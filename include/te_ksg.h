@@ -340,10 +340,13 @@ te_status te_ctx_set_trace(te_ctx *ctx, te_trace_fn fn, void *user);
 
 /* ---- execution options (tuning and measurement; the paper has no counterpart) --
  *
- * KSG estimates run on neighbour lists wherever a member's X values fit a
- * CTA's shared memory (dx * points up to about 41,000).  The member-lane
- * kernel serves the rest, and every estimate of a context in which one of its
- * own options (tile, members per lane, persistent, order) is set.
+ * KSG estimates run on neighbour lists where a member's X values fit a CTA's
+ * shared memory (dx * points up to about 41,000) and the lists are the faster
+ * path for the group's sizes.  The member-lane kernel serves the other groups, those
+ * whose data leave too many pairs beyond their lists (ties, heavy tails: found
+ * while the lists are walked, and then evaluated again), and every
+ * estimate of a context in which one of its own options (tile, members per
+ * lane, persistent, order) is set.
  *
  * te_ctx_set_option sets one option of a context for its later calls:
  *   TE_OPT_KSG_TILE              points per staged tile of the member-lane KSG
@@ -368,6 +371,9 @@ te_status te_ctx_set_trace(te_ctx *ctx, te_trace_fn fn, void *user);
  *                                prune by: 1 = Morton curve, 2 = k-d tree;
  *                                0 (default) = the k-d tree for groups of at
  *                                least 4096 members, the Morton curve below
+ *   TE_OPT_KSG_LISTS             1: neighbour lists for every group they can
+ *                                hold, none handed over; 0 (default): the
+ *                                faster path by the rule above
  * None of them changes a result.  Errors: TE_EINVAL for an unknown option or
  * value. */
 #define TE_OPT_KSG_TILE 1
@@ -375,6 +381,7 @@ te_status te_ctx_set_trace(te_ctx *ctx, te_trace_fn fn, void *user);
 #define TE_OPT_PERSISTENT 3
 #define TE_OPT_GRAPH 4
 #define TE_OPT_KSG_ORDER 5
+#define TE_OPT_KSG_LISTS 6
 te_status te_ctx_set_option(te_ctx *ctx, int32_t option, int64_t value);
 
 /* Counters of a context since its creation. */

@@ -81,9 +81,10 @@ class Context:
 
     def set_option(self, name: str, value: int):
         """Execution options (no change to any result): "ksg_tile" (64, 128,
-        256; 0 = neighbour lists), "ksg_members_per_lane" (1, 2; 0 = neighbour
-        lists), "persistent" (0/1), "graph" (0/1).  A forced tile, member count,
-        order or persistent grid takes the member-lane kernel."""
+        256; 0 = the tuning table), "ksg_members_per_lane" (1, 2; 0 = the tuning
+        table), "persistent" (0/1), "graph" (0/1), "ksg_order" (0..2),
+        "ksg_lists" (1 = wherever they fit).  A forced tile, member count, order
+        or persistent grid takes the member-lane kernel."""
         if name not in _abi.OPTIONS:
             raise ValueError(f"unknown option {name!r}; one of {sorted(_abi.OPTIONS)}")
         _check(self._h, self._lib.te_ctx_set_option(self._h, _abi.OPTIONS[name], int(value)))

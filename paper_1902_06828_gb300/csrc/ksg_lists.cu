@@ -216,6 +216,7 @@ __global__ void __launch_bounds__(kListBuildThreads) list_build_kernel(const Lis
     const int N = G.N, w = G.theiler, dy = G.dy, dz = G.dz, dyz = dy + dz;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int r0 = (int)(item - S.build_item) * Q, nq = S.nq;   // first row of the segment
+    const unsigned given_up = L.bad ? L.bad[S.group] : 0u;   // by the walk of an earlier launch
     const int i0 = S.q0 + r0;
     const int cap[2] = {G.cap_a, G.cap_b};
     for (int e = tid; e < Q * dyz; e += kListBuildThreads) {
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(kListBuildThreads) list_build_kernel(const Lis
         s_r[tid >> 1][tid & 1] = CUDART_INF_F;
         s_cnt[tid >> 1][tid & 1] = 0;
     }
+    if (given_up) return;
     __syncthreads();
     auto masked = [&](int q, int j) { return abs(j - (i0 + q)) <= w; };
     // per query [A sample | B sample], floats, in the entries' space
@@ -905,6 +907,8 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
     __shared__ uint32_t s_slow[kListWalkSmem / 4 / 32 + 1];
     __shared__ Aside s_aside[kAside];
     __shared__ int s_n_aside;
+    __shared__ unsigned s_given_up;
+    __shared__ int s_slow_limit;
     const long long item = blockIdx.x;
     const ListSeg &S = L.segs[last_at_or_below(L.n_segs, item,
                                                [&](int a) { return L.segs[a].walk_item; })];
@@ -927,6 +931,8 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
     float *coarse = xs + width * xn;
     const int nc = (N + 15) / 16;
     const bool xsorted = DXP == 1 && dz == 0;
+    unsigned given_up = 0;   // by another CTA
+    if (threadIdx.x == 0 && L.bad) given_up = *(volatile unsigned *)(L.bad + S.group);
 
     for (int m = 0; m < width; ++m) {
         // past the last member: the last one again, its results dropped
@@ -934,13 +940,14 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
         for (int d = 0; d < dx; ++d) {
             const float *src = Gr.base + L.cols[md.xcol + d];
             float *dst = xs + m * xn + d * sd;
+            bool finite = true;
 #pragma unroll 4
-            for (int j = threadIdx.x; j < N; j += blockDim.x)
-                dst[sp * (dz == 1 ? __ldg(Gr.rank + j) : j)] =
-                    __ldg(src + (md.perm ? __ldg(md.perm + j) : j));
-            if (L.nonfinite && !md.perm)   // a permutation has the original's values
-                for (int j = threadIdx.x; j < N; j += blockDim.x)
-                    if (!(fabsf(__ldg(src + j)) < CUDART_INF_F)) *L.nonfinite = 1;
+            for (int j = threadIdx.x; j < N; j += blockDim.x) {
+                const float v = __ldg(src + (md.perm ? __ldg(md.perm + j) : j));
+                dst[sp * (dz == 1 ? __ldg(Gr.rank + j) : j)] = v;
+                finite = finite && fabsf(v) < CUDART_INF_F;
+            }
+            if (!finite && L.nonfinite) *L.nonfinite = 1;
         }
         if (DXP > 2 && dx < DXP)   // the unused dimensions add nothing to a maximum
             for (int j = threadIdx.x; j < N; j += blockDim.x)
@@ -958,7 +965,11 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
     const int q_first = split * S.per_cta, q_last = min(S.nq, q_first + S.per_cta);
     const int n_words = (q_last - q_first) * width / 32 + 1;
     for (int a = threadIdx.x; a < n_words; a += blockDim.x) s_slow[a] = 0;
-    if (threadIdx.x == 0) s_n_aside = 0;
+    if (threadIdx.x == 0) {
+        s_n_aside = 0;
+        s_given_up = given_up;
+        s_slow_limit = L.bad ? list_slow_limit((q_last - q_first) * nm, N, dx) : 0x7fffffff;
+    }
     const char *xm = reinterpret_cast<const char *>(xs + gm * xn);
     // A pair's sum of digamma values: its group's lanes 0, 1, 2 sum those of
     // n_z, -n_xz and -n_yz (the low 32 bits and the rest apart, as the
@@ -967,6 +978,7 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
     long long sum_hi = 0, q_last_term = 0;
     unsigned evals = 0;   // member-pairs evaluated by the warp
     __syncthreads();
+    if (s_given_up) return;
 
     // the X values at byte offset o of the row x
     auto load_x = [&](const char *x, uint32_t o, float (&v)[XR]) {
@@ -1302,15 +1314,19 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
                 nxz = group_sum(c);
             }
         }
-        if (slow) {
-            if (u == 0 && live) {
+        if (__any_sync(kFull, slow)) {
+            bool give_up = false;
+            if (slow && u == 0 && live) {
                 const int bit = (row - q_first) * width + gm;
                 const int at = atomicAdd(&s_n_aside, 1);
                 if (at < kAside)
                     s_aside[at] = Aside{(uint32_t)bit | (eps > h.ra ? 0u : kExact), eps};
                 else
                     atomicOr(&s_slow[bit >> 5], 1u << (bit & 31));
+                give_up = at >= s_slow_limit;
             }
+            // the group's sums are not used: no further point
+            if (__any_sync(kFull, give_up)) first_row = q_last;
         }
         if (slow || !live) nz = nxz = nyz = -1;   // the digamma table's first value, 0
         add_term();
@@ -1338,6 +1354,15 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
     }
     // ---- pairs beyond the lists' radii: over all points, by the whole CTA ----
     __syncthreads();
+    if (s_n_aside > 32 && L.bad) {   // more than a batch of scans: are they still wanted?
+        if (threadIdx.x == 0) {
+            if (s_n_aside > s_slow_limit && atomicExch(L.bad + S.group, 1u) == 0u)
+                atomicAdd(L.n_bad, 1ull);
+            s_given_up = *(volatile unsigned *)(L.bad + S.group);
+        }
+        __syncthreads();
+        if (s_given_up) return;
+    }
     if (s_n_aside)
         scan_aside(L, Gr, s_col, s_aside, min(s_n_aside, kAside), q0 + q_first, width,
                    Gr.member_begin + mb * width, xs, xn, sp, sd,

@@ -78,11 +78,29 @@ struct ListLaunch {
     int *dbg_nxz, *dbg_nyz, *dbg_nz;
     int dbg_out;
     unsigned long long *work;   // as KsgLaunch::work [0], [1]; nullptr: not counted
+    // per group of the launch: set by a walking CTA that gives it up because more
+    // than its share of pairs (list_slow_limit) lies beyond the radii; n_bad:
+    // groups given up.  nullptr: none is.
+    unsigned *bad;
+    unsigned long long *n_bad;
     unsigned *nonfinite;        // set if a value is not finite; nullptr: checked by the caller
 };
 
 constexpr int kListBuildThreads = 512;
 constexpr int kListWalkThreads = 1024;   // of all walking CTAs on an SM
+
+// Pairs beyond the lists' radii that a walking CTA with `pairs` of them scans.
+// A scan visits every point twice: at N = 10^4 18 ns of the whole chip with two Z
+// variables, 36 with eight, against 1.15 and 1.55 a pair by the member-lane kernel
+// and 0.4 and 0.13 on lists, so the lists lose from 3% of such pairs on; at N =
+// 1000 the scan takes 2.3, the other kernel 0.45.  With several X variables that
+// is the fused kernel, 10 ns a pair.  A few dozen scans cost less than handing
+// the group over.
+__host__ __device__ inline int list_slow_limit(int pairs, int N, int dx)
+{
+    const float share = fminf(0.25f, dx == 1 ? 300.f / (float)N : 1.f);
+    return pairs < 256 ? 64 : max(64, (int)((float)pairs * share));
+}
 
 // capacities of the two lists for a group
 void list_caps(int N, int k, int dx, int dy, int dz, int *cap_a, int *cap_b);

@@ -118,6 +118,7 @@ te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &group
             .push_back(g);
 
     std::vector<ListGroup> lg;
+    std::vector<const HostGroup *> order;              // lg's groups
     std::vector<MemberDesc> mdesc;
     std::vector<std::pair<size_t, int>> msorted;       // (member, job)
     std::vector<int> cols;
@@ -208,6 +209,7 @@ te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &group
             }
             list_caps(N, g.k, g.dx, G.dy, G.dz, &G.cap_a, &G.cap_b);
             lg.push_back(G);
+            order.push_back(hg);
             const size_t row = list_row_bytes(G.cap_a, G.cap_b);
             for (int q0 = 0; q0 < N;) {
                 const size_t room = kListPoolBytes - std::min(kListPoolBytes, used + 256);
@@ -257,6 +259,7 @@ te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &group
     for (size_t a = 0; a < segs.size(); ++a)
         segs[a].rows = (unsigned char *)ctx->ws_lists.p + seg_off[a];
     for (auto &ms : msorted) mdesc[ms.first].xsorted = vjobs[ms.second].sorted;
+    const std::vector<unsigned> bad(lg.size(), 0);   // groups given up
     struct Table {
         const void *src;
         size_t bytes, at;
@@ -264,7 +267,8 @@ te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &group
                {segs.data(), segs.size() * sizeof(ListSeg), 0},
                {mdesc.data(), mdesc.size() * sizeof(MemberDesc), 0},
                {vjobs.data(), vjobs.size() * sizeof(RankSortJob), 0},
-               {cols.data(), cols.size() * sizeof(int), 0}};
+               {cols.data(), cols.size() * sizeof(int), 0},
+               {bad.data(), bad.size() * sizeof(unsigned), 0}};
     size_t bytes = 0;
     for (Table &t : tab) {
         t.at = bytes;
@@ -302,11 +306,19 @@ te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &group
     base.dbg_nz = dbg.nz;
     base.dbg_out = dbg.out;
     base.work = ctx->work_dev;
-    part.kernels = [ctx, plans, chunks, base]() -> te_status {
+    if (!ctx->opt_lists) {
+        base.bad = (unsigned *)(dtab + tab[5].at);
+        base.n_bad = ctx->work_dev + 4;
+        ctx->pend_bad = base.bad;
+        ctx->pend_lists = std::move(order);
+    }
+    part.kernels = [ctx, plans = std::move(plans), chunks = std::move(chunks),
+                    base]() -> te_status {
         for (const Chunk &ch : chunks) {
             const ClassPlan &cp = plans[ch.cls];
             ListLaunch L = base;
             L.groups += cp.first_group;
+            if (L.bad) L.bad += cp.first_group;
             L.segs += ch.first_seg;
             L.n_segs = ch.n_segs;
             CK(launch_list_build(L, ch.build_items, ch.queries, ch.cap_a, ch.cap_b, ctx->stream),

@@ -297,8 +297,12 @@ te_status run_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n_ou
 {
     te_status st = launch_groups(ctx, groups, n_out, dbg_out, dbg_eps, dbg_nxz, dbg_nyz, dbg_nz);
     if (st) return st;
+    if ((st = finish_groups(ctx)) || !groups_given_up(ctx)) return st;
+    if ((st = relaunch_given_up(ctx, n_out, dbg_out, dbg_eps, dbg_nxz, dbg_nyz, dbg_nz))) return st;
     return finish_groups(ctx);
 }
+
+bool groups_given_up(const te_ctx *ctx) { return ctx->pend_bad && ctx->work_host[4]; }
 
 te_status finish_groups(te_ctx *ctx)
 {
@@ -312,6 +316,10 @@ te_status finish_groups(te_ctx *ctx)
     ctx->stats.ksg_ops += ctx->work_host[1];
     ctx->stats.estimates += ctx->pend_members;
     ctx->pend_timed = 0;
+    if (ctx->pend_bad && !ctx->work_host[4]) {
+        ctx->pend_bad = nullptr;
+        ctx->pend_lists.clear();
+    }
     if (ctx->work_host[2])
         return fail(ctx, TE_ETIMEOUT, "a KSG tile copy did not complete in time");
     return TE_OK;
@@ -342,10 +350,48 @@ te_status submit_work(te_ctx *ctx, const std::function<te_status()> &work)
     return TE_OK;
 }
 
+// Queue the groups, each on its path, and the keys of all slots.
+static te_status launch_paths(te_ctx *ctx, const std::vector<const HostGroup *> &by_lists,
+                              const std::vector<const HostGroup *> &by_lanes, int n_out,
+                              const KsgDebug &dbg)
+{
+    te_status st;
+    ctx->pend_timed = 0;
+    ctx->pend_bad = nullptr;
+    ctx->pend_lists.clear();
+    KsgPart lanes, lists;
+    if (!by_lanes.empty() && (st = prepare_lanes(ctx, by_lanes, dbg, lanes))) return st;
+    if (!by_lists.empty() && (st = prepare_lists(ctx, by_lists, dbg, lists))) return st;
+    const bool graph = ctx->opt_graph != 0;
+    auto device_work = [&]() -> te_status {
+        te_status st;
+        CK(cudaMemsetAsync(ctx->work_dev, 0, 5 * sizeof(unsigned long long), ctx->stream),
+           "cudaMemsetAsync");
+        for (const KsgPart *p : {&lanes, &lists})
+            if (p->before && (st = p->before())) return st;
+        if (!graph) CK(cudaEventRecord(ctx->ev_a, ctx->stream), "cudaEventRecord");
+        for (const KsgPart *p : {&lanes, &lists})
+            if (p->kernels && (st = p->kernels())) return st;
+        if (!graph) CK(cudaEventRecord(ctx->ev_b, ctx->stream), "cudaEventRecord");
+        CK(copy_d2h(ctx, ctx->work_host, ctx->work_dev, 5 * sizeof(unsigned long long)),
+           "cudaMemcpyAsync");
+        CK(launch_finalize((const unsigned long long *)ctx->ws_acc.p, (long long *)ctx->ws_keys.p,
+                           n_out, ctx->stream),
+           "finalize launch");
+        ctx->stats.launches++;
+        return TE_OK;
+    };
+    if ((st = submit_work(ctx, device_work))) return st;
+    if (!lanes.members && !lists.members) return TE_OK;
+    ctx->pend_timed = 1;
+    ctx->pend_pair_evals = lanes.pair_evals + lists.pair_evals;
+    ctx->pend_members = lanes.members + lists.members;
+    return TE_OK;
+}
+
 te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n_out, int dbg_out,
                         float *dbg_eps, int *dbg_nxz, int *dbg_nyz, int *dbg_nz)
 {
-    ctx->pend_timed = 0;
     te_status st;
     int max_N = 0;
     for (const HostGroup &g : groups) max_N = std::max(max_N, g.data->T - g.max_lag);
@@ -371,36 +417,37 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
         if (g.members.empty()) continue;
         const ListCall c{g.data->T - g.max_lag, g.k, g.theiler, g.dx, (int)g.y.size(),
                          (int)g.z.size(), g.members.size()};
-        (!lane_only && list_serves(c, n_groups, rows, pairs) ? by_lists : by_lanes).push_back(&g);
+        const bool lists = !lane_only && (ctx->opt_lists ? list_fits(c.N, c.dx, c.dz, c.k)
+                                                         : list_serves(c, n_groups, rows, pairs));
+        (lists ? by_lists : by_lanes).push_back(&g);
     }
-    KsgPart lanes, lists;
-    if (!by_lanes.empty() && (st = prepare_lanes(ctx, by_lanes, dbg, lanes))) return st;
-    if (!by_lists.empty() && (st = prepare_lists(ctx, by_lists, dbg, lists))) return st;
-    const bool graph = ctx->opt_graph != 0;
-    auto device_work = [&]() -> te_status {
-        te_status st;
-        CK(cudaMemsetAsync(ctx->work_dev, 0, 3 * sizeof(unsigned long long), ctx->stream),
+    return launch_paths(ctx, by_lists, by_lanes, n_out, dbg);
+}
+
+te_status relaunch_given_up(te_ctx *ctx, int n_out, int dbg_out, float *dbg_eps, int *dbg_nxz,
+                            int *dbg_nyz, int *dbg_nz)
+{
+    std::vector<unsigned> bad(ctx->pend_lists.size());
+    CK(copy_d2h(ctx, bad.data(), ctx->pend_bad, bad.size() * sizeof(unsigned)), "cudaMemcpyAsync");
+    CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+    std::vector<const HostGroup *> again;
+    std::vector<int> out;
+    for (size_t a = 0; a < bad.size(); ++a) {
+        if (!bad[a]) continue;
+        again.push_back(ctx->pend_lists[a]);
+        for (const HostMember &m : ctx->pend_lists[a]->members) out.push_back(m.out);
+    }
+    // their sums start anew, run by run of slots; the other groups' stand
+    std::sort(out.begin(), out.end());
+    for (size_t a = 0, b; a < out.size(); a = b) {
+        for (b = a + 1; b < out.size() && out[b] == out[b - 1] + 1;) ++b;
+        CK(cudaMemsetAsync((char *)ctx->ws_acc.p + (size_t)out[a] * 16, 0, (b - a) * 16, ctx->stream),
            "cudaMemsetAsync");
-        for (const KsgPart *p : {&lanes, &lists})
-            if (p->before && (st = p->before())) return st;
-        if (!graph) CK(cudaEventRecord(ctx->ev_a, ctx->stream), "cudaEventRecord");
-        for (const KsgPart *p : {&lanes, &lists})
-            if (p->kernels && (st = p->kernels())) return st;
-        if (!graph) CK(cudaEventRecord(ctx->ev_b, ctx->stream), "cudaEventRecord");
-        CK(copy_d2h(ctx, ctx->work_host, ctx->work_dev, 3 * sizeof(unsigned long long)),
-           "cudaMemcpyAsync");
-        CK(launch_finalize((const unsigned long long *)ctx->ws_acc.p, (long long *)ctx->ws_keys.p,
-                           n_out, ctx->stream),
-           "finalize launch");
-        ctx->stats.launches++;
-        return TE_OK;
-    };
-    if ((st = submit_work(ctx, device_work))) return st;
-    if (!lanes.members && !lists.members) return TE_OK;
-    ctx->pend_timed = 1;
-    ctx->pend_pair_evals = lanes.pair_evals + lists.pair_evals;
-    ctx->pend_members = lanes.members + lists.members;
-    return TE_OK;
+    }
+    const te_status st = launch_paths(ctx, {}, again, n_out,
+                                      KsgDebug{dbg_out, dbg_eps, dbg_nxz, dbg_nyz, dbg_nz});
+    ctx->pend_pair_evals = ctx->pend_members = 0;   // counted with the first launch
+    return st;
 }
 
 te_status prepare_lanes(te_ctx *ctx, const std::vector<const HostGroup *> &groups,
@@ -767,7 +814,7 @@ te_status prepare_lanes(te_ctx *ctx, const std::vector<const HostGroup *> &group
         }
         return TE_OK;
     };
-    part.kernels = [ctx, plans, dbg]() -> te_status {
+    part.kernels = [ctx, plans = std::move(plans), dbg]() -> te_status {
         for (const Plan &p : plans) {
             KsgLaunch L{};
             L.groups = (const GroupDesc *)ctx->ws_groups.p + p.g_off;
@@ -843,8 +890,8 @@ te_status te_ctx_create(int device, te_ctx **out)
     if (cudaSetDevice(device) != cudaSuccess ||
         cudaStreamCreateWithFlags(&ctx->own_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&ctx->ev_a) != cudaSuccess || cudaEventCreate(&ctx->ev_b) != cudaSuccess ||
-        cudaMalloc(&ctx->work_dev, 4 * sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMallocHost(&ctx->work_host, 3 * sizeof(unsigned long long)) != cudaSuccess) {
+        cudaMalloc(&ctx->work_dev, 5 * sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMallocHost(&ctx->work_host, 5 * sizeof(unsigned long long)) != cudaSuccess) {
         te_ctx_destroy(ctx);
         return TE_ECUDA;
     }
@@ -869,8 +916,11 @@ te_status te_ctx_set_option(te_ctx *ctx, int32_t option, int64_t value)
         return TE_OK;
     case TE_OPT_PERSISTENT:
     case TE_OPT_GRAPH:
+    case TE_OPT_KSG_LISTS:
         if (value != 0 && value != 1) return fail(ctx, TE_EINVAL, "the option takes 0 or 1");
-        (option == TE_OPT_PERSISTENT ? ctx->opt_persistent : ctx->opt_graph) = (int)value;
+        (option == TE_OPT_PERSISTENT ? ctx->opt_persistent
+         : option == TE_OPT_GRAPH    ? ctx->opt_graph
+                                     : ctx->opt_lists) = (int)value;
         return TE_OK;
     case TE_OPT_KSG_ORDER:
         if (value < 0 || value > 2) return fail(ctx, TE_EINVAL, "the order option takes 0, 1 or 2");
@@ -1038,7 +1088,8 @@ static te_status cmi_common(te_ctx *ctx, const te_data *data, const te_var *x, i
     CK(launch_perms(perm, N, N, p->seed, p->stream_tag, 0, 0, 1, S, ctx->stream),
        "permutation launch");
     if (S > 0) ctx->stats.launches++;
-    HostGroup g;
+    std::vector<HostGroup> gs(1);
+    HostGroup &g = gs[0];
     g.data = data;
     g.max_lag = p->max_lag;
     g.k = p->k;
@@ -1047,9 +1098,9 @@ static te_status cmi_common(te_ctx *ctx, const te_data *data, const te_var *x, i
     if (dz) g.z.assign(z, z + dz);
     g.dx = dx;
     g.xvars.assign(x, x + dx);
+    g.members.reserve(S + 1);
     for (int s = 0; s <= S; ++s)
         g.members.push_back(HostMember{0, s == 0 ? nullptr : perm + (size_t)(s - 1) * N, s});
-    std::vector<HostGroup> gs{g};
     float *d_eps = nullptr;
     int *d_cnt = nullptr;
     if (dbg_member >= 0) {

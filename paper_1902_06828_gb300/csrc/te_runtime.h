@@ -136,10 +136,14 @@ struct te_ctx {
     // counters of the launch in flight, added to stats by finish_groups
     int pend_timed = 0;
     uint64_t pend_pair_evals = 0, pend_members = 0;
+    // its groups on lists and, on the device, which of them were given up
+    std::vector<const teksg::HostGroup *> pend_lists;
+    const unsigned *pend_bad = nullptr;
     struct te_server *server = nullptr;   // serving state (te_serve_*), created on demand
     std::mutex serve_start_mu;
     unsigned long long *work_dev = nullptr;   // KSG kernel work counters [2], error flag [1],
-                                              // persistent-grid item counter [1]
+                                              // persistent-grid item counter [1], groups that
+                                              // the list walk gave up [1]
     unsigned long long *work_host = nullptr;  // pinned copy
     cudaEvent_t ev_a = nullptr, ev_b = nullptr;
     // second stream for work that overlaps the context's stream (created on
@@ -152,7 +156,8 @@ struct te_ctx {
     void *trace_user = nullptr;
     // te_ctx_set_option: forced member-lane tile / members per lane (0 = the
     // tuning table), persistent member-lane grids, batches captured as graphs
-    int opt_jt = 0, opt_ms = 0, opt_persistent = 0, opt_graph = 0, opt_order = 0;
+    int opt_jt = 0, opt_ms = 0, opt_persistent = 0, opt_graph = 0, opt_order = 0,
+        opt_lists = 0;
 };
 
 namespace teksg {
@@ -204,6 +209,12 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
                         int dbg_out = -1, float *dbg_eps = nullptr, int *dbg_nxz = nullptr,
                         int *dbg_nyz = nullptr, int *dbg_nz = nullptr);
 te_status finish_groups(te_ctx *ctx);
+// After finish_groups: whether the list walk gave up some of the launch's
+// groups, and their evaluation by the member-lane kernel, queued like
+// launch_groups (which took the same groups, still in place; finish_groups follows).
+bool groups_given_up(const te_ctx *ctx);
+te_status relaunch_given_up(te_ctx *ctx, int n_out, int dbg_out = -1, float *dbg_eps = nullptr,
+                            int *dbg_nxz = nullptr, int *dbg_nyz = nullptr, int *dbg_nz = nullptr);
 // A launch's groups on one path: what precedes the timed kernels (orders,
 // sorted columns) and the kernels themselves, to be called on ctx->stream (or
 // under capture) once the tables are uploaded, which prepare_* has done.

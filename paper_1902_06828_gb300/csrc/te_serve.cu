@@ -51,6 +51,7 @@ struct Slot {
     bool busy = false;
     cudaEvent_t done = nullptr;
     std::vector<ServeJob *> jobs;
+    std::vector<HostGroup> groups;   // of the batch in flight
     std::vector<int> out0;
     int n_out = 0;
     int64_t *keys_pin = nullptr;
@@ -91,6 +92,26 @@ struct te_server {
 
 namespace {
 
+// Queue the copy of a queued batch's keys and the event after it.
+te_status queue_keys(Slot &sl)
+{
+    te_ctx *ctx = sl.ctx;
+    const size_t bytes = (size_t)sl.n_out * 16;
+    if (bytes > sl.keys_cap) {
+        if (sl.keys_pin) {
+            CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+            CK(cudaFreeHost(sl.keys_pin), "cudaFreeHost");
+            sl.keys_pin = nullptr;
+        }
+        const size_t want = std::max(bytes, sl.keys_cap * 2);
+        CK(cudaMallocHost(&sl.keys_pin, want), "cudaMallocHost");
+        sl.keys_cap = want;
+    }
+    CK(copy_d2h(ctx, sl.keys_pin, ctx->ws_keys.p, bytes), "cudaMemcpyAsync");
+    CK(cudaEventRecord(sl.done, ctx->stream), "cudaEventRecord");
+    return TE_OK;
+}
+
 // Build and queue one batch on the slot's stream (no host wait).
 te_status launch_batch(Slot &sl)
 {
@@ -122,7 +143,8 @@ te_status launch_batch(Slot &sl)
         ctx->stats.launches++;
     }
     std::map<std::vector<long long>, int> gid;
-    std::vector<HostGroup> groups;
+    std::vector<HostGroup> &groups = sl.groups;
+    groups.clear();
     for (size_t a = 0; a < sl.jobs.size(); ++a) {
         ServeJob *j = sl.jobs[a];
         std::vector<long long> key{(long long)(uintptr_t)j->data, j->p.max_lag, j->p.k,
@@ -155,19 +177,7 @@ te_status launch_batch(Slot &sl)
             hg.members.push_back(HostMember{xfirst, sets.perm(set[a], s), sl.out0[a] + s});
     }
     if ((st = launch_groups(ctx, groups, n_out))) return st;
-    if ((size_t)n_out * 16 > sl.keys_cap) {
-        if (sl.keys_pin) {
-            CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
-            CK(cudaFreeHost(sl.keys_pin), "cudaFreeHost");
-            sl.keys_pin = nullptr;
-        }
-        const size_t want = std::max((size_t)n_out * 16, sl.keys_cap * 2);
-        CK(cudaMallocHost(&sl.keys_pin, want), "cudaMallocHost");
-        sl.keys_cap = want;
-    }
-    CK(copy_d2h(ctx, sl.keys_pin, ctx->ws_keys.p, (size_t)n_out * 16), "cudaMemcpyAsync");
-    CK(cudaEventRecord(sl.done, ctx->stream), "cudaEventRecord");
-    return TE_OK;
+    return queue_keys(sl);
 }
 
 void serve_loop(te_server *S)
@@ -182,8 +192,18 @@ void serve_loop(te_server *S)
             const cudaError_t q = cudaEventQuery(sl.done);
             if (q == cudaErrorNotReady) continue;
             lk.unlock();
-            const te_status fst = q == cudaSuccess ? finish_groups(sl.ctx) : TE_ECUDA;
+            te_status fst = q == cudaSuccess ? finish_groups(sl.ctx) : TE_ECUDA;
+            bool again = fst == TE_OK && groups_given_up(sl.ctx);
+            if (again) {   // those groups by the member-lane kernel: the slot stays busy
+                fst = relaunch_given_up(sl.ctx, sl.n_out);
+                if (fst == TE_OK) fst = queue_keys(sl);
+                again = fst == TE_OK;
+            }
             lk.lock();
+            if (again) {
+                progressed = true;
+                continue;
+            }
             for (size_t a = 0; a < sl.jobs.size(); ++a) {
                 ServeJob *j = sl.jobs[a];
                 if (j->cancel_requested) {

@@ -54,7 +54,8 @@ unsigned char g_desc_host[sizeof(GroupDesc) + (kStaticMaxSurr + 1) * sizeof(Memb
                           4 * TE_MAX_DIMS + 64];
 constexpr int kStaticMaxSegs = 64;   // pieces of the points whose lists are in the scratch at once
 struct StaticListTables {
-    unsigned nonfinite, pad[3];   // set by the kernels, read back with the keys before it
+    unsigned nonfinite, bad;      // set by the kernels, read back with the keys before it
+    unsigned long long n_bad;
     ListGroup group;
     RankSortJob sort;
     ListSeg segs[kStaticMaxSegs];
@@ -182,9 +183,7 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
     const int qsz = dx1 ? kLaneQueries : 128;
     int jt = 0;
     size_t smem = 0;
-    if (lists) {
-        // no tile
-    } else if (dx1) {
+    if (dx1) {
         jt = 256;
         if (N < jt) jt = std::max(64, (N + 63) & ~63);
         smem = ksg_lane_smem_bytes(dy + dz, jt);
@@ -196,7 +195,7 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
             room_t = 190 * 1024 - 4LL * rows_q * 128 - 64 - 8 * 8 * 128;
             jt = (int)std::min<long long>((room_t / (4LL * rows_t + 8)) & ~7LL, 2048);
         }
-        if (jt < 8) return TE_EINVAL;
+        if (jt < 8 && !lists) return TE_EINVAL;
         jt = std::min(jt, (N + 7) & ~7);
         smem = ksg_smem_bytes(rows_t, rows_q, jt, 128);
     }
@@ -236,9 +235,36 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
         cudaMemsetAsync(acc, 0, (size_t)(S + 1) * 16, stream) != cudaSuccess)
         return TE_ECUDA;
 
+    auto run_lanes = [&]() -> bool {
+        if (cudaMemcpyAsync(sc + grp_off, h, sizeof(GroupDesc), cudaMemcpyHostToDevice, stream) !=
+            cudaSuccess)
+            return false;
+        KsgLaunch L{};
+        L.groups = (const GroupDesc *)(sc + grp_off);
+        L.n_groups = 1;
+        L.members = (const MemberDesc *)(sc + mem_off);
+        L.cols = (const int *)(sc + col_off);
+        L.q = q;
+        L.acc = acc;
+        L.dbg_out = -1;
+        L.jt = jt;
+        L.work = nullptr;
+        const long long items = (long long)gd.n_qtiles * gd.n_mblocks;
+        return launch_ksg(L, v, items, dx1, smem, stream) == cudaSuccess;
+    };
+    // the keys, and with lists the flags at most 256 bytes behind them: one copy
+    const size_t flag_at = tab_off - key_off;
+    auto read_keys = [&](size_t bytes) -> bool {
+        return launch_finalize(acc, keys, S + 1, stream) == cudaSuccess &&
+               cudaMemcpyAsync(g_keys_host, keys, bytes, cudaMemcpyDeviceToHost, stream) ==
+                   cudaSuccess &&
+               cudaStreamSynchronize(stream) == cudaSuccess;
+    };
+    bool lanes = !lists;
     if (lists) {
         StaticListTables &t = g_tables_host;
-        t.nonfinite = 0;
+        t.nonfinite = t.bad = 0;
+        t.n_bad = 0;
         lg.base = series_dev;
         lg.N = N;
         lg.k = p->k;
@@ -287,41 +313,26 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
             L.q = q;
             L.acc = acc;
             L.dbg_out = -1;
-            L.nonfinite = (unsigned *)(sc + tab_off);
+            L.nonfinite = (unsigned *)&dt->nonfinite;
+            if (jt >= 8) {   // the other kernel can take over
+                L.bad = (unsigned *)&dt->bad;
+                L.n_bad = (unsigned long long *)&dt->n_bad;
+            }
             if (launch_list_build(L, (t.segs[a].nq + queries - 1) / queries, queries, lg.cap_a,
                                   lg.cap_b, stream) != cudaSuccess ||
                 launch_list_walk(L, (long long)t.segs[a].n_splits * lg.n_mblocks, shape, xbytes,
                                  stream) != cudaSuccess)
                 return TE_ECUDA;
         }
-    } else {
-        if (cudaMemcpyAsync(sc + grp_off, h, sizeof(GroupDesc), cudaMemcpyHostToDevice, stream) !=
-            cudaSuccess)
+        if (!read_keys(flag_at + 16)) return TE_ECUDA;
+        unsigned flags[2];   // nonfinite, bad
+        std::memcpy(flags, g_keys_host + flag_at, sizeof flags);
+        if (flags[0]) return TE_EINVAL;
+        lanes = flags[1] != 0;   // too many pairs beyond the lists: evaluated anew
+        if (lanes && cudaMemsetAsync(acc, 0, (size_t)(S + 1) * 16, stream) != cudaSuccess)
             return TE_ECUDA;
-        KsgLaunch L{};
-        L.groups = (const GroupDesc *)(sc + grp_off);
-        L.n_groups = 1;
-        L.members = (const MemberDesc *)(sc + mem_off);
-        L.cols = (const int *)(sc + col_off);
-        L.q = q;
-        L.acc = acc;
-        L.dbg_out = -1;
-        L.jt = jt;
-        L.work = nullptr;
-        const long long items = (long long)gd.n_qtiles * gd.n_mblocks;
-        if (launch_ksg(L, v, items, dx1, smem, stream) != cudaSuccess) return TE_ECUDA;
     }
-    if (launch_finalize(acc, keys, S + 1, stream) != cudaSuccess) return TE_ECUDA;
-
-    // with lists the flag lies at most 256 bytes behind the keys: one copy
-    const size_t flag_at = tab_off - key_off;
-    if (cudaMemcpyAsync(g_keys_host, keys, lists ? flag_at + 16 : (size_t)(S + 1) * 16,
-                        cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
-        cudaStreamSynchronize(stream) != cudaSuccess)
-        return TE_ECUDA;
-    unsigned nonfinite = 0;
-    if (lists) std::memcpy(&nonfinite, g_keys_host + flag_at, sizeof nonfinite);
-    if (nonfinite) return TE_EINVAL;
+    if (lanes && (!run_lanes() || !read_keys((size_t)(S + 1) * 16))) return TE_ECUDA;
     const int64_t *kh = (const int64_t *)g_keys_host;
     if (out_key) std::memcpy(out_key, kh, (size_t)(S + 1) * 16);
     const double psi_k = std::ldexp((double)g_q_host[p->k], -52);

@@ -247,3 +247,78 @@ def test_batches_whose_groups_take_both_paths(env, T, n_groups, S):
     got, ref = _both(te, ctx, jobs)
     assert got == ref
     data.close()
+
+
+def _series(kind, T, seed=0):
+    rng = np.random.default_rng(seed)
+    if kind == "cauchy":
+        s = rng.standard_cauchy(size=(10, T))
+    elif kind == "ties":
+        s = np.clip(np.round(rng.standard_cauchy(size=(10, T)) * 7 / 20), -7, 7)
+    elif kind == "binary":
+        s = rng.integers(0, 2, size=(10, T))
+    else:   # most values zero
+        s = np.where(rng.random((10, T)) < 0.7, 0.0, rng.exponential(size=(10, T)))
+    return np.asarray(s, dtype=np.float32)
+
+
+@pytest.mark.parametrize("kind,T,dz,dx,k,w,S", [
+    ("cauchy", 38, 2, 1, 4, 0, 2), ("cauchy", 1500, 2, 1, 4, 0, 33), ("cauchy", 1500, 3, 2, 4, 5, 9),
+    ("cauchy", 1500, 1, 4, 16, 0, 9), ("ties", 2600, 2, 1, 4, 0, 400), ("binary", 2600, 0, 1, 4, 0, 9),
+    ("binary", 1200, 8, 1, 4, 0, 60), ("binary", 1200, 8, 3, 4, 0, 9), ("zero", 2600, 1, 1, 4, 2, 40),
+    ("zero", 1200, 0, 2, 9, 0, 9)])
+def test_pairs_beyond_the_radii_scanned_or_handed_over(env, kind, T, dz, dx, k, w, S):
+    """Data that leave many pairs beyond their lists: scanned by the walk when
+    nothing is handed over, otherwise given up and evaluated anew; one call,
+    its per-point values, a batch beside ordinary groups, and as a graph."""
+    te, ctx = env
+    data = te.te_data_create(ctx, _series(kind, T))
+    plain = te.te_data_create(ctx, synth.workload_var10(T=T, seed=3)["series"])
+    x, kw = [(2, 1 + a) for a in range(dx)], dict(k=k, theiler=w, max_lag=5, seed=3)
+    jobs = [te.Job(data, x, [(0, 0)], Z[:dz], n_surr=S, **kw),
+            te.Job(plain, [(3, 1)], [(0, 0)], Z[:2], n_surr=7, **kw),
+            te.Job(data, [(1, 2)], [(0, 0)], [(5, 1), (6, 2), (7, 3)], n_surr=2, **kw)]
+    got, ref = _both(te, ctx, jobs)
+    assert got == ref
+    one = te.cmi_ksg(ctx, data, x, [(0, 0)], Z[:dz], n_surr=S, return_keys=True, **kw)[1]
+    assert one == ref[0]
+    dbg = te.cmi_ksg_debug(ctx, data, x, [(0, 0)], Z[:dz], n_surr=S, member=S // 2, **kw)
+    try:
+        for name in ("ksg_lists", "graph"):
+            ctx.set_option(name, 1)
+            assert te.cmi_ksg_batch(ctx, jobs, return_keys=True)[1] == ref
+            if name == "ksg_lists":   # the scans' own per-point values
+                own = te.cmi_ksg_debug(ctx, data, x, [(0, 0)], Z[:dz], n_surr=S, member=S // 2, **kw)
+            ctx.set_option(name, 0)
+    finally:
+        ctx.set_option("ksg_lists", 0)
+        ctx.set_option("graph", 0)
+    for name in ("eps", "n_xz", "n_yz") + (("n_z",) if dz else ()):
+        np.testing.assert_array_equal(dbg[name], own[name])
+    data.close()
+    plain.close()
+
+
+@pytest.mark.parametrize("kind,T,dz,S", [("zero", 2600, 1, 90), ("binary", 1200, 8, 60),
+                                         ("cauchy", 2600, 8, 90)])
+def test_served_and_allocation_free_calls_hand_over(env, kind, T, dz, S):
+    """Groups that the list walk gives up, in served batches beside others and
+    in the allocation-free call: keys as everywhere."""
+    torch = pytest.importorskip("torch")
+    te, ctx = env
+    s = _series(kind, T)
+    data = te.te_data_create(ctx, s)
+    plain = te.te_data_create(ctx, synth.workload_var10(T=T, seed=3)["series"])
+    jobs = [te.Job(d, [(2 + a, 1)], [(0, 0)], Z[:dz], k=4, max_lag=5, n_surr=S, seed=a)
+            for a in range(3) for d in (data, plain)]
+    _, ref = _both(te, ctx, jobs)
+    for _ in range(2):
+        tickets = [te.te_serve_submit(ctx, j) for j in jobs]
+        for t, j, r in zip(tickets, jobs, ref):
+            assert te.te_serve_poll(ctx, t, j.n_surr, return_keys=True)[1] == r
+    te.te_serve_stop(ctx)
+    got = te.cmi_ksg_static(torch.from_numpy(s).cuda(), jobs[0].x, [(0, 0)], Z[:dz], k=4,
+                            max_lag=5, n_surr=S, seed=0, return_keys=True)[1]
+    assert got == ref[0]
+    data.close()
+    plain.close()
