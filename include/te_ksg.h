@@ -411,7 +411,11 @@ te_status te_get_stats(const te_ctx *ctx, te_stats *out);
  * Jobs (te_cmi_job, as for cmi_ksg_batch) are submitted from any host thread
  * and evaluated by a scheduler thread of the context.  Pending jobs are
  * admitted in arrival order while the device memory of the admitted jobs stays
- * within hbm_budget_bytes; each admitted set is fused into one batch, and up to
+ * within hbm_budget_bytes, the neighbour lists of their batches included: a
+ * batch's lists take a share of what its jobs leave of the budget, at most 256 MiB
+ * and their tables, and a batch that is left too little runs without lists
+ * (lists that an idle batch slot keeps are given back where they would not fit).
+ * Each admitted set is fused into one batch, and up to
  * max_inflight batches run on the device at once, each on its own stream.
  * Jobs submitted while batches run join the next batch.  A job's result does
  * not depend on the batch it lands in (exact keys), so it equals cmi_ksg's.
@@ -430,7 +434,7 @@ typedef struct {
 
 typedef struct {
     uint64_t submitted, completed, cancelled, batches;
-    size_t in_use_bytes, peak_bytes;   /* admitted footprint now / at most */
+    size_t in_use_bytes, peak_bytes;   /* admitted footprint and lists now / at most */
     uint64_t pending;                  /* jobs waiting for admission */
 } te_serve_stats;
 

@@ -126,6 +126,13 @@ struct ListCall {
     size_t members;
 };
 bool list_serves(const ListCall &c, int n_groups, long long rows, long long pairs);
+size_t list_bytes(const ListCall &c);   // of the group's lists, all in the pool
+// A batch whose lists do not all fit the pool needs this much of it: smaller
+// pieces leave the chip idle at the end of each. Member lanes / lists with
+// 64, 32 and 16 MiB, ms: 40 groups of 201 members, N = 10^4, two Z variables 128 /
+// 120, 163, 247 (one group 5.9 / 3.2, 4.3, 6.3; 45 candidates 102 / 40, 45, 55),
+// N = 3000 20.6 / 16.3, 19.8, 26.2; one group of 41 3.0 / 2.1, 2.9, 4.3.
+constexpr size_t kListPoolLeast = (size_t)64 << 20;
 // whether a group can take the list path
 bool list_fits(int N, int dx, int dz, int k);
 // Parts into which the walk splits the points of a launch, given its member

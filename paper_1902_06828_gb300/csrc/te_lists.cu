@@ -1,6 +1,6 @@
 // Host plan of the neighbour-list path (ksg_lists.cu): every group of a batch
-// in a few launches, with the lists of at most kListPoolBytes of query points
-// in device memory at a time.
+// in a few launches, with at most ctx->list_pool bytes of lists in device memory
+// at a time.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -17,10 +17,6 @@
 namespace teksg {
 
 namespace {
-
-// Lists in device memory at once: enough points to fill the chip several
-// times over at the longest lists (48 KB a point), small beside the X values.
-constexpr size_t kListPoolBytes = (size_t)256 << 20;
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
@@ -102,6 +98,13 @@ bool list_serves(const ListCall &c, int n_groups, long long rows, long long pair
     default:
         return !(full && m <= 32 && n_groups >= 200 && N <= 700);
     }
+}
+
+size_t list_bytes(const ListCall &c)
+{
+    int cap_a, cap_b;
+    list_caps(c.N, c.k, c.dx, c.dy, c.dz, &cap_a, &cap_b);
+    return (size_t)c.N * list_row_bytes(cap_a, cap_b) + 512;   // a piece begins at 256 bytes
 }
 
 te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &groups,
@@ -212,7 +215,7 @@ te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &group
             order.push_back(hg);
             const size_t row = list_row_bytes(G.cap_a, G.cap_b);
             for (int q0 = 0; q0 < N;) {
-                const size_t room = kListPoolBytes - std::min(kListPoolBytes, used + 256);
+                const size_t room = ctx->list_pool - std::min(ctx->list_pool, used + 256);
                 int nq = (int)std::min<size_t>((size_t)(N - q0), room / row);
                 if (nq < N - q0) nq &= ~31;
                 if (nq <= 0) {
@@ -242,7 +245,7 @@ te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &group
         plans.push_back(cp);
     }
     // workspaces, then the pointers into them, then one upload of all tables
-    if ((st = ensure_dev(ctx, ctx->ws_lists, pool))) return st;
+    if ((st = ensure_dev(ctx, ctx->ws_lists, pool, ctx->list_pool))) return st;
     if (vs_words && (st = ensure_dev(ctx, ctx->ws_lsort, vs_words * 4))) return st;
     int vitems = 0;
     for (size_t a = 0; a < vjobs.size(); ++a) {

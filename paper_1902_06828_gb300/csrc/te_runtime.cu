@@ -47,18 +47,28 @@ cudaError_t copy_d2h(te_ctx *ctx, void *dst, const void *src, size_t bytes)
     return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, ctx->stream);
 }
 
-te_status ensure_dev(te_ctx *ctx, DevBuf &b, size_t bytes)
+te_status free_dev(te_ctx *ctx, DevBuf &b)
+{
+    if (!b.p) return TE_OK;
+    CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+    CK(cudaFree(b.p), "cudaFree");
+    b.p = nullptr;
+    b.cap = 0;
+    return TE_OK;
+}
+
+te_status ensure_dev(te_ctx *ctx, DevBuf &b, size_t bytes, size_t most)
 {
     if (bytes <= b.cap) return TE_OK;
-    size_t want = std::max(bytes, b.cap + b.cap / 2);
+    size_t want = std::max(bytes, std::min(b.cap + b.cap / 2, most));
     want = (want + 255) & ~(size_t)255;
-    if (b.p) {
-        CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
-        CK(cudaFree(b.p), "cudaFree");
-        b.p = nullptr;
-        b.cap = 0;
-    }
-    CK(cudaMalloc(&b.p, want), "cudaMalloc");
+    te_status st = free_dev(ctx, b);
+    if (st) return st;
+    void *p = nullptr;
+    const cudaError_t e = cudaMalloc(&p, want);
+    if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();   // not the next launch's error
+    CK(e, "cudaMalloc");
+    b.p = p;
     b.cap = want;
     return TE_OK;
 }
@@ -352,7 +362,7 @@ te_status submit_work(te_ctx *ctx, const std::function<te_status()> &work)
 
 // Queue the groups, each on its path, and the keys of all slots.
 static te_status launch_paths(te_ctx *ctx, const std::vector<const HostGroup *> &by_lists,
-                              const std::vector<const HostGroup *> &by_lanes, int n_out,
+                              std::vector<const HostGroup *> by_lanes, int n_out,
                               const KsgDebug &dbg)
 {
     te_status st;
@@ -360,8 +370,13 @@ static te_status launch_paths(te_ctx *ctx, const std::vector<const HostGroup *> 
     ctx->pend_bad = nullptr;
     ctx->pend_lists.clear();
     KsgPart lanes, lists;
+    if (!by_lists.empty()) {
+        st = prepare_lists(ctx, by_lists, dbg, lists);
+        if (st && st != TE_ENOMEM) return st;
+        // no memory for the lists: the member lanes do without
+        if (st) by_lanes.insert(by_lanes.end(), by_lists.begin(), by_lists.end());
+    }
     if (!by_lanes.empty() && (st = prepare_lanes(ctx, by_lanes, dbg, lanes))) return st;
-    if (!by_lists.empty() && (st = prepare_lists(ctx, by_lists, dbg, lists))) return st;
     const bool graph = ctx->opt_graph != 0;
     auto device_work = [&]() -> te_status {
         te_status st;
@@ -413,6 +428,7 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
         pairs += N * (long long)g.members.size();
     }
     std::vector<const HostGroup *> by_lists, by_lanes;
+    size_t list_need = 0;
     for (const HostGroup &g : groups) {
         if (g.members.empty()) continue;
         const ListCall c{g.data->T - g.max_lag, g.k, g.theiler, g.dx, (int)g.y.size(),
@@ -420,6 +436,11 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
         const bool lists = !lane_only && (ctx->opt_lists ? list_fits(c.N, c.dx, c.dz, c.k)
                                                          : list_serves(c, n_groups, rows, pairs));
         (lists ? by_lists : by_lanes).push_back(&g);
+        if (lists) list_need += list_bytes(c);
+    }
+    if (ctx->list_pool < std::min(list_need, kListPoolLeast)) {   // a served batch's share
+        by_lanes.insert(by_lanes.end(), by_lists.begin(), by_lists.end());
+        by_lists.clear();
     }
     return launch_paths(ctx, by_lists, by_lanes, n_out, dbg);
 }

@@ -16,6 +16,10 @@
 
 namespace teksg {
 
+// Neighbour lists in device memory at once: enough points to fill the chip
+// several times over at the longest lists (54 KB a point), small beside the X values.
+constexpr size_t kListPoolBytes = (size_t)256 << 20;
+
 struct DevBuf {
     void *p = nullptr;
     size_t cap = 0;
@@ -126,6 +130,7 @@ struct te_ctx {
     // neighbour lists of the points in work, the list launches' tables and
     // sorted columns (a batch may need the member-lane kernel's beside them)
     teksg::DevBuf ws_lists, ws_ltables, ws_lsort;
+    size_t list_pool = teksg::kListPoolBytes;   // bytes of ws_lists at most
     teksg::DevBuf ws_gtile;  // cmi_gauss: the contraction's prepared B tiles and centred X
     // pinned host staging
     void *pin = nullptr;
@@ -174,7 +179,9 @@ te_status fail(te_ctx *ctx, te_status st, const std::string &msg);
 te_status autocorr_decay(te_ctx *ctx, const te_data *data, int32_t proc, int32_t *out_tau);
 te_status cuda_fail(te_ctx *ctx, cudaError_t e, const char *what);
 
-te_status ensure_dev(te_ctx *ctx, DevBuf &b, size_t bytes);
+// b holds at least `bytes`; where it grows, by half of what it had (up to `most`)
+te_status ensure_dev(te_ctx *ctx, DevBuf &b, size_t bytes, size_t most = SIZE_MAX);
+te_status free_dev(te_ctx *ctx, DevBuf &b);   // given back once the stream's work is done
 te_status ensure_pin(te_ctx *ctx, size_t bytes);
 te_status ensure_pin_lists(te_ctx *ctx, size_t bytes);
 te_status ensure_aux(te_ctx *ctx);   // ctx->aux_stream, ev_fork, ev_join

@@ -57,19 +57,40 @@ struct Slot {
     int64_t *keys_pin = nullptr;
     size_t keys_cap = 0;
     size_t fp = 0;
+    // device bytes for neighbour lists: what the batch in flight may take, of
+    // an idle slot what it keeps
+    size_t lists = 0;
+    bool give_back = false;   // an idle slot's, before the next batch starts
 };
 
 // device bytes of one job, as the member-lane path needs them: permutations
 // and their composed copies (8 S N), the X-value rows of the TMA-staged kernel
 // (4 (S + 1) N, rows padded to a multiple of 8 points), the order and sorted Y/Z
 // columns, the chunk boxes, accumulators, keys and descriptors.  The list path
-// keeps the permutations alone and, per batch in flight and whatever its
-// size, at most 256 MiB of lists.
+// keeps the permutations alone; its own buffers come out of what the admitted
+// jobs leave of the budget (list_room).
 size_t footprint(int N, int S, int dyz)
 {
     const size_t pitch = (size_t)std::max(32, (N + 7) & ~7);
     return (size_t)S * N * 8 + (size_t)(S + 1) * pitch * 4 + (size_t)N * (4 + 4 * (size_t)dyz) +
            8 * (size_t)dyz * (N / 8 + 1) + 64 * (size_t)(S + 1) + 4096;
+}
+
+// device bytes of a job on lists besides the pool: its tables and a sorted
+// column with its ranks, in buffers that grow by half
+size_t list_tables(int N, int S) { return 16 * (size_t)N + 36 * (size_t)(S + 1) + 2048; }
+
+size_t lists_held(const te_ctx *ctx)
+{
+    return ctx->ws_lists.cap + ctx->ws_ltables.cap + ctx->ws_lsort.cap;
+}
+
+te_status give_back_lists(te_ctx *ctx)
+{
+    te_status st;
+    for (DevBuf *b : {&ctx->ws_lists, &ctx->ws_ltables, &ctx->ws_lsort})
+        if ((st = free_dev(ctx, *b))) return st;
+    return TE_OK;
 }
 
 }  // namespace
@@ -110,6 +131,31 @@ te_status queue_keys(Slot &sl)
     CK(copy_d2h(ctx, sl.keys_pin, ctx->ws_keys.p, bytes), "cudaMemcpyAsync");
     CK(cudaEventRecord(sl.done, ctx->stream), "cudaEventRecord");
     return TE_OK;
+}
+
+// Lists for the slot's batch, whose jobs are admitted (in_use counts them): an
+// equal share of what the budget has left for each slot that is idle, at most
+// kListPoolBytes; without one the batch takes the member-lane kernel, which
+// the jobs' footprints pay for.  The lists that idle slots keep are given back
+// where they would pass the budget.  Called with the lock held.
+void list_room(te_server *S, Slot &sl)
+{
+    size_t busy = 0, kept = 0, tables = 0;
+    int idle = 1;
+    for (Slot &o : S->slots) {
+        if (&o == &sl) continue;
+        (o.busy ? busy : kept) += o.lists;
+        idle += o.busy ? 0 : 1;
+    }
+    for (const ServeJob *j : sl.jobs) tables += list_tables(j->N, j->S);
+    const size_t left = S->budget - S->in_use - busy;
+    const size_t share = std::min(left / idle, kListPoolBytes + tables);
+    sl.ctx->list_pool = share > tables ? (share - tables) & ~(size_t)255 : 0;
+    for (Slot &o : S->slots)
+        o.give_back = !o.busy && &o != &sl && o.lists && kept + share > left;
+    sl.give_back = sl.ctx->ws_lists.cap > sl.ctx->list_pool || sl.lists > share;
+    sl.lists = share;
+    S->peak = std::max(S->peak, S->in_use + busy + share);
 }
 
 // Build and queue one batch on the slot's stream (no host wait).
@@ -227,19 +273,21 @@ void serve_loop(te_server *S)
             }
             S->in_use -= sl.fp;
             sl.fp = 0;
+            sl.lists = lists_held(sl.ctx);
             sl.jobs.clear();
             sl.busy = false;
             progressed = true;
             S->cv_done.notify_all();
         }
-        // admissions: arrival order, footprint within the budget
+        // admissions: arrival order, footprints and the batches' lists within the budget
         for (Slot &sl : S->slots) {
             if (sl.busy) continue;
             std::vector<ServeJob *> batch;
-            size_t fp = 0;
+            size_t fp = 0, held = S->in_use;   // by the other batches
+            for (const Slot &o : S->slots) held += o.busy ? o.lists : 0;
             while (!S->pending.empty() && (int)batch.size() < S->max_batch) {
                 ServeJob *j = S->pending.front();
-                if (S->in_use + fp + j->fp > S->budget) break;
+                if (held + fp + j->fp > S->budget) break;
                 S->pending.pop_front();
                 fp += j->fp;
                 j->state = JS_RUNNING;
@@ -247,14 +295,21 @@ void serve_loop(te_server *S)
             }
             if (batch.empty()) break;
             S->in_use += fp;
-            S->peak = std::max(S->peak, S->in_use);
             sl.jobs = batch;
             sl.fp = fp;
             sl.busy = true;
+            list_room(S, sl);
             S->st.batches++;
             lk.unlock();
-            const te_status lst = launch_batch(sl);
+            te_status lst = TE_OK;   // (this thread alone touches the slots' contexts)
+            for (Slot &o : S->slots)
+                if (o.give_back && !lst) lst = give_back_lists(o.ctx);
+            if (!lst) lst = launch_batch(sl);
             lk.lock();
+            for (Slot &o : S->slots) {
+                if (o.give_back && &o != &sl) o.lists = lists_held(o.ctx);
+                o.give_back = false;
+            }
             if (lst) {
                 for (ServeJob *j : sl.jobs) {
                     j->state = JS_FAILED;
@@ -262,6 +317,7 @@ void serve_loop(te_server *S)
                 }
                 S->in_use -= sl.fp;
                 sl.fp = 0;
+                sl.lists = lists_held(sl.ctx);
                 sl.jobs.clear();
                 sl.busy = false;
                 S->cv_done.notify_all();
@@ -459,6 +515,7 @@ te_status te_serve_get_stats(te_ctx *ctx, te_serve_stats *out)
     std::lock_guard<std::mutex> lk(ctx->server->mu);
     *out = ctx->server->st;
     out->in_use_bytes = ctx->server->in_use;
+    for (const Slot &sl : ctx->server->slots) out->in_use_bytes += sl.busy ? sl.lists : 0;
     out->peak_bytes = ctx->server->peak;
     out->pending = ctx->server->pending.size();
     return TE_OK;

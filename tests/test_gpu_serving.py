@@ -159,3 +159,37 @@ def test_greedy_loops_served_equal_direct_and_oracle():
                                         max_lag=j.max_lag)
         assert got == want
     ctx.close()
+
+
+@pytest.mark.parametrize("budget_mib,inflight", [(24, 2), (200, 1), (330, 2), (1200, 4)])
+def test_lists_stay_within_the_memory_budget(env, budget_mib, inflight):
+    """The neighbour lists of served batches come out of the budget: device
+    memory and the reported peak stay within it, whether a batch's share of
+    it holds lists or not, and the keys are cmi_ksg_batch's.  (The largest batch's
+    lists take up to 256 MiB at any budget if nothing bounds them.)"""
+    torch = pytest.importorskip("torch")
+    te, ctx = env
+    d = te.te_data_create(ctx, synth.workload_var10(T=6005, seed=3)["series"])
+    z = [(0, 1), (4, 2), (7, 1)]
+    jobs = [te.Job(d, [(1 + a % 9, 1 + a // 9)], [(0, 0)], z[:a % 4], k=4, max_lag=5,
+                   n_surr=20 + 30 * (a % 3), seed=a) for a in range(24)]
+    _, ref = te.cmi_ksg_batch(ctx, jobs, return_keys=True)
+    budget = budget_mib << 20
+    te.te_serve_start(ctx, hbm_budget_bytes=budget, max_inflight=inflight, max_batch_jobs=5)
+    try:
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        low = before
+        for _ in range(3):
+            tickets = [te.te_serve_submit(ctx, j) for j in jobs]
+            for t, j, r in zip(tickets, jobs, ref):
+                assert te.te_serve_poll(ctx, t, j.n_surr, return_keys=True)[1] == r
+                low = min(low, torch.cuda.mem_get_info()[0])
+        st = te.te_serve_get_stats(ctx)
+    finally:
+        te.te_serve_stop(ctx)
+    assert st["in_use_bytes"] == 0 and 0 < st["peak_bytes"] <= budget
+    # beside the admitted bytes: what every slot's buffers are rounded up to (2 MiB
+    # each) and grow by beyond a job's need (half)
+    assert before - low <= budget + inflight * (24 << 20), (before - low) / 2 ** 20
+    d.close()
