@@ -36,6 +36,14 @@ struct Chunk {
 
 }  // namespace
 
+static bool list_serves_other_k(const ListCall &c, int n_groups, bool full);
+
+// mean n_yz of a member's k nearest: how deep in list A they lie
+static double list_depth(const ListCall &c)
+{
+    return c.N * std::pow((double)c.k / c.N, (double)(c.dy + c.dz) / (c.dx + c.dy + c.dz));
+}
+
 // Measured line between the two paths (whole calls on one GB300, member-lane
 // or fused kernel / lists, microseconds).  Lists pay for themselves by a row
 // per point that all members of the group walk; the member-lane kernel shares
@@ -51,18 +59,18 @@ struct Chunk {
 // Y and Z variables there are, and pairs beyond its capacity scan all points.
 // The line is at the expected depth: 201 members at N = 9000, k = 4, empty Z, two X
 // variables (depth 686) 17,220 / 18,689, four (1922) 28,342 / 147,900; one Z and four
-// (686) equal; two Z 3.3 to 7 times in the lists' favour.  With k other than 4
-// a point's dimensions lie apart (list_shape) and the line is nearer: k = 6,
-// one Z, four X variables, N = 4000 9981 / 12,455.
+// (686) equal; two Z 3.3 to 7 times in the lists' favour.
 bool list_serves(const ListCall &c, int n_groups, long long rows, long long pairs)
 {
     const int N = c.N, dz = c.dz;
     const long long m = (long long)c.members;
     if (!list_fits(N, c.dx, dz, c.k)) return false;
+    const bool full = rows >= 24000;   // points of all groups: several waves of CTAs
+    if (c.dx == 1 && (c.theiler > 0 || N > kMaxOrderN))
+        return true;   // the member lanes cannot prune then
+    if (c.k != 4) return list_serves_other_k(c, n_groups, full);
     if (c.dx > 1) {
         if (dz > 1 || m < 8) return true;
-        const double d = c.dx + c.dy + dz;
-        const double depth = N * std::pow((double)c.k / N, (c.dy + dz) / d);   // mean n_yz
         const bool packed = list_shape(N, c.dx, dz, c.k, c.members).dxp > 0;
         double most;
         if (dz == 0)
@@ -72,10 +80,8 @@ bool list_serves(const ListCall &c, int n_groups, long long rows, long long pair
             most = 680;
         else
             most = m >= 64 && (c.dx > 2 || (m >= 100 && N < 5000)) ? 0 : 500;
-        return depth <= most;
+        return list_depth(c) <= most;
     }
-    if (c.theiler > 0 || N > kMaxOrderN) return true;   // the member lanes cannot prune then
-    const bool full = rows >= 24000;   // points of all groups: several waves of CTAs
     const bool block = m <= 32 || (m >= 48 && m <= 64);   // one well-filled block of members
     if (n_groups >= 200 && m <= 8 && N <= 700 && dz > 0) return false;
     if (N < 250) return true;
@@ -98,6 +104,38 @@ bool list_serves(const ListCall &c, int n_groups, long long rows, long long pair
     default:
         return !(full && m <= 32 && n_groups >= 200 && N <= 700);
     }
+}
+
+// With another k the member-lane kernel keeps its k smallest by insertion and
+// takes about 1.6 times as long as with four, the lists hardly longer; the fused
+// kernel serves two members at a time and, from k = 9 on, its longer buffer. The
+// lines are those of 2130 measured sizes (k 1 to 16, one to six X variables, 1 to
+// 9045 members): 11 of them are 6 to 12% faster on the other side.
+// Member lanes / lists, one X variable: 9 groups of 201, N = 4000, empty Z, k = 3
+// and 9: 1.90 and 1.43; 64 of 5, N = 9990 0.90 and 1.02; 64 of 21, N = 8000, two Z
+// 0.70 and 0.86, three 1.30 and 0.94, five 2.5 and 2.0. Fused / lists: four X,
+// one Z, 201 members, N = 2200, k = 3 and 9 0.67 and 1.47; 21 members 1.24 and 1.89;
+// three X, empty Z, 12 members, N = 2200, 4000, 9000, k = 5 1.92, 1.48, 0.53.
+static bool list_serves_other_k(const ListCall &c, int n_groups, bool full)
+{
+    const int N = c.N, dz = c.dz, k = c.k;
+    const double m = (double)c.members;
+    if (c.dx == 1) {
+        if (dz == 0)
+            return !(full && m >= 4 && m < 16 && N >= 1500 &&
+                     k <= (N < 3000 ? 8 : N < 6000 ? 6 : 3));
+        return !(dz == 2 && k > 1 && k <= 9 && full && N >= 3500 && m <= 32 && n_groups >= 8);
+    }
+    if (dz > 1 || m < 8) return true;
+    const double depth = list_depth(c);
+    if (dz == 0) {
+        if (m < 100) return depth * m * N <= 6.5e7;
+        return N <= (c.dx == 2 ? 2500 : 1500) && (c.dx <= 3 || k > 8);
+    }
+    if (k > 8) return m >= 48 ? depth <= 860 : depth * N <= 8e6;
+    if (m < 48) return depth * N <= 6.5e6;
+    if (m < 100) return c.dx == 2 || N < 600 || (c.dx == 3 && (N < 1500 || (N > 3000 && k <= 3)));
+    return c.dx == 2 && (k <= 2 || N >= 5000);
 }
 
 size_t list_bytes(const ListCall &c)

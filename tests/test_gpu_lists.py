@@ -249,6 +249,26 @@ def test_batches_whose_groups_take_both_paths(env, T, n_groups, S):
     data.close()
 
 
+@pytest.mark.parametrize("k", [1, 3, 8, 9, 16])
+def test_batches_of_another_k_take_both_paths(env, k):
+    """As above with k other than 4, whose lines lie elsewhere: many groups of
+    5 and of 21 over zero, two and three Z variables, and several X variables
+    with few and many members."""
+    te, ctx = env
+    T = 3805
+    s = np.asarray(synth.workload_var10(T=T, seed=k)["series"], dtype=np.float32)
+    data = te.te_data_create(ctx, s)
+    kw = dict(k=k, max_lag=5, seed=3)
+    jobs = [te.Job(data, [((g + 7) % 10, 2)], [(g % 10, g // 10)],
+                   [((g + 1 + d) % 10, 1 + d) for d in range((0, 2, 3)[g % 3])],
+                   n_surr=4 if g % 2 else 20, **kw) for g in range(18)]
+    jobs += [te.Job(data, [(a, 1 + a % 5) for a in range(dx)], [(0, 0)], Z[:dz], n_surr=S, **kw)
+             for dx, dz, S in ((2, 0, 11), (3, 0, 63), (3, 1, 20), (4, 1, 70))]
+    got, ref = _both(te, ctx, jobs)
+    assert got == ref
+    data.close()
+
+
 def _series(kind, T, seed=0):
     rng = np.random.default_rng(seed)
     if kind == "cauchy":
