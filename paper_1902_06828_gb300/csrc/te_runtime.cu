@@ -212,7 +212,8 @@ te_status ensure_q(te_ctx *ctx, int n_needed)
             ctx->q_host.push_back(dd_to_q(ctx->dd_hi, ctx->dd_lo));  // n = 1
         }
         int target = std::max(n_needed + 1, (int)ctx->q_host.size() * 2);
-        target = std::max(target, 4096);
+        // (a short table for a context's first small call: 4096 entries took it 60 us)
+        target = std::max(target, 512);
         for (int n = (int)ctx->q_host.size(); n < target; ++n) {
             double rh, rl;
             dd_recip((double)(n - 1), rh, rl);
