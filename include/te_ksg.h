@@ -498,8 +498,8 @@ te_status te_serve_get_stats(te_ctx *ctx, te_serve_stats *out);
  * out_cmi: host double[1 + S]; out_key: NULL or host int64[2 (1 + S)].
  * Errors: status codes only (no context carries a message): TE_EINVAL for any
  * rule cmi_ksg checks plus the scratch limit, TE_ECUDA for a failed CUDA call.
- * A value of x, y or z that is not finite is found while the lists are built
- * (TE_EINVAL); a call that runs without lists does not look for one.
+ * Values that are not finite are not refused here (no host check has read them);
+ * a difference that is not a number counts as no distance in its dimension.
  *
  * The first call on a device resolves the device address of the scratch array
  * (cudaGetSymbolAddress, with that device current).  No call may be made while

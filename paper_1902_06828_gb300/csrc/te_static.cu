@@ -327,8 +327,10 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
         if (!read_keys(flag_at + 16)) return TE_ECUDA;
         unsigned flags[2];   // nonfinite, bad
         std::memcpy(flags, g_keys_host + flag_at, sizeof flags);
-        if (flags[0]) return TE_EINVAL;
-        lanes = flags[1] != 0;   // too many pairs beyond the lists: evaluated anew
+        // values that are not finite (no host check has read them), or too many
+        // pairs beyond the lists: evaluated anew
+        lanes = flags[0] || flags[1];
+        if (lanes && jt < 8) return TE_EINVAL;
         if (lanes && cudaMemsetAsync(acc, 0, (size_t)(S + 1) * 16, stream) != cudaSuccess)
             return TE_ECUDA;
     }
