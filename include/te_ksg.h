@@ -390,7 +390,8 @@ typedef struct {
     uint64_t launches;        /* kernel launches issued (all kernels of the library) */
     uint64_t pair_evals;      /* member x point-pair distance evaluations the KSG kernel
                                  executed (both passes; pairs of skipped chunks, or beyond
-                                 the lists' prefixes, excluded) */
+                                 the lists' prefixes, excluded, as are the lists' build,
+                                 once per group, and counts by search in a sorted column) */
     double kernel_ms;         /* summed device time of the KSG kernels (CUDA events on the
                                  context's stream) */
     uint64_t ksg_launches;    /* launches of the KSG kernel (the list walk, or the member-lane kernel) */
@@ -401,7 +402,8 @@ typedef struct {
     uint64_t ksg_ops;         /* algorithmic ops of the executed evaluations: 3 per kNN-pass
                                  pair (subtract, max, compare), 7 per count-pass pair
                                  (subtract, 3 compares, 3 increments); on neighbour lists 3
-                                 per pair (a count is a subtract, a compare, an increment) */
+                                 per pair (a count is a subtract, a compare, an increment),
+                                 pairs beyond their radii, which scan all points, as before */
 } te_stats;
 
 te_status te_get_stats(const te_ctx *ctx, te_stats *out);

@@ -497,6 +497,14 @@ __device__ __forceinline__ void group_window(const float *__restrict__ z, int n,
     if (!(e > 0.f) || hi < lo) hi = lo;   // hi < lo: values out of order (not finite)
 }
 
+// Work counters of one pair's scan over all points: the search, then the counts
+__device__ __forceinline__ void count_scan(const ListLaunch &L, int N, bool search)
+{
+    if (!L.work) return;
+    atomicAdd(&L.work[0], (search ? 2ull : 1ull) * (unsigned)N);
+    atomicAdd(&L.work[1], (search ? 10ull : 7ull) * (unsigned)N);
+}
+
 // One member at query point i over all points, by the whole CTA: its k-th
 // smallest joint distance and the three counts, added to the accumulators.
 // Blocks of 32 points go round the warps, four of a warp's in flight; every
@@ -589,6 +597,7 @@ __device__ __noinline__ void scan_member(const ListLaunch &L, const ListGroup &G
     }
     __syncthreads();
     if (threadIdx.x == 0) {
+        count_scan(L, N, true);
         // an empty Z: d_Z is below every eps for every point that is not masked
         if (G.dz == 0) cnt[0] = N - (min(i + w, N - 1) - max(i - w, 0) + 1);
         const long long t = L.q[cnt[0] + 1] - L.q[cnt[1] + 1] - L.q[cnt[2] + 1];
@@ -743,6 +752,7 @@ __device__ __noinline__ void scan_aside(const ListLaunch &L, const ListGroup &G,
         __syncthreads();
         if (threadIdx.x < ne) {
             const int e = threadIdx.x, i = point(e);
+            count_scan(L, N, !(aside[base + e].pair & kExact));
             if (W.n_near[e] > kScanNear) {
                 const uint32_t b = aside[base + e].pair & ~kExact;
                 atomicOr(&left[b >> 5], 1u << (b & 31));
@@ -1288,6 +1298,7 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
                     cx += fmaxf(d, v) < ec ? 1 : 0;
                 }
                 __syncwarp();
+                evals += NG * (last - first + 1);
                 nz -= group_sum(cz);
                 nxz -= group_sum(cx);
             }
@@ -1304,12 +1315,14 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
                 c = 0;
                 for (int j = first + u; j <= last; j += G)
                     c += dist_x(xm, xi, oi, 4u * j) < ec ? 1 : 0;
+                evals += NG * (last - first + 1);
                 __syncwarp();
                 nxz = hi - lo - group_sum(c);
             } else {
                 c = 0;
                 for (int j = u; j < N; j += G)
                     if (j < first || j > last) c += dist_x(xm, xi, oi, 4u * j) < ec ? 1 : 0;
+                evals += NG * nz;
                 __syncwarp();
                 nxz = group_sum(c);
             }

@@ -345,3 +345,27 @@ def test_served_and_allocation_free_calls_hand_over(env, kind, T, dz, S):
     assert got == ref[0]
     data.close()
     plain.close()
+
+
+@pytest.mark.parametrize("dz,dx,w", [(8, 1, 0), (8, 1, 3), (0, 2, 0), (0, 2, 5)])
+def test_work_counters_include_scans_over_all_points(env, dz, dx, w):
+    """Binary values: with eight Z variables two points in 1100 share a query
+    point's (Y, Z) and the rest are tied at one, so that lists end before k
+    neighbours and every pair scans every point; over an empty Z a count of several X variables visits every point: at
+    least one evaluation a point for each pair, no more than two scans."""
+    te, ctx = env
+    N, S = 1100, 4
+    data = te.te_data_create(ctx, _series("binary", N + 5))
+    x = [(2, 1 + a) for a in range(dx)]
+    try:
+        ctx.set_option("ksg_lists", 1)
+        before = ctx.stats()
+        te.cmi_ksg(ctx, data, x, [(0, 0)], Z[:dz], k=4, theiler=w, max_lag=5, n_surr=S)
+        after = ctx.stats()
+    finally:
+        ctx.set_option("ksg_lists", 0)
+    evals, ops = (after[n] - before[n] for n in ("pair_evals", "ksg_ops"))
+    pairs = (S + 1) * N
+    assert pairs * (N - 2 * w - 1) <= evals <= 5 * pairs * N
+    assert 3 * evals <= ops <= 7 * evals
+    data.close()
