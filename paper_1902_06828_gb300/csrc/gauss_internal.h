@@ -60,10 +60,6 @@ struct GaussArgs {
     int group;              // chunks per FP32 accumulation group of the tensor-core contraction
     double *cross_part;
 };
-// splits of the points for (S + 1) * dx rows of N points in the batched
-// FP64 / float-float contraction (every split keeps at least one accumulation
-// group)
-int gauss_cross_splits(int rows, int N);
 // chunks of 32 points per split of the tensor-core contraction (two CTAs an SM)
 // and per FP32 accumulation group
 int gauss_tc_split_chunks(int N, int rows, int sms, int *group);

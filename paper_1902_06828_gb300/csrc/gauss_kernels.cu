@@ -1461,21 +1461,6 @@ cudaError_t gauss_launch_keys(const double *v, int n, long long *keys, int *bad,
     return cudaGetLastError();
 }
 
-int gauss_cross_splits(int rows, int N)
-{
-    // enough CTAs for four resident per SM (each split ends in an FP64
-    // partial-sum row that the reduction adds); the SM count is the device's
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        sms < 1)
-        sms = 1;
-    const int tiles = (rows + kGaussTileM - 1) / kGaussTileM;
-    const int groups = (N + kGaussKC * kGaussGroup - 1) / (kGaussKC * kGaussGroup);
-    int splits = (4 * sms + tiles - 1) / tiles;
-    return splits < 1 ? 1 : (splits > groups ? groups : splits);
-}
-
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // byte offsets of the parts of the buffer (btile first), and their end

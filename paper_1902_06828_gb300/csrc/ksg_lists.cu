@@ -1422,7 +1422,7 @@ void list_caps(int N, int k, int dx, int dy, int dz, int *cap_a, int *cap_b)
     *cap_b = dz > 1 ? cap(28.0 * nz, kListCapB) : 0;
 }
 
-// X variables as stored for the walk (ListWalk's DXP): the dimensions of a
+// X variables as stored for the walk (its DXP): the dimensions of a
 // point together where that fits, a row per dimension (0) otherwise
 static int list_dxp(int N, int dx, int k)
 {
@@ -1449,9 +1449,9 @@ ListShape list_shape(int N, int dx, int dz, int k, size_t members)
     s.k4 = k == 4;
     s.lanes = k <= 8 ? 8 : 16;
     s.width = 32 / s.lanes;
-    // one member: a warp per point (fewer than 2^17 pairs leave warps idle, and
-    // a point's chain of steps is shorter over 32 lanes)
-    if (members == 1 && N <= 131072) {
+    // one member: a warp per point (so few pairs leave warps idle, and a point's
+    // chain of steps is shorter over 32 lanes)
+    if (members == 1) {
         s.lanes = 32;
         s.width = 1;
         return s;

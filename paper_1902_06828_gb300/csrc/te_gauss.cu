@@ -171,7 +171,7 @@ te_status run_groups_gauss(te_ctx *ctx, const std::vector<HostGroup> &groups, in
             const int blocks = A.perm_t_pitch ? (A.S + 256) / 256 * A.dx
                                               : ((A.S + 1) * A.dx + 127) / 128;
             const bool col = A.perm_t_pitch != 0;
-            const int splits = ((col ? 32 : 8) * 152 + b.n * blocks - 1) / (b.n * blocks);
+            const int splits = ((col ? 32 : 8) * ctx->sms + b.n * blocks - 1) / (b.n * blocks);
             off[i] = w;
             w += gauss_shape(A, A.N, A.S, A.dx, A.dy, A.d - A.dx - A.dy, splits, true);
         }
@@ -276,7 +276,7 @@ extern "C" te_status cmi_gauss(te_ctx *ctx, const te_data *data, const te_var *x
         GaussArgs A{};
         const size_t ws =
             gauss_shape(A, N, S, dx, dy, dz, 1, false,
-                        gauss_tc_split_chunks(N, (S + 1) * dx, 152, &A.group));
+                        gauss_tc_split_chunks(N, (S + 1) * dx, ctx->sms, &A.group));
         const size_t nd = ws + 2 * (size_t)(S + 1);
         if ((st = ensure_dev(ctx, ctx->ws_gauss, nd * 8 + (size_t)(d + 8) * 4))) return st;
         // permutations as 16-bit rows (pitch a multiple of 8 entries) when the

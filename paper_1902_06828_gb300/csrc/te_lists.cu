@@ -149,9 +149,6 @@ te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &group
                         const KsgDebug &dbg, KsgPart &part)
 {
     te_status st;
-    int sms = 0;
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device),
-       "cudaDeviceGetAttribute");
     std::map<ListShape, std::vector<const HostGroup *>> classes;
     for (const HostGroup *g : groups)
         classes[list_shape(g->data->T - g->max_lag, g->dx, (int)g->z.size(), g->k,
@@ -193,7 +190,7 @@ te_status prepare_lists(te_ctx *ctx, const std::vector<const HostGroup *> &group
                 blocks += lg[cp.first_group + segs[s].group].n_mblocks;
                 max_nq = std::max(max_nq, segs[s].nq);
             }
-            const int splits = list_splits(blocks, max_nq, cp.smem, sms);
+            const int splits = list_splits(blocks, max_nq, cp.smem, ctx->sms);
             for (int s = ch.first_seg; s < ch.first_seg + ch.n_segs; ++s) {
                 segs[s].build_item = ch.build_items;
                 ch.build_items += (segs[s].nq + ch.queries - 1) / ch.queries;

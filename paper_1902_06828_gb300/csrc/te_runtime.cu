@@ -910,6 +910,7 @@ te_status te_ctx_create(int device, te_ctx **out)
     }
     ctx->device = device;
     if (cudaSetDevice(device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaStreamCreateWithFlags(&ctx->own_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&ctx->ev_a) != cudaSuccess || cudaEventCreate(&ctx->ev_b) != cudaSuccess ||
         cudaMalloc(&ctx->work_dev, 5 * sizeof(unsigned long long)) != cudaSuccess ||

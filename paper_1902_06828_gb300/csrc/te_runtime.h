@@ -114,6 +114,7 @@ struct te_data {
 
 struct te_ctx {
     int device = 0;
+    int sms = 0;   // of the device
     cudaStream_t own_stream = nullptr;
     cudaStream_t stream = nullptr;
     std::string err;
