@@ -213,3 +213,60 @@ def test_more_permutation_sets_in_a_round_than_a_grid_dimension(te, ctx):
         assert g["n_estimates"] == r["n_estimates"] and g["omnibus_p"] == r["omnibus_p"]
         assert g["omnibus_cmi"] == r["omnibus_cmi"] or abs(g["omnibus_cmi"] - r["omnibus_cmi"]) <= TOL
     data.close()
+
+
+@pytest.mark.parametrize("T,S", [(1501, 40), (26001, 3), (26002, 3)])
+def test_every_width_of_the_conditioning_set(te, ctx, T, S):
+    """A target driven by twenty sources with equal weights selects them one by
+    one: W has every width from 1 to 18 (the shared-memory contraction ends
+    at 16), at N = 1500 and on both sides of the N = 26,000 whose X column still
+    fits shared memory; sampled estimates against FP64."""
+    from oracle import ksg as oksg
+    n, alpha = 21, 0.05 if S > 20 else 0.4
+    rng = np.random.default_rng(T)
+    s = rng.normal(size=(n, T))
+    s[0, 1:] = 0.5 * s[1:, :-1].sum(0) + 0.2 * rng.normal(size=T - 1)
+    s = synth.standardise_jitter(s, T).astype(np.float32)
+    N = T - 1
+    col = lambda v: s[v[0], 1 - v[1]:T - v[1]].astype(np.float64)
+    sel, widths, errs = [], set(), []
+
+    def value(key):   # inverse of the order-preserving image
+        k = key & ((1 << 64) - 1)
+        k = k - (1 << 64) if k >= 1 << 63 else k
+        return np.int64(k if k >= 0 else k ^ 0x7FFFFFFFFFFFFFFF).view(np.float64)
+
+    def check(target, stage, it, vs, n_cand, n_surr, keys):
+        if stage not in (1, 2):
+            return
+        got = np.array([[value(k) for k in row] for row in keys])
+        W = np.array([col((0, 0))] + [col(v) for v in sel])
+        W -= W.mean(1, keepdims=True)
+        widths.add(len(W))
+        inv = np.linalg.inv(W @ W.T / (N - 1))
+        inv_z = np.linalg.inv(W[1:] @ W[1:].T / (N - 1)) if sel else None
+        for c in (0, len(vs) // 2, len(vs) - 1):
+            for a in (0, 1, n_surr):
+                x = col(vs[c]) - col(vs[c]).mean()
+                if a:
+                    x = x[oksg.permutation(9, 0, stage, it, a, N)]
+                cw, sxx = W @ x / (N - 1), x @ x / (N - 1)
+                z = cw[1:] @ inv_z @ cw[1:] if sel else 0.0
+                ref = 0.5 * (np.log(sxx - z) - np.log(sxx - cw @ inv @ cw))
+                errs.append(abs(got[c, a] - ref))
+        best = int(np.argmax(got[:, 0]))
+        if np.sum(got[:, 1:].max(0) > got[best, 0]) / n_surr < alpha:
+            sel.append(tuple(vs[best]))
+
+    data = te.te_data_create(ctx, s)
+    ctx.set_trace(check)
+    try:
+        te.te_network_infer(ctx, data, max_lag_target=1, max_lag_sources=1, n_surr=S,
+                            alpha_max=alpha, alpha_min=alpha, alpha_omnibus=alpha, seed=9,
+                            targets=[0], estimator="gauss")
+    except te.TEError as e:   # more than 8 sources left for the omnibus block
+        assert "dx <= 8" in str(e)
+    finally:
+        ctx.set_trace(None)
+    assert set(range(1, 19)) <= widths and max(errs) <= TOL
+    data.close()

@@ -93,6 +93,33 @@ def test_largest_point_counts_of_every_width(env, N):
     data.close()
 
 
+@pytest.mark.parametrize("dz,N", [(0, 9876), (0, 9877), (0, 19756), (0, 19757), (0, 39512),
+                                  (0, 39513), (1, 10332), (1, 10333), (1, 20352), (1, 20353),
+                                  (1, 39512), (1, 39513)])
+def test_largest_point_counts_with_a_coarse_column_beside_the_x_values(env, dz, N):
+    """With one Z variable or none a CTA also holds every 16th value of the
+    sorted columns, so its widths end earlier. The executed evaluations tell
+    which kernel ran: equal to the member-lane kernel's past the last N only."""
+    te, ctx = env
+    rng = np.random.default_rng(N)
+    s = rng.normal(size=(3, N + 1)).astype(np.float32)
+    s[1, 1:] += 0.5 * s[0, :-1]
+    data = te.te_data_create(ctx, s)
+    runs = []
+    for option, value in (("ksg_lists", 1), ("ksg_tile", 256)):
+        try:
+            ctx.set_option(option, value)
+            before = ctx.stats()["pair_evals"]
+            keys = te.cmi_ksg(ctx, data, [(0, 1)], [(1, 0)], [(2, 1)][:dz], k=4, max_lag=1,
+                              n_surr=4, seed=2, return_keys=True)[1]
+            runs.append((keys, ctx.stats()["pair_evals"] - before))
+        finally:
+            ctx.set_option(option, 0)
+    assert runs[0][0] == runs[1][0]
+    assert (runs[0][1] == runs[1][1]) == (N > 39512)
+    data.close()
+
+
 def test_columns_of_different_point_sets_in_one_batch(env):
     """Jobs whose maximum lags differ read the same memory as columns of
     different lengths; each sorts its own."""
@@ -145,6 +172,29 @@ def test_permutations_past_the_parallel_shuffle(env, N):
         x = s[0].astype(np.float64)[oksg.permutation(8, 1, 0, 0, a, N)]
         r = np.corrcoef(x, s[1].astype(np.float64))[0, 1]
         assert abs(got[a] - -0.5 * np.log1p(-r * r)) < 1e-7
+    data.close()
+
+
+@pytest.mark.parametrize("N", [65535, 65536, 70001])
+def test_gaussian_estimates_past_16_bit_permutations(env, N):
+    """The largest N whose surrogates are drawn as 16-bit rows and the first past
+    it, where the contraction reads 32-bit ones: every surrogate with two Z
+    variables against FP64, within the call's own bound."""
+    from oracle import ksg as oksg
+    te, ctx = env
+    rng = np.random.default_rng(N)
+    s = rng.normal(size=(4, N)).astype(np.float32)
+    s[1] += 0.3 * s[0] + 0.2 * s[2]
+    data = te.te_data_create(ctx, s)
+    got, err = te.cmi_gauss(ctx, data, [(0, 0)], [(1, 0)], [(2, 0), (3, 0)], max_lag=0, n_surr=5,
+                            seed=8, stream_tag=1)
+    v = s.astype(np.float64)
+    logdet = lambda rows: np.linalg.slogdet(np.cov(rows))[1]
+    for a in range(6):
+        x = v[0] if a == 0 else v[0][oksg.permutation(8, 1, 0, 0, a, N)]
+        ref = 0.5 * (logdet(np.array([x, v[2], v[3]])) + logdet(v[1:]) - logdet(v[2:])
+                     - logdet(np.array([x, v[1], v[2], v[3]])))
+        assert abs(got[a] - ref) <= err[a] + 1e-12
     data.close()
 
 
