@@ -978,7 +978,9 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
     if (threadIdx.x == 0) {
         s_n_aside = 0;
         s_given_up = given_up;
-        s_slow_limit = L.bad ? list_slow_limit((q_last - q_first) * nm, N, dx) : 0x7fffffff;
+        s_slow_limit = L.bad ? list_slow_limit((q_last - q_first) * nm, N, dx, Gr.n_members,
+                                               w == 0 && N <= kMaxOrderN)
+                             : 0x7fffffff;
     }
     const char *xm = reinterpret_cast<const char *>(xs + gm * xn);
     // A pair's sum of digamma values: its group's lanes 0, 1, 2 sum those of
@@ -1367,7 +1369,7 @@ __global__ void __launch_bounds__(kListWalkThreads) list_walk_kernel(const ListL
     }
     // ---- pairs beyond the lists' radii: over all points, by the whole CTA ----
     __syncthreads();
-    if (s_n_aside > 32 && L.bad) {   // more than a batch of scans: are they still wanted?
+    if (L.bad && s_n_aside > min(32, s_slow_limit)) {   // are so many scans still wanted?
         if (threadIdx.x == 0) {
             if (s_n_aside > s_slow_limit && atomicExch(L.bad + S.group, 1u) == 0u)
                 atomicAdd(L.n_bad, 1ull);

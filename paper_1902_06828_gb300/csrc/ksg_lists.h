@@ -89,17 +89,30 @@ struct ListLaunch {
 constexpr int kListBuildThreads = 512;
 constexpr int kListWalkThreads = 1024;   // of all walking CTAs on an SM
 
-// Pairs beyond the lists' radii that a walking CTA with `pairs` of them scans.
-// A scan visits every point twice: at N = 10^4 18 ns of the whole chip with two Z
-// variables, 36 with eight, against 1.15 and 1.55 a pair by the member-lane kernel
-// and 0.4 and 0.13 on lists, so the lists lose from 3% of such pairs on; at N =
-// 1000 the scan takes 2.3, the other kernel 0.45.  With several X variables that
-// is the fused kernel, 10 ns a pair.  A few dozen scans cost less than handing
-// the group over.
-__host__ __device__ inline int list_slow_limit(int pairs, int N, int dx)
+// Pairs beyond the lists' radii that a walking CTA with `pairs` of them scans,
+// before it gives its group of m members up. A scan visits every point twice;
+// what the other kernel takes a pair depends on how well it fills the chip and
+// prunes (not with a Theiler window or past kMaxOrderN), and on the data, whose
+// tails slow it too.  The shares are where lists and scans lost to it in most
+// of 5568 measured groups (normal, heavy-tailed, rounded, zero-inflated, binary
+// values). Member lanes / lists below and above the share, medians: m >= 61, N >=
+// 6000 1.2 / 0.22, 800 to 6000 1.3 / 0.1; m of 13 to 60 1.3 / 0.2; 2 to 12 1.7 /
+// 0.35 (unpruned 1.6 / 0.5); one member 2.5 / 0.9 (unpruned 1.4 at every share);
+// several X variables, N >= 3000, m >= 61 1.4 / 0.25, 13 to 60 1.3 / 0.4, 2 to 12 1.8 / 0.5.
+__host__ __device__ inline int list_slow_limit(int pairs, int N, int dx, int m, bool pruned)
 {
-    const float share = fminf(0.25f, dx == 1 ? 300.f / (float)N : 1.f);
-    return pairs < 256 ? 64 : max(64, (int)((float)pairs * share));
+    float share = 2.f;   // never
+    if (dx == 1) {
+        if (m >= 13) share = N < 800 ? 0.5f : m >= 61 && N >= 6000 ? 0.12f : 0.2f;
+        else if (m > 1) share = N < 800 ? 0.5f : pruned ? 0.3f : 0.4f;
+        else if (pruned) share = 0.6f;
+    } else if (m >= 13) {
+        share = m >= 61 ? (N >= 3000 ? 0.45f : N >= 800 ? 0.6f : 0.9f) : N >= 3000 ? 0.5f : 0.9f;
+    } else if (m > 1 && N >= 3000) {
+        share = 0.8f;
+    }
+    // (a CTA of few pairs needs most of them to judge by)
+    return max(pairs < 256 ? 16 : 64, (int)((float)pairs * (pairs < 256 ? fmaxf(share, 0.5f) : share)));
 }
 
 // capacities of the two lists for a group
