@@ -68,20 +68,11 @@ bool list_serves(const ListCall &c, int n_groups, long long rows, long long pair
     const bool full = rows >= 24000;   // points of all groups: several waves of CTAs
     if (c.dx == 1 && (c.theiler > 0 || N > kMaxOrderN))
         return true;   // the member lanes cannot prune then
-    if (c.k != 4) return list_serves_other_k(c, n_groups, full);
-    if (c.dx > 1) {
-        if (dz > 1 || m < 8) return true;
-        const bool packed = list_shape(N, c.dx, dz, c.k, c.members).dxp > 0;
-        double most;
-        if (dz == 0)
-            most = m >= 64 ? (packed ? 650 : std::min(290.0, 0.42 * N))
-                           : packed ? 1150 : m >= 24 ? 430 : 700;
-        else if (packed)
-            most = 680;
-        else
-            most = m >= 64 && (c.dx > 2 || (m >= 100 && N < 5000)) ? 0 : 500;
-        return list_depth(c) <= most;
-    }
+    // (a point's X values one by one in shared memory: as with another k)
+    if (c.k != 4 || list_shape(N, c.dx, dz, c.k, c.members).dxp == 0)
+        return list_serves_other_k(c, n_groups, full);
+    if (c.dx > 1)
+        return dz > 1 || m < 8 || list_depth(c) <= (dz == 1 ? 680 : m >= 64 ? 650 : 1150);
     const bool block = m <= 32 || (m >= 48 && m <= 64);   // one well-filled block of members
     if (n_groups >= 200 && m <= 8 && N <= 700 && dz > 0) return false;
     if (N < 250) return true;
@@ -115,7 +106,8 @@ bool list_serves(const ListCall &c, int n_groups, long long rows, long long pair
 // and 9: 1.90 and 1.43; 64 of 5, N = 9990 0.90 and 1.02; 64 of 21, N = 8000, two Z
 // 0.70 and 0.86, three 1.30 and 0.94, five 2.5 and 2.0. Fused / lists: four X,
 // one Z, 201 members, N = 2200, k = 3 and 9 0.67 and 1.47; 21 members 1.24 and 1.89;
-// three X, empty Z, 12 members, N = 2200, 4000, 9000, k = 5 1.92, 1.48, 0.53.
+// three X, empty Z, 12 members, N = 2200, 4000, 9000, k = 5 1.92, 1.48, 0.53; five X,
+// empty Z, k = 4, 29 members, N = 2500 1.46, 201, N = 700 0.75.
 static bool list_serves_other_k(const ListCall &c, int n_groups, bool full)
 {
     const int N = c.N, dz = c.dz, k = c.k;
@@ -124,13 +116,14 @@ static bool list_serves_other_k(const ListCall &c, int n_groups, bool full)
         if (dz == 0)
             return !(full && m >= 4 && m < 16 && N >= 1500 &&
                      k <= (N < 3000 ? 8 : N < 6000 ? 6 : 3));
-        return !(dz == 2 && k > 1 && k <= 9 && full && N >= 3500 && m <= 32 && n_groups >= 8);
+        return !(dz == 2 && k > 1 && k <= 9 && full && N >= 3500 && m >= 4 && m <= 32 &&
+                 n_groups >= 8);
     }
-    if (dz > 1 || m < 8) return true;
+    if (dz > 1 || m < 8 || N < 150) return true;
     const double depth = list_depth(c);
     if (dz == 0) {
-        if (m < 100) return depth * m * N <= 6.5e7;
-        return N <= (c.dx == 2 ? 2500 : 1500) && (c.dx <= 3 || k > 8);
+        if (m <= 100) return depth * m * N <= 6.5e7;
+        return (k == 4 && N < 400) || (N <= (c.dx == 2 ? 2500 : 1500) && (c.dx <= 3 || k > 8));
     }
     if (k > 8) return m >= 48 ? depth <= 860 : depth * N <= 8e6;
     if (m < 48) return depth * N <= 6.5e6;
