@@ -133,10 +133,15 @@ te_status queue_keys(Slot &sl)
     return TE_OK;
 }
 
+// What a batch of several jobs leaves for its lists: filling the budget with
+// jobs sent a saturated server to the member-lane kernel (100 loops on 16 GiB
+// 310,000 estimates/s, 590,000 on lists).
+size_t list_reserve(const te_server *S) { return std::min(kListPoolBytes, S->budget / 4); }
+
 // Lists for the slot's batch, whose jobs are admitted (in_use counts them): an
-// equal share of what the budget has left for each slot that is idle, at most
-// kListPoolBytes; without one the batch takes the member-lane kernel, which
-// the jobs' footprints pay for.  The lists that idle slots keep are given back
+// equal share of what the budget has left for each slot that is idle, but the
+// reserve if it can be had, at most kListPoolBytes; without one the batch takes
+// the member-lane kernel, which the jobs' footprints pay for.  The lists that idle slots keep are given back
 // where they would pass the budget.  Called with the lock held.
 void list_room(te_server *S, Slot &sl)
 {
@@ -149,7 +154,9 @@ void list_room(te_server *S, Slot &sl)
     }
     for (const ServeJob *j : sl.jobs) tables += list_tables(j->N, j->S);
     const size_t left = S->budget - S->in_use - busy;
-    const size_t share = std::min(left / idle, kListPoolBytes + tables);
+    const size_t share =
+        std::min(left, std::min(std::max(left / idle, list_reserve(S) + tables),
+                                kListPoolBytes + tables));
     sl.ctx->list_pool = share > tables ? (share - tables) & ~(size_t)255 : 0;
     for (Slot &o : S->slots)
         o.give_back = !o.busy && &o != &sl && o.lists && kept + share > left;
@@ -283,11 +290,13 @@ void serve_loop(te_server *S)
         for (Slot &sl : S->slots) {
             if (sl.busy) continue;
             std::vector<ServeJob *> batch;
-            size_t fp = 0, held = S->in_use;   // by the other batches
+            size_t fp = 0, tables = 0, held = S->in_use;   // held: by the other batches
             for (const Slot &o : S->slots) held += o.busy ? o.lists : 0;
             while (!S->pending.empty() && (int)batch.size() < S->max_batch) {
                 ServeJob *j = S->pending.front();
-                if (held + fp + j->fp > S->budget) break;
+                tables += list_tables(j->N, j->S);
+                const size_t lists = batch.empty() ? 0 : list_reserve(S) + tables;
+                if (held + fp + j->fp + lists > S->budget) break;
                 S->pending.pop_front();
                 fp += j->fp;
                 j->state = JS_RUNNING;
