@@ -36,7 +36,11 @@ sys.path.insert(0, ROOT)
 
 METRIC = "KSG CMI estimates/s incl. surrogates at T=10000"
 UNIT = "estimates/s"
-TRAFFIC_PER_MEMBER_POINT = 3453012224.0 / (9045 * 9995)
+# DRAM bytes (read + write) of list builds and walks per member and point at T = 10^4, from
+# counters (profiles/list_walk_kernel_*): 17,889 members of coupled maps with eight Z variables
+# (their lists stay in L2), 9045 members of a VAR with two (lists of up to 50 KB a point)
+TRAFFIC_PER_MEMBER_POINT = {"clm100": 235681792.0 / (17889 * 9995),
+                            "var10": 3453012224.0 / (9045 * 9995)}
 
 
 def _peaks():
@@ -653,12 +657,14 @@ def main():
     sm_count = torch.cuda.get_device_properties(local).multi_processor_count
     peak = sm_count * 128 * sm_max * 1e6 / 1e12
     # DRAM traffic of the KSG kernels per launch pair (lists built, then walked):
-    # the ncu capture of the same kernels (profiles/list_walk_kernel_*) by
-    # member-point; scaled here by the member-points one launch processes.
+    # counters of the same kernels on one batch (profiles/list_walk_kernel_*) by
+    # member-point; scaled here by the member-points one launch processes: an
+    # estimate, no measurement of these launches, whose Z variables differ.
     # Algorithmic bytes: 4 N per member (its X values) + 16 (key).
     n_pts = args.T - 5
     mp_per_launch = (n_est / world) * n_pts / max(ksg_launches, 1)   # this rank's launches
-    traffic = TRAFFIC_PER_MEMBER_POINT * mp_per_launch if ksg_launches else None
+    per_mp = TRAFFIC_PER_MEMBER_POINT.get(args.workload)
+    traffic = per_mp * mp_per_launch if ksg_launches and per_mp and args.T == 10000 else None
     alg_bytes = (4.0 * n_pts + 16.0) * (n_est / world) / max(ksg_launches, 1)
     value = n_est / (ms / 1e3)
     # measured ceiling of the counted instruction mix (te_alu_peak, after the
@@ -689,8 +695,9 @@ def main():
         "gpu_launches": s1["launches"] - s0["launches"],
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s",
                      "frac": (achieved / peak) if achieved else None, "traffic": traffic,
-                     "traffic_note": "dram read+write bytes per launch, scaled from the ncu "
-                                     "capture of these kernels at T=10000 by member-points",
+                     "traffic_note": "dram read+write bytes per launch, estimated: counters of "
+                                     "one batch of this kind of data at T=10000, scaled by "
+                                     "member-points",
                      "algorithmic_bytes_per_launch": alg_bytes,
                      "kernel": "list_build_kernel + list_walk_kernel", "kernel_ms_per_launch":
                      kernel_ms / max(ksg_launches, 1), "launches": ksg_launches,
@@ -705,8 +712,9 @@ def main():
                                        "note": "te_alu_peak: each pass's counted instruction "
                                                "pattern from registers at full occupancy, this "
                                                "run; the mix weights them by this run's ops"},
-                     "work": "3 ops per list entry evaluated for a member (member-lane kernel: 3 per "
-                             "kNN-pass member-pair, 7 per count-pass one)",
+                     "work": "3 ops per list entry evaluated for a member (member-lane kernel and scans "
+                             "over all points: 3 per kNN-pass member-pair, 7 per count-pass one); "
+                             "list builds and binary searches not counted",
                      "pair_evals_executed": pair_evals, "pair_evals_bruteforce": pair_evals_bf,
                      "pruned_fraction": (1.0 - pair_evals / pair_evals_bf) if pair_evals_bf
                      else None},

@@ -1030,8 +1030,9 @@ __global__ void __launch_bounds__(256) gauss_turn_kernel(const PermTurnJob *jobs
 // turned permutations, so that a warp's 32 gathers cost their bank conflicts
 // (about 7 cycles of 8-byte loads) and its 32 indices one line, where gathers
 // through L1 took a cycle per row each for the indices and the values (64
-// cycles a point, against 12 of arithmetic at dw = 4).  319 estimates of 201
-// rows, dw = 4, N = 9995: 3.1 -> 1.5 ms, the FMA pipe 58% and issue 73% busy.
+// cycles a point, against 12 of arithmetic at dw = 4).  All launches of a
+// 10-node network (N = 9995, 201 rows an estimate): 22.1 -> 9.5 ms; issue 56 to 69%
+// and the shared-memory pipe 59 to 74% busy.
 // smem: N float2
 //
 // The CTA's H parts of `rows` threads take consecutive splits of the points

@@ -157,8 +157,8 @@ extern "C" te_status cmi_ksg_static(const float *series_dev, int32_t n_proc, int
     // Neighbour lists (as the context path) where the scratch beyond the seven
     // parts holds the lists of at least a 64th of the points (the tables and
     // sorted columns lie before them); else the member-lane kernel, which
-    // needs no more.  A call of 201 members at T = 1000: 426 us with the
-    // member-lane kernel, 167 with lists.
+    // needs no more.  A call of 201 members at T = 1000: 445 us with the
+    // member-lane kernel, 165 with lists.
     const ListShape shape = list_shape(N, dx, dz, p->k, (size_t)S + 1);
     ListGroup lg{};
     list_caps(N, p->k, dx, dy, dz, &lg.cap_a, &lg.cap_b);
