@@ -426,24 +426,26 @@ te_status launch_groups(te_ctx *ctx, const std::vector<HostGroup> &groups, int n
         int n_groups = 0;
         long long rows = 0, pairs = 0;
     };
-    Sums all;
-    std::map<std::pair<bool, size_t>, Sums> like;   // one X variable, Z variables
-    for (const HostGroup &g : groups) {
+    auto add = [](Sums &s, const HostGroup &g) {
+        if (g.members.empty()) return;
         const long long N = g.data->T - g.max_lag;
-        if (g.members.empty()) continue;
-        for (Sums *s : {&all, &like[{g.dx == 1, g.z.size()}]}) {
-            s->n_groups++;
-            s->rows += N;
-            s->pairs += N * (long long)g.members.size();
-        }
-    }
+        s.n_groups++;
+        s.rows += N;
+        s.pairs += N * (long long)g.members.size();
+    };
+    Sums all;
+    for (const HostGroup &g : groups) add(all, g);
+    std::map<std::pair<bool, size_t>, Sums> like;   // one X variable, Z variables
+    const bool small = all.n_groups > 1 && all.pairs < 1000000;
+    if (small)
+        for (const HostGroup &g : groups) add(like[{g.dx == 1, g.z.size()}], g);
     std::vector<const HostGroup *> by_lists, by_lanes;
     size_t list_need = 0;
     for (const HostGroup &g : groups) {
         if (g.members.empty()) continue;
         const ListCall c{g.data->T - g.max_lag, g.k, g.theiler, g.dx, (int)g.y.size(),
                          (int)g.z.size(), g.members.size()};
-        const Sums &s = all.pairs < 1000000 ? like[{g.dx == 1, g.z.size()}] : all;
+        const Sums &s = small ? like[{g.dx == 1, g.z.size()}] : all;
         const bool lists = !lane_only && (ctx->opt_lists ? list_fits(c.N, c.dx, c.dz, c.k)
                                                          : list_serves(c, s.n_groups, s.rows, s.pairs));
         (lists ? by_lists : by_lanes).push_back(&g);
